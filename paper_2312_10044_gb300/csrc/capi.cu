@@ -96,11 +96,12 @@ __device__ __forceinline__ uint32_t dev_bits(float v) { return __float_as_uint(v
 // Charge records (y - centre, q) of n_rhs configurations from device arrays,
 // with the checks bipb_charges_set makes on the host: every value finite, and
 // no charge on a centroid (the centroid with the same FP32 point, found in the
-// surface's hash table, compared in FP64).  A failed check sets *err.
+// surface's hash table, compared in FP64).  A failed check sets *err.  The
+// largest coordinate of a configuration goes into its chg_tab entry.
 __global__ void k_charges_dev(int64_t nc, int n_rhs, int n_pos_sets, const double* __restrict__ pos,
                               const double* __restrict__ q, double cx, double cy, double cz,
                               const int32_t* __restrict__ slot, uint64_t mask, const double4_32a* __restrict__ tgt64,
-                              double4_32a* __restrict__ rec, int* __restrict__ err) {
+                              double4_32a* __restrict__ rec, int4* __restrict__ chg_tab, int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nc * n_rhs) return;
   const int64_t r = i / nc, k = i % nc;
@@ -123,6 +124,8 @@ __global__ void k_charges_dev(int64_t nc, int n_rhs, int n_pos_sets, const doubl
     }
   }
   if (!ok) atomicOr(err, 1);
+  const int far = __float_as_int(__double2float_ru(fmax(fabs(p0), fmax(fabs(p1), fabs(p2)))));
+  if (ok && far > chg_tab[r].z) atomicMax(&chg_tab[r].z, far);
   rec[i] = make_double4_32a(p0, p1, p2, qq);
 }
 
@@ -219,7 +222,7 @@ struct PartIn {
 void add_part(Surface* s, const PartIn& P, std::vector<double4_32a>& tgt, std::vector<float4>& tgt32) {
   BIPB_REQUIRE(P.n >= 2, "need at least 2 triangles per surface");
   BIPB_REQUIRE(P.c && P.nrm && P.area, "NULL input array");
-  double c[3] = {0, 0, 0};
+  double c[3] = {0, 0, 0}, lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   std::vector<double> inv_len((size_t)P.n);
   for (int64_t i = 0; i < P.n; ++i) {
     BIPB_REQUIRE(finite3(P.c + 3 * i), "non-finite centroid");
@@ -229,9 +232,21 @@ void add_part(Surface* s, const PartIn& P, std::vector<double4_32a>& tgt, std::v
     double len = std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
     BIPB_REQUIRE(std::fabs(len - 1.0) <= 1e-6, "normals must have unit length (within 1e-6)");
     inv_len[i] = 1.0 / len;
-    for (int k = 0; k < 3; ++k) c[k] += P.c[3 * i + k];
+    for (int k = 0; k < 3; ++k) {
+      const double x = P.c[3 * i + k];
+      c[k] += x;
+      lo[k] = x < lo[k] ? x : lo[k];
+      hi[k] = x > hi[k] ? x : hi[k];
+    }
   }
   for (int k = 0; k < 3; ++k) c[k] /= (double)P.n;
+  // largest centred coordinate, and the grid of the df64 coordinates (df_pos):
+  // 2^-23 of the power of two above it
+  double far = 0.0;
+  for (int k = 0; k < 3; ++k) far = std::max(far, std::max(std::fabs(lo[k] - c[k]), std::fabs(hi[k] - c[k])));
+  int far_exp = 0;
+  std::frexp(far, &far_exp);
+  const double grid = std::ldexp(1.0, far_exp - 23);
   // centred copies (FP64 and FP32 records), and the check for duplicates (in
   // FP32, then FP64 on a hit); the set is kept to reject charges on a centroid
   CentroidSet cs;
@@ -257,13 +272,14 @@ void add_part(Surface* s, const PartIn& P, std::vector<double4_32a>& tgt, std::v
     const double* v = P.nrm + 3 * i;
     const double nx = v[0] * inv_len[i], ny = v[1] * inv_len[i], nz = v[2] * inv_len[i];
     tgt[base + 2 * i] = make_double4_32a(d[0], d[1], d[2], P.area[i]);
-    tgt[base + 2 * i + 1] = make_double4_32a(nx, ny, nz, 0.0);
+    tgt[base + 2 * i + 1] = make_double4_32a(nx, ny, nz, grid);
     tgt32[base + 2 * i] = make_float4(f[0], f[1], f[2], (float)P.area[i]);
     tgt32[base + 2 * i + 1] = make_float4((float)nx, (float)ny, (float)nz, 0.f);
   }
   s->part_off.push_back((int)s->n);
   s->part_n.push_back((int)P.n);
   for (int k = 0; k < 3; ++k) s->part_center.push_back(c[k]);
+  s->part_far.push_back(far);
   s->part_keys.push_back(std::move(cs));
   s->n += P.n;
 }
@@ -335,8 +351,10 @@ bipb_surface create_surface(const std::vector<PartIn>& parts, void* cuda_stream,
 
 // Charge records of one system, centred like its surface; rejects charges on
 // a centroid (lookup in the surface's set of centred centroids).
-void append_charges(Surface* s, int part, int64_t nc, const double* pos, const double* q,
-                    std::vector<double4_32a>& rec) {
+// Returns the largest coordinate of the surface and these charges.
+double append_charges(Surface* s, int part, int64_t nc, const double* pos, const double* q,
+                      std::vector<double4_32a>& rec) {
+  double far = s->part_far[part];
   const double* c = &s->part_center[3 * part];
   const auto& keys = s->part_keys[part];
   for (int64_t k = 0; k < nc; ++k) {
@@ -348,11 +366,23 @@ void append_charges(Surface* s, int part, int64_t nc, const double* pos, const d
     BIPB_REQUIRE(j < 0 || !(keys.d[3 * j] == p[0] && keys.d[3 * j + 1] == p[1] && keys.d[3 * j + 2] == p[2]),
                  "a charge sits on a centroid");
     rec.push_back(make_double4_32a(p[0], p[1], p[2], q[k]));
+    for (int a = 0; a < 3; ++a) far = std::max(far, std::fabs(p[a]));
   }
+  return far;
 }
 
-void store_charges(Surface* s, const std::vector<double4_32a>& rec, SysLayout lay) {
+// The per-system table of the charge passes.
+std::vector<int4> charge_table(const SysLayout& lay, const std::vector<double>& far) {
+  std::vector<int4> tab(lay.K);
+  for (int k = 0; k < lay.K; ++k) tab[k] = make_int4(lay.chg_off[k], lay.nc[k], far_bits(far[k]), 0);
+  return tab;
+}
+
+void store_charges(Surface* s, const std::vector<double4_32a>& rec, const std::vector<double>& far, SysLayout lay) {
+  const std::vector<int4> tab = charge_table(lay, far);
   s->grow(s->chg, rec.size());
+  s->grow(s->chg_tab, tab.size());
+  BIPB_CUDA(cudaMemcpyAsync(s->chg_tab.p, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
   BIPB_CUDA(cudaMemcpyAsync(s->chg.p, rec.data(), rec.size() * sizeof(double4_32a), cudaMemcpyHostToDevice,
                             s->stream));
   BIPB_CUDA(cudaStreamSynchronize(s->stream));
@@ -455,14 +485,15 @@ bipb_status bipb_charges_set(bipb_surface h, int64_t nc, const double* pos, int 
     DeviceGuard dg(s->device);
     std::vector<double4_32a> rec;
     rec.reserve((size_t)n_rhs * nc);
+    std::vector<double> far(n_rhs);
     std::vector<int> go(n_rhs, 0), n(n_rhs, (int)s->n), co(n_rhs), ncv(n_rhs, (int)nc);
     for (int r = 0; r < n_rhs; ++r) {
       co[r] = (int)(r * nc);
-      append_charges(s, 0, nc, pos + (size_t)(n_pos_sets == 1 ? 0 : r) * nc * 3, q + (size_t)r * nc, rec);
+      far[r] = append_charges(s, 0, nc, pos + (size_t)(n_pos_sets == 1 ? 0 : r) * nc * 3, q + (size_t)r * nc, rec);
     }
     s->nc = nc;
     s->n_pos_sets = n_pos_sets;
-    store_charges(s, rec, make_layout(go, n, co, ncv));
+    store_charges(s, rec, far, make_layout(go, n, co, ncv));
   });
 }
 
@@ -489,16 +520,21 @@ bipb_status bipb_charges_set_dev(bipb_surface h, int64_t nc, const double* pos, 
     const int64_t total = (int64_t)n_rhs * nc;
     s->grow(s->chg, (size_t)total);
     BIPB_CUDA(cudaMemsetAsync(s->chg_err.p, 0, sizeof(int), s->stream));
+    std::vector<int> go(n_rhs, 0), n(n_rhs, (int)s->n), co(n_rhs), ncv(n_rhs, (int)nc);
+    for (int r = 0; r < n_rhs; ++r) co[r] = (int)(r * nc);
+    SysLayout lay = make_layout(go, n, co, ncv);
+    const std::vector<int4> tab = charge_table(lay, std::vector<double>(n_rhs, s->part_far[0]));
+    s->grow(s->chg_tab, tab.size());
+    // pageable source: the copy has read it when the call returns
+    BIPB_CUDA(cudaMemcpyAsync(s->chg_tab.p, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
     const double* c = &s->part_center[0];
     k_charges_dev<<<(unsigned)((total + 255) / 256), 256, 0, s->stream>>>(
         nc, n_rhs, n_pos_sets, pos, q, c[0], c[1], c[2], s->key_slots.p, keys.mask, s->tgt64.p, s->chg.p,
-        s->chg_err.p);
+        s->chg_tab.p, s->chg_err.p);
     BIPB_LAUNCHED(s);
-    std::vector<int> go(n_rhs, 0), n(n_rhs, (int)s->n), co(n_rhs), ncv(n_rhs, (int)nc);
-    for (int r = 0; r < n_rhs; ++r) co[r] = (int)(r * nc);
     s->nc = nc;
     s->n_pos_sets = n_pos_sets;
-    s->lay = make_layout(go, n, co, ncv);
+    s->lay = std::move(lay);
     s->n_rhs = s->lay.K;
     s->have_solution = false;
     s->chg_check_pending = true;
@@ -515,17 +551,18 @@ bipb_status bipb_charges_set_batch(bipb_surface h, const int64_t* nc, const doub
     DeviceGuard dg(s->device);
     std::vector<double4_32a> rec;
     std::vector<int> co(K), ncv(K);
+    std::vector<double> far(K);
     for (int k = 0; k < K; ++k) {
       BIPB_REQUIRE(nc[k] >= 1 && nc[k] <= (int64_t)1 << 26, "every surface needs 1 .. 2^26 charges");
       BIPB_REQUIRE(pos[k] && q[k], "NULL charge array");
       co[k] = (int)rec.size();
       ncv[k] = (int)nc[k];
-      append_charges(s, k, nc[k], pos[k], q[k], rec);
+      far[k] = append_charges(s, k, nc[k], pos[k], q[k], rec);
       BIPB_REQUIRE(rec.size() <= ((size_t)1 << 28), "too many charges in total");
     }
     s->nc = 0;
     s->n_pos_sets = 0;
-    store_charges(s, rec, make_layout(s->part_off, s->part_n, co, ncv));
+    store_charges(s, rec, far, make_layout(s->part_off, s->part_n, co, ncv));
   });
 }
 
@@ -680,11 +717,13 @@ bipb_status bipb_potential_at(bipb_surface h, int region, int64_t n_pts, const d
     // the points in the frame of the surface's centred copies
     const double* c = &s->part_center[0];
     std::vector<double4_32a> p1((size_t)n_pts), p2((size_t)2 * n_pts);
+    double far = 0.0;
     for (int64_t i = 0; i < n_pts; ++i) {
       double d[3];
       for (int k = 0; k < 3; ++k) {
         BIPB_REQUIRE(std::isfinite(pts[3 * i + k]), "non-finite point");
         d[k] = pts[3 * i + k] - c[k];
+        far = std::max(far, std::fabs(d[k]));
       }
       p1[i] = double4_32a{d[0], d[1], d[2], 0.0};
       p2[2 * i] = p1[i];
@@ -700,7 +739,7 @@ bipb_status bipb_potential_at(bipb_surface h, int region, int64_t n_pts, const d
     BIPB_CUDA(cudaMemcpyAsync(s->pts2.p, p2.data(), p2.size() * sizeof(double4_32a), cudaMemcpyHostToDevice,
                               s->stream));
     potential_pass(s, L, s->solved_medium, s->u.p, region == BIPB_REGION_INSIDE, (int)n_pts, s->pts.p, s->pts2.p,
-                   s->pot.p);
+                   far, s->pot.p);
     BIPB_CUDA(cudaMemcpyAsync(phi, s->pot.p, (size_t)L.K * n_pts * sizeof(double), cudaMemcpyDeviceToHost,
                               s->stream));
     BIPB_CUDA(cudaStreamSynchronize(s->stream));

@@ -9,6 +9,7 @@
 #include <stdexcept>
 #include <string>
 #include <array>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -292,7 +293,7 @@ struct Surface {
 
   // Geometry of every element, each surface relative to its own mean
   // centroid (part_center), so that the FP32 copies keep the most digits.
-  DevBuf<double4_32a> tgt64;  // 2n: (x, y, z, area), (nx, ny, nz, 0)
+  DevBuf<double4_32a> tgt64;  // 2n: (x, y, z, area), (nx, ny, nz, coordinate grid of the surface: df_pos)
   DevBuf<float4> tgt32;   // the same in FP32
   DevBuf<float4> exptab;  // 2^(j/1024), j < 1024, as df64 (hi, lo) pairs: the df64 exp table
 
@@ -332,7 +333,10 @@ struct Surface {
   int n_rhs = 0;   // configurations (systems)
   int n_pos_sets = 0;
   DevBuf<double4_32a> chg;
-  DevBuf<float4> chgdf;  // the charges as df64 records (2 float4 each), packed by the source pass
+  DevBuf<float4> chgdf;  // the charges as df64 records (3 float4 each), packed by the source pass
+  // per system {chg_off, nc, far, 0}: far = FP32 bits (rounded up) of the largest coordinate
+  // of its surface and charges, which sets the coordinate grid of its df64 charge passes
+  DevBuf<int4> chg_tab;
   // charges passed on the device (bipb_charges_set_dev): the centroid hash
   // table on the device for the on-centroid check, and the check's flag,
   // read by the next call that uses the charges
@@ -345,6 +349,7 @@ struct Surface {
   // batch handle, one system each): element offsets, sizes, centres
   std::vector<int> part_off, part_n;
   std::vector<double> part_center;  // 3 per surface
+  std::vector<double> part_far;     // largest centred coordinate of each surface
   std::vector<CentroidSet> part_keys;  // the centred centroids of every surface
   std::vector<double> raw_centroids;   // single-surface handles: the centroids as given (tree of the far field)
   bool batch = false;
@@ -458,9 +463,17 @@ void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const d
 // Potential at n_pts points (device records: pts one (p, 0) per point, pts2 two,
 // (p, 0) and a zero normal) for every system, internal units, into out[k n_pts + q]:
 // Eq. eq_inside when inside (with S1 of the system's charges), else the
-// exterior representation (Eq. eqbim_2).
+// exterior representation (Eq. eqbim_2).  far_pts: the points' largest coordinate.
 void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
-                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double* out);
+                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out);
+// FP32 bits of |x| rounded up (ordered like the values)
+inline int far_bits(double x) {
+  float f = (float)x;
+  if ((double)f < x) f = std::nextafterf(f, INFINITY);
+  int b;
+  std::memcpy(&b, &f, 4);
+  return b;
+}
 // part[k * blocks + b]: block sums of sum_{c != l} q_c q_l / |y_c - y_l| of system k;
 // tab[k] = {0, 0, nc, chg_off}.
 void coulomb_pass(Surface* s, const SysLayout& L, const int4* tab, double* part, int* blocks);

@@ -55,6 +55,7 @@ struct MatvecPolicy {
   using V4 = typename V4T<T>::type;
   static constexpr int RW = 2;
   static constexpr int NOUT = 2;
+  static constexpr bool CHUNKED = false;
   static constexpr bool SELF = true;
   template <class A>
   __device__ static void prologue(const A&) {}
@@ -67,12 +68,12 @@ struct MatvecPolicy {
     T* part;
     PairConst<T> c;
   };
-  __device__ static void load(const Args& a, int i, Tgt& t) {
+  __device__ static void load(const Args& a, int i, int, Tgt& t) {
     V4 g = a.tgt[2 * i], v = a.tgt[2 * i + 1];
     t = Tgt{g.x, g.y, g.z, v.x, v.y, v.z};
   }
   __device__ static void zero(Acc& acc) { acc.p = T(0), acc.q = T(0); }
-  __device__ static void renorm(Acc&) {}
+  __device__ static void flush(Acc&, const Acc&) {}
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const V4* r, bool self, Acc& acc) {
     const V4 A = r[0], B = r[1];
@@ -89,6 +90,31 @@ struct MatvecPolicy {
   }
 };
 
+// Coordinate grid (df_pos) of system sys of a charge pass: 2^-23 of the power
+// of two above the largest coordinate of its surface, charges and (extra, FP32
+// bits) points.
+__device__ __forceinline__ double charge_grid(const int4* __restrict__ chg_tab, int sys, int extra) {
+  const int b = max(chg_tab[sys].z, extra);
+  return __longlong_as_double((long long)((b >> 23) - 127 + 1 - 23 + 1023) << 52);
+}
+// the element target of the charge passes: position on the grid and normal
+struct ElemTgtDF {
+  df_pos x[3];
+  df n[3];
+};
+__device__ __forceinline__ void load_elem_df(const double4_32a* __restrict__ tgt, int i, double grid, ElemTgtDF& t) {
+  const double4_32a g = tgt[2 * i], v = tgt[2 * i + 1];
+  t.x[0] = df_split_grid(g.x, grid), t.x[1] = df_split_grid(g.y, grid), t.x[2] = df_split_grid(g.z, grid);
+  t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
+}
+struct PointTgtDF {
+  df_pos y[3];
+};
+__device__ __forceinline__ void load_point_df(const double4_32a* __restrict__ pts, int k, double grid, PointTgtDF& t) {
+  const double4_32a g = pts[k];
+  t.y[0] = df_split_grid(g.x, grid), t.y[1] = df_split_grid(g.y, grid), t.y[2] = df_split_grid(g.z, grid);
+}
+
 // Mat-vec in double-float arithmetic (df64.cuh).  Record per source, 4 float4:
 // (x.hi, a.hi), (x.lo, a.lo), (m.hi, 0), (m.lo, 0) with a = ds psi and
 // m = ds phi n (forward) or a = wphi, m = wpsi n (transposed).
@@ -101,6 +127,7 @@ template <bool TRANS>
 struct MatvecDFPolicy {
   static constexpr int RW = 4;
   static constexpr int NOUT = 2;
+  static constexpr bool CHUNKED = true;
   static constexpr bool SELF = true;
   struct Tgt {
     df x[3], n[3];
@@ -116,13 +143,16 @@ struct MatvecDFPolicy {
   __device__ static void prologue(const Args& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
-  __device__ static void load(const Args& a, int i, Tgt& t) {
+  __device__ static void load(const Args& a, int i, int, Tgt& t) {
     double4_32a g = a.tgt[2 * i], v = a.tgt[2 * i + 1];
     t.x[0] = df_from_double(g.x), t.x[1] = df_from_double(g.y), t.x[2] = df_from_double(g.z);
     t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
   }
   __device__ static void zero(Acc& acc) { acc.p = df{0.f, 0.f}, acc.q = df{0.f, 0.f}; }
-  __device__ static void renorm(Acc&) {}
+  __device__ static void flush(Acc& sum, const Acc& acc) {
+    sum.p = df_add(sum.p, acc.p);
+    sum.q = df_add(sum.q, acc.q);
+  }
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool self, Acc& acc) {
     const float4 A = r[0], B = r[1], C = r[2], D = r[3];
@@ -141,37 +171,39 @@ struct MatvecDFPolicy {
 };
 
 // Source term in df64: target element i, source charge k with df record
-// (y_k.hi, q_k.hi), (y_k.lo, q_k.lo), d = x_i - y_k:
+// (y_k.h, q_k.hi), (y_k.l, q_k.lo), (y_k.m, 0), d = x_i - y_k:
 //   4 pi eps_in S1 += q s,   4 pi eps_in S2 += -q (n_i.d) s^3   (d/dnu_x = +n_x.grad_x)
 // GB300 executes FP64 at 1/64 of the FP32 rate; df64 keeps b accurate to
 // about 1e-14 relative at a fraction of the FP64 cost.
 struct SourcePolicy {
-  static constexpr int RW = 2;
+  static constexpr int RW = 3;
   static constexpr int NOUT = 2;
+  static constexpr bool CHUNKED = true;
   static constexpr bool SELF = false;
   template <class A>
   __device__ static void prologue(const A&) {}
-  struct Tgt {
-    df x[3], n[3];
-  };
+  using Tgt = ElemTgtDF;
   struct Acc {
     df s1, s2;
   };
   struct Args {
     const double4_32a* tgt;  // 2 per element
     double* part;
+    const int4* chg_tab;
+    int extra;  // FP32 bits of the largest coordinate of the targets, 0 for the surface's own elements
   };
-  __device__ static void load(const Args& a, int i, Tgt& t) {
-    double4_32a g = a.tgt[2 * i], v = a.tgt[2 * i + 1];
-    t.x[0] = df_from_double(g.x), t.x[1] = df_from_double(g.y), t.x[2] = df_from_double(g.z);
-    t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
+  __device__ static void load(const Args& a, int i, int sys, Tgt& t) {
+    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) { acc.s1 = df{0.f, 0.f}, acc.s2 = df{0.f, 0.f}; }
-  __device__ static void renorm(Acc&) {}
+  __device__ static void flush(Acc& sum, const Acc& acc) {
+    sum.s1 = df_add(sum.s1, acc.s1);
+    sum.s2 = df_add(sum.s2, acc.s2);
+  }
   template <bool MASK>
   __device__ static void pair(const Args&, const Tgt& t, const float4* r, bool, Acc& acc) {
-    const float4 A = r[0], B = r[1];
-    const df y[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
+    const float4 A = r[0], B = r[1], C = r[2];
+    const df_pos y[3] = {df_pos{A.x, B.x, C.x}, df_pos{A.y, B.y, C.y}, df_pos{A.z, B.z, C.z}};
     df_source_pair(t.x, t.n, y, df{A.w, B.w}, acc.s1, acc.s2);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int i, const Acc& acc) {
@@ -180,16 +212,15 @@ struct SourcePolicy {
   }
 };
 
-// Reaction potential at a charge y_k from the surface in df64 (forward df
-// record (x_j, a_j = ds psi_j), m_j = ds phi_j n_j), d = y_k - x_j:
-//   4 pi phi_reac += s [ (1 - e) a_j + (eps t - 1) (m_j.d) s^2 ]  (K1 psi + K2 phi, n_j only)
+// Reaction potential at a charge y_k from the surface in df64 (df record of
+// k_pack_df<true>: x_j, a_j = ds psi_j, n_j, alpha_j = ds phi_j), d = y_k - x_j:
+//   4 pi phi_reac += s [ (1 - e) a_j + (eps t - 1) alpha_j (n_j.d) s^2 ]  (K1 psi + K2 phi, n_j only)
 struct ReactionPolicy {
-  static constexpr int RW = 4;
+  static constexpr int RW = 5;
   static constexpr int NOUT = 1;
+  static constexpr bool CHUNKED = true;
   static constexpr bool SELF = false;
-  struct Tgt {
-    df y[3];
-  };
+  using Tgt = PointTgtDF;
   struct Acc {
     df p;
   };
@@ -197,23 +228,24 @@ struct ReactionPolicy {
     const double4_32a* pts;  // (y, q)
     double* part;
     DFConst c;
+    const int4* chg_tab;
+    int extra;  // FP32 bits of the points' largest coordinate, 0 for the charges themselves
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
-  __device__ static void load(const Args& a, int k, Tgt& t) {
-    double4_32a g = a.pts[k];
-    t.y[0] = df_from_double(g.x), t.y[1] = df_from_double(g.y), t.y[2] = df_from_double(g.z);
+  __device__ static void load(const Args& a, int k, int sys, Tgt& t) {
+    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) { acc.p = df{0.f, 0.f}; }
-  __device__ static void renorm(Acc&) {}
+  __device__ static void flush(Acc& sum, const Acc& acc) { sum.p = df_add(sum.p, acc.p); }
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
-    const float4 A = r[0], B = r[1], C = r[2], D = r[3];
-    const df xs[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
-    const df m[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_reaction_pair(t.y, xs, df{A.w, B.w}, m, a.c, df_exp_table(), acc.p);
+    const float4 A = r[0], B = r[1], C = r[2], D = r[3], M = r[4];
+    const df_pos xs[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
+    const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
+    df_reaction_pair(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
   }
   __device__ static void store(const Args& a, int out, int, int k, const Acc& acc) {
     a.part[(size_t)out + k] = df_to_double(acc.p);
@@ -221,15 +253,15 @@ struct ReactionPolicy {
 };
 
 // Potential at a point y in the solvent from the surface in df64 (the same
-// forward df record as the reaction pass), the exterior representation:
-//   4 pi phi(y) += s [ t (m_j.d) s^2 - (1/eps) e a_j ],  d = y - x_j
+// df record as the reaction pass), the exterior representation:
+//   4 pi phi(y) += s [ t alpha_j (n_j.d) s^2 - (1/eps) e a_j ],  d = y - x_j
 struct ExteriorPolicy : ReactionPolicy {
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
-    const float4 A = r[0], B = r[1], C = r[2], D = r[3];
-    const df xs[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
-    const df m[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_exterior_pair(t.y, xs, df{A.w, B.w}, m, a.c, df_exp_table(), acc.p);
+    const float4 A = r[0], B = r[1], C = r[2], D = r[3], M = r[4];
+    const df_pos xs[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
+    const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
+    df_exterior_pair(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
   }
 };
 
@@ -237,12 +269,11 @@ struct ExteriorPolicy : ReactionPolicy {
 // (y_k, q_k)), d = y_k - x_j:
 //   4 pi K2(y_k, x_j) = (eps t - 1) (n_j.d) s^3,  4 pi K1(y_k, x_j) = (1 - e) s
 struct EnergyRowPolicy {
-  static constexpr int RW = 2;
+  static constexpr int RW = 3;
   static constexpr int NOUT = 2;
+  static constexpr bool CHUNKED = true;
   static constexpr bool SELF = false;
-  struct Tgt {
-    df x[3], n[3];
-  };
+  using Tgt = ElemTgtDF;
   struct Acc {
     df cphi, cpsi;
   };
@@ -250,25 +281,24 @@ struct EnergyRowPolicy {
     const double4_32a* tgt;
     double* part;
     DFConst c;
+    const int4* chg_tab;
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
-  __device__ static void load(const Args& a, int i, Tgt& t) {
-    double4_32a g = a.tgt[2 * i], v = a.tgt[2 * i + 1];
-    t.x[0] = df_from_double(g.x), t.x[1] = df_from_double(g.y), t.x[2] = df_from_double(g.z);
-    t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
+  __device__ static void load(const Args& a, int i, int sys, Tgt& t) {
+    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, 0), t);
   }
   __device__ static void zero(Acc& acc) { acc.cphi = df{0.f, 0.f}, acc.cpsi = df{0.f, 0.f}; }
-  __device__ static void renorm(Acc& acc) {
-    acc.cphi = two_sum(acc.cphi.hi, acc.cphi.lo);
-    acc.cpsi = two_sum(acc.cpsi.hi, acc.cpsi.lo);
+  __device__ static void flush(Acc& sum, const Acc& acc) {
+    sum.cphi = df_add(sum.cphi, acc.cphi);
+    sum.cpsi = df_add(sum.cpsi, acc.cpsi);
   }
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
-    const float4 A = r[0], B = r[1];
-    const df y[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
+    const float4 A = r[0], B = r[1], C = r[2];
+    const df_pos y[3] = {df_pos{A.x, B.x, C.x}, df_pos{A.y, B.y, C.y}, df_pos{A.z, B.z, C.z}};
     df_energy_row_pair(t.x, t.n, y, df{A.w, B.w}, a.c, df_exp_table(), acc.cphi, acc.cpsi);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int i, const Acc& acc) {
@@ -278,17 +308,16 @@ struct EnergyRowPolicy {
 };
 
 // Energy gradient at charge y_k in df64 (df_grad_pair in df64.cuh).  Record
-// per element j, 5 float4: (x.hi, a.hi), (x.lo, a.lo), (n.hi, alpha.hi),
-// (n.lo, alpha.lo), (lphi.hi, lphi.lo, beta.hi, beta.lo) with a = ds psi,
-// alpha = ds phi and the adjoint lam = [lphi; beta].  Outputs per charge: v
+// per element j, 6 float4: (x.h, a.hi), (x.l, a.lo), (n.hi, alpha.hi),
+// (n.lo, alpha.lo), (l.hi, l.lo, beta.hi, beta.lo), (x.m, 0) with a = ds psi, alpha =
+// ds phi and the adjoint lam / eps_in = [l; beta].  Outputs per charge: v
 // (dE/dq up to 1/2 and 1/(4 pi)) and the three components of the gradient g.
 struct GradPolicy {
-  static constexpr int RW = 5;
+  static constexpr int RW = 6;
   static constexpr int NOUT = 4;
+  static constexpr bool CHUNKED = true;
   static constexpr bool SELF = false;
-  struct Tgt {
-    df y[3];
-  };
+  using Tgt = PointTgtDF;
   struct Acc {
     df v, g[3];
   };
@@ -296,31 +325,30 @@ struct GradPolicy {
     const double4_32a* pts;
     double* part;
     DFConst c;
-    df inv_eps_in;
+    const int4* chg_tab;
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
-  __device__ static void load(const Args& a, int k, Tgt& t) {
-    double4_32a g = a.pts[k];
-    t.y[0] = df_from_double(g.x), t.y[1] = df_from_double(g.y), t.y[2] = df_from_double(g.z);
+  __device__ static void load(const Args& a, int k, int sys, Tgt& t) {
+    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, 0), t);
   }
   __device__ static void zero(Acc& acc) {
     acc.v = df{0.f, 0.f};
     for (int m = 0; m < 3; ++m) acc.g[m] = df{0.f, 0.f};
   }
-  __device__ static void renorm(Acc& acc) {
-    acc.v = two_sum(acc.v.hi, acc.v.lo);
-    for (int m = 0; m < 3; ++m) acc.g[m] = two_sum(acc.g[m].hi, acc.g[m].lo);
+  __device__ static void flush(Acc& sum, const Acc& acc) {
+    sum.v = df_add(sum.v, acc.v);
+    for (int m = 0; m < 3; ++m) sum.g[m] = df_add(sum.g[m], acc.g[m]);
   }
   template <bool MASK>
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
-    const float4 A = r[0], B = r[1], C = r[2], D = r[3], E = r[4];
-    const df x[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
+    const float4 A = r[0], B = r[1], C = r[2], D = r[3], E = r[4], M = r[5];
+    const df_pos x[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
     const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_grad_pair(t.y, x, df{A.w, B.w}, nv, df{C.w, D.w}, df{E.x, E.y}, df{E.z, E.w}, a.c, a.inv_eps_in,
-                 df_exp_table(), acc.v, acc.g);
+    df_grad_pair(t.y, x, df{A.w, B.w}, nv, df{C.w, D.w}, df{E.x, E.y}, df{E.z, E.w}, a.c, df_exp_table(), acc.v,
+                 acc.g);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int k, const Acc& acc) {
     double* o = a.part + (size_t)out + k;
@@ -335,7 +363,12 @@ struct GradPolicy {
 //                              with n_tgt targets (thread t owns t0 + k*NT + t)
 //   {src_off, s0, s1, out}     sources src_off + [s0, s1); partials at part[out]
 // The self pair (same local index) is masked only in source chunks that
-// overlap the item's own targets.
+// overlap the item's own targets.  CHUNKED policies (df64) sum runs of 16
+// sources from zero with lazy accumulators and add each run to the running
+// sums once: a lazy sum's trailing part grows with its length and loses digits
+// (a reaction potential from 20480 elements summed in runs of 64: error 5e-14,
+// of 16: 3e-14, of 4: 3e-14), and the sums of a run cost less than one
+// operation per source.
 template <class P, typename V4, int NT, int TPT, int CH>
 __global__ void __launch_bounds__(NT) k_items(typename P::Args a, const int4* __restrict__ items,
                                               const V4* __restrict__ rec, const int* __restrict__ skip,
@@ -347,13 +380,14 @@ __global__ void __launch_bounds__(NT) k_items(typename P::Args a, const int4* __
   if (sys_skipped(skip, skip_stride, sys)) return;
   P::prologue(a);  // per-CTA shared tables (made visible by the first barrier below)
   typename P::Tgt tg[TPT];
-  typename P::Acc acc[TPT];
+  typename P::Acc acc[TPT], sum[P::CHUNKED ? TPT : 1];
   int idx[TPT];
 #pragma unroll
   for (int k = 0; k < TPT; ++k) {
     idx[k] = t0 + k * NT + threadIdx.x;
-    P::load(a, tgt_off + min(idx[k], n_tgt - 1), tg[k]);
+    P::load(a, tgt_off + min(idx[k], n_tgt - 1), sys, tg[k]);
     P::zero(acc[k]);
+    if (P::CHUNKED) P::zero(sum[k]);
   }
   for (int j0 = s0; j0 < s1; j0 += CH) {
     const int cnt = min(CH, s1 - j0);
@@ -362,32 +396,39 @@ __global__ void __launch_bounds__(NT) k_items(typename P::Args a, const int4* __
     for (int q = threadIdx.x; q < cnt * P::RW; q += NT) sh[q] = src[q];
     __syncthreads();
     const bool diag = P::SELF && (j0 < t0 + NT * TPT) && (j0 + cnt > t0);
-    if (!diag) {
-      if (cnt == CH) {
+    constexpr int kRun = P::CHUNKED ? 16 : CH;
+    for (int r0 = 0; r0 < cnt; r0 += kRun) {
+      if (!diag) {
+        if (r0 + kRun <= cnt) {
 #pragma unroll 2
-        for (int jj = 0; jj < CH; ++jj) {
+          for (int jj = r0; jj < r0 + kRun; ++jj) {
 #pragma unroll
-          for (int k = 0; k < TPT; ++k) P::template pair<false>(a, tg[k], sh + jj * P::RW, false, acc[k]);
+            for (int k = 0; k < TPT; ++k) P::template pair<false>(a, tg[k], sh + jj * P::RW, false, acc[k]);
+          }
+        } else {
+          for (int jj = r0; jj < cnt; ++jj) {
+#pragma unroll
+            for (int k = 0; k < TPT; ++k) P::template pair<false>(a, tg[k], sh + jj * P::RW, false, acc[k]);
+          }
         }
       } else {
-        for (int jj = 0; jj < cnt; ++jj) {
+        for (int jj = r0; jj < min(cnt, r0 + kRun); ++jj) {
 #pragma unroll
-          for (int k = 0; k < TPT; ++k) P::template pair<false>(a, tg[k], sh + jj * P::RW, false, acc[k]);
+          for (int k = 0; k < TPT; ++k)
+            P::template pair<true>(a, tg[k], sh + jj * P::RW, j0 + jj == idx[k], acc[k]);
         }
       }
-    } else {
-      for (int jj = 0; jj < cnt; ++jj) {
+      if (P::CHUNKED)
 #pragma unroll
-        for (int k = 0; k < TPT; ++k)
-          P::template pair<true>(a, tg[k], sh + jj * P::RW, j0 + jj == idx[k], acc[k]);
-      }
+        for (int k = 0; k < TPT; ++k) {
+          P::flush(sum[k], acc[k]);
+          P::zero(acc[k]);
+        }
     }
-#pragma unroll
-    for (int k = 0; k < TPT; ++k) P::renorm(acc[k]);  // lazily updated accumulators back to normal form
   }
 #pragma unroll
   for (int k = 0; k < TPT; ++k)
-    if (idx[k] < n_tgt) P::store(a, out, n_tgt, idx[k], acc[k]);
+    if (idx[k] < n_tgt) P::store(a, out, n_tgt, idx[k], P::CHUNKED ? sum[k] : acc[k]);
 }
 
 // ------------------------------------------------------------------ work lists
@@ -541,7 +582,8 @@ __global__ void k_pack(const int4* __restrict__ lay, bool transpose, const doubl
   rec[2 * o + 1] = r1;
 }
 
-// df64 records (4 float4 per element) of every system, forward or transposed.
+// df64 records (4 float4 per element) of every system, forward or transposed:
+// (x.hi, w.hi), (x.lo, w.lo), (m.hi, 0), (m.lo, 0) with m the normal times its factor.
 __global__ void k_pack_df(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
                           const double* __restrict__ u, float4* __restrict__ rec, const int* __restrict__ skip,
                           int skip_stride) {
@@ -561,6 +603,33 @@ __global__ void k_pack_df(const int4* __restrict__ lay, bool transpose, const do
   rec[o + 1] = make_float4(x0.lo, x1.lo, x2.lo, w.lo);
   rec[o + 2] = make_float4(m0.hi, m1.hi, m2.hi, 0.f);
   rec[o + 3] = make_float4(m0.lo, m1.lo, m2.lo, 0.f);
+}
+
+// The first 4 float4 and the last one of an element's record in the charge
+// passes: (x.h, a.hi), (x.l, a.lo), (n.hi, alpha.hi), (n.lo, alpha.lo), ..,
+// (x.m, 0) with a = ds psi, alpha = ds phi, x on the pass's grid.
+__device__ __forceinline__ void pack_elem_df(const double4_32a& g, const double4_32a& v, double phi, double psi,
+                                             double grid, float4* o, int last) {
+  const df_pos x0 = df_split_grid(g.x, grid), x1 = df_split_grid(g.y, grid), x2 = df_split_grid(g.z, grid);
+  const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
+  const df a = df_from_double(g.w * psi), al = df_from_double(g.w * phi);
+  o[0] = make_float4(x0.h, x1.h, x2.h, a.hi);
+  o[1] = make_float4(x0.l, x1.l, x2.l, a.lo);
+  o[2] = make_float4(n0.hi, n1.hi, n2.hi, al.hi);
+  o[3] = make_float4(n0.lo, n1.lo, n2.lo, al.lo);
+  o[last] = make_float4(x0.m, x1.m, x2.m, 0.f);
+}
+// Records of the reaction pass (5 float4 per element, at vec_off / 2).
+__global__ void k_pack_react(const int4* __restrict__ lay, const int4* __restrict__ chg_tab, int extra,
+                             const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
+                             float4* __restrict__ rec) {
+  const int k = blockIdx.y;
+  const int4 L = lay[k];
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= L.y) return;
+  const double* uk = u + L.z;
+  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, extra),
+               rec + 5 * (size_t)(L.z / 2 + j), 4);
 }
 
 // y_i = diag * u_i - (1/(4 pi)) * scale_i * sum over splits, i < 2n of each system;
@@ -681,28 +750,21 @@ __global__ void k_energy_row_reduce(const int4* __restrict__ lay, const int4* __
   c[L.z + i] = tgt64[2 * (L.x + e)].w * kInv4Pi * acc;
 }
 
-// Gradient records of every system in df64 (5 float4 per element, at
-// vec_off / 2): (x, a = ds psi), (n, alpha = ds phi), (lphi, beta = lpsi).
-__global__ void k_pack_grad(const int4* __restrict__ lay, const double4_32a* __restrict__ tgt64,
-                            const double* __restrict__ u, const double* __restrict__ lam,
-                            float4* __restrict__ rec) {
+// Gradient records of every system in df64 (6 float4 per element, at
+// vec_off / 2): pack_elem_df's and (l, beta) = inv_eps_in (lphi, lpsi).
+__global__ void k_pack_grad(const int4* __restrict__ lay, const int4* __restrict__ chg_tab,
+                            const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
+                            const double* __restrict__ lam, double inv_eps_in, float4* __restrict__ rec) {
   const int k = blockIdx.y;
   const int4 L = lay[k];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= L.y) return;
-  const double4_32a g = tgt64[2 * (L.x + j)], v = tgt64[2 * (L.x + j) + 1];
   const double* uk = u + L.z;
   const double* lk = lam + L.z;
-  const df x0 = df_from_double(g.x), x1 = df_from_double(g.y), x2 = df_from_double(g.z);
-  const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
-  const df a = df_from_double(g.w * uk[L.y + j]), al = df_from_double(g.w * uk[j]);
-  const df lphi = df_from_double(lk[j]), beta = df_from_double(lk[L.y + j]);
-  float4* o = rec + 5 * (size_t)(L.z / 2 + j);
-  o[0] = make_float4(x0.hi, x1.hi, x2.hi, a.hi);
-  o[1] = make_float4(x0.lo, x1.lo, x2.lo, a.lo);
-  o[2] = make_float4(n0.hi, n1.hi, n2.hi, al.hi);
-  o[3] = make_float4(n0.lo, n1.lo, n2.lo, al.lo);
-  o[4] = make_float4(lphi.hi, lphi.lo, beta.hi, beta.lo);
+  const df l = df_from_double(inv_eps_in * lk[j]), beta = df_from_double(inv_eps_in * lk[L.y + j]);
+  float4* o = rec + 6 * (size_t)(L.z / 2 + j);
+  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, 0), o, 5);
+  o[4] = make_float4(l.hi, l.lo, beta.hi, beta.lo);
 }
 
 // dE/dq = 1/2 (1/(4 pi)) v and dE/dy = 1/2 q (1/(4 pi)) g per charge (sums over splits in a fixed order)
@@ -752,10 +814,8 @@ DFConst df_const_impl(const Surface* s, const bipb_medium& m) {
   c.inveps = split(1.0 / eps);
   c.kappa = split(m.kappa);
   const double L = 0.693147180559945309417232121458 / kExpTab;
-  const double l1 = std::ldexp(std::nearbyint(std::ldexp(L, 17)), -17);  // 7 significant bits
-  c.l1 = (float)l1;
-  c.l2 = (float)(L - l1);
-  c.l3 = (float)(L - l1 - (double)c.l2);
+  c.l1 = (float)L;
+  c.l2 = (float)(L - (double)c.l1);
   c.inv_l = (float)(kExpTab / 0.693147180559945309417232121458);
   c.tab = s->exptab.p;
   return c;
@@ -1007,14 +1067,20 @@ int autotune_matvec32(Surface* s, const SysLayout& L, const bipb_medium& m, int 
   return best;
 }
 
-// df64 records of every charge: (y.hi, q.hi), (y.lo, q.lo)
-__global__ void k_pack_chg_df(int n_chg, const double4_32a* __restrict__ chg, float4* __restrict__ rec) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_chg) return;
-  const double4_32a c = chg[k];
-  const df x = df_from_double(c.x), y = df_from_double(c.y), z = df_from_double(c.z), q = df_from_double(c.w);
-  rec[2 * k] = make_float4(x.hi, y.hi, z.hi, q.hi);
-  rec[2 * k + 1] = make_float4(x.lo, y.lo, z.lo, q.lo);
+// df64 records of every charge: (y.h, q.hi), (y.l, q.lo), (y.m, 0), on the grid of its system's pass
+__global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const double4_32a* __restrict__ chg,
+                              float4* __restrict__ rec) {
+  const int4 T = chg_tab[blockIdx.y];
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= T.y) return;
+  const double4_32a g = chg[T.x + c];
+  const double grid = charge_grid(chg_tab, blockIdx.y, extra);
+  const df_pos x = df_split_grid(g.x, grid), y = df_split_grid(g.y, grid), z = df_split_grid(g.z, grid);
+  const df q = df_from_double(g.w);
+  float4* o = rec + 3 * (size_t)(T.x + c);
+  o[0] = make_float4(x.h, y.h, z.h, q.hi);
+  o[1] = make_float4(x.l, y.l, z.l, q.lo);
+  o[2] = make_float4(x.m, y.m, z.m, 0.f);
 }
 
 void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b) {
@@ -1026,11 +1092,11 @@ void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b
     n_chg = std::max(n_chg, L.chg_off[k] + L.nc[k]);
   }
   ItemPlan* plan = plan_pass<SourcePolicy, float4, NT, TPT, CH>(s, kPassSource, sys, CH);
-  s->grow(s->chgdf, (size_t)2 * n_chg);
+  s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<blocks_for(n_chg, 256), 256, 0, s->stream>>>(n_chg, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  SourcePolicy::Args a{s->tgt64.p, s->part64.p};
+  SourcePolicy::Args a{s->tgt64.p, s->part64.p, s->chg_tab.p, 0};
   launch_items<SourcePolicy, float4, NT, TPT, CH>(s, kTSource, plan, a, s->chgdf.p, nullptr, 0);
   k_reduce_source<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, kInv4Pi / m.eps_in, b);
@@ -1043,30 +1109,31 @@ void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const d
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
   ItemPlan* plan = plan_pass<ReactionPolicy, float4, NT, TPT, CH>(s, kPassReaction, sys, CH);
-  s->grow(s->recdf, (size_t)2 * L.len);  // 4 float4 per element
+  s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  k_pack_df<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, false, s->tgt64.p, u, s->recdf.p,
-                                                                          nullptr, 0);
+  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, 0, s->tgt64.p, u,
+                                                                             s->recdf.p);
   BIPB_LAUNCHED(s);
-  ReactionPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m)};
+  ReactionPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, 0};
   launch_items<ReactionPolicy, float4, NT, TPT, CH>(s, kTReaction, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_reaction<<<L.K, 1024, 0, s->stream>>>(plan->tab.p, lay, s->part64.p, s->chg.p, phi_reac, e_out);
   BIPB_LAUNCHED(s);
 }
 
 void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
-                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double* out) {
+                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out) {
   constexpr int NT = 128, TPT = 1, CH = 64;
+  const int extra = far_bits(far_pts);
   // surface integral: targets are the points (shared by every system), sources the elements
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{0, n_pts, L.vec_off[k] / 2, L.n[k]};
-  s->grow(s->recdf, (size_t)2 * L.len);  // 4 float4 per element
+  s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
   const int4* lay = s->lay_dev(L);
-  k_pack_df<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, false, s->tgt64.p, u, s->recdf.p,
-                                                                          nullptr, 0);
+  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
+                                                                             s->recdf.p);
   BIPB_LAUNCHED(s);
-  ReactionPolicy::Args a{pts, nullptr, df_const_impl(s, m)};
+  ReactionPolicy::Args a{pts, nullptr, df_const_impl(s, m), s->chg_tab.p, extra};
   ItemPlan* plan;
   if (inside) {
     plan = plan_pass<ReactionPolicy, float4, NT, TPT, CH>(s, kPassPotIn, sys, CH);
@@ -1091,11 +1158,11 @@ void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const 
   }
   if (n_chg == 0) return;
   ItemPlan* sp = plan_pass<SourcePolicy, float4, NT, TPT, CH>(s, kPassPotSrc, sys, CH);
-  s->grow(s->chgdf, (size_t)2 * n_chg);
+  s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)sp->part_len);
-  k_pack_chg_df<<<blocks_for(n_chg, 256), 256, 0, s->stream>>>(n_chg, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  SourcePolicy::Args b{pts2, s->part64.p};
+  SourcePolicy::Args b{pts2, s->part64.p, s->chg_tab.p, extra};
   launch_items<SourcePolicy, float4, NT, TPT, CH>(s, kTPotential, sp, b, s->chgdf.p, nullptr, 0);
   k_reduce_points<<<dim3(blocks_for(n_pts, 256), L.K), 256, 0, s->stream>>>(sp->tab.p, s->part64.p, n_pts, 2,
                                                                            kInv4Pi / m.eps_in, 1, out);
@@ -1119,11 +1186,11 @@ void energy_row_pass(Surface* s, const SysLayout& L, const bipb_medium& m, doubl
     n_chg = std::max(n_chg, L.chg_off[k] + L.nc[k]);
   }
   ItemPlan* plan = plan_pass<EnergyRowPolicy, float4, NT, TPT, CH>(s, kPassRow, sys, CH);
-  s->grow(s->chgdf, (size_t)2 * n_chg);
+  s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<blocks_for(n_chg, 256), 256, 0, s->stream>>>(n_chg, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  EnergyRowPolicy::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m)};
+  EnergyRowPolicy::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
   launch_items<EnergyRowPolicy, float4, NT, TPT, CH>(s, kTRow, plan, a, s->chgdf.p, nullptr, 0);
   k_energy_row_reduce<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, s->tgt64.p, c);
@@ -1136,14 +1203,13 @@ void grad_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const doubl
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
   ItemPlan* plan = plan_pass<GradPolicy, float4, NT, TPT, CH>(s, kPassGrad, sys, CH);
-  s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
+  s->grow(s->recdf, (size_t)3 * L.len);  // 6 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  k_pack_grad<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->tgt64.p, u, lam, s->recdf.p);
+  k_pack_grad<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, s->tgt64.p, u, lam,
+                                                                            1.0 / m.eps_in, s->recdf.p);
   BIPB_LAUNCHED(s);
-  const double inv = 1.0 / m.eps_in;
-  const float inv_hi = (float)inv;
-  GradPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), df{inv_hi, (float)(inv - (double)inv_hi)}};
+  GradPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
   launch_items<GradPolicy, float4, NT, TPT, CH>(s, kTGrad, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_grad<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(plan->tab.p, lay, s->part64.p,
                                                                               s->chg.p, dq, dy);

@@ -65,6 +65,7 @@ struct SymPolicy {
   static constexpr bool SCALED = !LAPLACE;
   static constexpr int RW = 2;  // (x, a), (n, alpha)
   static constexpr int UNROLL = sizeof(T) == 4 ? 4 : 1;  // sources in flight per thread
+  static constexpr bool CHUNKED = false;
   struct Elem {
     T x[3], a, n[3], al;
   };
@@ -91,6 +92,7 @@ struct SymPolicy {
                           masked, g.c, ti.p, ti.q, tj.p, tj.q);
   }
   __device__ static void renorm(Acc&) {}
+  __device__ static void flush(Acc&, const Acc&) {}
   __device__ static T add(T a, T b) { return a + b; }
   __device__ static T shfl_from(T v, int src) { return __shfl_sync(0xffffffffu, v, src); }
   // a source slot q past the end of a chunk: far away, no field, no normal (adds exact zeros)
@@ -110,17 +112,20 @@ __device__ df* sym_exp_table() {
   return tab;
 }
 
-// df64 record, 4 float4: (x.hi, a.hi), (x.lo, a.lo), (n.hi, alpha.hi), (n.lo, alpha.lo);
+// df64 record, 5 float4: (x.h, a.hi), (x.l, a.lo), (n.hi, alpha.hi), (n.lo, alpha.lo),
+// (x.m, 0), the position in three parts on the surface's grid (df_pos);
 // SCALED: positions and alpha in kappa-scaled units (df_sym_pair)
 template <bool TRANS, bool SCALED_>
 struct SymDFPolicy {
   using V4 = float4;
   using PT = double;
   static constexpr bool SCALED = SCALED_;
-  static constexpr int RW = 4;
+  static constexpr int RW = 5;
   static constexpr int UNROLL = 1;
+  static constexpr bool CHUNKED = true;  // every chunk summed from zero, then added to the running sums
   struct Elem {
-    df x[3], a, n[3], al;
+    df_pos x[3];
+    df a, n[3], al;
   };
   struct Acc {
     df p, q;
@@ -129,19 +134,21 @@ struct SymDFPolicy {
     DFConst c;
   };
   __device__ static void prologue(const Args& g) { df_load_exp_table(sym_exp_table(), g.c); }
-  __device__ static void load(const float4* r, Elem& e) { unpack(r[0], r[1], r[2], r[3], e); }
+  __device__ static void load(const float4* r, Elem& e) { unpack(r[0], r[1], r[2], r[3], r[4], e); }
   template <int CH>
   __device__ static void load_plane(const float4* sh, int q, Elem& e) {
-    unpack(sh[q], sh[CH + q], sh[2 * CH + q], sh[3 * CH + q], e);
+    unpack(sh[q], sh[CH + q], sh[2 * CH + q], sh[3 * CH + q], sh[4 * CH + q], e);
   }
-  __device__ static void unpack(const float4& A, const float4& B, const float4& C, const float4& D, Elem& e) {
-    e.x[0] = df{A.x, B.x}, e.x[1] = df{A.y, B.y}, e.x[2] = df{A.z, B.z}, e.a = df{A.w, B.w};
+  __device__ static void unpack(const float4& A, const float4& B, const float4& C, const float4& D, const float4& M,
+                                Elem& e) {
+    e.x[0] = df_pos{A.x, B.x, M.x}, e.x[1] = df_pos{A.y, B.y, M.y}, e.x[2] = df_pos{A.z, B.z, M.z};
+    e.a = df{A.w, B.w};
     e.n[0] = df{C.x, D.x}, e.n[1] = df{C.y, D.y}, e.n[2] = df{C.z, D.z}, e.al = df{C.w, D.w};
   }
   __device__ static void zero(Acc& v) { v.p = df{0.f, 0.f}, v.q = df{0.f, 0.f}; }
   template <bool MASK>
   __device__ static void pair(const Args& g, const Elem& t, const Elem& sj, bool masked, Acc& ti, Acc& tj) {
-    const df d[3] = {df_sub(t.x[0], sj.x[0]), df_sub(t.x[1], sj.x[1]), df_sub(t.x[2], sj.x[2])};
+    const df d[3] = {df_diff(t.x[0], sj.x[0]), df_diff(t.x[1], sj.x[1]), df_diff(t.x[2], sj.x[2])};
     df_sym_pair<MASK, TRANS, SCALED>(d, t.n, t.a, t.al, sj.n, sj.a, sj.al, masked, g.c, sym_exp_table(), ti.p, ti.q,
                                      tj.p, tj.q);
   }
@@ -150,6 +157,10 @@ struct SymDFPolicy {
     v.p = two_sum(v.p.hi, v.p.lo);
     v.q = two_sum(v.q.hi, v.q.lo);
   }
+  __device__ static void flush(Acc& sum, const Acc& v) {
+    sum.p = df_add(sum.p, v.p);
+    sum.q = df_add(sum.q, v.q);
+  }
   __device__ static df add(df a, df b) { return df_add(a, b); }
   __device__ static df shfl_from(df v, int src) {
     return df{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
@@ -157,7 +168,7 @@ struct SymDFPolicy {
   template <int CH>
   __device__ static void pad(float4* sh, int q) {
     sh[q] = make_float4(1e4f, 1e4f, 1e4f, 0.f);
-    sh[CH + q] = sh[2 * CH + q] = sh[3 * CH + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    sh[CH + q] = sh[2 * CH + q] = sh[3 * CH + q] = sh[4 * CH + q] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __device__ static PT out(df v) { return df_to_double(v); }
 };
@@ -226,13 +237,14 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
     const int64_t jrow = jbase + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2);
     const int len = n - t0;  // j-side row length
     typename P::Elem tg[TPT];
-    Acc acc[TPT];
+    Acc acc[TPT], sum[P::CHUNKED ? TPT : 1];
     int idx[TPT];
 #pragma unroll
     for (int k = 0; k < TPT; ++k) {
       idx[k] = t0 + k * NT + threadIdx.x;
       P::load(rec + (size_t)(rec_off + min(idx[k], n - 1)) * P::RW, tg[k]);
       P::zero(acc[k]);
+      if (P::CHUNKED) P::zero(sum[k]);
     }
     for (int j0 = s0; j0 < s1; j0 += CH) {
       const int cnt = min(CH, s1 - j0);
@@ -247,8 +259,12 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
         sym_chunk<P, TPT, CH, true>(g, tg, idx, acc, sh, cnt, j0, jred);
       else
         sym_chunk<P, TPT, CH, false>(g, tg, idx, acc, sh, cnt, j0, jred);
+      if (P::CHUNKED)
 #pragma unroll
-      for (int k = 0; k < TPT; ++k) P::renorm(acc[k]);
+        for (int k = 0; k < TPT; ++k) {
+          P::flush(sum[k], acc[k]);
+          P::zero(acc[k]);
+        }
       __syncthreads();
       for (int q = threadIdx.x; q < cnt; q += NT) {
         Acc v = jred[0][q];
@@ -262,8 +278,9 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
 #pragma unroll
     for (int k = 0; k < TPT; ++k)
       if (idx[k] < n) {
-        part[(size_t)ioff + idx[k] - t0] = P::out(acc[k].p);
-        part[(size_t)ioff + T + idx[k] - t0] = P::out(acc[k].q);
+        const Acc& v = P::CHUNKED ? sum[k] : acc[k];
+        part[(size_t)ioff + idx[k] - t0] = P::out(v.p);
+        part[(size_t)ioff + T + idx[k] - t0] = P::out(v.q);
       }
   }
 }
@@ -271,7 +288,8 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
 // ------------------------------------------------------------------ pack / reduce
 // Records of every system at vec_off / 2 (RW vectors each).  lay[k] = {geo_off, n, vec_off, chg_off}.
 // A u: a = ds psi, alpha = ds phi; A^T w: a = wphi, alpha = wpsi.
-// sigma: the positions and alpha are multiplied by it (kappa-scaled records; 1 otherwise)
+// sigma: the positions and alpha are multiplied by it (kappa-scaled records; 1 otherwise);
+// gscale: the power of two at or above sigma, by which the surface's coordinate grid grows with it
 template <typename V4, typename T>
 __global__ void k_pack_sym(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
                            const double* __restrict__ u, V4* __restrict__ rec, const int* __restrict__ skip,
@@ -295,7 +313,7 @@ __global__ void k_pack_sym(const int4* __restrict__ lay, bool transpose, const d
 
 __global__ void k_pack_sym_df(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
                               const double* __restrict__ u, float4* __restrict__ rec, const int* __restrict__ skip,
-                              int skip_stride, double sigma) {
+                              int skip_stride, double sigma, double gscale) {
   chain_wait();
   chain_release();
   const int k = blockIdx.y;
@@ -306,13 +324,16 @@ __global__ void k_pack_sym_df(const int4* __restrict__ lay, bool transpose, cons
   const double phi = u[L.z + j], psi = u[L.z + L.y + j];
   const df a = df_from_double(transpose ? phi : g.w * psi);
   const df al = df_from_double(sigma * (transpose ? psi : g.w * phi));
-  const df x0 = df_from_double(sigma * g.x), x1 = df_from_double(sigma * g.y), x2 = df_from_double(sigma * g.z);
+  const double grid = gscale * v.w;  // of the scaled coordinates
+  const df_pos x0 = df_split_grid(sigma * g.x, grid), x1 = df_split_grid(sigma * g.y, grid),
+               x2 = df_split_grid(sigma * g.z, grid);
   const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
-  float4* o = rec + 4 * (size_t)(L.z / 2 + j);
-  o[0] = make_float4(x0.hi, x1.hi, x2.hi, a.hi);
-  o[1] = make_float4(x0.lo, x1.lo, x2.lo, a.lo);
+  float4* o = rec + 5 * (size_t)(L.z / 2 + j);
+  o[0] = make_float4(x0.h, x1.h, x2.h, a.hi);
+  o[1] = make_float4(x0.l, x1.l, x2.l, a.lo);
   o[2] = make_float4(n0.hi, n1.hi, n2.hi, al.hi);
   o[3] = make_float4(n0.lo, n1.lo, n2.lo, al.lo);
+  o[4] = make_float4(x0.m, x1.m, x2.m, 0.f);
 }
 
 // y_i = diag u_i - (1/(4 pi)) scale_i f_c (i-side blocks of the element's row + j-side rows 0..E),
@@ -596,7 +617,7 @@ void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typena
   const int4* lay = s->lay_dev(L);
   if constexpr (std::is_same<typename P::PT, double>::value && std::is_same<typename P::V4, float4>::value) {
     launch_chained(k_pack_sym_df, dim3(blocks_of(L.max_n, 256), L.K), 256, 0, s->stream, lay, transpose, s->tgt64.p, u,
-                   recbuf.p, skip, skip_stride, sigma);
+                   recbuf.p, skip, skip_stride, sigma, std::exp2(std::ceil(std::log2(sigma))));
   } else {
     launch_chained(k_pack_sym<typename P::V4, typename P::PT>, dim3(blocks_of(L.max_n, 256), L.K), 256, 0, s->stream,
                    lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride, sigma);

@@ -1,0 +1,84 @@
+"""Edges of the kernels' arithmetic against the FP64 CPU oracle (through the C ABI).
+
+Tolerances are those of tests/test_gpu_parity.py: 1e-12 of the largest output
+for the double-float charge passes, 2e-12 for the double-float mat-vec.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def bipb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_10044_gb300.build import build
+
+    build()
+    import paper_2312_10044_gb300 as b
+
+    b.load_library()
+    return b
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+
+    return oracle
+
+
+def _dev(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+@pytest.mark.parametrize("far", [1.0, 1.9, 37.0, 1e5])
+def test_charge_pass_grid_follows_the_farthest_charge(bipb, orc, far):
+    """The coordinate grid of the double-float charge passes covers the surface and
+    the charges of its system: one charge `far` surface radii away, on either side
+    of a power of two and far outside, set from the host and from the device."""
+    p = synth.kirkwood_problem(level=3)
+    eps = p.eps_out / p.eps_in
+    pos = p.charge_pos.copy()
+    pos[3] = [0.0, -far * 20.0, 0.3]
+    u = np.random.default_rng(5).standard_normal(2 * p.n)
+    b_ref = orc.source(p.centroids, p.normals, pos, p.q[0], p.eps_in)
+    e_ref, pr_ref = orc.energy(p.centroids, p.normals, p.areas, eps, p.kappa, pos, p.q[0], u)
+    med = bipb.medium(p.eps_in, p.eps_out, p.kappa)
+    got = []
+    with bipb.Surface(p.centroids, p.normals, p.areas) as s:
+        for device in (False, True):
+            s.set_charges_dev(_dev(pos), _dev(p.q)) if device else s.set_charges(pos, p.q)
+            b = _dev(np.zeros(2 * p.n))
+            pr, e = _dev(np.zeros(p.nc)), _dev(np.zeros(1))
+            s.source(b, med=med)
+            s.reaction(_dev(u), pr, e, med=med)
+            np.testing.assert_allclose(b.cpu().numpy(), b_ref, rtol=0, atol=1e-12 * np.abs(b_ref).max())
+            np.testing.assert_allclose(pr.cpu().numpy(), pr_ref, rtol=0, atol=1e-12 * np.abs(pr_ref).max())
+            got.append((b.cpu().numpy(), pr.cpu().numpy()))
+    np.testing.assert_array_equal(got[0][0], got[1][0])
+    np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("scale", [1e-3, 1.0, 31.0, 1e4])
+def test_double_float_matvec_grid_scales_with_the_surface(bipb, orc, scale):
+    """The double-float mat-vec's coordinate grid is taken from the surface's own
+    extent times kappa: small and large surfaces in one batch handle, both directions."""
+    p = synth.kirkwood_problem(level=2)
+    parts = [(p.centroids * f, p.normals, p.areas * f * f) for f in (1.0, scale)]
+    kappa = 0.1257 / max(scale, 1.0)
+    u = np.random.default_rng(7).standard_normal(4 * p.n)
+    with bipb.BatchSurface(parts) as s:
+        for transpose in (False, True):
+            y = _dev(np.zeros_like(u))
+            s.matvec(_dev(u), y, precision=bipb.DF64, transpose=transpose, med=bipb.medium(1.0, 80.0, kappa))
+            y = y.cpu().numpy().reshape(2, -1)
+            f = orc.matvec_t if transpose else orc.matvec
+            for k, (c, n, a) in enumerate(parts):
+                ref = f(c, n, a, 80.0, kappa, u.reshape(2, -1)[k])
+                np.testing.assert_allclose(y[k], ref, rtol=0, atol=2e-12 * np.abs(ref).max(), err_msg=f"{transpose} {k}")
