@@ -24,6 +24,12 @@ __device__ __forceinline__ f2 f2_splat(float a) { return f2_make(a, a); }
 __device__ __forceinline__ void f2_get(f2 a, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
 }
+// the two values added
+__device__ __forceinline__ float f2_sum(f2 a) {
+  float lo, hi;
+  f2_get(a, lo, hi);
+  return lo + hi;
+}
 __device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
   f2 r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));

@@ -192,7 +192,7 @@ struct ItemPlan {
 // sources per shared-memory chunk): every ordered pair: 0 (256,2,128)
 // 1 (256,1,128) 2 (128,2,128) 3 (256,4,128) 4 (128,4,64) 5 (512,1,128)
 // 6 (256,2,64); every unordered pair once (sym.cu): 7 (256,2,64)
-// 8 (128,4,64) 9 (256,4,64, two CTAs per SM).
+// 8 (128,4,64) 9 (a shape by the size of the surfaces: matvec_sym32).
 constexpr int kNumMv32Variants = 10;
 constexpr int kFirstSymVariant = 7;
 

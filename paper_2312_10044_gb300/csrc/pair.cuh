@@ -29,6 +29,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "f32x2.cuh"
+
 namespace bipb {
 
 constexpr float kSMaxF = 1.0e6f;   // 1/r is capped at its value at 1e-6 A (an overflow guard, not a model)
@@ -219,6 +221,63 @@ __device__ __forceinline__ void sym_pair(T dx, T dy, T dz, const T* nt, T at, T 
       Qt = ome_s * as - ((te1_s3 * cj) * als - Qt);
       Ps = U_s3 * alt + ((et1_s3 * cj) * at + Ps);
       Qs = ome_s * at + ((te1_s3 * ci) * alt + Qs);
+    }
+  }
+}
+
+// The symmetric pair in FP32 for two targets t (packed) and one source s (every
+// value in both halves), the formulas of sym_pair with signs placed so that no
+// packed operand needs a negation: 1 - t for t - 1, -U, -(eps t - 1) s^3 and
+// -(t/eps - 1) s^3, and in scaled units (1 - e) s = (1 - t) s + e (kappa r s =
+// 1).  ft: a, -alpha and alpha (A u) or -a (A^T w) of the targets; fs: a,
+// -alpha and -a (A u) or alpha (A^T w) of the source.  A masked pair has s = e = 0.
+template <bool MASK, bool TRANS, bool LAPLACE>
+__device__ __forceinline__ void sym_pair2(const f2* xt, const f2* nt, const f2* ft, const f2* xs, const f2* ns,
+                                          const f2* fs, bool m0, bool m1, const PairConst<float>& c, f2& Pt, f2& Qt,
+                                          f2& Ps, f2& Qs) {
+  const f2 dx = f2_sub(xt[0], xs[0]), dy = f2_sub(xt[1], xs[1]), dz = f2_sub(xt[2], xs[2]);
+  const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
+  float ra, rb;
+  f2_get(r2, ra, rb);
+  float sa = fminf(rsqrt_approx(ra), c.smax), sb = fminf(rsqrt_approx(rb), c.smax);
+  if (MASK) sa = m0 ? 0.f : sa, sb = m1 ? 0.f : sb;
+  const f2 s = f2_make(sa, sb);
+  const f2 ci = f2_fma(nt[0], dx, f2_fma(nt[1], dy, f2_mul(nt[2], dz)));
+  const f2 cj = f2_fma(ns[0], dx, f2_fma(ns[1], dy, f2_mul(ns[2], dz)));
+  const f2 s2 = f2_mul(s, s), s3 = f2_mul(s2, s);
+  if constexpr (LAPLACE) {
+    const f2 E = f2_mul(f2_splat(1.f - c.eps), s3), F = f2_mul(f2_splat(1.f - c.inveps), s3);
+    const f2 A = f2_mul(E, cj), B = f2_mul(F, ci), C = f2_mul(E, ci), D = f2_mul(F, cj);
+    Pt = TRANS ? f2_fma(C, fs[0], Pt) : f2_fma(A, fs[1], Pt);
+    Qt = TRANS ? f2_fma(D, fs[2], Qt) : f2_fma(B, fs[2], Qt);
+    Ps = TRANS ? f2_fma(A, ft[2], Ps) : f2_fma(C, ft[2], Ps);
+    Qs = TRANS ? f2_fma(B, ft[1], Qs) : f2_fma(D, ft[0], Qs);
+  } else {
+    const f2 kr = f2_mul(r2, s);
+    float ea, eb;
+    f2_get(f2_mul(kr, f2_splat(-1.4426950408889634f)), ea, eb);
+    ea = ex2_approx(ea), eb = ex2_approx(eb);
+    if (MASK) ea = m0 ? 0.f : ea, eb = m1 ? 0.f : eb;
+    const f2 e = f2_make(ea, eb);
+    const f2 t = f2_fma(e, kr, e);
+    const f2 omt = f2_sub(f2_splat(1.f), t);
+    const f2 w = f2_fma(omt, f2_mul(f2_splat(-3.f), s2), e);  // (w - 3) s^2
+    const f2 cij = f2_fma(nt[0], ns[0], f2_fma(nt[1], ns[1], f2_mul(nt[2], ns[2])));
+    const f2 V = f2_mul(f2_fma(w, f2_mul(ci, cj), f2_mul(omt, cij)), s3);  // -U s^3
+    const f2 K1 = f2_fma(omt, s, e);
+    const f2 ts3 = f2_mul(t, s3);
+    const f2 E = f2_fma(f2_splat(-c.eps), ts3, s3), F = f2_fma(f2_splat(-c.inveps), ts3, s3);
+    const f2 A = f2_mul(E, cj), B = f2_mul(F, ci), C = f2_mul(E, ci), D = f2_mul(F, cj);
+    if (!TRANS) {
+      Pt = f2_fma(A, fs[1], f2_fma(K1, fs[0], Pt));
+      Qt = f2_fma(V, fs[1], f2_fma(B, fs[2], Qt));
+      Ps = f2_fma(C, ft[2], f2_fma(K1, ft[0], Ps));
+      Qs = f2_fma(V, ft[1], f2_fma(D, ft[0], Qs));
+    } else {
+      Pt = f2_fma(V, fs[1], f2_fma(C, fs[0], Pt));
+      Qt = f2_fma(K1, fs[0], f2_fma(D, fs[2], Qt));
+      Ps = f2_fma(V, ft[1], f2_fma(A, ft[2], Ps));
+      Qs = f2_fma(K1, ft[0], f2_fma(B, ft[1], Qs));
     }
   }
 }

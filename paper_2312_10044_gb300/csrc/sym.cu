@@ -33,6 +33,7 @@
 #include <queue>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "internal.cuh"
 
 namespace bipb {
@@ -41,70 +42,147 @@ namespace {
 
 constexpr double kInv4PiS = 1.0 / (4.0 * kPi);
 
-template <typename T>
-struct SymV4;
-template <>
-struct SymV4<float> {
-  using type = float4;
-};
-template <>
-struct SymV4<double> {
-  using type = double4_32a;
-};
-
 // ------------------------------------------------------------------ policies
-// Record of an element (both roles): position, a, normal, alpha, where
-// (a, alpha) = (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w.
+// A policy: the record of an element (RW vectors of 4 values; both roles), a
+// pack of PACK targets of one thread (Tgt, with its accumulators Acc), a source
+// (Src), and the pair update of a pack with one source.  PACK = 2: two targets
+// in packed FP32 (f32x2.cuh), the source's values duplicated in its record so
+// that one 64-bit load gives a packed operand; the j side stays packed (one
+// half per target of the pack) until a block of 32 sources is done.  Red is the
+// j side of one source over a warp.
 
+// FP64, one target per pack.  Record (x, a), (n, alpha), where (a, alpha) =
+// (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w.
 // LAPLACE: the kappa = 0 form of sym_pair (pair.cuh); otherwise the records
 // are in kappa-scaled units (SCALED).
-template <typename T, bool TRANS, bool LAPLACE>
-struct SymPolicy {
-  using V4 = typename SymV4<T>::type;
-  using PT = T;  // partial sums are stored in this type
+template <bool TRANS, bool LAPLACE>
+struct Sym64Policy {
+  using V4 = double4_32a;
+  using PT = double;  // partial sums are stored in this type
   static constexpr bool SCALED = !LAPLACE;
-  static constexpr int RW = 2;  // (x, a), (n, alpha)
-  static constexpr int UNROLL = sizeof(T) == 4 ? 4 : 1;  // sources in flight per thread
+  static constexpr int RW = 2, PACK = 1, UNROLL = 1;
   static constexpr bool CHUNKED = false;
-  struct Elem {
-    T x[3], a, n[3], al;
+  struct Tgt {
+    double x[3], a, n[3], al;
   };
+  using Src = Tgt;
   struct Acc {
-    T p, q;
+    double p, q;
   };
+  using Red = Acc;
   struct Args {
-    PairConst<T> c;
+    PairConst<double> c;
   };
   __device__ static void prologue(const Args&) {}
-  __device__ static void load(const V4* r, Elem& e) { unpack(r[0], r[1], e); }
+  __device__ static void load(const V4* rec, const int* i, Tgt& t) { unpack(rec[2 * (size_t)i[0]], rec[2 * (size_t)i[0] + 1], t); }
   // record q of a chunk staged as planes (vector r of record q at sh[r * CH + q])
   template <int CH>
-  __device__ static void load_plane(const V4* sh, int q, Elem& e) { unpack(sh[q], sh[CH + q], e); }
-  __device__ static void unpack(const V4& A, const V4& B, Elem& e) {
+  __device__ static void load_src(const V4* sh, int q, Src& e) { unpack(sh[q], sh[CH + q], e); }
+  __device__ static void unpack(const V4& A, const V4& B, Tgt& e) {
     e.x[0] = A.x, e.x[1] = A.y, e.x[2] = A.z, e.a = A.w;
     e.n[0] = B.x, e.n[1] = B.y, e.n[2] = B.z, e.al = B.w;
   }
-  __device__ static void zero(Acc& v) { v.p = T(0), v.q = T(0); }
-  // i-side of target t and j-side of source sj for the pair d = x_t - x_sj
+  __device__ static void zero(Acc& v) { v.p = 0.0, v.q = 0.0; }
+  // i side of the targets t and j side of source sj for the pairs d = x_t - x_sj
   template <bool MASK>
-  __device__ static void pair(const Args& g, const Elem& t, const Elem& sj, bool masked, Acc& ti, Acc& tj) {
-    sym_pair<MASK, TRANS, LAPLACE>(t.x[0] - sj.x[0], t.x[1] - sj.x[1], t.x[2] - sj.x[2], t.n, t.a, t.al, sj.n, sj.a, sj.al,
-                          masked, g.c, ti.p, ti.q, tj.p, tj.q);
+  __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
+    sym_pair<MASK, TRANS, LAPLACE>(t.x[0] - sj.x[0], t.x[1] - sj.x[1], t.x[2] - sj.x[2], t.n, t.a, t.al, sj.n, sj.a,
+                                   sj.al, masked[0], g.c, ti.p, ti.q, tj.p, tj.q);
   }
-  __device__ static void renorm(Acc&) {}
   __device__ static void flush(Acc&, const Acc&) {}
-  __device__ static T add(T a, T b) { return a + b; }
-  __device__ static T shfl_from(T v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+  __device__ static Red reduced(const Acc& v) { return v; }
+  __device__ static double add(double a, double b) { return a + b; }
+  __device__ static void rotate(Acc& v, int src) {
+    v.p = __shfl_sync(0xffffffffu, v.p, src);
+    v.q = __shfl_sync(0xffffffffu, v.q, src);
+  }
   // a source slot q past the end of a chunk: far away, no field, no normal (adds exact zeros)
   template <int CH>
   __device__ static void pad(V4* sh, int q) {
-    V4 z;
-    z.x = T(1e4), z.y = T(1e4), z.z = T(1e4), z.w = T(0);
-    sh[q] = z;
-    z.x = z.y = z.z = T(0);
-    sh[CH + q] = z;
+    sh[q] = make_double4_32a(1e4, 1e4, 1e4, 0.0);
+    sh[CH + q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
   }
-  __device__ static PT out(T v) { return v; }
+  __device__ static PT out(double v) { return v; }
+  __device__ static void store(PT* p, int T, const int* o, const bool* in, const Acc& v) {
+    if (in[0]) p[o[0]] = v.p, p[T + o[0]] = v.q;
+  }
+};
+
+// FP32, two targets per pack.  What bounds it: the FP32 pipe's register ports.  An
+// FFMA with three register operands takes 1.5 issue cycles (FFMA2 three for two
+// results; measured), FADD and FMUL one, so a pair of 24 FFMA and 23 others
+// takes 59 cycles of a scheduler however it is issued, and the scalar form
+// waited for its loads, shuffles and MUFU calls on top (64.5).  Packed, they
+// hide behind it: N = 20480 0.387 -> 0.358 ms, N = 65537 3.43 -> 3.20 ms a
+// mat-vec (59.7 cycles a pair).  Record, 5 float4, every value twice: (x, x, y, y),
+// (z, z, a, a), (nx, nx, ny, ny), (nz, nz, -alpha, -alpha), (f, f, 0, 0) with f
+// = -a (A u) or alpha (A^T w): packed FP32 has no negated operands, so every
+// sign of sym_pair2 is one that a record, a constant or a subtraction brings.
+template <bool TRANS, bool LAPLACE>
+struct Sym32Policy {
+  using V4 = float4;
+  using PT = float;
+  static constexpr bool SCALED = !LAPLACE;
+  static constexpr int RW = 5, PACK = 2, UNROLL = 4;
+  static constexpr bool CHUNKED = false;
+  struct Tgt {
+    f2 x[3], n[3], f[3];  // f: a, -alpha and alpha (A u) or -a (A^T w)
+  };
+  struct Src {
+    f2 x[3], n[3], f[3];  // f: a, -alpha and -a (A u) or alpha (A^T w)
+  };
+  struct Acc {
+    f2 p, q;
+  };
+  struct Red {
+    float p, q;
+  };
+  struct Args {
+    PairConst<float> c;
+  };
+  __device__ static void prologue(const Args&) {}
+  __device__ static void load(const V4* rec, const int* i, Tgt& t) {
+    const V4 *r = rec + 5 * (size_t)i[0], *q = rec + 5 * (size_t)i[1];
+    const V4 A = r[0], B = r[1], C = r[2], D = r[3], E = q[0], F = q[1], G = q[2], H = q[3];
+    t.x[0] = f2_make(A.x, E.x), t.x[1] = f2_make(A.z, E.z), t.x[2] = f2_make(B.x, F.x);
+    t.n[0] = f2_make(C.x, G.x), t.n[1] = f2_make(C.z, G.z), t.n[2] = f2_make(D.x, H.x);
+    t.f[0] = f2_make(B.z, F.z), t.f[1] = f2_make(D.z, H.z);
+    t.f[2] = TRANS ? f2_make(-B.z, -F.z) : f2_make(-D.z, -H.z);
+  }
+  template <int CH>
+  __device__ static void load_src(const V4* sh, int q, Src& e) {
+    const ulonglong2* v = reinterpret_cast<const ulonglong2*>(sh);
+    const ulonglong2 A = v[q], B = v[CH + q], C = v[2 * CH + q], D = v[3 * CH + q];
+    e.x[0].v = A.x, e.x[1].v = A.y, e.x[2].v = B.x, e.f[0].v = B.y;
+    e.n[0].v = C.x, e.n[1].v = C.y, e.n[2].v = D.x, e.f[1].v = D.y;
+    e.f[2].v = v[4 * CH + q].x;
+  }
+  __device__ static void zero(Acc& v) { v.p = f2_splat(0.f), v.q = f2_splat(0.f); }
+  template <bool MASK>
+  __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
+    sym_pair2<MASK, TRANS, LAPLACE>(t.x, t.n, t.f, sj.x, sj.n, sj.f, masked[0], masked[1], g.c, ti.p, ti.q, tj.p, tj.q);
+  }
+  __device__ static void flush(Acc&, const Acc&) {}
+  __device__ static Red reduced(const Acc& v) { return Red{f2_sum(v.p), f2_sum(v.q)}; }
+  __device__ static float add(float a, float b) { return a + b; }
+  __device__ static void rotate(Acc& v, int src) {
+    v.p.v = __shfl_sync(0xffffffffu, v.p.v, src);
+    v.q.v = __shfl_sync(0xffffffffu, v.q.v, src);
+  }
+  template <int CH>
+  __device__ static void pad(V4* sh, int q) {
+    sh[q] = make_float4(1e4f, 1e4f, 1e4f, 1e4f);
+    sh[CH + q] = make_float4(1e4f, 1e4f, 0.f, 0.f);
+    sh[2 * CH + q] = sh[3 * CH + q] = sh[4 * CH + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ static PT out(float v) { return v; }
+  __device__ static void store(PT* p, int T, const int* o, const bool* in, const Acc& v) {
+    float a, b, c, d;
+    f2_get(v.p, a, b);
+    f2_get(v.q, c, d);
+    if (in[0]) p[o[0]] = a, p[T + o[0]] = c;
+    if (in[1]) p[o[1]] = b, p[T + o[1]] = d;
+  }
 };
 
 __device__ df* sym_exp_table() {
@@ -120,73 +198,78 @@ struct SymDFPolicy {
   using V4 = float4;
   using PT = double;
   static constexpr bool SCALED = SCALED_;
-  static constexpr int RW = 5;
-  static constexpr int UNROLL = 1;
+  static constexpr int RW = 5, PACK = 1, UNROLL = 1;
   static constexpr bool CHUNKED = true;  // every chunk summed from zero, then added to the running sums
-  struct Elem {
+  struct Tgt {
     df_pos x[3];
     df a, n[3], al;
   };
+  using Src = Tgt;
   struct Acc {
     df p, q;
   };
+  using Red = Acc;
   struct Args {
     DFConst c;
   };
   __device__ static void prologue(const Args& g) { df_load_exp_table(sym_exp_table(), g.c); }
-  __device__ static void load(const float4* r, Elem& e) { unpack(r[0], r[1], r[2], r[3], r[4], e); }
+  __device__ static void load(const V4* rec, const int* i, Tgt& t) {
+    const V4* r = rec + 5 * (size_t)i[0];
+    unpack(r[0], r[1], r[2], r[3], r[4], t);
+  }
   template <int CH>
-  __device__ static void load_plane(const float4* sh, int q, Elem& e) {
+  __device__ static void load_src(const V4* sh, int q, Src& e) {
     unpack(sh[q], sh[CH + q], sh[2 * CH + q], sh[3 * CH + q], sh[4 * CH + q], e);
   }
   __device__ static void unpack(const float4& A, const float4& B, const float4& C, const float4& D, const float4& M,
-                                Elem& e) {
+                                Tgt& e) {
     e.x[0] = df_pos{A.x, B.x, M.x}, e.x[1] = df_pos{A.y, B.y, M.y}, e.x[2] = df_pos{A.z, B.z, M.z};
     e.a = df{A.w, B.w};
     e.n[0] = df{C.x, D.x}, e.n[1] = df{C.y, D.y}, e.n[2] = df{C.z, D.z}, e.al = df{C.w, D.w};
   }
   __device__ static void zero(Acc& v) { v.p = df{0.f, 0.f}, v.q = df{0.f, 0.f}; }
   template <bool MASK>
-  __device__ static void pair(const Args& g, const Elem& t, const Elem& sj, bool masked, Acc& ti, Acc& tj) {
+  __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
     const df d[3] = {df_diff(t.x[0], sj.x[0]), df_diff(t.x[1], sj.x[1]), df_diff(t.x[2], sj.x[2])};
-    df_sym_pair<MASK, TRANS, SCALED>(d, t.n, t.a, t.al, sj.n, sj.a, sj.al, masked, g.c, sym_exp_table(), ti.p, ti.q,
+    df_sym_pair<MASK, TRANS, SCALED>(d, t.n, t.a, t.al, sj.n, sj.a, sj.al, masked[0], g.c, sym_exp_table(), ti.p, ti.q,
                                      tj.p, tj.q);
-  }
-  // the accumulators are updated lazily (df_mac): bring them back to normal form
-  __device__ static void renorm(Acc& v) {
-    v.p = two_sum(v.p.hi, v.p.lo);
-    v.q = two_sum(v.q.hi, v.q.lo);
   }
   __device__ static void flush(Acc& sum, const Acc& v) {
     sum.p = df_add(sum.p, v.p);
     sum.q = df_add(sum.q, v.q);
   }
+  // the accumulators are updated lazily (df_mac): bring them back to normal form
+  __device__ static Red reduced(const Acc& v) { return Red{two_sum(v.p.hi, v.p.lo), two_sum(v.q.hi, v.q.lo)}; }
   __device__ static df add(df a, df b) { return df_add(a, b); }
-  __device__ static df shfl_from(df v, int src) {
+  __device__ static df shfl(df v, int src) {
     return df{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
   }
+  __device__ static void rotate(Acc& v, int src) { v.p = shfl(v.p, src), v.q = shfl(v.q, src); }
   template <int CH>
   __device__ static void pad(float4* sh, int q) {
     sh[q] = make_float4(1e4f, 1e4f, 1e4f, 0.f);
     sh[CH + q] = sh[2 * CH + q] = sh[3 * CH + q] = sh[4 * CH + q] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __device__ static PT out(df v) { return df_to_double(v); }
+  __device__ static void store(PT* p, int T, const int* o, const bool* in, const Acc& v) {
+    if (in[0]) p[o[0]] = out(v.p), p[T + o[0]] = out(v.q);
+  }
 };
 
 // ------------------------------------------------------------------ kernel
 // One shared-memory chunk of cnt sources (starting at j0) against the
-// thread's TPT targets.  MASK: the chunk overlaps the tile's own targets, and
-// pairs with j <= i are masked.  The j side rotates through the warp: the
-// chunk is taken in blocks of 32 sources (the slots past cnt padded with
-// records that add exact zeros); at step k of a block, lane l evaluates
+// thread's NP packs of targets.  MASK: the chunk overlaps the tile's own
+// targets, and pairs with j <= i are masked.  The j side rotates through the
+// warp: the chunk is taken in blocks of 32 sources (the slots past cnt padded
+// with records that add exact zeros); at step k of a block, lane l evaluates
 // source (l + k) mod 32 against its targets, then takes over the accumulator
 // of the next source from lane l + 1.  After 32 steps lane l holds the
 // complete j-side sum of source (l + 31) mod 32 over the warp's targets,
 // accumulated in a fixed order; it leaves it in jred[warp][source].
-template <class P, int TPT, int CH, bool MASK>
-__device__ __forceinline__ void sym_chunk(const typename P::Args& g, const typename P::Elem* tg, const int* idx,
-                                              typename P::Acc* acc, const typename P::V4* sh, int cnt, int j0,
-                                              typename P::Acc (*jred)[CH]) {
+template <class P, int NP, int CH, bool MASK>
+__device__ __forceinline__ void sym_chunk(const typename P::Args& g, const typename P::Tgt* tg,
+                                          const int (*idx)[P::PACK], typename P::Acc* acc, const typename P::V4* sh,
+                                          int cnt, int j0, typename P::Red (*jred)[CH]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int next = (lane + 1) & 31;
   for (int r0 = 0; r0 < cnt; r0 += 32) {
@@ -195,18 +278,19 @@ __device__ __forceinline__ void sym_chunk(const typename P::Args& g, const typen
 #pragma unroll P::UNROLL
     for (int k = 0; k < 32; ++k) {
       const int jj = r0 + ((lane + k) & 31);
-      typename P::Elem sj;
-      P::template load_plane<CH>(sh, jj, sj);
+      typename P::Src sj;
+      P::template load_src<CH>(sh, jj, sj);
 #pragma unroll
-      for (int t = 0; t < TPT; ++t) P::template pair<MASK>(g, tg[t], sj, MASK && j0 + jj <= idx[t], acc[t], tj);
-      if (k < 31) {
-        tj.p = P::shfl_from(tj.p, next);
-        tj.q = P::shfl_from(tj.q, next);
+      for (int t = 0; t < NP; ++t) {
+        bool masked[P::PACK];
+#pragma unroll
+        for (int h = 0; h < P::PACK; ++h) masked[h] = MASK && j0 + jj <= idx[t][h];
+        P::template pair<MASK>(g, tg[t], sj, masked, acc[t], tj);
       }
+      if (k < 31) P::rotate(tj, next);
     }
-    P::renorm(tj);
     const int mine = r0 + ((lane + 31) & 31);
-    if (mine < cnt) jred[warp][mine] = tj;
+    if (mine < cnt) jred[warp][mine] = P::reduced(tj);
   }
 }
 
@@ -221,9 +305,10 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
                                             const int* __restrict__ skip, int skip_stride) {
   using V4 = typename P::V4;
   using Acc = typename P::Acc;
-  constexpr int NW = NT / 32, T = NT * TPT;
+  constexpr int NW = NT / 32, T = NT * TPT, NP = TPT / P::PACK;
+  static_assert(TPT % P::PACK == 0, "whole packs of targets");
   __shared__ V4 sh[CH * P::RW];
-  __shared__ Acc jred[NW][CH];
+  __shared__ typename P::Red jred[NW][CH];
   chain_wait();  // the records of the pack kernel (no early release: this kernel is long)
   const int4 H = items[3 * blockIdx.x];
   const int rec_off = H.x, n = H.y, sys = H.z, jbase = H.w;
@@ -236,13 +321,18 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
     const int I = t0 / T;
     const int64_t jrow = jbase + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2);
     const int len = n - t0;  // j-side row length
-    typename P::Elem tg[TPT];
-    Acc acc[TPT], sum[P::CHUNKED ? TPT : 1];
-    int idx[TPT];
+    typename P::Tgt tg[NP];
+    Acc acc[NP], sum[P::CHUNKED ? NP : 1];
+    int idx[NP][P::PACK];
 #pragma unroll
-    for (int k = 0; k < TPT; ++k) {
-      idx[k] = t0 + k * NT + threadIdx.x;
-      P::load(rec + (size_t)(rec_off + min(idx[k], n - 1)) * P::RW, tg[k]);
+    for (int k = 0; k < NP; ++k) {
+      int r[P::PACK];
+#pragma unroll
+      for (int h = 0; h < P::PACK; ++h) {
+        idx[k][h] = t0 + (k * P::PACK + h) * NT + threadIdx.x;
+        r[h] = rec_off + min(idx[k][h], n - 1);
+      }
+      P::load(rec, r, tg[k]);
       P::zero(acc[k]);
       if (P::CHUNKED) P::zero(sum[k]);
     }
@@ -256,18 +346,18 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
       for (int q = cnt + threadIdx.x; q < ((cnt + 31) & ~31); q += NT) P::template pad<CH>(sh, q);
       __syncthreads();
       if (j0 < t0 + T)
-        sym_chunk<P, TPT, CH, true>(g, tg, idx, acc, sh, cnt, j0, jred);
+        sym_chunk<P, NP, CH, true>(g, tg, idx, acc, sh, cnt, j0, jred);
       else
-        sym_chunk<P, TPT, CH, false>(g, tg, idx, acc, sh, cnt, j0, jred);
+        sym_chunk<P, NP, CH, false>(g, tg, idx, acc, sh, cnt, j0, jred);
       if (P::CHUNKED)
 #pragma unroll
-        for (int k = 0; k < TPT; ++k) {
+        for (int k = 0; k < NP; ++k) {
           P::flush(sum[k], acc[k]);
           P::zero(acc[k]);
         }
       __syncthreads();
       for (int q = threadIdx.x; q < cnt; q += NT) {
-        Acc v = jred[0][q];
+        typename P::Red v = jred[0][q];
 #pragma unroll
         for (int w = 1; w < NW; ++w) v.p = P::add(v.p, jred[w][q].p), v.q = P::add(v.q, jred[w][q].q);
         const int o = j0 + q - t0;
@@ -276,12 +366,13 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
       }
     }
 #pragma unroll
-    for (int k = 0; k < TPT; ++k)
-      if (idx[k] < n) {
-        const Acc& v = P::CHUNKED ? sum[k] : acc[k];
-        part[(size_t)ioff + idx[k] - t0] = P::out(v.p);
-        part[(size_t)ioff + T + idx[k] - t0] = P::out(v.q);
-      }
+    for (int k = 0; k < NP; ++k) {
+      int o[P::PACK];
+      bool in[P::PACK];
+#pragma unroll
+      for (int h = 0; h < P::PACK; ++h) o[h] = idx[k][h] - t0, in[h] = idx[k][h] < n;
+      P::store(part + ioff, T, o, in, P::CHUNKED ? sum[k] : acc[k]);
+    }
   }
 }
 
@@ -290,10 +381,9 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
 // A u: a = ds psi, alpha = ds phi; A^T w: a = wphi, alpha = wpsi.
 // sigma: the positions and alpha are multiplied by it (kappa-scaled records; 1 otherwise);
 // gscale: the power of two at or above sigma, by which the surface's coordinate grid grows with it
-template <typename V4, typename T>
-__global__ void k_pack_sym(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
-                           const double* __restrict__ u, V4* __restrict__ rec, const int* __restrict__ skip,
-                           int skip_stride, double sigma) {
+__global__ void k_pack_sym64(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
+                             const double* __restrict__ u, double4_32a* __restrict__ rec, const int* __restrict__ skip,
+                             int skip_stride, double sigma) {
   chain_wait();
   chain_release();
   const int k = blockIdx.y;
@@ -304,11 +394,33 @@ __global__ void k_pack_sym(const int4* __restrict__ lay, bool transpose, const d
   const double phi = u[L.z + j], psi = u[L.z + L.y + j];
   const double a = transpose ? phi : g.w * psi;
   const double al = sigma * (transpose ? psi : g.w * phi);
-  V4 r0, r1;
-  r0.x = (T)(sigma * g.x), r0.y = (T)(sigma * g.y), r0.z = (T)(sigma * g.z), r0.w = (T)a;
-  r1.x = (T)v.x, r1.y = (T)v.y, r1.z = (T)v.z, r1.w = (T)al;
-  V4* o = rec + 2 * (size_t)(L.z / 2 + j);
-  o[0] = r0, o[1] = r1;
+  double4_32a* o = rec + 2 * (size_t)(L.z / 2 + j);
+  o[0] = make_double4_32a(sigma * g.x, sigma * g.y, sigma * g.z, a);
+  o[1] = make_double4_32a(v.x, v.y, v.z, al);
+}
+
+// every value twice, with the negated fields (Sym32Policy)
+__global__ void k_pack_sym32(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
+                             const double* __restrict__ u, float4* __restrict__ rec, const int* __restrict__ skip,
+                             int skip_stride, double sigma) {
+  chain_wait();
+  chain_release();
+  const int k = blockIdx.y;
+  const int4 L = lay[k];
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= L.y || (skip != nullptr && skip[(size_t)k * skip_stride] != 0)) return;
+  const double4_32a g = tgt64[2 * (L.x + j)], v = tgt64[2 * (L.x + j) + 1];
+  const double phi = u[L.z + j], psi = u[L.z + L.y + j];
+  const float a = (float)(transpose ? phi : g.w * psi);
+  const float al = (float)(sigma * (transpose ? psi : g.w * phi));
+  const float x = (float)(sigma * g.x), y = (float)(sigma * g.y), z = (float)(sigma * g.z);
+  const float nx = (float)v.x, ny = (float)v.y, nz = (float)v.z, f = transpose ? al : -a;
+  float4* o = rec + 5 * (size_t)(L.z / 2 + j);
+  o[0] = make_float4(x, x, y, y);
+  o[1] = make_float4(z, z, a, a);
+  o[2] = make_float4(nx, nx, ny, ny);
+  o[3] = make_float4(nz, nz, -al, -al);
+  o[4] = make_float4(f, f, 0.f, 0.f);
 }
 
 __global__ void k_pack_sym_df(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
@@ -615,12 +727,16 @@ void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typena
   s->grow(recbuf, (size_t)(L.len / 2) * P::RW);
   s->grow(partbuf, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  if constexpr (std::is_same<typename P::PT, double>::value && std::is_same<typename P::V4, float4>::value) {
-    launch_chained(k_pack_sym_df, dim3(blocks_of(L.max_n, 256), L.K), 256, 0, s->stream, lay, transpose, s->tgt64.p, u,
-                   recbuf.p, skip, skip_stride, sigma, std::exp2(std::ceil(std::log2(sigma))));
+  const dim3 pgrid(blocks_of(L.max_n, 256), L.K);
+  if constexpr (std::is_same<typename P::V4, double4_32a>::value) {
+    launch_chained(k_pack_sym64, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+                   sigma);
+  } else if constexpr (std::is_same<typename P::PT, double>::value) {
+    launch_chained(k_pack_sym_df, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+                   sigma, std::exp2(std::ceil(std::log2(sigma))));
   } else {
-    launch_chained(k_pack_sym<typename P::V4, typename P::PT>, dim3(blocks_of(L.max_n, 256), L.K), 256, 0, s->stream,
-                   lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride, sigma);
+    launch_chained(k_pack_sym32, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+                   sigma);
   }
   BIPB_LAUNCHED(s);
   {
@@ -653,16 +769,25 @@ bool sym_form(double kappa, PairConst<T>& c, bool& laplace) {
 bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, double kappa, bool transpose,
                   int variant, const double* u, double* y, double dphi, double dpsi, const int* skip,
                   int skip_stride) {
-  static const int kT[3] = {512, 512, 1024};  // NT x TPT of the variants below
   if (variant < 0 || variant > 2) throw Error(BIPB_ERR_INVALID_ARG, "unknown symmetric FP32 mat-vec variant");
+  // Shapes (threads, targets per thread, tile of targets): 0 (256, 2, 512), 1
+  // (128, 4, 512), 2 (256, 4, 1024), 3 (128, 2, 256).  Variant 2 takes the
+  // shape by size.  A tile of T targets evaluates n T / 2 masked pairs of its
+  // own diagonal beside the n^2 / 2 real ones, and a small surface needs small
+  // tiles to give every SM work, while the large tile shares each source load
+  // among more targets.  Whole mat-vec, us, tile 1024 / 512 / 256: N = 1280 34.9
+  // / 26.9 / 24.7; 2500 47.2 / 37.0 / 41.1; 20480 367 / 358 / 387; 40000 1253 /
+  // 1283 / 1342; 65537 3196 / 3229 / 3702.
+  int shape = variant;
+  if (variant == 2) shape = L.max_n < 1536 ? 3 : L.max_n < 32768 ? 1 : 2;
+  static const int kT[4] = {512, 512, 1024, 256};
   PairConst<float> c = c0;
   bool lap = false;
-  if (!sym_fits(L, kT[variant]) || !sym_form(kappa, c, lap)) return false;
+  if (!sym_fits(L, kT[shape]) || !sym_form(kappa, c, lap)) return false;
   const int kind = transpose ? kTMv32T : kTMv32;
-#define BIPB_SYM32_RUN(TR_, LAP_, V_, NT_, TPT_, CH_, MINB_)                                                    \
-  run_sym<SymPolicy<float, TR_, LAP_>, NT_, TPT_, CH_, MINB_>(s, (TR_ ? 0x100 : 0x200) + V_, kind, L, {c}, TR_, \
-                                                               s->rec32, s->part32, u, y, dphi, dpsi, skip,      \
-                                                               skip_stride, kappa)
+#define BIPB_SYM32_RUN(TR_, LAP_, V_, NT_, TPT_, CH_, MINB_)                                                       \
+  run_sym<Sym32Policy<TR_, LAP_>, NT_, TPT_, CH_, MINB_>(s, (TR_ ? 0x100 : 0x200) + V_, kind, L, {c}, TR_, s->rec32, \
+                                                         s->part32, u, y, dphi, dpsi, skip, skip_stride, kappa)
 #define BIPB_SYM32(V_, NT_, TPT_, CH_, MINB_)                     \
   case V_:                                                         \
     if (transpose) {                                               \
@@ -677,10 +802,11 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
         BIPB_SYM32_RUN(false, false, V_, NT_, TPT_, CH_, MINB_);   \
     }                                                              \
     return true;
-  switch (variant) {
-    BIPB_SYM32(0, 256, 2, 64, 4)
-    BIPB_SYM32(1, 128, 4, 64, 5)
+  switch (shape) {
+    BIPB_SYM32(0, 256, 2, 64, 3)
+    BIPB_SYM32(1, 128, 4, 64, 4)
     BIPB_SYM32(2, 256, 4, 64, 2)
+    BIPB_SYM32(3, 128, 2, 32, 6)
   }
 #undef BIPB_SYM32
 #undef BIPB_SYM32_RUN
@@ -693,7 +819,7 @@ bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c0, d
   bool lap = false;
   if (!sym_fits(L, 256) || !sym_form(kappa, c, lap)) return false;
 #define BIPB_SYM64_RUN(TR_, LAP_)                                                                                \
-  run_sym<SymPolicy<double, TR_, LAP_>, 128, 2, 64, 1>(s, TR_ ? 0x300 : 0x400, TR_ ? kTMv64T : kTMv64, L, {c}, TR_, \
+  run_sym<Sym64Policy<TR_, LAP_>, 128, 2, 64, 1>(s, TR_ ? 0x300 : 0x400, TR_ ? kTMv64T : kTMv64, L, {c}, TR_, \
                                                       s->rec64, s->part64, u, y, dphi, dpsi, skip, skip_stride,     \
                                                       kappa)
   if (transpose) {

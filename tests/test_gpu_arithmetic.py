@@ -82,3 +82,25 @@ def test_double_float_matvec_grid_scales_with_the_surface(bipb, orc, scale):
             for k, (c, n, a) in enumerate(parts):
                 ref = f(c, n, a, 80.0, kappa, u.reshape(2, -1)[k])
                 np.testing.assert_allclose(y[k], ref, rtol=0, atol=2e-12 * np.abs(ref).max(), err_msg=f"{transpose} {k}")
+
+
+@pytest.mark.parametrize("n", [2, 3, 31, 33, 255, 257, 513, 1279, 1535, 1536, 1537])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_fp32_symmetric_shapes_small_and_ragged(bipb, orc, n, transpose):
+    """Every shape of the packed symmetric FP32 mat-vec (and the default's choice by
+    size) on surfaces around its tiles of 256 and 512 targets, its chunks of 32 and 64
+    sources and the line between shapes: the FP32 bounds of test_matvec_fp64_and_fp32."""
+    p = synth.protein_like_problem(level=4, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, n, replace=False))
+    c, nv, a = p.centroids[keep], p.normals[keep], p.areas[keep]
+    u = np.random.default_rng(3).standard_normal(2 * n)
+    for kappa in (p.kappa, 0.0):
+        ref = (orc.matvec_t if transpose else orc.matvec)(c, nv, a, 80.0, kappa, u)
+        with bipb.Surface(c, nv, a) as s:
+            for variant in (7, 8, 9):
+                s.set_variant(variant)
+                y = _dev(np.zeros_like(u))
+                s.matvec(_dev(u), y, precision=bipb.FP32, transpose=transpose, med=bipb.medium(1.0, 80.0, kappa))
+                y = y.cpu().numpy()
+                assert np.linalg.norm(y - ref) < 3e-6 * np.linalg.norm(ref), (variant, kappa)
+                assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max(), (variant, kappa)
