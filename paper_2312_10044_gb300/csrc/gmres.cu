@@ -27,12 +27,14 @@
 #include <mutex>
 
 #include "internal.cuh"
+#include "symstep.cuh"
 
 namespace bipb {
 
 namespace {
 
 constexpr int kBS = 256;
+constexpr double kInv4PiG = 1.0 / (4.0 * kPi);
 
 struct DevState {
   int k;       // Arnoldi steps done in this cycle
@@ -53,8 +55,9 @@ struct DevState {
 constexpr int kStateInts = (int)(sizeof(DevState) / sizeof(int));
 static_assert(offsetof(DevState, skip) == sizeof(int), "skip must be the second int");
 
+template <int NT>
 __device__ double block_sum(double v) {
-  __shared__ double red[kBS / 32];
+  __shared__ double red[NT / 32];
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __syncthreads();
@@ -62,15 +65,16 @@ __device__ double block_sum(double v) {
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x < 32) {
-    t = threadIdx.x < kBS / 32 ? red[threadIdx.x] : 0.0;
+    t = threadIdx.x < NT / 32 ? red[threadIdx.x] : 0.0;
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
   }
   return t;  // valid in thread 0
 }
 
-// Block table: blk[b] = {system, start, end, first block of the system},
-// sysb[k] = {first block, end block, 0, 0}.  Every block covers one
-// contiguous range of one system's unknowns.
+// Block table: blk[b] = {system, first element, end element, first block of
+// the system}, sysb[k] = {first block, end block, 0, 0}, lay[k] = {geo_off, n,
+// vec_off, chg_off}.  A block owns a range of one system's elements: their phi
+// unknowns vec_off + e and their psi unknowns vec_off + n + e.
 
 // Sum of v over a warp in a fixed order (tree of shuffles down), then
 // broadcast from lane 0, so every lane holds the same, reproducible value.
@@ -80,24 +84,35 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // sum over blocks b in [b0, b1) of part[b * stride + i], by one warp, fixed order
-__device__ __forceinline__ double warp_sum_parts(const double* __restrict__ part, int stride, int i, int b0, int b1) {
+__device__ __forceinline__ double warp_sum_parts(const double* part, int stride, int i, int b0, int b1) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
+#pragma unroll 4
   for (int b = b0 + lane; b < b1; b += 32) s += part[(size_t)b * stride + i];
-  return warp_sum(s);
+  if (b1 - b0 > 8) return warp_sum(s);
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);  // lanes 0..7 hold all of it
+  return __shfl_sync(0xffffffffu, s, 0);
 }
 
-// part[b * m1 + i] = V_i . w over block b's range, i <= j (warp i % 8 takes vector i)
-__device__ __forceinline__ void block_dots(int j, int m1, int64_t len, const double* __restrict__ V,
-                                           const double* w, double* __restrict__ part, int4 B) {
+// part[b * m1 + i] = V_i . w over block b's unknowns, i <= j: one warp per
+// vector and half (phi, psi), the two halves added at the end.  V and w hold
+// values that other threads of the cluster or block wrote in this kernel.
+template <int NT>
+__device__ __forceinline__ void block_dots(int j, int m1, int64_t len, const double* V, const double* w,
+                                           double* part, int b, int4 B, int4 Lk) {
+  __shared__ double half[2 * (kMaxRestart + 1)];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = warp; i <= j; i += kBS / 32) {
-    const double* v = V + (size_t)i * len;
+  for (int t = warp; t < 2 * (j + 1); t += NT / 32) {
+    const int64_t o = Lk.z + (t & 1) * Lk.y;
+    const double *v = V + (size_t)(t >> 1) * len + o, *x = w + o;
     double acc = 0.0;
-    for (int x = B.y + lane; x < B.z; x += 32) acc += v[x] * w[x];
+#pragma unroll 4
+    for (int e = B.y + lane; e < B.z; e += 32) acc += v[e] * x[e];
     acc = warp_sum(acc);
-    if (lane == 0) part[(size_t)blockIdx.x * m1 + i] = acc;
+    if (lane == 0) half[t] = acc;
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i <= j; i += NT) part[(size_t)b * m1 + i] = half[2 * i] + half[2 * i + 1];
 }
 
 // Preconditioning by the element self blocks (Sec. 2.2.4 with one element per
@@ -105,80 +120,91 @@ __device__ __forceinline__ void block_dots(int j, int m1, int64_t len, const dou
 // diag(1/2 (1 + eps), 1/2 (1 + 1/eps)), so M^-1 scales the phi rows by pre.x
 // and the psi rows by pre.y.  It is applied on the right, A M^-1 y = r,
 // d = M^-1 y: GMRES then minimises the true residual, which is what the
-// stopping tests and the refinement read.  lay[k] = {geo_off, n, vec_off,
-// chg_off} of system k.
-__device__ __forceinline__ double precond_factor(int x, int4 Lk, double2 pre) {
-  return (x - Lk.z < Lk.y) ? pre.x : pre.y;
-}
+// stopping tests and the refinement read.
 
-__global__ void k_dots(int j, int m1, int64_t len, const double* __restrict__ V, const double* __restrict__ w,
-                       double* __restrict__ part, const DevState* st, const int4* __restrict__ blk) {
-  chain_wait();
-  chain_release();
-  const int4 B = blk[blockIdx.x];
-  if (st[B.x].skip) return;
-  block_dots(j, m1, len, V, w, part, B);
+// One Arnoldi step after the mat-vec, in three phases with a reduction over the
+// system's blocks between them: the dot products V^T w (with FUSED, w first
+// summed from the symmetric FP32 mat-vec's partial sums); w -= V h and ||w||;
+// the next basis vector, the Givens rotation and (FUSED) the next mat-vec's
+// records.  As three kernels (a block per about 128 elements), or, for small
+// systems, as one kernel with one cluster of CTAs per system, whose barrier
+// takes the place of the kernel boundaries.
+struct StepArgs {
+  int j, m;
+  int64_t len;
+  double *V, *w;
+  double *part, *part2, *part1;  // per block: dots, second-pass dots, norm
+  double *H, *cs, *sn, *g;
+  DevState* st;
+  const int4 *blk, *sysb, *lay;
+  double* tz;    // M^-1 v_{j+1} (preconditioned), or nullptr
+  double2 pre;   // M^-1
+  SymStep mv;    // FUSED: the symmetric mat-vec
+  const double* u;  // FUSED: its input
+  const double4_32a* tgt64;
+};
+
+template <int NT, bool FUSED>
+__device__ __forceinline__ void step_dots(const StepArgs& a, int b, int4 B, int4 Lk) {
+  if (FUSED) {
+    const int4 S = a.mv.tab[B.x];
+    const int cnt = B.z - B.y;
+    for (int t = threadIdx.x; t < 2 * cnt; t += NT) {
+      const int c = t < cnt ? 0 : 1, e = B.y + t - c * cnt;
+      const double acc = sym_sum(a.mv.tab, S, a.mv.part, e, c);
+      const double sc = kInv4PiG * (a.mv.transpose ? a.tgt64[2 * (Lk.x + e)].w : 1.0);
+      const int64_t x = Lk.z + (int64_t)c * Lk.y + e;
+      a.w[x] = (c ? a.mv.dpsi : a.mv.dphi) * a.u[x] - sc * (c ? a.mv.f.y : a.mv.f.x) * acc;
+    }
+    __syncthreads();  // the block's w is visible to all its threads
+  }
+  block_dots<NT>(a.j, a.m + 1, a.len, a.V, a.w, a.part, b, B, Lk);
 }
 
 // h_i = sum over the system's blocks of part[.][i]; w -= sum_i h_i V_i; H[:, j] (+)= h;
-// with want_norm, also part1[b] = sum of the updated w^2 over block b's range;
-// with part_next, also the block's dot products of the updated w for the
-// second Gram-Schmidt pass (block-local, so they need no extra launch).
-__global__ void k_orth(int j, int m, int64_t len, const double* __restrict__ V, double* __restrict__ w,
-                       const double* __restrict__ part, double* __restrict__ H, int accumulate, const DevState* st,
-                       const int4* __restrict__ blk, const int4* __restrict__ sysb, double* __restrict__ part1,
-                       int want_norm, double* __restrict__ part_next) {
-  chain_wait();
-  chain_release();
-  const int4 B = blk[blockIdx.x];
-  if (st[B.x].skip) return;
-  const int m1 = m + 1;
-  const int4 S = sysb[B.x];
+// with NORM, also part1[b] = sum of the updated w^2 over block b's unknowns;
+// otherwise the block's dot products of the updated w for the second
+// Gram-Schmidt pass (block-local, so they need no reduction in between).
+template <int NT, bool NORM>
+__device__ __forceinline__ void step_orth(const StepArgs& a, const double* part, int accumulate, int b, int4 B,
+                                          int4 S, int4 Lk) {
+  const int j = a.j, m1 = a.m + 1;
   __shared__ double h[kMaxRestart + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = warp; i <= j; i += kBS / 32) {
+  __syncthreads();  // h of an earlier phase has been read
+  for (int i = warp; i <= j; i += NT / 32) {
     const double v = warp_sum_parts(part, m1, i, S.x, S.y);
     if (lane == 0) h[i] = v;
   }
   __syncthreads();
-  if ((int)blockIdx.x == S.x) {
-    double* Hs = H + (size_t)B.x * m1 * m + (size_t)j * m1;
-    for (int i = threadIdx.x; i <= j; i += kBS) Hs[i] = accumulate ? Hs[i] + h[i] : h[i];
+  if (b == S.x) {
+    double* Hs = a.H + (size_t)B.x * m1 * a.m + (size_t)j * m1;
+    for (int i = threadIdx.x; i <= j; i += NT) Hs[i] = accumulate ? Hs[i] + h[i] : h[i];
   }
   double ss = 0.0;
-  for (int x = B.y + threadIdx.x; x < B.z; x += kBS) {
-    double acc = w[x];
-    for (int i = 0; i <= j; ++i) acc -= h[i] * V[(size_t)i * len + x];
-    w[x] = acc;
-    ss += acc * acc;
+  const int cnt = B.z - B.y;
+  for (int t = threadIdx.x; t < 2 * cnt; t += NT) {
+    const int64_t x = Lk.z + B.y + (t < cnt ? t : t - cnt + Lk.y);
+    double p = a.w[x];
+#pragma unroll 8
+    for (int i = 0; i <= j; ++i) p -= h[i] * a.V[(size_t)i * a.len + x];
+    a.w[x] = p;
+    ss += p * p;
   }
-  if (want_norm) {
-    ss = block_sum(ss);
-    if (threadIdx.x == 0) part1[blockIdx.x] = ss;
-  }
-  if (part_next != nullptr) {
+  if (NORM) {
+    ss = block_sum<NT>(ss);
+    if (threadIdx.x == 0) a.part1[b] = ss;
+  } else {
     __syncthreads();  // the block's updated w is visible to all its threads
-    block_dots(j, m1, len, V, w, part_next, B);
+    block_dots<NT>(j, m1, a.len, a.V, a.w, a.part2, b, B, Lk);
   }
-}
-
-// part1[b] = sum of w^2 over block b's range (mode 0: systems not skipped,
-// mode 1: active systems, mode 2: every system)
-__global__ void k_sumsq(const double* __restrict__ w, double* __restrict__ part1, const DevState* st,
-                        const int4* __restrict__ blk, int mode) {
-  const int4 B = blk[blockIdx.x];
-  if ((mode == 0 && st[B.x].skip) || (mode == 1 && !st[B.x].active)) return;
-  double acc = 0.0;
-  for (int x = B.y + threadIdx.x; x < B.z; x += kBS) acc += w[x] * w[x];
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) part1[blockIdx.x] = acc;
 }
 
 // Per system: apply earlier rotations to column j, make rotation j, update g,
 // test.  The column (j + 2 entries, h[j + 1] = ||w||) and the earlier
 // rotations are in shared memory (ch, csh, snh), staged by the caller's
 // block in parallel, so the serial recurrence waits on no global load.
-__device__ void givens_step(int j, int m, int sys, double* ch, const double* csh, const double* snh,
+__device__ void givens_step(int j, int m, int sys, const double* ch, const double* csh, const double* snh,
                             double* __restrict__ H, double* __restrict__ cs, double* __restrict__ sn,
                             double* __restrict__ g, DevState* __restrict__ st) {
   DevState& S = st[sys];
@@ -187,15 +213,21 @@ __device__ void givens_step(int j, int m, int sys, double* ch, const double* csh
   double* g_ = g + (size_t)sys * m1;
   const double gj = g_[j], bnorm = S.bnorm, tol = S.tol;
   const int iters = S.iters + 1, max_iter = S.max_iter, Sm = S.m;
+  double a = ch[0];
   for (int i = 0; i < j; ++i) {
-    const double t = csh[i] * ch[i] + snh[i] * ch[i + 1];
-    ch[i + 1] = -snh[i] * ch[i] + csh[i] * ch[i + 1];
-    ch[i] = t;
+    const double c = csh[i], t = snh[i], x = ch[i + 1];
+    h[i] = c * a + t * x;
+    a = c * x - t * a;
   }
-  const double a = ch[j], b = ch[j + 1];
-  const double den = hypot(a, b);
-  const double c = den > 0.0 ? a / den : 1.0, s = den > 0.0 ? b / den : 0.0;
-  for (int i = 0; i < j; ++i) h[i] = ch[i];
+  const double b = ch[j + 1];
+  // den = sqrt(a^2 + b^2) = |(a, b)| of the pair scaled by a power of two near its larger part
+  const int big = max((__double2hiint(a) >> 20) & 0x7ff, (__double2hiint(b) >> 20) & 0x7ff);
+  const int up = min(max(big, 1), 2045);
+  const double down = __hiloint2double((2046 - up) << 20, 0), back = __hiloint2double(up << 20, 0);  // 2^(1023 - up), 2^(up - 1023)
+  const double as = a * down, bs = b * down, q = as * as + bs * bs;
+  const double inv = q > 0.0 ? rsqrt(q) : 0.0;
+  const double den = q * inv * back;
+  const double c = q > 0.0 ? as * inv : 1.0, s = bs * inv;
   h[j] = den;
   h[j + 1] = 0.0;
   cs[(size_t)sys * m + j] = c;
@@ -214,93 +246,212 @@ __device__ void givens_step(int j, int m, int sys, double* ch, const double* csh
   if (conv || stop || j + 1 == Sm) S.skip = 1;
 }
 
-// out = w / ||w|| per system (and tz = M^-1 out when preconditioned); j >= 0:
-// H[j+1, j] = ||w|| and the Givens step of
-// column j, both by the last block of the system to finish (every block has
-// then passed its skip test, so the step may set skip; the blocks' arrival
-// is counted with an atomic after a fence, no block waits); j < 0: start of
-// a cycle, beta = ||w|| (and bnorm = ||w|| if set_bnorm).
-__global__ void k_normalize(int j, int m, const double* __restrict__ w, double* __restrict__ out,
-                            const double* __restrict__ part1, double* __restrict__ H, DevState* st,
-                            const int4* __restrict__ blk, const int4* __restrict__ sysb, int set_bnorm,
-                            double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-                            double* __restrict__ tz, const int4* __restrict__ lay, double2 pre) {
-  chain_wait();
-  chain_release();
-  const int4 B = blk[blockIdx.x];
-  if (j >= 0 ? st[B.x].skip : !st[B.x].active) return;
-  const int4 S = sysb[B.x];
-  __shared__ double nrm;
+// (||w||, 1 / ||w||) of the system from the blocks' sums, in every thread (0, 0 for w = 0)
+__device__ __forceinline__ double2 step_norm(const double* part1, int4 S) {
+  __shared__ double2 nrm;
   if (threadIdx.x < 32) {
     const double s = warp_sum_parts(part1, 1, 0, S.x, S.y);
-    if (threadIdx.x == 0) nrm = sqrt(s);
+    if (threadIdx.x == 0) {
+      const double inv = s > 0.0 ? rsqrt(s) : 0.0;
+      nrm = make_double2(s * inv, inv);
+    }
   }
   __syncthreads();
-  const double v = nrm;
-  const double inv = v > 0.0 ? 1.0 / v : 0.0;
-  for (int x = B.y + threadIdx.x; x < B.z; x += kBS) out[x] = w[x] * inv;
-  if (tz != nullptr) {  // the next mat-vec's input M^-1 out
-    const int4 Lk = lay[B.x];
-    for (int x = B.y + threadIdx.x; x < B.z; x += kBS) tz[x] = precond_factor(x, Lk, pre) * (w[x] * inv);
-  }
-  if (j < 0) {
-    if (threadIdx.x == 0 && (int)blockIdx.x == S.x) {
-      if (set_bnorm) st[B.x].bnorm = v;
-      st[B.x].beta = v;
+  return nrm;
+}
+
+// v_{j+1} = inv w (and tz = M^-1 v_{j+1} when preconditioned, and FUSED the
+// next mat-vec's records), by the block's first NT threads.
+template <int NT, bool FUSED>
+__device__ __forceinline__ void step_next(const StepArgs& a, double inv, int4 B, int4 Lk) {
+  double* out = a.V + (size_t)(a.j + 1) * a.len;
+  const bool pack = FUSED && a.j + 1 < a.m;
+  for (int e = B.y + threadIdx.x; e < B.z; e += NT) {
+    const int64_t x = Lk.z + e, y = x + Lk.y;
+    double p = a.w[x] * inv, q = a.w[y] * inv;
+    out[x] = p;
+    out[y] = q;
+    if (a.tz != nullptr) {
+      p *= a.pre.x;
+      q *= a.pre.y;
+      a.tz[x] = p;
+      a.tz[y] = q;
     }
-    return;
+    if (pack)
+      sym32_refresh(a.tgt64[2 * (Lk.x + e)].w, p, q, a.mv.transpose, a.mv.sigma,
+                    a.mv.rec + 5 * (size_t)(Lk.z / 2 + e));
   }
+}
+
+// H[j+1, j] = ||w|| and the Givens step of column j, by one warp of the system
+__device__ __forceinline__ void step_givens(const StepArgs& a, int sys, double norm) {
+  __shared__ double ch[kMaxRestart + 2], csh[kMaxRestart], snh[kMaxRestart];
+  const int j = a.j, m = a.m, lane = threadIdx.x & 31;
+  const double* Hc = a.H + (size_t)sys * (m + 1) * m + (size_t)j * (m + 1);
+  for (int i = lane; i <= j; i += 32) ch[i] = Hc[i];
+  for (int i = lane; i < j; i += 32) csh[i] = a.cs[(size_t)sys * m + i], snh[i] = a.sn[(size_t)sys * m + i];
+  if (lane == 0) ch[j + 1] = norm;
+  __syncwarp();
+  if (lane == 0) givens_step(j, m, sys, ch, csh, snh, a.H, a.cs, a.sn, a.g, a.st);
+}
+
+template <bool FUSED>
+__global__ void __launch_bounds__(kBS) k_dots(StepArgs a) {
+  chain_wait();
+  chain_release();
+  const int4 B = a.blk[blockIdx.x];
+  if (a.st[B.x].skip) return;
+  step_dots<kBS, FUSED>(a, blockIdx.x, B, a.lay[B.x]);
+}
+
+template <bool NORM>
+__global__ void __launch_bounds__(kBS) k_orth(StepArgs a, const double* part, int accumulate) {
+  chain_wait();
+  chain_release();
+  const int4 B = a.blk[blockIdx.x];
+  if (a.st[B.x].skip) return;
+  step_orth<kBS, NORM>(a, part, accumulate, blockIdx.x, B, a.sysb[B.x], a.lay[B.x]);
+}
+
+// The Givens step is made by the last block of the system to finish (every
+// block has then passed its skip test, so the step may set skip; the blocks'
+// arrival is counted with an atomic after a fence, no block waits).
+template <bool FUSED>
+__global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
+  chain_wait();
+  chain_release();
+  const int4 B = a.blk[blockIdx.x];
+  if (a.st[B.x].skip) return;
+  const int4 S = a.sysb[B.x];
+  const double2 v = step_norm(a.part1, S);
+  step_next<kBS, FUSED>(a, v.y, B, a.lay[B.x]);
   __shared__ int last;
   if (threadIdx.x == 0) {
     __threadfence();
-    last = atomicAdd(&st[B.x].arrive, 1) == S.y - S.x - 1;
+    last = atomicAdd(&a.st[B.x].arrive, 1) == S.y - S.x - 1;
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  __shared__ double ch[kMaxRestart + 1], csh[kMaxRestart], snh[kMaxRestart];
-  const double* Hc = H + (size_t)B.x * (m + 1) * m + (size_t)j * (m + 1);
-  for (int i = threadIdx.x; i <= j; i += kBS) ch[i] = Hc[i];
-  for (int i = threadIdx.x; i < j; i += kBS) csh[i] = cs[(size_t)B.x * m + i], snh[i] = sn[(size_t)B.x * m + i];
-  if (threadIdx.x == 0) ch[j + 1] = v;
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  st[B.x].arrive = 0;
-  givens_step(j, m, B.x, ch, csh, snh, H, cs, sn, g, st);
+  if (threadIdx.x == 0) a.st[B.x].arrive = 0;
+  if (threadIdx.x < 32) step_givens(a, B.x, v.x);
 }
 
-// Per system: least squares R y = g (k x k) and the restart coefficients
-// z = Q^T (g_k e_k) / |g_k|.
-__global__ void k_lsq(int m, int K, const double* __restrict__ H, const double* __restrict__ cs,
+// The whole step in one launch: a cluster of kClu CTAs per system (its blocks).
+// The cluster barrier orders the phases and makes each CTA's partial sums,
+// w and H visible to the others.
+constexpr int kClu = 8;      // CTAs of a cluster (the portable size)
+constexpr int kCluNT = 512;  // threads of each
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <bool CGS2, bool FUSED>
+__global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluNT) k_step(StepArgs a) {
+  chain_wait();
+  chain_release();
+  const int4 B = a.blk[blockIdx.x];
+  if (a.st[B.x].skip) return;  // the same for every CTA of the cluster
+  const int4 S = a.sysb[B.x], Lk = a.lay[B.x];
+  step_dots<kCluNT, FUSED>(a, blockIdx.x, B, Lk);
+  cluster_sync();
+  if (CGS2) {
+    step_orth<kCluNT, false>(a, a.part, 0, blockIdx.x, B, S, Lk);
+    cluster_sync();
+    step_orth<kCluNT, true>(a, a.part2, 1, blockIdx.x, B, S, Lk);
+  } else {
+    step_orth<kCluNT, true>(a, a.part, 0, blockIdx.x, B, S, Lk);
+  }
+  cluster_sync();  // also: every CTA has passed its skip test
+  // the last warp of the system's first block makes the Givens step beside the others' vector work
+  const double2 v = step_norm(a.part1, S);
+  if (threadIdx.x < kCluNT - 32)
+    step_next<kCluNT - 32, FUSED>(a, v.y, B, Lk);
+  else if ((int)blockIdx.x == S.x)
+    step_givens(a, B.x, v.x);
+}
+
+// part1[b] = sum of w^2 over block b's unknowns (mode 0: systems not skipped,
+// mode 1: active systems, mode 2: every system)
+__global__ void k_sumsq(const double* __restrict__ w, double* __restrict__ part1, const DevState* st,
+                        const int4* __restrict__ blk, const int4* __restrict__ lay, int mode) {
+  const int4 B = blk[blockIdx.x];
+  if ((mode == 0 && st[B.x].skip) || (mode == 1 && !st[B.x].active)) return;
+  const int4 Lk = lay[B.x];
+  double acc = 0.0;
+  for (int e = B.y + threadIdx.x; e < B.z; e += kBS) {
+    const double p = w[Lk.z + e], q = w[Lk.z + Lk.y + e];
+    acc += p * p + q * q;
+  }
+  acc = block_sum<kBS>(acc);
+  if (threadIdx.x == 0) part1[blockIdx.x] = acc;
+}
+
+// Start of a solve, per active system: beta = bnorm = ||r0||, v_0 = r0 / beta
+// (and tz = M^-1 v_0 when preconditioned).
+__global__ void k_start(const double* __restrict__ r0, double* __restrict__ V, const double* __restrict__ part1,
+                        DevState* st, const int4* __restrict__ blk, const int4* __restrict__ sysb,
+                        const int4* __restrict__ lay, double* __restrict__ tz, double2 pre) {
+  const int4 B = blk[blockIdx.x];
+  if (!st[B.x].active) return;
+  const int4 S = sysb[B.x], Lk = lay[B.x];
+  const double2 v = step_norm(part1, S);
+  const double inv = v.y;
+  for (int e = B.y + threadIdx.x; e < B.z; e += kBS) {
+    const int64_t x = Lk.z + e, y = x + Lk.y;
+    const double p = r0[x] * inv, q = r0[y] * inv;
+    V[x] = p;
+    V[y] = q;
+    if (tz != nullptr) tz[x] = pre.x * p, tz[y] = pre.y * q;
+  }
+  if (threadIdx.x == 0 && (int)blockIdx.x == S.x) {
+    st[B.x].bnorm = v.x;
+    st[B.x].beta = v.x;
+  }
+}
+
+// Per system (one block): least squares R y = g (k x k) and the restart
+// coefficients z = Q^T (g_k e_k) / |g_k|, from shared copies of the rotations
+// and of g (one thread makes the serial recurrences).
+__global__ void __launch_bounds__(64) k_lsq(int m, const double* __restrict__ H, const double* __restrict__ cs,
                       const double* __restrict__ sn, const double* __restrict__ g, double* __restrict__ y,
                       double* __restrict__ z, DevState* st) {
-  const int sys = blockIdx.x * blockDim.x + threadIdx.x;
-  if (sys >= K) return;
+  chain_wait();
+  chain_release();
+  const int sys = blockIdx.x;
   DevState& S = st[sys];
   const int k = S.k;
   if (!S.active || k == 0) return;
   const int m1 = m + 1;
+  __shared__ double c_[kMaxRestart], s_[kMaxRestart], r_[kMaxRestart + 1], z_[kMaxRestart + 1];
   const double* Hs = H + (size_t)sys * m1 * m;
-  const double* c_ = cs + (size_t)sys * m;
-  const double* s_ = sn + (size_t)sys * m;
-  const double* g_ = g + (size_t)sys * m1;
-  double* y_ = y + (size_t)sys * m;
-  double* z_ = z + (size_t)sys * m1;
-  for (int i = k - 1; i >= 0; --i) {
-    double s = g_[i];
-    for (int l = i + 1; l < k; ++l) s -= Hs[(size_t)l * m1 + i] * y_[l];
-    y_[i] = s / Hs[(size_t)i * m1 + i];
+  for (int i = threadIdx.x; i <= k; i += 64) {
+    if (i < k) c_[i] = cs[(size_t)sys * m + i], s_[i] = sn[(size_t)sys * m + i];
+    r_[i] = g[(size_t)sys * m1 + i];
   }
-  const double gk = g_[k];
-  const double beta = fabs(gk);
-  for (int i = 0; i <= k; ++i) z_[i] = 0.0;
-  z_[k] = beta > 0.0 ? gk / beta : 0.0;
-  for (int i = k - 1; i >= 0; --i) {
-    double a = z_[i], b = z_[i + 1];
-    z_[i] = c_[i] * a - s_[i] * b;
-    z_[i + 1] = s_[i] * a + c_[i] * b;
+  __syncthreads();
+  const double gk = r_[k], beta = fabs(gk);
+  if (threadIdx.x >= 32) {  // second warp: the restart coefficients
+    if (threadIdx.x == 32) {
+      for (int i = 0; i <= k; ++i) z_[i] = 0.0;
+      z_[k] = beta > 0.0 ? gk / beta : 0.0;
+      for (int i = k - 1; i >= 0; --i) {
+        const double a = z_[i], b = z_[i + 1];
+        z_[i] = c_[i] * a - s_[i] * b;
+        z_[i + 1] = s_[i] * a + c_[i] * b;
+      }
+      S.beta = beta;
+    }
+    __syncwarp();
+    for (int i = threadIdx.x - 32; i <= k; i += 32) z[(size_t)sys * m1 + i] = z_[i];
+  } else {  // first warp: back substitution by columns, the solved entries in r_
+    for (int i = k - 1; i >= 0; --i) {
+      const double yi = r_[i] / Hs[(size_t)i * m1 + i];
+      __syncwarp();
+      for (int l = threadIdx.x; l < i; l += 32) r_[l] -= Hs[(size_t)i * m1 + l] * yi;
+      if (threadIdx.x == 0) y[(size_t)sys * m + i] = yi;
+      __syncwarp();
+    }
   }
-  S.beta = beta;
 }
 
 // x += M^-1 sum_{i<k} y_i V_i ; V_0 <- sum_{i<=k} z_i V_i (per system); when
@@ -309,31 +460,40 @@ __global__ void k_update(int m, int64_t len, double* __restrict__ V, double* __r
                          const double* __restrict__ y, const double* __restrict__ z, const DevState* st,
                          const int4* __restrict__ blk, double* __restrict__ tz, const int4* __restrict__ lay,
                          double2 pre) {
+  chain_wait();
+  chain_release();
   const int4 B = blk[blockIdx.x];
   const DevState& S = st[B.x];
   const int k = S.k;
   if (!S.active || k == 0) return;
+  const int4 Lk = lay[B.x];
   const double* y_ = y + (size_t)B.x * m;
   const double* z_ = z + (size_t)B.x * (m + 1);
-  for (int e = B.y + threadIdx.x; e < B.z; e += kBS) {
-    double dx = 0.0, v0 = 0.0;
-    for (int i = 0; i <= k; ++i) {
-      double v = V[(size_t)i * len + e];
-      if (i < k) dx += y_[i] * v;
-      v0 += z_[i] * v;
+  for (int c = 0; c < 2; ++c) {
+    const double f = c ? pre.y : pre.x;
+    for (int o = B.y + threadIdx.x; o < B.z; o += kBS) {
+      const int64_t e = Lk.z + c * Lk.y + o;
+      double dx = 0.0, v0 = 0.0;
+#pragma unroll 4
+      for (int i = 0; i <= k; ++i) {
+        double v = V[(size_t)i * len + e];
+        if (i < k) dx += y_[i] * v;
+        v0 += z_[i] * v;
+      }
+      if (tz != nullptr) {
+        x[e] += f * dx;
+        tz[e] = f * v0;
+      } else {
+        x[e] += dx;
+      }
+      V[e] = v0;
     }
-    if (tz != nullptr) {
-      const double f = precond_factor(e, lay[B.x], pre);
-      x[e] += f * dx;
-      tz[e] = f * v0;
-    } else {
-      x[e] += dx;
-    }
-    V[e] = v0;
   }
 }
 
 __global__ void k_next_cycle(int m, int K, double* __restrict__ g, DevState* st) {
+  chain_wait();
+  chain_release();
   const int sys = blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= K) return;
   DevState& S = st[sys];
@@ -378,11 +538,12 @@ struct Recorded {
 
 struct GmresWork {
   uint64_t lay_key = 0;
-  int m = 0, K = 0, nblk = 0;
+  int m = 0, K = 0, nblk = 0;  // nblk: blocks of blk
   int precond = 0;  // bipb_precond of the current call
   int64_t len = 0;
   DevBuf<double> V, w, H, cs, sn, g, y, z, part, part2, part1, r, d, t, tz;
-  DevBuf<int4> blk, sysb;
+  DevBuf<int4> blk, sysb;      // blocks of about 128 elements
+  DevBuf<int4> cblk, csysb;    // kClu blocks per system (the cluster step)
   DevBuf<int> mask;  // per system: 1 = leave out of the FP64 residual
   std::vector<int4> sysb_host;
   DevBuf<DevState> st_buf;
@@ -478,19 +639,20 @@ GmresWork* workspace(Surface* s, const SysLayout& L, int m) {
   w->m = m;
   w->K = L.K;
   w->len = L.len;
-  // blocks: each covers one contiguous range (about 256 unknowns, at most
-  // 1024 blocks per system) of one system
-  std::vector<int4> blk;
-  std::vector<int4> sysb(L.K);
+  // blocks: each covers a range of one system's elements, about 128 of them (at
+  // most 1024 blocks per system); for the cluster step, kClu blocks per system
+  std::vector<int4> blk, cblk;
+  std::vector<int4> sysb(L.K), csysb(L.K);
   for (int k = 0; k < L.K; ++k) {
-    const int64_t lk = 2 * (int64_t)L.n[k];
-    const int nb = (int)std::min<int64_t>(1024, std::max<int64_t>(1, (lk + 255) / 256));
-    const int64_t chunk = (lk + nb - 1) / nb;
-    sysb[k] = make_int4((int)blk.size(), (int)blk.size() + nb, 0, 0);
-    for (int b = 0; b < nb; ++b) {
-      const int64_t a = L.vec_off[k] + b * chunk, e = std::min<int64_t>(L.vec_off[k] + lk, a + chunk);
-      blk.push_back(make_int4(k, (int)a, (int)e, sysb[k].x));
-    }
+    const int n = L.n[k];
+    auto cut = [&](int nb, std::vector<int4>& out, int4& range) {
+      const int chunk = (n + nb - 1) / nb, first = (int)out.size();
+      range = make_int4(first, first + nb, 0, 0);
+      for (int b = 0; b < nb; ++b)
+        out.push_back(make_int4(k, std::min(n, b * chunk), std::min(n, (b + 1) * chunk), first));
+    };
+    cut(std::min(1024, std::max(1, (n + 127) / 128)), blk, sysb[k]);
+    cut(kClu, cblk, csysb[k]);
   }
   w->nblk = (int)blk.size();
   w->sysb_host = sysb;
@@ -507,11 +669,14 @@ GmresWork* workspace(Surface* s, const SysLayout& L, int m) {
   w->g.ensure((size_t)L.K * (m + 1), s->stream);
   w->y.ensure((size_t)L.K * m, s->stream);
   w->z.ensure((size_t)L.K * (m + 1), s->stream);
-  w->part.ensure((size_t)w->nblk * (m + 1), s->stream);
-  w->part2.ensure((size_t)w->nblk * (m + 1), s->stream);
-  w->part1.ensure(w->nblk, s->stream);
+  const size_t nb_max = std::max(blk.size(), cblk.size());
+  w->part.ensure(nb_max * (m + 1), s->stream);
+  w->part2.ensure(nb_max * (m + 1), s->stream);
+  w->part1.ensure(nb_max, s->stream);
   w->blk.ensure(blk.size(), s->stream);
   w->sysb.ensure(L.K, s->stream);
+  w->cblk.ensure(cblk.size(), s->stream);
+  w->csysb.ensure(L.K, s->stream);
   w->mask.ensure(L.K, s->stream);
   w->st_buf.ensure(L.K, s->stream);
   w->st = w->st_buf.p;
@@ -520,6 +685,8 @@ GmresWork* workspace(Surface* s, const SysLayout& L, int m) {
   w->mask_host.resize(L.K);
   BIPB_CUDA(cudaMemcpyAsync(w->blk.p, blk.data(), blk.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
   BIPB_CUDA(cudaMemcpyAsync(w->sysb.p, sysb.data(), sysb.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
+  BIPB_CUDA(cudaMemcpyAsync(w->cblk.p, cblk.data(), cblk.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
+  BIPB_CUDA(cudaMemcpyAsync(w->csysb.p, csysb.data(), csysb.size() * sizeof(int4), cudaMemcpyHostToDevice, s->stream));
   BIPB_CUDA(cudaStreamSynchronize(s->stream));
   ++s->alloc_gen;
   return w;
@@ -532,47 +699,76 @@ double2 precond_factors(const bipb_medium& m) {
   return make_double2(2.0 / (1.0 + eps), 2.0 / (1.0 + 1.0 / eps));
 }
 
+// Whether one cluster per system takes an Arnoldi step in one launch.  GB300
+// has two FP64 lanes per SM, so eight SMs make the (j + 1) 4n multiply-adds of a
+// step as fast as the three kernels' launches and block reductions take only
+// for small systems, and only while every cluster has its SMs.  With the fused
+// FP32 mat-vec they also sum its partial sums.  Whole solves, cluster /
+// kernels: one system of 1280 elements 1.59 / 1.98 ms; 12 of 320 .. 5120, fused,
+// 3.00 / 2.91 ms; 16 charge sets on 5120 elements, not fused, 8.0 / 8.2 ms.
+bool cluster_step(const SysLayout& L, bool fused) {
+  return L.max_n <= (fused ? 2560 : 5120) && L.K * kClu <= 160;
+}
+
 void issue_cycle(Surface* s, const SysLayout& L, GmresWork* w, const bipb_medium& med, int precision,
                  bool transpose) {
-  const int4* lay = w->precond ? s->lay_dev(L) : nullptr;
+  const int4* lay = s->lay_dev(L);
   double* tz = w->precond ? w->tz.p : nullptr;
   const double2 pre = precond_factors(med);
-  const int m = w->m, m1 = m + 1, K = w->K, nb = w->nblk;
+  const int m = w->m, K = w->K, nb = w->nblk;
   const int64_t len = w->len;
   const int kg = (K + 127) / 128;
+  const int* skip = &w->st->skip;
+  // CGS2 for FP64 and df64 Krylov mat-vecs: the first pass also takes the
+  // dot products of the second, the second also forms the block norms.
+  // The FP32 / split-FP16 tensor-core Krylov solve of the mixed modes stops at a
+  // relative 1e-6 (its true residual is measured in higher precision by
+  // the refinement), and its FP64 basis of at most m vectors loses
+  // orthogonality in one classical pass only at about eps_64 cond(A)^2:
+  // one pass, which also forms the block norms.
   const bool cgs2 = precision == BIPB_FP64 || precision == BIPB_DF64;
+  StepArgs a{0,       m,       len,     w->V.p, w->w.p, w->part.p, w->part2.p, w->part1.p, w->H.p, w->cs.p,
+             w->sn.p, w->g.p, w->st, w->blk.p, w->sysb.p, lay,      tz,         pre,         {},     nullptr,
+             s->tgt64.p};
+  // the symmetric FP32 mat-vec fused into the step: its first records here, its
+  // sums and the next records in the step's kernels
+  const bool fused = precision == BIPB_FP32 &&
+                     matvec_sym32_stages(s, L, med, transpose, tz ? tz : w->V.p, w->w.p, skip, kStateInts, kSymPack, &a.mv);
+  const bool cluster = cluster_step(L, fused);
+  if (cluster) a.blk = w->cblk.p, a.sysb = w->csysb.p;
   for (int j = 0; j < m; ++j) {
     double* vj = w->V.p + (size_t)j * len;
-    matvec(s, L, med, precision, transpose, tz ? tz : vj, w->w.p, &w->st->skip, kStateInts);
-    // CGS2 for FP64 and df64 Krylov mat-vecs: the first pass also takes the
-    // dot products of the second, the second also forms the block norms.
-    // The FP32 / split-FP16 tensor-core Krylov solve of the mixed modes stops at a
-    // relative 1e-6 (its true residual is measured in higher precision by
-    // the refinement), and its FP64 basis of at most m vectors loses
-    // orthogonality in one classical pass only at about eps_64 cond(A)^2:
-    // one pass, which also forms the block norms.
-    launch_chained(k_dots, nb, kBS, 0, s->stream, j, m1, len, w->V.p, w->w.p, w->part.p, w->st, w->blk.p);
+    a.j = j;
+    a.u = tz ? tz : vj;
+    if (fused)
+      matvec_sym32_stages(s, L, med, transpose, a.u, w->w.p, skip, kStateInts, kSymPairs, nullptr);
+    else
+      matvec(s, L, med, precision, transpose, a.u, w->w.p, skip, kStateInts);
+    if (cluster) {
+      launch_chained(cgs2 ? k_step<true, false> : fused ? k_step<false, true> : k_step<false, false>, K * kClu, kCluNT, 0,
+                     s->stream, a);
+      BIPB_LAUNCHED(s);
+      continue;
+    }
+    launch_chained(fused ? k_dots<true> : k_dots<false>, nb, kBS, 0, s->stream, a);
     BIPB_LAUNCHED(s);
     if (cgs2) {
-      launch_chained(k_orth, nb, kBS, 0, s->stream, j, m, len, w->V.p, w->w.p, w->part.p, w->H.p, 0, w->st, w->blk.p,
-                     w->sysb.p, w->part1.p, 0, w->part2.p);
+      launch_chained(k_orth<false>, nb, kBS, 0, s->stream, a, a.part, 0);
       BIPB_LAUNCHED(s);
-      launch_chained(k_orth, nb, kBS, 0, s->stream, j, m, len, w->V.p, w->w.p, w->part2.p, w->H.p, 1, w->st,
-                     w->blk.p, w->sysb.p, w->part1.p, 1, nullptr);
+      launch_chained(k_orth<true>, nb, kBS, 0, s->stream, a, a.part2, 1);
     } else {
-      launch_chained(k_orth, nb, kBS, 0, s->stream, j, m, len, w->V.p, w->w.p, w->part.p, w->H.p, 0, w->st, w->blk.p,
-                     w->sysb.p, w->part1.p, 1, nullptr);
+      launch_chained(k_orth<true>, nb, kBS, 0, s->stream, a, a.part, 0);
     }
     BIPB_LAUNCHED(s);
-    launch_chained(k_normalize, nb, kBS, 0, s->stream, j, m, w->w.p, vj + len, w->part1.p, w->H.p, w->st, w->blk.p,
-                   w->sysb.p, 0, w->cs.p, w->sn.p, w->g.p, tz, lay, pre);
+    launch_chained(fused ? k_normalize<true> : k_normalize<false>, nb, kBS, 0, s->stream, a);
     BIPB_LAUNCHED(s);
   }
-  k_lsq<<<kg, 128, 0, s->stream>>>(m, K, w->H.p, w->cs.p, w->sn.p, w->g.p, w->y.p, w->z.p, w->st);
+  launch_chained(k_lsq, K, 64, 0, s->stream, m, w->H.p, w->cs.p, w->sn.p, w->g.p, w->y.p, w->z.p, w->st);
   BIPB_LAUNCHED(s);
-  k_update<<<nb, kBS, 0, s->stream>>>(m, len, w->V.p, w->d.p, w->y.p, w->z.p, w->st, w->blk.p, tz, lay, pre);
+  launch_chained(k_update, nb, kBS, 0, s->stream, m, len, w->V.p, w->d.p, w->y.p, w->z.p, w->st, w->blk.p, tz, lay,
+                 pre);
   BIPB_LAUNCHED(s);
-  k_next_cycle<<<kg, 128, 0, s->stream>>>(m, K, w->g.p, w->st);
+  launch_chained(k_next_cycle, kg, 128, 0, s->stream, m, K, w->g.p, w->st);
   BIPB_LAUNCHED(s);
 }
 
@@ -640,8 +836,8 @@ void read_states(Surface* s, GmresWork* w) {
 }
 
 // Per-system 2-norms of a batched vector (all systems, fixed summation order).
-std::vector<double> norms(Surface* s, GmresWork* w, const double* v) {
-  k_sumsq<<<w->nblk, kBS, 0, s->stream>>>(v, w->part1.p, w->st, w->blk.p, 2);
+std::vector<double> norms(Surface* s, const SysLayout& L, GmresWork* w, const double* v) {
+  k_sumsq<<<w->nblk, kBS, 0, s->stream>>>(v, w->part1.p, w->st, w->blk.p, s->lay_dev(L), 2);
   BIPB_LAUNCHED(s);
   BIPB_CUDA(cudaMemcpyAsync(w->part1_host.data(), w->part1.p, w->nblk * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
   BIPB_CUDA(cudaStreamSynchronize(s->stream));
@@ -677,11 +873,11 @@ std::vector<int> gmres_core(Surface* s, const SysLayout& L, GmresWork* w, const 
   }
   BIPB_CUDA(cudaMemcpyAsync(w->st, w->st_host.data(), K * sizeof(DevState), cudaMemcpyHostToDevice, s->stream));
   const int kg = (K + 127) / 128;
-  k_sumsq<<<w->nblk, kBS, 0, s->stream>>>(r0, w->part1.p, w->st, w->blk.p, 1);
+  const int4* lay = s->lay_dev(L);
+  k_sumsq<<<w->nblk, kBS, 0, s->stream>>>(r0, w->part1.p, w->st, w->blk.p, lay, 1);
   BIPB_LAUNCHED(s);
-  k_normalize<<<w->nblk, kBS, 0, s->stream>>>(-1, w->m, r0, w->V.p, w->part1.p, w->H.p, w->st, w->blk.p, w->sysb.p,
-                                              1, w->cs.p, w->sn.p, w->g.p, w->precond ? w->tz.p : nullptr,
-                                              w->precond ? s->lay_dev(L) : nullptr, precond_factors(med));
+  k_start<<<w->nblk, kBS, 0, s->stream>>>(r0, w->V.p, w->part1.p, w->st, w->blk.p, w->sysb.p, lay,
+                                          w->precond ? w->tz.p : nullptr, precond_factors(med));
   BIPB_LAUNCHED(s);
   k_next_cycle<<<kg, 128, 0, s->stream>>>(w->m, K, w->g.p, w->st);
   BIPB_LAUNCHED(s);
@@ -717,7 +913,7 @@ std::vector<SolveResult> gmres_solve(Surface* s, const SysLayout& L, const bipb_
   w->precond = p.precond;
   const int64_t len = L.len;
   const int nb = grid_for(len);
-  const std::vector<double> bnorm = norms(s, w, rhs);
+  const std::vector<double> bnorm = norms(s, L, w, rhs);
   const bool mixed = p.precision == BIPB_MIXED || p.precision == BIPB_MIXED_DF64 || p.precision == BIPB_MIXED_TENSOR ||
                      p.precision == BIPB_MIXED_TREE;
   // arithmetic of the Krylov mat-vecs and of the residual r = b - A x
@@ -737,7 +933,7 @@ std::vector<SolveResult> gmres_solve(Surface* s, const SysLayout& L, const bipb_
   }
   std::vector<double> rel(K, 1.0);
   if (warm) {
-    std::vector<double> rn = norms(s, w, w->r.p);
+    std::vector<double> rn = norms(s, L, w, w->r.p);
     for (int k = 0; k < K; ++k) rel[k] = bnorm[k] > 0 ? rn[k] / bnorm[k] : 0.0;
   }
   for (int k = 0; k < K; ++k)
@@ -776,7 +972,7 @@ std::vector<SolveResult> gmres_solve(Surface* s, const SysLayout& L, const bipb_
     matvec(s, L, med, resid, transpose, x, w->t.p, w->mask.p, 1);
     k_sub<<<nb, kBS, 0, s->stream>>>(len, rhs, w->t.p, w->r.p);
     BIPB_LAUNCHED(s);
-    std::vector<double> rn = norms(s, w, w->r.p);
+    std::vector<double> rn = norms(s, L, w, w->r.p);
     for (int k = 0; k < K; ++k) {
       if (!active[k]) continue;
       iters[k] += used[k];

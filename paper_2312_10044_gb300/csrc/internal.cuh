@@ -426,9 +426,28 @@ int autotune_matvec32(Surface* s, const SysLayout& L, const bipb_medium& m, int 
 // ---- sym.cu: mat-vecs visiting every unordered pair once; false when the
 // layout is too large for the symmetric work list, or 0 < kappa < 1e-6
 // (nothing launched then)
+struct SymStep;
 bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c, double kappa, bool transpose,
                   int variant, const double* u, double* y, double dphi, double dpsi, const int* skip,
-                  int skip_stride);
+                  int skip_stride, int stages, SymStep* step);
+// The FP32 symmetric mat-vec in parts, for a caller that fuses its pack and its
+// reduction into kernels of its own (the Krylov step): what those need.
+struct SymStep {
+  const int4* tab = nullptr;   // reduction table (symstep.cuh)
+  const float* part = nullptr; // partial sums
+  float4* rec = nullptr;       // records, 5 float4 per element at vec_off / 2
+  double sigma = 1.0;          // positions and alpha are multiplied by it
+  double2 f{1.0, 1.0};         // factors of the phi and psi sums
+  double dphi = 0.0, dpsi = 0.0;  // the diagonal
+  bool transpose = false;
+};
+enum { kSymPack = 1, kSymPairs = 2, kSymReduce = 4, kSymAll = 7 };
+// y = A u (or A^T u) by the handle's FP32 variant if it is a symmetric one that
+// takes this layout and medium (false otherwise, nothing launched); stages is
+// a sum of kSym* (the others are left to the caller), step (may be null)
+// receives what they need.
+bool matvec_sym32_stages(Surface* s, const SysLayout& L, const bipb_medium& m, bool transpose, const double* u,
+                         double* y, const int* skip, int skip_stride, int stages, SymStep* step);
 bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c, double kappa, bool transpose,
                   const double* u, double* y, double dphi, double dpsi, const int* skip, int skip_stride);
 bool matvec_sym_df(Surface* s, const SysLayout& L, const DFConst& c, double kappa, bool transpose, const double* u,

@@ -976,7 +976,8 @@ void matvec(Surface* s, const SysLayout& L, const bipb_medium& m, int precision,
   PairConst<float> c = pair_const<float>(m);
   int variant = s->mv32_variant;
   if (variant >= kFirstSymVariant) {
-    if (matvec_sym32(s, L, c, m.kappa, transpose, variant - kFirstSymVariant, u, y, dphi, dpsi, skip, skip_stride))
+    if (matvec_sym32(s, L, c, m.kappa, transpose, variant - kFirstSymVariant, u, y, dphi, dpsi, skip, skip_stride,
+                     kSymAll, nullptr))
       return;
     variant = 0;  // too large for the symmetric work list
   }
@@ -1001,6 +1002,14 @@ void matvec(Surface* s, const SysLayout& L, const bipb_medium& m, int precision,
   }
 }
 
+
+bool matvec_sym32_stages(Surface* s, const SysLayout& L, const bipb_medium& m, bool transpose, const double* u,
+                         double* y, const int* skip, int skip_stride, int stages, SymStep* step) {
+  const double eps = m.eps_out / m.eps_in;
+  if (s->mv32_variant < kFirstSymVariant) return false;
+  return matvec_sym32(s, L, pair_const<float>(m), m.kappa, transpose, s->mv32_variant - kFirstSymVariant, u, y,
+                      0.5 * (1.0 + eps), 0.5 * (1.0 + 1.0 / eps), skip, skip_stride, stages, step);
+}
 
 void launch_reduce_matvec64(Surface* s, const SysLayout& L, const int4* tab, const double* part, const double* u,
                             double* y, double dphi, double dpsi, const int* skip, int skip_stride) {

@@ -35,6 +35,7 @@
 
 #include "f32x2.cuh"
 #include "internal.cuh"
+#include "symstep.cuh"
 
 namespace bipb {
 
@@ -411,16 +412,7 @@ __global__ void k_pack_sym32(const int4* __restrict__ lay, bool transpose, const
   if (j >= L.y || (skip != nullptr && skip[(size_t)k * skip_stride] != 0)) return;
   const double4_32a g = tgt64[2 * (L.x + j)], v = tgt64[2 * (L.x + j) + 1];
   const double phi = u[L.z + j], psi = u[L.z + L.y + j];
-  const float a = (float)(transpose ? phi : g.w * psi);
-  const float al = (float)(sigma * (transpose ? psi : g.w * phi));
-  const float x = (float)(sigma * g.x), y = (float)(sigma * g.y), z = (float)(sigma * g.z);
-  const float nx = (float)v.x, ny = (float)v.y, nz = (float)v.z, f = transpose ? al : -a;
-  float4* o = rec + 5 * (size_t)(L.z / 2 + j);
-  o[0] = make_float4(x, x, y, y);
-  o[1] = make_float4(z, z, a, a);
-  o[2] = make_float4(nx, nx, ny, ny);
-  o[3] = make_float4(nz, nz, -al, -al);
-  o[4] = make_float4(f, f, 0.f, 0.f);
+  sym32_record(g, v, phi, psi, transpose, sigma, rec + 5 * (size_t)(L.z / 2 + j));
 }
 
 __global__ void k_pack_sym_df(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
@@ -448,9 +440,8 @@ __global__ void k_pack_sym_df(const int4* __restrict__ lay, bool transpose, cons
   o[4] = make_float4(x0.m, x1.m, x2.m, 0.f);
 }
 
-// y_i = diag u_i - (1/(4 pi)) scale_i f_c (i-side blocks of the element's row + j-side rows 0..E),
-// f_c = f.x for the phi rows and f.y for the psi rows (the factors of kappa-scaled records).
-// tab[k] = {n, first row entry, j-side base, T}; tab[row entry + E] = {first i-side block, blocks, 0, 0}.
+// y_i = diag u_i - (1/(4 pi)) scale_i f_c sym_sum, f_c = f.x for the phi rows
+// and f.y for the psi rows (the factors of kappa-scaled records).
 template <typename PT>
 __global__ void k_reduce_sym(const int4* __restrict__ lay, const int4* __restrict__ tab, const PT* __restrict__ part,
                              const double* __restrict__ u, double* __restrict__ y, double d_phi, double d_psi,
@@ -459,32 +450,14 @@ __global__ void k_reduce_sym(const int4* __restrict__ lay, const int4* __restric
   chain_wait();
   chain_release();
   const int k = blockIdx.y;
-  const int4 L = lay[k], S = tab[k];
-  const int n = L.y, T = S.w;
+  const int4 L = lay[k];
+  const int n = L.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n || (skip != nullptr && skip[(size_t)k * skip_stride] != 0)) return;
-  const int c = i < n ? 0 : 1;
-  const int e = i - c * n;
-  const int E = e / T;
-  const int4 R = tab[S.y + E];
-  double acc = 0.0;
-  for (int b = 0; b < R.y; ++b) acc += (double)part[(size_t)R.x + (size_t)b * 2 * T + (size_t)c * T + (e - E * T)];
-  // rows 0..E in order; four loads in flight at a time
-  auto at = [&](int I) {
-    const int64_t row = (int64_t)S.z + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2);
-    return (double)part[row + (int64_t)c * (n - I * T) + (e - I * T)];
-  };
-  int I = 0;
-  for (; I + 4 <= E + 1; I += 4) {
-    const double v0 = at(I), v1 = at(I + 1), v2 = at(I + 2), v3 = at(I + 3);
-    acc += v0;
-    acc += v1;
-    acc += v2;
-    acc += v3;
-  }
-  for (; I <= E; ++I) acc += at(I);
-  const double sc = tgt64_for_area ? tgt64_for_area[2 * (L.x + e)].w : 1.0;
-  y[L.z + i] = (c == 0 ? d_phi : d_psi) * u[L.z + i] - kInv4PiS * sc * (c == 0 ? f.x : f.y) * acc;
+  const int c = i < n ? 0 : 1, e = i - c * n;
+  const double acc = sym_sum(tab, tab[k], part, e, c);
+  const double sc = kInv4PiS * (tgt64_for_area ? tgt64_for_area[2 * (L.x + e)].w : 1.0);
+  y[L.z + i] = (c == 0 ? d_phi : d_psi) * u[L.z + i] - sc * (c == 0 ? f.x : f.y) * acc;
 }
 
 int blocks_of(int64_t n, int bs) { return (int)std::max<int64_t>(1, (n + bs - 1) / bs); }
@@ -717,7 +690,8 @@ int sym_occupancy() {
 template <class P, int NT, int TPT, int CH, int MINB>
 void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typename P::Args& g, bool transpose,
              DevBuf<typename P::V4>& recbuf, DevBuf<typename P::PT>& partbuf, const double* u, double* y,
-             double dphi, double dpsi, const int* skip, int skip_stride, double sigma = 1.0) {
+             double dphi, double dpsi, const int* skip, int skip_stride, double sigma = 1.0, int stages = kSymAll,
+             SymStep* step = nullptr) {
   constexpr int T = NT * TPT;
   if (!P::SCALED) sigma = 1.0;
   // A u: P ~ sigma, Q ~ sigma^2; A^T w: P ~ sigma^2, Q ~ sigma (pair.cuh)
@@ -727,27 +701,33 @@ void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typena
   s->grow(recbuf, (size_t)(L.len / 2) * P::RW);
   s->grow(partbuf, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  const dim3 pgrid(blocks_of(L.max_n, 256), L.K);
-  if constexpr (std::is_same<typename P::V4, double4_32a>::value) {
-    launch_chained(k_pack_sym64, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+  if constexpr (std::is_same<typename P::PT, float>::value) {
+    if (step != nullptr) *step = SymStep{plan->tab.p, partbuf.p, recbuf.p, sigma, f, dphi, dpsi, transpose};
+  }
+  const dim3 pgrid(blocks_of(L.max_n, 128), L.K);
+  if (!(stages & kSymPack)) {
+  } else if constexpr (std::is_same<typename P::V4, double4_32a>::value) {
+    launch_chained(k_pack_sym64, pgrid, 128, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
                    sigma);
   } else if constexpr (std::is_same<typename P::PT, double>::value) {
-    launch_chained(k_pack_sym_df, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+    launch_chained(k_pack_sym_df, pgrid, 128, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
                    sigma, std::exp2(std::ceil(std::log2(sigma))));
   } else {
-    launch_chained(k_pack_sym32, pgrid, 256, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
+    launch_chained(k_pack_sym32, pgrid, 128, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
                    sigma);
   }
-  BIPB_LAUNCHED(s);
-  {
+  if (stages & kSymPack) BIPB_LAUNCHED(s);
+  if (stages & kSymPairs) {
     TimedLaunch tl(s, kind);
     launch_chained(k_sym<P, NT, TPT, CH, MINB>, plan->n_items, NT, 0, s->stream, g, plan->items.p, recbuf.p,
                    partbuf.p, skip, skip_stride);
     BIPB_LAUNCHED(s);
   }
-  launch_chained(k_reduce_sym<typename P::PT>, dim3(blocks_of(2 * (int64_t)L.max_n, 256), L.K), 256, 0, s->stream, lay,
-                 plan->tab.p, partbuf.p, u, y, dphi, dpsi, transpose ? s->tgt64.p : nullptr, skip, skip_stride, f);
-  BIPB_LAUNCHED(s);
+  if (stages & kSymReduce) {
+    launch_chained(k_reduce_sym<typename P::PT>, dim3(blocks_of(2 * (int64_t)L.max_n, 128), L.K), 128, 0, s->stream, lay, plan->tab.p, partbuf.p, u, y, dphi,
+                   dpsi, transpose ? s->tgt64.p : nullptr, skip, skip_stride, f);
+    BIPB_LAUNCHED(s);
+  }
 }
 
 }  // namespace
@@ -768,7 +748,7 @@ bool sym_form(double kappa, PairConst<T>& c, bool& laplace) {
 
 bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, double kappa, bool transpose,
                   int variant, const double* u, double* y, double dphi, double dpsi, const int* skip,
-                  int skip_stride) {
+                  int skip_stride, int stages, SymStep* step) {
   if (variant < 0 || variant > 2) throw Error(BIPB_ERR_INVALID_ARG, "unknown symmetric FP32 mat-vec variant");
   // Shapes (threads, targets per thread, tile of targets): 0 (256, 2, 512), 1
   // (128, 4, 512), 2 (256, 4, 1024), 3 (128, 2, 256).  Variant 2 takes the
@@ -787,7 +767,7 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
   const int kind = transpose ? kTMv32T : kTMv32;
 #define BIPB_SYM32_RUN(TR_, LAP_, V_, NT_, TPT_, CH_, MINB_)                                                       \
   run_sym<Sym32Policy<TR_, LAP_>, NT_, TPT_, CH_, MINB_>(s, (TR_ ? 0x100 : 0x200) + V_, kind, L, {c}, TR_, s->rec32, \
-                                                         s->part32, u, y, dphi, dpsi, skip, skip_stride, kappa)
+                                                         s->part32, u, y, dphi, dpsi, skip, skip_stride, kappa, stages, step)
 #define BIPB_SYM32(V_, NT_, TPT_, CH_, MINB_)                     \
   case V_:                                                         \
     if (transpose) {                                               \

@@ -104,3 +104,27 @@ def test_fp32_symmetric_shapes_small_and_ragged(bipb, orc, n, transpose):
                 y = y.cpu().numpy()
                 assert np.linalg.norm(y - ref) < 3e-6 * np.linalg.norm(ref), (variant, kappa)
                 assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max(), (variant, kappa)
+
+
+@pytest.mark.parametrize("n,sets,precond", [(2, 1, 0), (37, 20, 1), (37, 21, 1), (2560, 1, 0), (2561, 1, 0), (2561, 2, 1)])
+def test_krylov_step_as_cluster_and_as_kernels(bipb, orc, n, sets, precond):
+    """The Arnoldi step as one cluster launch per system (small systems, up to 20 of
+    them) and as three kernels, on both sides of the lines between them, with the
+    fused FP32 mat-vec and (FP64) without: mixed and FP64 solves against the
+    oracle's, 1e-7 and 1e-9 of the energy (test_kirkwood_solve's bounds or looser)."""
+    p = synth.protein_like_problem(level=4, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, n, replace=False))
+    p.centroids, p.normals, p.areas = p.centroids[keep], p.normals[keep], p.areas[keep]
+    q = np.random.default_rng(1).uniform(-1.0, 1.0, (sets, p.nc))
+    p.q = q
+    ref = [orc.solve(p, rhs=r, method="gmres", tol=1e-12).energy_kcal for r in range(min(sets, 2))]
+    for prec, tol, rt in ((bipb.MIXED_DF64, 1e-9, 1e-7), (bipb.FP64, 1e-11, 1e-9)):
+        if prec == bipb.FP64 and n > 2560:
+            continue
+        for restart in (10, 3):
+            with bipb.Surface(p.centroids, p.normals, p.areas) as s:
+                s.set_charges(p.charge_pos, q)
+                info = s.solve(eps_in=p.eps_in, eps_out=p.eps_out, kappa=p.kappa, tol=tol, precision=prec,
+                               precond=precond, restart=restart)
+                assert all(i["converged"] for i in info)
+                np.testing.assert_allclose(s.energy()[:2], ref, rtol=rt)
