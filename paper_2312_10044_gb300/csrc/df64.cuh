@@ -127,12 +127,16 @@ __device__ __forceinline__ df df_fma(df a, df b, df x) {
   const df s = two_sum(x.hi, p.hi);
   return df{s.hi, __fadd_rn(x.lo, __fadd_rn(s.lo, plo))};
 }
-// The same for a float x, normalised (14 operations).
-__device__ __forceinline__ df df_fma_f(df a, df b, float x) {
+// The same for a float x (11 operations), and normalised (14).
+__device__ __forceinline__ df df_fma_lazy(df a, df b, float x) {
   const df p = two_prod(a.hi, b.hi);
   const float plo = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
   const df s = two_sum(x, p.hi);
-  return fast_two_sum(s.hi, __fadd_rn(s.lo, plo));
+  return df{s.hi, __fadd_rn(s.lo, plo)};
+}
+__device__ __forceinline__ df df_fma_f(df a, df b, float x) {
+  const df r = df_fma_lazy(a, b, x);
+  return fast_two_sum(r.hi, r.lo);
 }
 // x + 3 a (11 operations).
 __device__ __forceinline__ df df_add_3(df a, df x) {
@@ -332,33 +336,38 @@ __device__ __forceinline__ void df_pair_transpose(const df* xj, const df* nj, co
 // element i gathering input element j (the transposed pair of pair.cuh, d =
 // x_i - x_j): k[0] = K2_ji, k[1] = K4_ji (the phi row), k[2] = K1_ji, k[3] =
 // K3_ji (the psi row), i.e. ((1 - eps t) c_i s^3, K4, (1 - e) s,
-// (1 - t/eps) c_j s^3), times `area` (the output's area goes on the sums).
+// (1 - t/eps) c_j s^3), without an area (the output's goes on the sums).
+// SCALED: kappa-scaled coordinates; the phi (A^T: psi) column is multiplied by
+// kappa here, the sums by (kappa, kappa^2) (A^T: (kappa^2, kappa)) elsewhere.
+// r0, r1: factors of the phi and psi row (powers of two).
 // The values are normalised: where a factor has cancelled, its trailing part
 // is far above an ulp of its leading one, which the digits of the exact
 // tensor-core form could not hold.
-template <bool MASK, bool TRANS = false>
-__device__ __forceinline__ void df_kernel_block(const df* xi, const df* ni, const df* xj, const df* nj, df area,
-                                                bool self, const DFConst& c, const df* tab, df* k) {
-  const df d[3] = {df_sub(xi[0], xj[0]), df_sub(xi[1], xj[1]), df_sub(xi[2], xj[2])};
-  const DfRadial R = df_radial<MASK, false>(d, self, c, tab);
-  const df s2 = df_sqr(R.s), sa = df_mul(R.s, area), s3a = df_mul(s2, sa);
+template <bool MASK, bool TRANS, bool SCALED>
+__device__ __forceinline__ void df_kernel_block(const df_pos* xi, const df* ni, const df_pos* xj, const df* nj,
+                                                df area, bool self, const DFConst& c, const df* tab, float r0,
+                                                float r1, df* k) {
+  const df d[3] = {df_diff(xi[0], xj[0]), df_diff(xi[1], xj[1]), df_diff(xi[2], xj[2])};
+  const DfRadial R = df_radial<MASK, SCALED>(d, self, c, tab);
+  const df s2 = df_sqr(R.s), sa = TRANS ? R.s : df_mul(R.s, area), s3 = df_mul(s2, sa);
+  const df s3k = SCALED ? df_mul(s3, c.kappa) : s3;  // of the phi (A^T: psi) column
   const df ci = df_dot(ni, d), cj = df_dot(nj, d), cij = df_dot_unit(ni, nj);
-  const df k1 = df_neg(df_mul(R.e1, sa));                                            // K1 ds
-  const df k4 = df_mul(df_det(R.t1, cij, df_wm3s2<false>(R, s2, c), df_mul(ci, cj)), s3a);  // K4 ds
-  const df et1 = df_fma_f(c.eps, R.t, -1.0f), te1 = df_fma_f(R.t, c.inveps, -1.0f);
+  const df k1 = df_neg(df_mul(R.e1, df_scale(sa, TRANS ? r1 : r0)));
+  const df k4 = df_mul(df_det(R.t1, cij, df_wm3s2<SCALED>(R, s2, c), df_mul(ci, cj)), df_scale(s3k, TRANS ? r0 : r1));
+  const df et1 = df_fma_lazy(c.eps, R.t, -1.0f), te1 = df_fma_lazy(R.t, c.inveps, -1.0f);
   if (!TRANS) {
-    k[1] = k1;
-    k[0] = df_mul(df_mul(et1, cj), s3a);          // K2 ds
-    k[3] = df_mul(df_mul(te1, ci), s3a);          // K3 ds
-    k[2] = k4;
+    k[0] = df_mul(df_mul(et1, cj), df_scale(s3k, r0));         // K2 ds
+    k[1] = k1;                                    // K1 ds
+    k[2] = k4;                                    // K4 ds
+    k[3] = df_mul(df_mul(te1, ci), df_scale(s3, r1));          // K3 ds
   } else {
-    k[0] = df_neg(df_mul(df_mul(et1, ci), s3a));  // K2_ji
+    k[0] = df_neg(df_mul(df_mul(et1, ci), df_scale(s3, r0)));  // K2_ji
     k[1] = k4;                                    // K4_ji
     k[2] = k1;                                    // K1_ji
-    k[3] = df_neg(df_mul(df_mul(te1, cj), s3a));  // K3_ji
+    k[3] = df_neg(df_mul(df_mul(te1, cj), df_scale(s3k, r1)));  // K3_ji
   }
 #pragma unroll
-  for (int v = 0; v < 4; ++v) k[v] = two_sum(k[v].hi, k[v].lo);
+  for (int v = 0; v < 4; ++v) k[v] = df_norm(k[v]);
 }
 
 // The symmetric pair of pair.cuh (sym_pair) in df64.  The four accumulators

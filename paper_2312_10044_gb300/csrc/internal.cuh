@@ -315,7 +315,7 @@ struct Surface {
   DevBuf<float> part32;
   DevBuf<double> part64;
   DevBuf<int> rhs_idx;  // right-hand-side indices of a compacted multi-RHS pass
-  DevBuf<float4> geodf;  // multi-RHS df64 pass: geometry as df64 records (4 float4 each)
+  DevBuf<float4> geodf;  // multi-RHS df64 pass: geometry as df64 records (5 float4 each)
   DevBuf<float4> udf;    // multi-RHS df64 pass: right-hand sides as df64 (phi, psi) pairs
   DevBuf<int2> tcx_rowexp[2];  // exact tensor-core df64 pass, per direction (A u, A^T u): row scale exponents (phi, psi row)
   DevBuf<unsigned> tcx_colmax;  // exact tensor-core df64 pass: max |u| per right-hand side (FP32 bits)

@@ -17,6 +17,7 @@
 // converged) uses fewer groups.  Partial sums per source split are written in
 // FP64 and added by the FP64 reduction of kernels.cu.
 #include <algorithm>
+#include <cmath>
 
 #include <cuda_fp16.h>
 
@@ -37,13 +38,17 @@ constexpr int kTcxMinRHS = 16;  // the exact tensor-core form from this many rig
 // Double-float copies made once per pass, so that the hot loop stages plain
 // float4 records and never converts from FP64 (GB300 runs FP64 and its
 // conversions at a small fraction of the FP32 rate):
-//   geo[4 j .. 4 j + 3] = (x.hi, a.hi), (x.lo, a.lo), (n.hi, 0), (n.lo, 0) of element j
-//     (x the centred centroid as a 3-vector, a = ds_j, n the normal);
+//   geo[5 j .. 5 j + 4] = (x.h, a.hi), (x.l, a.lo), (n.hi, 0), (n.lo, 0), (x.m, 0) of element j
+//     (x sigma times the centred centroid on the surface's grid, a = ds_j, n the normal);
 //   u4[b n + j] = (phi.hi, phi.lo, psi.hi, psi.lo) of right-hand side b (the
 //     rhs[b]-th of u when rhs is given), element j.
-// blockIdx.y < nb packs right-hand side blockIdx.y, blockIdx.y == nb the geometry.
+// sigma = kappa for the kappa-scaled form (df_kernel_block), 1 otherwise; gscale
+// the power of two at or above it.  blockIdx.y < nb packs right-hand side
+// blockIdx.y, blockIdx.y == nb the geometry.
+constexpr int kGeo = 5;  // float4 per geometry record
 __global__ void k_pack_mrhs_df(int n, int nb, const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
-                               const int* __restrict__ rhs, float4* __restrict__ geo, float4* __restrict__ u4) {
+                               const int* __restrict__ rhs, float4* __restrict__ geo, float4* __restrict__ u4,
+                               double sigma, double gscale) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const int b = blockIdx.y;
@@ -54,34 +59,50 @@ __global__ void k_pack_mrhs_df(int n, int nb, const double4_32a* __restrict__ tg
     return;
   }
   const double4_32a g = tgt64[2 * j], v = tgt64[2 * j + 1];
-  const df x0 = df_from_double(g.x), x1 = df_from_double(g.y), x2 = df_from_double(g.z), a = df_from_double(g.w);
+  const double grid = gscale * v.w;
+  const df_pos x0 = df_split_grid(sigma * g.x, grid), x1 = df_split_grid(sigma * g.y, grid),
+               x2 = df_split_grid(sigma * g.z, grid);
+  const df a = df_from_double(g.w);
   const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
-  geo[4 * j] = make_float4(x0.hi, x1.hi, x2.hi, a.hi);
-  geo[4 * j + 1] = make_float4(x0.lo, x1.lo, x2.lo, a.lo);
-  geo[4 * j + 2] = make_float4(n0.hi, n1.hi, n2.hi, 0.f);
-  geo[4 * j + 3] = make_float4(n0.lo, n1.lo, n2.lo, 0.f);
+  float4* o = geo + kGeo * (int64_t)j;
+  o[0] = make_float4(x0.h, x1.h, x2.h, a.hi);
+  o[1] = make_float4(x0.l, x1.l, x2.l, a.lo);
+  o[2] = make_float4(n0.hi, n1.hi, n2.hi, 0.f);
+  o[3] = make_float4(n0.lo, n1.lo, n2.lo, 0.f);
+  o[4] = make_float4(x0.m, x1.m, x2.m, 0.f);
+}
+// position, normal and area of a geometry record
+struct GeoDF {
+  df_pos x[3];
+  df n[3], a;
+};
+__device__ __forceinline__ GeoDF load_geo(const float4* r) {
+  const float4 A = r[0], B = r[1], C = r[2], D = r[3], M = r[4];
+  return GeoDF{{df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}},
+               {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}},
+               df{A.w, B.w}};
 }
 
 // Dynamic shared memory of one CTA with G groups: kernel blocks (hi, lo),
 // right-hand-side values, source records, exp table.
 template <int G>
 constexpr int smem_bytes() {
-  return 2 * kCh * kTgt * 16 + kGB * G * kCh * 16 + kCh * 4 * 16 + kExpTab * 8;
+  return 2 * kCh * kTgt * 16 + kGB * G * kCh * 16 + kCh * kGeo * 16 + kExpTab * 8;
 }
 
 // items: {t0, s0, s1, split}; geo, u4: the packed records of k_pack_mrhs_df;
-// part: [b][split][2n]
-template <int G>
+// part: [b][split][2n], times (sigma, sigma^2) when SCALED
+template <int G, bool SCALED>
 __global__ void __launch_bounds__(kTgt * G, 512 / (kTgt * G))
     k_mrhs_df(int n, int nb, int n_splits, const int4* __restrict__ items, const float4* __restrict__ geo,
-              const float4* __restrict__ u4, double* __restrict__ part, DFConst c) {
+              const float4* __restrict__ u4, double* __restrict__ part, DFConst c, double sigma) {
   constexpr int NT = kTgt * G;
   extern __shared__ __align__(16) unsigned char smem[];
   float4* kbh = reinterpret_cast<float4*>(smem);           // [kCh][kTgt]: (K2, K1, K4, K3) ds, hi parts
   float4* kbl = kbh + kCh * kTgt;                           // lo parts
   float4* ush = kbl + kCh * kTgt;                           // [8 G][kCh]: (phi.hi, phi.lo, psi.hi, psi.lo)
-  float4* srec = ush + kGB * G * kCh;                       // [kCh][4]: x, n split as below
-  df* tab = reinterpret_cast<df*>(srec + kCh * 4);          // 2^(j/1024)
+  float4* srec = ush + kGB * G * kCh;                       // [kCh][kGeo]: geometry records
+  df* tab = reinterpret_cast<df*>(srec + kCh * kGeo);          // 2^(j/1024)
   const int tid = threadIdx.x;
   const int g = tid / kTgt, tl = tid % kTgt;  // MAC phase: group g (warp-uniform), target tl
   const int4 item = items[blockIdx.x];
@@ -89,13 +110,7 @@ __global__ void __launch_bounds__(kTgt * G, 512 / (kTgt * G))
   df_load_exp_table(tab, c);
   const int ti = t0 + tl;
   const bool tvalid = ti < n;
-  df xi[3], ni[3];
-  {
-    const int64_t r = 4 * (int64_t)min(ti, n - 1);
-    const float4 A = geo[r], B = geo[r + 1], C = geo[r + 2], D = geo[r + 3];
-    xi[0] = df{A.x, B.x}, xi[1] = df{A.y, B.y}, xi[2] = df{A.z, B.z};
-    ni[0] = df{C.x, D.x}, ni[1] = df{C.y, D.y}, ni[2] = df{C.z, D.z};
-  }
+  const GeoDF T = load_geo(geo + kGeo * (int64_t)min(ti, n - 1));
   df accp[kGB], accq[kGB];
 #pragma unroll
   for (int b = 0; b < kGB; ++b) accp[b] = df{0.f, 0.f}, accq[b] = df{0.f, 0.f};
@@ -103,7 +118,7 @@ __global__ void __launch_bounds__(kTgt * G, 512 / (kTgt * G))
   for (int j0 = s0; j0 < s1; j0 += kCh) {
     const int cnt = min(kCh, s1 - j0);
     __syncthreads();  // the previous chunk's blocks and values have been used
-    for (int e = tid; e < 4 * cnt; e += NT) srec[e] = geo[4 * (int64_t)j0 + e];
+    for (int e = tid; e < kGeo * cnt; e += NT) srec[e] = geo[kGeo * (int64_t)j0 + e];
     // right-hand-side values, e = b * cnt + q (q fastest: coalesced reads)
     for (int e = tid; e < kGB * G * cnt; e += NT) {
       const int q = e % cnt, b = e / cnt;
@@ -112,11 +127,9 @@ __global__ void __launch_bounds__(kTgt * G, 512 / (kTgt * G))
     __syncthreads();
     // kernel blocks of (target tl, source q) for q = g, g + G, ...
     for (int q = g; q < cnt; q += G) {
-      const float4 A = srec[4 * q], B = srec[4 * q + 1], C = srec[4 * q + 2], D = srec[4 * q + 3];
-      const df xj[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
-      const df nj[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
+      const GeoDF S = load_geo(srec + kGeo * q);
       df k[4];
-      df_kernel_block<true>(xi, ni, xj, nj, df{A.w, B.w}, !tvalid || j0 + q == ti, c, tab, k);
+      df_kernel_block<true, false, SCALED>(T.x, T.n, S.x, S.n, S.a, !tvalid || j0 + q == ti, c, tab, 1.f, 1.f, k);
       kbh[q * kTgt + tl] = make_float4(k[0].hi, k[1].hi, k[2].hi, k[3].hi);
       kbl[q * kTgt + tl] = make_float4(k[0].lo, k[1].lo, k[2].lo, k[3].lo);
     }
@@ -146,8 +159,8 @@ __global__ void __launch_bounds__(kTgt * G, 512 / (kTgt * G))
     const int bb = kGB * g + b;
     if (bb >= nb) break;
     double* o = part + ((int64_t)bb * n_splits + split) * 2 * n;
-    o[ti] = df_to_double(accp[b]);
-    o[n + ti] = df_to_double(accq[b]);
+    o[ti] = sigma * df_to_double(accp[b]);
+    o[n + ti] = sigma * sigma * df_to_double(accq[b]);
   }
 }
 
@@ -155,9 +168,10 @@ template <int G>
 int mrhs_df_occupancy() {
   static int occ = [] {
     int o = 0;
-    if (cudaFuncSetAttribute(k_mrhs_df<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<G>()) !=
+    if (cudaFuncSetAttribute(k_mrhs_df<G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<G>()) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_mrhs_df<G>, kTgt * G, smem_bytes<G>()) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_mrhs_df<G, true>, kTgt * G, smem_bytes<G>()) !=
+            cudaSuccess) {
       (void)cudaGetLastError();
       o = 1;
     }
@@ -167,10 +181,12 @@ int mrhs_df_occupancy() {
 }
 
 template <int G>
-void launch_mrhs_df(Surface* s, const ItemPlan* plan, int n, int nb, int S, const DFConst& c) {
-  BIPB_CUDA(cudaFuncSetAttribute(k_mrhs_df<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<G>()));
-  k_mrhs_df<G><<<plan->n_items, kTgt * G, smem_bytes<G>(), s->stream>>>(n, nb, S, plan->items.p, s->geodf.p,
-                                                                       s->udf.p, s->part64.p, c);
+void launch_mrhs_df(Surface* s, const ItemPlan* plan, int n, int nb, int S, const DFConst& c, bool scaled,
+                    double sigma) {
+  auto kernel = scaled ? k_mrhs_df<G, true> : k_mrhs_df<G, false>;
+  BIPB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<G>()));
+  kernel<<<plan->n_items, kTgt * G, smem_bytes<G>(), s->stream>>>(n, nb, S, plan->items.p, s->geodf.p, s->udf.p,
+                                                                 s->part64.p, c, sigma);
   BIPB_LAUNCHED(s);
 }
 
@@ -230,6 +246,13 @@ ItemPlan* mrhs_df_plan(Surface* s, int n, int G, int slots, int* S_out) {
 // nothing on the CUDA cores.  A^T U is the same pass over the transposed
 // blocks (df_kernel_block<.., true>, area 1), with its own row scales and the
 // output element's area applied to the FP64 sums.
+//
+// What bounds it: the generation, about 490 instructions a (target, source)
+// pair on the CUDA cores (FP32 pipe 60 % busy, tensor pipe 36 %, under the
+// generation).  At N = 20001 and 64 right-hand sides a pass takes 6.83 ms
+// (8.72 with unscaled, unfused df64 blocks and digit-by-digit rounding), and
+// a first pass in a medium 7.5 ms (18.0 when one thread per target found the
+// row scales in df64).
 namespace tcx {
 
 constexpr int kRHS = 64;                        // right-hand sides per CTA (all of a launch)
@@ -243,7 +266,7 @@ constexpr int kAStage = kChunks * kLv * kPlane; // A of one step: 56 KB
 constexpr int kBRows = kLv * kRHS;              // 448 rows: digit plane l of U in rows 64 l ..
 constexpr int kBChunk = kBRows * kKC * 2;       // 14 KB per K chunk
 constexpr int kBBytes = kChunks * kBChunk;      // 28 KB per step
-constexpr int kSRec = kStep * 64;               // source records of one step: 1 KB
+constexpr int kSRec = kStep * kGeo * 16;        // source records of one step
 constexpr int kRing = 3;                        // B and source buffers (step it in buffer it % 3)
 constexpr int kGroupChunks = 32;                // K chunks per exact accumulation group (K = 512)
 constexpr int kGroup = kGroupChunks / kChunks;  // steps per group
@@ -285,63 +308,87 @@ __device__ __forceinline__ int scale_exp(float m) {
   return max(-100, min(100, 5 - lg));
 }
 
-// a (df64, |a| below 64 up to rounding) as seven base-128 digits, exactly
-// up to 2^-43: a = sum_k d[k] 128^-k + rest.  The leading part gives three
-// digits by exact FP32 steps; the trailing part (at most 2^-19) joins at the
-// fourth, which may then reach 68 in magnitude.
-__device__ __forceinline__ void digits7(df a, float* d) {
-  float r = a.hi;
-  d[0] = rintf(r);
-  r = __fsub_rn(r, d[0]);
-  d[1] = rintf(__fmul_rn(r, 128.f));
-  r = __fsub_rn(__fmul_rn(r, 128.f), d[1]);
-  d[2] = rintf(__fmul_rn(r, 128.f));
-  r = __fsub_rn(__fmul_rn(r, 128.f), d[2]);
-  const df t = two_sum(__fmul_rn(r, 128.f), __fmul_rn(a.lo, 2097152.f));  // units 128^-3
-  d[3] = rintf(t.hi);
-  r = __fadd_rn(__fsub_rn(t.hi, d[3]), t.lo);
-  d[4] = rintf(__fmul_rn(r, 128.f));
-  r = __fsub_rn(__fmul_rn(r, 128.f), d[4]);
-  d[5] = rintf(__fmul_rn(r, 128.f));
-  r = __fsub_rn(__fmul_rn(r, 128.f), d[5]);
-  d[6] = rintf(__fmul_rn(r, 128.f));
+// (x & mask) as FP16 integers in both halves, plus the FP16 pair `off`
+__device__ __forceinline__ uint32_t fields(uint32_t x, uint32_t mask, uint32_t off) {
+  const uint32_t h = (x & mask) | 0x64006400u;  // FP16 1024 + field
+  uint32_t r;
+  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(off));
+  return r;
+}
+// Two values (df64, normalised, below 128 in magnitude) as seven balanced
+// base-128 digits each, in FP16 pairs (value 0 in the low half): out[k] holds
+// digit k, value = sum_k d_k 128^-k up to 2^-43.  Added to 1.5 2^23 grid units,
+// a float shows its multiple of the grid in its mantissa bits, so three
+// additions bring out 3 + 3 + 1 digits as integers (grids 2^-14, 2^-35, 2^-42;
+// the remainders are exact, and the trailing part joins at the second), each
+// with 64 added at the two lower digits so that their 7-bit fields are the
+// balanced digits plus 64.  A field f is put into the mantissa of FP16 1024 + f
+// by one logical operation and 1024 and its offset are taken away by one packed
+// FP16 addition: 20 instructions a value, 9 of them on the FP32 pipe (rounding
+// and scaling digit by digit took 29 and seven conversions of the slow pipe).
+// Digits lie in [-64, 64], the fourth in [-68, 68].
+__device__ __forceinline__ void digits7_pair(df a, df b, uint32_t* out) {
+  constexpr float C1 = (12582912.0f + 8256.0f) * 0x1p-14f, C2 = (12582912.0f + 8256.0f) * 0x1p-35f,
+                  C3 = (12582912.0f + 128.0f) * 0x1p-42f;
+  const float ta = __fadd_rn(a.hi, C1), tb = __fadd_rn(b.hi, C1);
+  const float ra = __fsub_rn(a.hi, __fsub_rn(ta, C1)), rb = __fsub_rn(b.hi, __fsub_rn(tb, C1));
+  const float ua = __fadd_rn(__fadd_rn(ra, a.lo), C2), ub = __fadd_rn(__fadd_rn(rb, b.lo), C2);
+  const float va = __fadd_rn(__fadd_rn(__fsub_rn(ra, __fsub_rn(ua, C2)), a.lo), C3);
+  const float vb = __fadd_rn(__fadd_rn(__fsub_rn(rb, __fsub_rn(ub, C2)), b.lo), C3);
+  auto three = [](float x, float y, uint32_t* o) {
+    const uint32_t lo = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x5410);  // bits 0..15 of both
+    const uint32_t hi = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x6521);  // bits 8..23 of both
+    o[0] = fields(hi >> 6, 0x01ff01ffu, 0xe500e500u);   // 256 + digit: -1280
+    o[1] = fields(lo >> 7, 0x007f007fu, 0xe440e440u);   // 64 + digit: -1088
+    o[2] = fields(lo, 0x007f007fu, 0xe440e440u);
+  };
+  three(ta, tb, out);
+  three(ua, ub, out + 3);
+  out[6] = fields(__byte_perm(__float_as_uint(va), __float_as_uint(vb), 0x5410), 0x01ff01ffu, 0xe480e480u);  // 128 + digit
 }
 
-// Row scale exponents: for target i the largest |K2 ds|, |K1 ds| (phi row)
-// and |K4 ds|, |K3 ds| (psi row) over all sources j != i, in df64 (the same
-// values the kernel digitises).  One thread per target.
-template <bool TRANS>
-__global__ void __launch_bounds__(128) k_tcx_rowexp(int n, const float4* __restrict__ geo, DFConst c,
-                                                    int2* __restrict__ rowexp) {
-  __shared__ float4 sh[4 * 64];
-  __shared__ __align__(16) df tab[kExpTab];
-  df_load_exp_table(tab, c);
+// rowmax[i] = (largest |K2 ds|, |K1 ds| and largest |K4 ds|, |K3 ds|) over the
+// sources j != i of split blockIdx.y, as FP32 bits (zeroed before); FP32 values
+// (in the units of SCALED and TRANS) do, since a digit may exceed its range by
+// a factor near 1.  Split over blockIdx.y: one thread per target alone left the
+// chip idle (n / 128 CTAs).
+template <bool SCALED, bool TRANS>
+__global__ void __launch_bounds__(128) k_tcx_rowmax(int n, const float4* __restrict__ tgt32, PairConst<float> c,
+                                                    uint2* __restrict__ rowmax) {
+  __shared__ float4 sh[2 * 64];
+  const float ks = SCALED ? c.kappa : 1.f;
   const int i = blockIdx.x * 128 + threadIdx.x;
   const int ii = min(i, n - 1);
-  df xi[3], ni[3];
-  {
-    const float4 A = geo[4 * (size_t)ii], B = geo[4 * (size_t)ii + 1], C = geo[4 * (size_t)ii + 2],
-                 D = geo[4 * (size_t)ii + 3];
-    xi[0] = df{A.x, B.x}, xi[1] = df{A.y, B.y}, xi[2] = df{A.z, B.z};
-    ni[0] = df{C.x, D.x}, ni[1] = df{C.y, D.y}, ni[2] = df{C.z, D.z};
-  }
+  const float4 gi = tgt32[2 * ii], ni = tgt32[2 * ii + 1];
   float m0 = 0.f, m1 = 0.f;
-  for (int j0 = 0; j0 < n; j0 += 64) {
+  const int s0 = (int)((int64_t)blockIdx.y * n / gridDim.y), s1 = (int)((int64_t)(blockIdx.y + 1) * n / gridDim.y);
+  for (int j0 = s0; j0 < s1; j0 += 64) {
     __syncthreads();
-    for (int e = threadIdx.x; e < 4 * 64; e += 128) sh[e] = geo[4 * (size_t)min(j0 + e / 4, n - 1) + e % 4];
+    sh[threadIdx.x] = tgt32[2 * min(j0 + (int)threadIdx.x / 2, n - 1) + (threadIdx.x & 1)];
     __syncthreads();
-    const int cnt = min(64, n - j0);
+    const int cnt = min(64, s1 - j0);
     for (int q = 0; q < cnt; ++q) {
-      const float4 A = sh[4 * q], B = sh[4 * q + 1], C = sh[4 * q + 2], D = sh[4 * q + 3];
-      const df xj[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
-      const df nj[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-      df k[4];
-      df_kernel_block<true, TRANS>(xi, ni, xj, nj, TRANS ? df{1.f, 0.f} : df{A.w, B.w}, j0 + q == ii, c, tab, k);
-      m0 = fmaxf(m0, fmaxf(fabsf(k[0].hi), fabsf(k[1].hi)));
-      m1 = fmaxf(m1, fmaxf(fabsf(k[2].hi), fabsf(k[3].hi)));
+      const float4 g = sh[2 * q];
+      float v[4];
+      kernel_block<SCALED, TRANS>(ks * gi.x, ks * gi.y, ks * gi.z, ni.x, ni.y, ni.z,
+                                  make_float4(ks * g.x, ks * g.y, ks * g.z, TRANS ? 1.f : g.w), sh[2 * q + 1],
+                                  j0 + q == ii, c, v);
+      // the phi (A^T: psi) column takes kappa, as in df_kernel_block
+      m0 = fmaxf(m0, fmaxf(fabsf(v[0]) * (TRANS ? 1.f : ks), fabsf(v[1]) * (TRANS ? ks : 1.f)));
+      m1 = fmaxf(m1, fmaxf(fabsf(v[2]) * (TRANS ? 1.f : ks), fabsf(v[3]) * (TRANS ? ks : 1.f)));
     }
   }
-  if (i < n) rowexp[i] = make_int2(scale_exp(m0), scale_exp(m1));
+  if (i < n) {
+    atomicMax(&rowmax[i].x, __float_as_uint(m0));
+    atomicMax(&rowmax[i].y, __float_as_uint(m1));
+  }
+}
+// Row scale exponents from the row maxima (in place)
+__global__ void k_tcx_rowexp(int n, int2* __restrict__ rowexp) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int2 m = rowexp[i];
+  rowexp[i] = make_int2(scale_exp(__int_as_float(m.x)), scale_exp(__int_as_float(m.y)));
 }
 
 // colmax[b] = max |u_b| over the 2n values (FP32 bits; colmax zeroed before): grid (x, nb)
@@ -359,25 +406,27 @@ __global__ void k_tcx_colmax(int n, const double* __restrict__ u, const int* __r
 
 // U digit tiles: for step x and K chunk kc, row 64 l + b holds digit l of
 // u_b 2^f(b), K = 2 j' + c (phi_j, psi_j of the chunk's sources), K-major.
-// One thread per (x, kc, b, k).
+// One thread per (x, kc, b, source): its phi and psi digits are one FP16 pair.
+// The digits are taken from a df64 copy on the FP32 pipe (in FP64, seven
+// roundings a value on two FP64 lanes per SM took 125 us at N = 20001).
 __global__ void k_tcx_pack_u(int n, int nb, int n_steps, const double* __restrict__ u, const int* __restrict__ rhs,
                              const unsigned* __restrict__ colmax, __half* __restrict__ upk) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)n_steps * kChunks * kRHS * kKC) return;
-  const int k = (int)(e % kKC), b = (int)((e / kKC) % kRHS);
-  const int kc = (int)((e / (kKC * kRHS)) % kChunks);
-  const int64_t x = e / ((int64_t)kKC * kRHS * kChunks);
-  const int j = (int)(x * kStep) + kc * (kKC / 2) + (k >> 1), c = k & 1;
-  double v = 0.0;
-  if (b < nb && j < n)
-    v = u[(int64_t)(rhs ? rhs[b] : b) * 2 * n + (int64_t)c * n + j] * p2d(scale_exp(__uint_as_float(colmax[b])));
+  constexpr int kSrc = kKC / 2;
+  if (e >= (int64_t)n_steps * kChunks * kRHS * kSrc) return;
+  const int q = (int)(e % kSrc), b = (int)((e / kSrc) % kRHS);
+  const int kc = (int)((e / (kSrc * kRHS)) % kChunks);
+  const int64_t x = e / ((int64_t)kSrc * kRHS * kChunks);
+  const int j = (int)(x * kStep) + kc * kSrc + q;
+  uint32_t d[kLv] = {0, 0, 0, 0, 0, 0, 0};
+  if (b < nb && j < n) {
+    const double* ub = u + (int64_t)(rhs ? rhs[b] : b) * 2 * n;
+    const double s = p2d(scale_exp(__uint_as_float(colmax[b])));
+    digits7_pair(df_from_double(s * ub[j]), df_from_double(s * ub[n + j]), d);
+  }
   unsigned char* tile = reinterpret_cast<unsigned char*>(upk) + x * (int64_t)kBBytes + kc * kBChunk;
 #pragma unroll
-  for (int l = 0; l < kLv; ++l) {
-    const double d = rint(v);
-    *reinterpret_cast<__half*>(tile + koff(kRHS * l + b, k)) = __float2half_rn((float)d);
-    v = (v - d) * 128.0;
-  }
+  for (int l = 0; l < kLv; ++l) *reinterpret_cast<uint32_t*>(tile + koff(kRHS * l + b, 2 * q)) = d[l];
 }
 
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -398,47 +447,35 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // target tg: the df64 block, scaled per row, as digit planes written into
 // the K chunk's planes at `a` (digit k at a + k kPlane; byte offsets offp and
 // offq of the target's phi and psi rows at the pair's K columns).
-template <bool EDGE, bool TRANS>
-__device__ __forceinline__ void tcx_gen(const df* xi, const df* ni, const float4* Sq, int jq, int tg, int n,
-                                        bool tvalid, const DFConst& c, const df* tab, float r0, float r1,
-                                        unsigned char* a, uint32_t offp, uint32_t offq) {
-  float dg[2][4][kLv];  // [source][value: K2, K1, K4, K3][digit]
+template <bool EDGE, bool TRANS, bool SCALED>
+__device__ __forceinline__ void tcx_gen(const GeoDF& T, const float4* Sq, int jq, int tg, int n, bool tvalid,
+                                        const DFConst& c, const df* tab, float r0, float r1, unsigned char* a,
+                                        uint32_t offp, uint32_t offq) {
+  uint32_t dp[2][kLv], dq[2][kLv];  // [source]: digits of (K2, K1) and of (K4, K3)
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
-    const float4 A = Sq[4 * u], B = Sq[4 * u + 1], C = Sq[4 * u + 2], D = Sq[4 * u + 3];
-    const df xj[3] = {df{A.x, B.x}, df{A.y, B.y}, df{A.z, B.z}};
-    const df nj[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
+    const GeoDF S = load_geo(Sq + kGeo * u);
     const bool z = EDGE && (!tvalid || jq + u >= n || jq + u == tg);
     df k[4];
-    df_kernel_block<EDGE, TRANS>(xi, ni, xj, nj, TRANS ? df{1.f, 0.f} : df{A.w, B.w}, z, c, tab, k);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      df w = df_scale(k[v], v < 2 ? r0 : r1);
-      if (EDGE && z) w = df{0.f, 0.f};
-      digits7(w, dg[u][v]);
-    }
+    df_kernel_block<EDGE, TRANS, SCALED>(T.x, T.n, S.x, S.n, S.a, z, c, tab, r0, r1, k);
+    if (EDGE && z) k[0] = k[1] = k[2] = k[3] = df{0.f, 0.f};
+    digits7_pair(k[0], k[1], dp[u]);
+    digits7_pair(k[2], k[3], dq[u]);
   }
-  // phi row: (K2, K1) of sources 0, 1 in the pair's four K columns; psi row: (K4, K3)
 #pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int k = 0; k < kLv; ++k) {
-      const __half2 p0 = __floats2half2_rn(dg[0][2 * m][k], dg[0][2 * m + 1][k]);
-      const __half2 p1 = __floats2half2_rn(dg[1][2 * m][k], dg[1][2 * m + 1][k]);
-      uint2 w;
-      w.x = *reinterpret_cast<const uint32_t*>(&p0);
-      w.y = *reinterpret_cast<const uint32_t*>(&p1);
-      *reinterpret_cast<uint2*>(a + k * kPlane + (m ? offq : offp)) = w;
-    }
+  for (int k = 0; k < kLv; ++k) {
+    *reinterpret_cast<uint2*>(a + k * kPlane + offp) = make_uint2(dp[0][k], dp[1][k]);
+    *reinterpret_cast<uint2*>(a + k * kPlane + offq) = make_uint2(dq[0][k], dq[1][k]);
+  }
 }
 
 // items: {t0, first step, end step, split}; part: [b][split][2n] for the nb
-// right-hand sides of this pass.
-template <bool TRANS>
+// right-hand sides of this pass, times rowf.x (phi) and rowf.y (psi rows).
+template <bool TRANS, bool SCALED>
 __global__ void __launch_bounds__(kThreads, 1)
     k_mrhs_tcx(int n, int nb, int n_splits, const int4* __restrict__ items, const float4* __restrict__ geo,
                const int2* __restrict__ rowexp, const unsigned* __restrict__ colmax, const __half* __restrict__ upk,
-               double* __restrict__ part, DFConst c, int* __restrict__ err) {
+               double* __restrict__ part, DFConst c, double2 rowf, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* ufull = reinterpret_cast<uint64_t*>(smem + kOffBar);  // kRing: U digit tiles landed
   uint64_t* sfull = ufull + kRing;                                 // kRing: source records landed
@@ -487,8 +524,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) break;
         const int st = x0 + x;
         const int cnt = min(kStep, n - st * kStep);
-        arrive_expect_tx(&sfull[q], cnt * 64);
-        bulk_load(smem + kOffS + q * kSRec, geo + 4 * (int64_t)st * kStep, cnt * 64, &sfull[q]);
+        arrive_expect_tx(&sfull[q], cnt * kGeo * 16);
+        bulk_load(smem + kOffS + q * kSRec, geo + kGeo * (int64_t)st * kStep, cnt * kGeo * 16, &sfull[q]);
         arrive_expect_tx(&ufull[q], kBBytes);
         bulk_load(smem + kOffB + q * kBBytes, reinterpret_cast<const unsigned char*>(upk) + (int64_t)st * kBBytes,
                   kBBytes, &ufull[q]);
@@ -542,13 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tr = 8 * (warp & 7) + (lane & 7), sp = 4 * (warp >> 3) + (lane >> 3);
     const int tg = t0 + tr;  // the generated target
     const bool gvalid = tg < n;
-    df xi[3], ni[3];
-    {
-      const int64_t r = 4 * (int64_t)min(tg, n - 1);
-      const float4 A = geo[r], B = geo[r + 1], C = geo[r + 2], D = geo[r + 3];
-      xi[0] = df{A.x, B.x}, xi[1] = df{A.y, B.y}, xi[2] = df{A.z, B.z};
-      ni[0] = df{C.x, D.x}, ni[1] = df{C.y, D.y}, ni[2] = df{C.z, D.z};
-    }
+    const GeoDF T = load_geo(geo + kGeo * (int64_t)min(tg, n - 1));
     const int2 rg_e = rowexp[min(tg, n - 1)];
     const float r0 = p2f(rg_e.x), r1 = p2f(rg_e.y);
     const uint32_t offp = koff(tr, 4 * (sp & 3)), offq = koff(kTgt + tr, 4 * (sp & 3));
@@ -562,16 +593,31 @@ __global__ void __launch_bounds__(kThreads, 1)
     df acc[16];
 #pragma unroll
     for (int b = 0; b < 16; ++b) acc[b] = df{0.f, 0.f};
-    auto read_back = [&]() {  // acc += sum_L level L 128^-L, exact levels, df64 sums
+    // acc += sum_L level L 128^-L: the exact levels 0 .. 3 by TwoSums, 4 .. 6 (below
+    // 2^-28 of level 0's weight) in FP32 with the trailing parts
+    auto read_back = [&]() {
+      float tail[16];
 #pragma unroll
-      for (int L = 0; L < kLv; ++L) {
+      for (int L = kLv - 1; L >= 0; --L) {
         uint32_t v[16];
         tc::tmem_ld16_async(dthr + kRHS * L, v);
         tc::tmem_wait_ld16(v);
-        const float sc = p2f(-7 * L);
 #pragma unroll
-        for (int b = 0; b < 16; ++b) acc[b] = df_add_f(acc[b], __fmul_rn(__uint_as_float(v[b]), sc));
+        for (int b = 0; b < 16; ++b) {
+          const float x = __uint_as_float(v[b]);
+          if (L == kLv - 1) {
+            tail[b] = x;
+          } else if (L >= 4) {
+            tail[b] = __fmaf_rn(tail[b], 0x1p-7f, x);
+          } else {
+            const df t = two_sum(acc[b].hi, __fmul_rn(x, p2f(-7 * L)));
+            acc[b].hi = t.hi;
+            acc[b].lo = __fadd_rn(acc[b].lo, L == 3 ? __fmaf_rn(tail[b], 0x1p-28f, t.lo) : t.lo);
+          }
+        }
       }
+#pragma unroll
+      for (int b = 0; b < 16; ++b) acc[b] = two_sum(acc[b].hi, acc[b].lo);
     };
     auto drain = [&](int d) {
       ok = ok && tc::mbar_wait_timed(done, d & 1, kWaitLimitNs);
@@ -600,12 +646,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const int j0 = (x0 + it) * kStep;
       const bool edge = tile_edge || (j0 + kStep > n) || (j0 < t0 + kTgt && j0 + kStep > t0);
-      const float4* Sq = reinterpret_cast<const float4*>(smem + kOffS + q * kSRec) + 4 * 2 * sp;
+      const float4* Sq = reinterpret_cast<const float4*>(smem + kOffS + q * kSRec) + kGeo * 2 * sp;
       unsigned char* a = smem + kOffA + s * kAStage + (sp >> 2) * kLv * kPlane;
       if (edge)
-        tcx_gen<true, TRANS>(xi, ni, Sq, j0 + 2 * sp, tg, n, gvalid, c, tab, r0, r1, a, offp, offq);
+        tcx_gen<true, TRANS, SCALED>(T, Sq, j0 + 2 * sp, tg, n, gvalid, c, tab, r0, r1, a, offp, offq);
       else
-        tcx_gen<false, TRANS>(xi, ni, Sq, j0 + 2 * sp, tg, n, gvalid, c, tab, r0, r1, a, offp, offq);
+        tcx_gen<false, TRANS, SCALED>(T, Sq, j0 + 2 * sp, tg, n, gvalid, c, tab, r0, r1, a, offp, offq);
       tc::fence_proxy_async_smem();  // the generic stores, before the tensor core reads them
       __syncwarp();
       if (lane == 0) mbar_arrive(&ready[s]);
@@ -617,7 +663,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int comp = rr / kTgt;
       const int2 re = rowexp[ti];
       const int e = comp ? re.y : re.x;
-      const double area = TRANS ? (double)geo[4 * (int64_t)ti].w + (double)geo[4 * (int64_t)ti + 1].w : 1.0;
+      const double area = (TRANS ? (double)geo[kGeo * (int64_t)ti].w + (double)geo[kGeo * (int64_t)ti + 1].w : 1.0) *
+                          (comp ? rowf.y : rowf.x);
 #pragma unroll
       for (int b = 0; b < 16; ++b) {
         const int bg = 16 * cb + b;
@@ -682,15 +729,29 @@ ItemPlan* tcx_plan(Surface* s, int n, int* S_out) {
   return it->second.get();
 }
 
+// The kappa-scaled form of the multi-RHS df64 passes (kappa >= 1e-6 / A, the
+// rule of the single-system pass): sigma = kappa, else 1.
+struct MrhsScale {
+  bool scaled;
+  double sigma, gscale;
+};
+MrhsScale mrhs_scale(const DFConst& c) {
+  const double kappa = (double)c.kappa.hi + (double)c.kappa.lo;
+  if (kappa < 1e-6) return MrhsScale{false, 1.0, 1.0};
+  return MrhsScale{true, kappa, std::exp2(std::ceil(std::log2(kappa)))};
+}
+
 // The exact tensor-core pass for nb <= 64 right-hand sides (u at ub, or the
 // rows rhs[b] of u when rhs is given): row exponents (cached per surface and
 // medium), right-hand-side digits, the kernel; writes part64 [b][split][2n]
 // and returns the number of splits.
-int launch_tcx(Surface* s, int n, int nb, bool transpose, const double* ub, const int* rhs, const DFConst& c) {
+int launch_tcx(Surface* s, int n, int nb, bool transpose, const double* ub, const int* rhs, const DFConst& c,
+               const MrhsScale& sc) {
   const int dir = transpose ? 1 : 0;
   const int n_steps = (n + tcx::kStep - 1) / tcx::kStep;
-  s->grow(s->geodf, (size_t)4 * n);
-  k_pack_mrhs_df<<<dim3((n + 255) / 256, 1), 256, 0, s->stream>>>(n, 0, s->tgt64.p, ub, rhs, s->geodf.p, s->udf.p);
+  s->grow(s->geodf, (size_t)kGeo * n);
+  k_pack_mrhs_df<<<dim3((n + 127) / 128, 1), 128, 0, s->stream>>>(n, 0, s->tgt64.p, ub, rhs, s->geodf.p, s->udf.p,
+                                                                  sc.sigma, sc.gscale);
   BIPB_LAUNCHED(s);
   const uint64_t gen0 = s->alloc_gen;
   s->grow(s->tcx_rowexp[dir], (size_t)n);
@@ -698,20 +759,34 @@ int launch_tcx(Surface* s, int n, int nb, bool transpose, const double* ub, cons
   float* key = s->tcx_key[dir];
   if (s->alloc_gen != gen0 || s->tcx_n[dir] != n || key[0] != c.eps.hi || key[1] != c.eps.lo ||
       key[2] != c.kappa.hi || key[3] != c.kappa.lo) {
-    if (transpose)
-      tcx::k_tcx_rowexp<true><<<(n + 127) / 128, 128, 0, s->stream>>>(n, s->geodf.p, c, rowexp);
+    BIPB_CUDA(cudaMemsetAsync(rowexp, 0, (size_t)n * sizeof(int2), s->stream));
+    PairConst<float> pc;
+    pc.eps = c.eps.hi, pc.inveps = c.inveps.hi, pc.kappa = c.kappa.hi;
+    pc.nkl2e = sc.scaled ? -1.4426950408889634f : (float)(-(double)c.kappa.hi * 1.4426950408889634);
+    pc.smax = sc.scaled ? (float)(kSMaxD / sc.sigma) : kSMaxF;
+    const int tiles = (n + 127) / 128;
+    const dim3 grid(tiles, std::min((n + 255) / 256, std::max(1, (16 * s->num_sms + tiles - 1) / tiles)));
+    auto* rm = reinterpret_cast<uint2*>(rowexp);
+    if (sc.scaled && transpose)
+      tcx::k_tcx_rowmax<true, true><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+    else if (sc.scaled)
+      tcx::k_tcx_rowmax<true, false><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+    else if (transpose)
+      tcx::k_tcx_rowmax<false, true><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
     else
-      tcx::k_tcx_rowexp<false><<<(n + 127) / 128, 128, 0, s->stream>>>(n, s->geodf.p, c, rowexp);
+      tcx::k_tcx_rowmax<false, false><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+    BIPB_LAUNCHED(s);
+    tcx::k_tcx_rowexp<<<tiles, 128, 0, s->stream>>>(n, rowexp);
     BIPB_LAUNCHED(s);
     s->tcx_n[dir] = n;
     key[0] = c.eps.hi, key[1] = c.eps.lo, key[2] = c.kappa.hi, key[3] = c.kappa.lo;
   }
   s->grow(s->tcx_colmax, (size_t)kNB);
   BIPB_CUDA(cudaMemsetAsync(s->tcx_colmax.p, 0, kNB * sizeof(unsigned), s->stream));
-  tcx::k_tcx_colmax<<<dim3((unsigned)std::min(64, (2 * n + 255) / 256), nb), 256, 0, s->stream>>>(n, ub, rhs,
-                                                                                                  s->tcx_colmax.p);
+  tcx::k_tcx_colmax<<<dim3((unsigned)std::min(64, (2 * n + 255) / 256), nb), 256, 0, s->stream>>>(
+      n, ub, rhs, s->tcx_colmax.p);
   BIPB_LAUNCHED(s);
-  const int64_t pk = (int64_t)n_steps * tcx::kChunks * tcx::kRHS * tcx::kKC;
+  const int64_t pk = (int64_t)n_steps * tcx::kChunks * tcx::kRHS * (tcx::kKC / 2);
   s->grow(s->tcx_upk, (size_t)n_steps * tcx::kBBytes / sizeof(float));
   __half* upk = reinterpret_cast<__half*>(s->tcx_upk.p);
   tcx::k_tcx_pack_u<<<(int)((pk + 255) / 256), 256, 0, s->stream>>>(n, nb, n_steps, ub, rhs, s->tcx_colmax.p, upk);
@@ -723,12 +798,15 @@ int launch_tcx(Surface* s, int n, int nb, bool transpose, const double* ub, cons
     s->grow(s->tc_err, 1);
     BIPB_CUDA(cudaMemsetAsync(s->tc_err.p, 0, sizeof(int), s->stream));
   }
-  auto kernel = transpose ? tcx::k_mrhs_tcx<true> : tcx::k_mrhs_tcx<false>;
+  auto kernel = transpose ? (sc.scaled ? tcx::k_mrhs_tcx<true, true> : tcx::k_mrhs_tcx<true, false>)
+                          : (sc.scaled ? tcx::k_mrhs_tcx<false, true> : tcx::k_mrhs_tcx<false, false>);
+  // row factors of the kappa-scaled form
+  const double2 rowf = transpose ? make_double2(sc.sigma * sc.sigma, sc.sigma) : make_double2(sc.sigma, sc.sigma * sc.sigma);
   BIPB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tcx::kSmemBytes));
   {
     TimedLaunch tl(s, transpose ? kTMvDFT : kTMvDF);
     kernel<<<plan->n_items, tcx::kThreads, tcx::kSmemBytes, s->stream>>>(
-        n, nb, S, plan->items.p, s->geodf.p, rowexp, s->tcx_colmax.p, upk, s->part64.p, c, s->tc_err.p);
+        n, nb, S, plan->items.p, s->geodf.p, rowexp, s->tcx_colmax.p, upk, s->part64.p, c, rowf, s->tc_err.p);
     BIPB_LAUNCHED(s);
   }
   return S;
@@ -756,6 +834,7 @@ void matvec_df_mrhs(Surface* s, const SysLayout& L, const DFConst& c, bool trans
     for (int k = 0; k < L.K; ++k) act.push_back(k);
   }
   const int n_act = (int)act.size();
+  const MrhsScale sc = mrhs_scale(c);
   for (int g0 = 0; g0 < n_act; g0 += kNB) {
     const int nb = std::min(kNB, n_act - g0);
     // 16 or more right-hand sides, or A^T: the exact tensor-core form; fewer: df64 on the CUDA cores
@@ -796,7 +875,7 @@ void matvec_df_mrhs(Surface* s, const SysLayout& L, const DFConst& c, bool trans
       rhs = s->rhs_idx.p;
       ub = u;
     }
-    if (tensor) S = launch_tcx(s, n, nb, transpose, ub, rhs, c);
+    if (tensor) S = launch_tcx(s, n, nb, transpose, ub, rhs, c, sc);
     const uint64_t tkey = 0x7f0000000000ull ^ ((uint64_t)n << 16) ^ ((uint64_t)S << 8) ^ (uint64_t)nb;
     auto tt = s->plans.find(tkey);
     if (tt == s->plans.end()) {
@@ -813,21 +892,21 @@ void matvec_df_mrhs(Surface* s, const SysLayout& L, const DFConst& c, bool trans
       launch_reduce_matvec64(s, Lb, tt->second->tab.p, s->part64.p, u, y, dphi, dpsi, nullptr, 0);
       continue;
     }
-    s->grow(s->geodf, (size_t)4 * n);
+    s->grow(s->geodf, (size_t)kGeo * n);
     s->grow(s->udf, (size_t)nb * n);
     k_pack_mrhs_df<<<dim3((n + 255) / 256, nb + 1), 256, 0, s->stream>>>(n, nb, s->tgt64.p, ub, rhs, s->geodf.p,
-                                                                          s->udf.p);
+                                                                          s->udf.p, sc.sigma, sc.gscale);
     BIPB_LAUNCHED(s);
     {
       TimedLaunch tl(s, kTMvDF);
       if (G == 1)
-        launch_mrhs_df<1>(s, plan, n, nb, S, c);
+        launch_mrhs_df<1>(s, plan, n, nb, S, c, sc.scaled, sc.sigma);
       else if (G == 2)
-        launch_mrhs_df<2>(s, plan, n, nb, S, c);
+        launch_mrhs_df<2>(s, plan, n, nb, S, c, sc.scaled, sc.sigma);
       else if (G == 4)
-        launch_mrhs_df<4>(s, plan, n, nb, S, c);
+        launch_mrhs_df<4>(s, plan, n, nb, S, c, sc.scaled, sc.sigma);
       else
-        launch_mrhs_df<8>(s, plan, n, nb, S, c);
+        launch_mrhs_df<8>(s, plan, n, nb, S, c, sc.scaled, sc.sigma);
     }
     launch_reduce_matvec64(s, Lb, tt->second->tab.p, s->part64.p, u, y, dphi, dpsi, nullptr, 0);
   }

@@ -281,4 +281,51 @@ __device__ __forceinline__ void sym_pair2(const f2* xt, const f2* nt, const f2* 
     }
   }
 }
+
+// ------------------------------------------------------------------ kernel blocks
+// The four kernel values of pair (target i, source j) times ds_j (times 4 pi),
+// in FP32: returns (K2, K1) in v[0], v[1] and (K4, K3) in v[2], v[3].
+// TRANS: the block of A^T instead, output element i gathering input element
+// j (pair_transpose of pair.cuh with d = x_i - x_j): the phi row (K2_ji,
+// K4_ji) in v[0], v[1], the psi row (K1_ji, K3_ji) in v[2], v[3], times the
+// record's area field (the output's area is applied to the sums), i.e.
+// ((1 - eps t) c_i s^3, K4, (1 - e) s, (1 - t/eps) c_j s^3).
+// SCALED: positions, area and normal in kappa-scaled units (k_tc_colexp,
+// mrhs_tc.cu: kappa r = r2 s and (w - 3) s^2 = 3 (t - 1) s^2 + e; one row
+// comes out with an extra power of kappa); c.nkl2e and c.smax are then
+// -log2(e) and the 1/r cap in those units.
+template <bool SCALED, bool TRANS>
+__device__ __forceinline__ void kernel_block(float xi, float yi, float zi, float nxi, float nyi, float nzi, float4 g,
+                                             float4 nv, bool zero, const PairConst<float>& c, float* v) {
+  const float dx = xi - g.x, dy = yi - g.y, dz = zi - g.z;
+  const float r2 = dx * dx + dy * dy + dz * dz;
+  float s = fminf(rsqrt_approx(r2), c.smax);
+  s = zero ? 0.f : s;
+  const float r = r2 * s;
+  const float e = ex2_approx(r * c.nkl2e);
+  const float kr = SCALED ? r : r * c.kappa;
+  const float ci = nxi * dx + nyi * dy + nzi * dz;
+  const float cj = nv.x * dx + nv.y * dy + nv.z * dz;
+  const float cij = nxi * nv.x + nyi * nv.y + nzi * nv.z;
+  const float t = e * kr + e;
+  const float tm1 = t - 1.f;
+  const float sa = s * g.w;
+  const float s2 = s * s;
+  const float s3a = s2 * sa;
+  // (w - 3) s^2
+  const float wm3s2 = SCALED ? (3.f * tm1) * s2 + e : ((t - e) * kr + 3.f * tm1) * s2;
+  const float k4 = (tm1 * cij - wm3s2 * (ci * cj)) * s3a;
+  if (!TRANS) {
+    v[1] = sa - e * sa;                                  // K1 ds = (1 - e) s ds
+    v[0] = ((c.eps * t - 1.f) * cj) * s3a;               // K2 ds
+    v[3] = ((t * c.inveps - 1.f) * ci) * s3a;            // K3 ds
+    v[2] = k4;                                           // K4 ds
+  } else {
+    v[0] = ((1.f - c.eps * t) * ci) * s3a;               // K2_ji
+    v[1] = k4;                                           // K4_ji
+    v[2] = sa - e * sa;                                  // K1_ji
+    v[3] = ((1.f - t * c.inveps) * cj) * s3a;            // K3_ji
+  }
+}
+
 }  // namespace bipb

@@ -128,3 +128,26 @@ def test_krylov_step_as_cluster_and_as_kernels(bipb, orc, n, sets, precond):
                                precond=precond, restart=restart)
                 assert all(i["converged"] for i in info)
                 np.testing.assert_allclose(s.energy()[:2], ref, rtol=rt)
+
+
+@pytest.mark.parametrize("n", [2, 63, 65, 515])
+@pytest.mark.parametrize("kappa", [0.0, 9e-7, 1.1e-6, 0.1257, 2.5])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_multi_rhs_double_float_scaling_rule(bipb, orc, n, kappa, transpose):
+    """The multi-RHS double-float passes on both sides of the rule that scales their
+    coordinates by kappa (1e-6), on surfaces around one tile of 64 targets and one
+    step of 16 sources, on the CUDA cores (3 right-hand sides, forward) and as exact
+    digits (17): the bound of test_multi_rhs_df64_matvec_matches_oracle."""
+    p = synth.protein_like_problem(level=3, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, n, replace=False))
+    c, nv, a = p.centroids[keep], p.normals[keep], p.areas[keep]
+    f = orc.matvec_t if transpose else orc.matvec
+    for n_rhs in (3, 17):
+        U = np.random.default_rng(n + n_rhs).standard_normal((n_rhs, 2 * n))
+        with bipb.Surface(c, nv, a) as s:
+            yd = torch.full_like(_dev(U), float("nan"))
+            s.matvec(_dev(U), yd, precision=bipb.DF64, transpose=transpose, med=bipb.medium(1.0, 80.0, kappa))
+            Y = yd.cpu().numpy()
+        for r in (0, n_rhs - 1):
+            ref = f(c, nv, a, 80.0, kappa, U[r])
+            np.testing.assert_allclose(Y[r], ref, rtol=0, atol=2e-12 * np.abs(ref).max(), err_msg=f"{n_rhs} {r}")
