@@ -278,7 +278,7 @@ struct FarField {
   DevBuf<float> nodes;     // per slot 3 x (degree+1) Chebyshev nodes, centred FP32
   DevBuf<float4> rec;      // records, 2 float4 each, rec_stride per system
   DevBuf<float> part;      // partial sums, 2 lmax per item and system
-  DevBuf<double> upart;    // partial proxy weights, 4 (degree+1)^3 per piece and system
+  DevBuf<float2> upart;    // partial proxy weights (sum, trailing part), 4 (degree+1)^3 per piece and system
 };
 
 struct Surface {
@@ -441,6 +441,7 @@ struct SymStep {
   double dphi = 0.0, dpsi = 0.0;  // the diagonal
   bool transpose = false;
 };
+constexpr double kSymKappaMin = 1e-6;  // smallest kappa (1/A) of the kappa-scaled FP32 and FP64 pairs
 enum { kSymPack = 1, kSymPairs = 2, kSymReduce = 4, kSymAll = 7 };
 // y = A u (or A^T u) by the handle's FP32 variant if it is a symmetric one that
 // takes this layout and medium (false otherwise, nothing launched); stages is
@@ -453,8 +454,8 @@ bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c, do
 bool matvec_sym_df(Surface* s, const SysLayout& L, const DFConst& c, double kappa, bool transpose, const double* u,
                    double* y, double dphi, double dpsi, const int* skip, int skip_stride);
 // y = A u (or A^T u) for right-hand sides of one surface by the far-field treecode (tree.cu)
-void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c, bool transpose, const double* u, double* y,
-                 double dphi, double dpsi, const int* skip, int skip_stride);
+void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c, double kappa, bool transpose,
+                 const double* u, double* y, double dphi, double dpsi, const int* skip, int skip_stride);
 // the far-field operator of the handle's parameters (built on first use; synchronises then)
 FarField* far_field(Surface* s);
 // y = A u (or A^T u) for right-hand sides of one surface with the split-FP16

@@ -945,7 +945,7 @@ void matvec(Surface* s, const SysLayout& L, const bipb_medium& m, int precision,
     return;
   }
   if (precision == BIPB_TREE32) {
-    matvec_tree(s, L, pair_const<float>(m), transpose, u, y, dphi, dpsi, skip, skip_stride);
+    matvec_tree(s, L, pair_const<float>(m), m.kappa, transpose, u, y, dphi, dpsi, skip, skip_stride);
     return;
   }
   if (precision == BIPB_DF64) {

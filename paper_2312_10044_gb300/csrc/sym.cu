@@ -736,7 +736,6 @@ void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typena
 // records for kappa >= kSymKappaMin; in between (a Debye length above 1e6 A)
 // the scaled 1/r^3 could leave the FP32 range, and the caller takes the
 // ordered kernels.
-constexpr double kSymKappaMin = 1e-6;
 
 template <typename T>
 bool sym_form(double kappa, PairConst<T>& c, bool& laplace) {

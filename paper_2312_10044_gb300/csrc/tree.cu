@@ -6,7 +6,7 @@
 // sum: output element t gathers column t of A, whose entries of row element
 // j depend on n_j only through K3 and K4, linearly, so the sources carry
 // a_j = wphi_j and m_j = wpsi_j n_j, the pair is the transposed one
-// (pair_transpose, pair.cuh) and the output element's area multiplies the
+// (tree_pair2) and the output element's area multiplies the
 // sums.  The tree, the lists and the proxies serve both directions.  The elements form a binary tree of
 // clusters; a cluster holding more than `leaf` elements is split in two at
 // the median of its longest box side (ties by element index), so every
@@ -26,18 +26,18 @@
 // for the kernel over a far cluster, as the Taylor series about the cluster
 // centre does in the paper.  Because proxies and elements are records of the
 // same form (position, a, m), every list entry is summed by the one ordered
-// pair formula (pair_forward, pair.cuh) and the far-field pass has the shape
+// pair formula (tree_pair2) and the far-field pass has the shape
 // of the direct pass.
 //
 // One mat-vec is five launches on the handle's stream:
 //   k_tree_pack   element records in tree order (gathered through perm);
-//   k_tree_up     partial proxy weights, one CTA per piece of <= 2048
-//                 elements of a far cluster (FP32 per 32 elements, FP64 across);
-//   k_tree_proxy  proxy records (pieces added in order, FP64);
+//   k_tree_up     partial proxy weights, one CTA per piece of <= 512
+//                 elements of a far cluster (FP32 runs of 32 elements, TwoSums across);
+//   k_tree_proxy  proxy records (pieces added in order, TwoSums);
 //   k_tree_far    one CTA per work item: a target leaf (one target per thread)
 //                 against a run of its list's records, streamed through shared
 //                 memory; FP32 partial sums per item;
-//   k_tree_reduce per target, its leaf's items in order (FP64), 1/(4 pi) and
+//   k_tree_reduce per target, its leaf's items in order (TwoSums), 1/(4 pi) and
 //                 the diagonal, scattered back to element order.
 // Every sum is in a fixed order, so the pass is bitwise reproducible.
 #include <algorithm>
@@ -45,25 +45,27 @@
 #include <numeric>
 
 #include "internal.cuh"
+#include "symstep.cuh"
 
 namespace bipb {
 
 namespace {
 
 constexpr double kInv4PiT = 1.0 / (4.0 * kPi);
-constexpr int kUpPiece = 2048;  // elements per piece of the upward pass
-constexpr int kUpChunk = 32;    // elements staged per step of the upward pass
-constexpr int kFarCH = 256;     // records per shared-memory chunk of the far-field kernel
+constexpr int kUpPiece = 512;  // elements per piece of the upward pass
+constexpr int kUpRun = 32;      // elements per FP32 run of the upward pass
+constexpr int kFarCH = 512;     // records per shared-memory chunk of the far-field kernel
 constexpr int kMaxLeaf = 512;
+constexpr int kFarMinB = 2;     // resident CTAs of kMaxLeaf threads the far-field kernel's registers allow
 
 __device__ __forceinline__ bool tree_skipped(const int* skip, int stride, int sys) {
   return skip != nullptr && skip[(size_t)sys * stride] != 0;
 }
 
 // ------------------------------------------------------------------ kernels
-// rec[k][t] = (x, a = ds psi), (m = ds phi n, 0) of element perm[t], system k;
-// transposed: (x, a = wphi), (m = wpsi n, 0)
-__global__ void k_tree_pack(int n, int rec_stride, bool transpose, const int* __restrict__ perm,
+// rec[k][t] = (sigma x, a = ds psi), (m = sigma ds phi n, 0) of element perm[t],
+// system k; transposed: a = wphi, m = sigma wpsi n.  sigma: see tree_pair2.
+__global__ void k_tree_pack(int n, int rec_stride, bool transpose, double sigma, const int* __restrict__ perm,
                             const double4_32a* __restrict__ tgt64, const int4* __restrict__ lay,
                             const double* __restrict__ u, float4* __restrict__ rec, const int* __restrict__ skip,
                             int skip_stride) {
@@ -74,9 +76,9 @@ __global__ void k_tree_pack(int n, int rec_stride, bool transpose, const int* __
   const int e = perm[t];
   const double4_32a g = tgt64[2 * (L.x + e)], v = tgt64[2 * (L.x + e) + 1];
   const double phi = u[L.z + e], psi = u[L.z + L.y + e];
-  const double a = transpose ? phi : g.w * psi, f = transpose ? psi : g.w * phi;
+  const double a = transpose ? phi : g.w * psi, f = sigma * (transpose ? psi : g.w * phi);
   const size_t o = 2 * ((size_t)k * rec_stride + t);
-  rec[o] = make_float4((float)g.x, (float)g.y, (float)g.z, (float)a);
+  rec[o] = make_float4((float)(sigma * g.x), (float)(sigma * g.y), (float)(sigma * g.z), (float)a);
   rec[o + 1] = make_float4((float)(f * v.x), (float)(f * v.y), (float)(f * v.z), 0.f);
 }
 
@@ -85,30 +87,51 @@ __global__ void k_tree_pack(int n, int rec_stride, bool transpose, const int* __
 // with l_i the barycentric Lagrange basis at the cluster's Chebyshev nodes
 // (weights (-1)^i, halved at both ends).  An element on a node takes the
 // node's basis value 1 exactly.
+//
+// Bound by the FP32 pipe: thread (g, q0, q1) of G groups adds every G-th
+// element of a chunk to its column of DEG + 1 proxies, one multiplication and
+// four multiply-adds (two packed) each, so the product of the first two basis
+// values and the loads are shared by the column.  FP32 over 32 elements, the
+// runs and the groups by TwoSums (PartSum); upart holds (sum, trailing part).
+// At N = 120001, degree 6, 0.10 ms; one proxy per thread with FP64 sums took
+// 0.29 ms.
+template <int DEG>
+struct UpShape {
+  static constexpr int NP = DEG + 1, P = NP * NP * NP, Q = NP * NP;
+  static constexpr int NT = 256, G = NT / Q;  // groups of elements
+  static constexpr int CH = kUpRun * G;       // elements staged at once
+  static constexpr int NB = (NP + 3) / 4 * 4;
+};
 template <int DEG>
 __global__ void __launch_bounds__(256) k_tree_up(const int4* __restrict__ pieces, const float* __restrict__ nodes,
-                                                 int rec_stride, const float4* __restrict__ rec,
-                                                 double* __restrict__ upart, int n_pieces,
+                                                 float sigma, int rec_stride, const float4* __restrict__ rec,
+                                                 float2* __restrict__ upart, int n_pieces,
                                                  const int* __restrict__ skip, int skip_stride) {
-  constexpr int NP = DEG + 1, P = NP * NP * NP, PT = (P + 255) / 256;
-  __shared__ float bas[kUpChunk][3][NP];
-  __shared__ float4 val[kUpChunk];
+  using U = UpShape<DEG>;
+  constexpr int NP = U::NP, P = U::P, G = U::G, CH = U::CH, NB = U::NB;
+  __shared__ __align__(16) float bas[CH][3][NB];
+  __shared__ float4 val[CH];
   __shared__ float nd[3][NP];
+  __shared__ float2 comb[G * P];
   const int k = blockIdx.y;
   if (tree_skipped(skip, skip_stride, k)) return;
   const int4 pc = pieces[blockIdx.x];  // {slot, first position, count, 0}
-  if (threadIdx.x < 3 * NP) nd[threadIdx.x / NP][threadIdx.x % NP] = nodes[(size_t)pc.x * 3 * NP + threadIdx.x];
-  double acc[PT][4];
-#pragma unroll
-  for (int r = 0; r < PT; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.0;
+  const int tid = threadIdx.x;
+  if (tid < 3 * NP) nd[tid / NP][tid % NP] = sigma * nodes[(size_t)pc.x * 3 * NP + tid];
+  const int g = tid / U::Q, q01 = tid % U::Q, q0 = q01 / NP, q1 = q01 % NP;  // g == G: idle
+  PartSum<float> acc[NP][4];
   const float4* R = rec + 2 * (size_t)k * rec_stride;
-  for (int c0 = 0; c0 < pc.z; c0 += kUpChunk) {
-    const int cnt = min(kUpChunk, pc.z - c0);
+  for (int c0 = 0; c0 < pc.z; c0 += CH) {
+    const int cnt = min(CH, pc.z - c0);
     __syncthreads();  // nodes staged; the previous chunk consumed
-    const int q = threadIdx.x;
-    if (q < 3 * cnt) {  // basis values of element q / 3 along coordinate q % 3
+    for (int q = tid; q < 3 * cnt; q += U::NT) {  // basis values of element q / 3 along coordinate q % 3
       const int e = q / 3, d = q % 3;
-      const float4 r0 = R[2 * (size_t)(pc.y + c0 + e)];
+      const size_t o = 2 * (size_t)(pc.y + c0 + e);
+      const float4 r0 = R[o];
+      if (d == 0) {
+        const float4 r1 = R[o + 1];
+        val[e] = make_float4(r0.w, r1.x, r1.y, r1.z);
+      }
       const float t = d == 0 ? r0.x : (d == 1 ? r0.y : r0.z);
       float w[NP];
       float sum = 0.f;
@@ -124,44 +147,59 @@ __global__ void __launch_bounds__(256) k_tree_up(const int4* __restrict__ pieces
       const float inv = 1.f / sum;
 #pragma unroll
       for (int i = 0; i < NP; ++i) bas[e][d][i] = hit >= 0 ? (i == hit ? 1.f : 0.f) : w[i] * inv;
-    } else if (q >= 128 && q < 128 + cnt) {
-      const int e = q - 128;
-      const size_t o = 2 * (size_t)(pc.y + c0 + e);
-      const float4 r0 = R[o], r1 = R[o + 1];
-      val[e] = make_float4(r0.w, r1.x, r1.y, r1.z);
     }
     __syncthreads();
+    if (g < G) {
+      f2 sa[NP], sm[NP];  // (a, mx), (my, mz)
 #pragma unroll
-    for (int r = 0; r < PT; ++r) {
-      const int kp = threadIdx.x + 256 * r;
-      if (kp >= P) continue;
-      const int k0 = kp / (NP * NP), k1 = (kp / NP) % NP, k2 = kp % NP;
-      float sa = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
-      for (int e = 0; e < cnt; ++e) {
-        const float w = bas[e][0][k0] * bas[e][1][k1] * bas[e][2][k2];
+      for (int i = 0; i < NP; ++i) sa[i] = sm[i] = f2_splat(0.f);
+#pragma unroll 2
+      for (int e = g; e < cnt; e += G) {
         const float4 v = val[e];
-        sa = fmaf(w, v.x, sa);
-        sx = fmaf(w, v.y, sx);
-        sy = fmaf(w, v.z, sy);
-        sz = fmaf(w, v.w, sz);
+        const f2 va = f2_make(v.x, v.y), vm = f2_make(v.z, v.w);
+        const float w01 = bas[e][0][q0] * bas[e][1][q1];
+        float b2[NB];
+#pragma unroll
+        for (int i = 0; i < NB; i += 4) *reinterpret_cast<float4*>(b2 + i) = *reinterpret_cast<float4*>(&bas[e][2][i]);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          const f2 w = f2_splat(w01 * b2[i]);
+          sa[i] = f2_fma(w, va, sa[i]);
+          sm[i] = f2_fma(w, vm, sm[i]);
+        }
       }
-      acc[r][0] += sa, acc[r][1] += sx, acc[r][2] += sy, acc[r][3] += sz;
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        float x, y;
+        f2_get(sa[i], x, y);
+        acc[i][0].add(x), acc[i][1].add(y);
+        f2_get(sm[i], x, y);
+        acc[i][2].add(x), acc[i][3].add(y);
+      }
     }
   }
+  // the groups in order, one component at a time
+  float2* o = upart + 4 * (size_t)(k * n_pieces + blockIdx.x) * P;
 #pragma unroll
-  for (int r = 0; r < PT; ++r) {
-    const int kp = threadIdx.x + 256 * r;
-    if (kp >= P) continue;
-    double* o = upart + 4 * ((size_t)(k * n_pieces + blockIdx.x) * P + kp);
-    o[0] = acc[r][0], o[1] = acc[r][1], o[2] = acc[r][2], o[3] = acc[r][3];
+  for (int c = 0; c < 4; ++c) {
+    __syncthreads();
+    if (g < G)
+#pragma unroll
+      for (int i = 0; i < NP; ++i) comb[g * P + q01 * NP + i] = make_float2(acc[i][c].hi, acc[i][c].lo);
+    __syncthreads();
+    for (int q = tid; q < P; q += U::NT) {
+      PartSum<float> t;
+      for (int x = 0; x < G; ++x) t.add(comb[x * P + q].x), t.lo += comb[x * P + q].y;
+      o[c * P + q] = make_float2(t.hi, t.lo);
+    }
   }
 }
 
-// Proxy records after the element records: (s_q, a_q), (m_q, 0), the pieces
-// of the slot's cluster added in order.
+// Proxy records after the element records: (sigma s_q, a_q), (m_q, 0), the
+// pieces of the slot's cluster added in order.
 template <int DEG>
-__global__ void k_tree_proxy(int n_slots, const int2* __restrict__ up_tab, const float* __restrict__ nodes,
-                             const double* __restrict__ upart, int n_pieces, int n, int rec_stride,
+__global__ void k_tree_proxy(int n_slots, const int2* __restrict__ up_tab, const float* __restrict__ nodes, float sigma,
+                             const float2* __restrict__ upart, int n_pieces, int n, int rec_stride,
                              float4* __restrict__ rec, const int* __restrict__ skip, int skip_stride) {
   constexpr int NP = DEG + 1, P = NP * NP * NP;
   const int k = blockIdx.y;
@@ -170,40 +208,105 @@ __global__ void k_tree_proxy(int n_slots, const int2* __restrict__ up_tab, const
   const int slot = idx / P, kp = idx % P;
   const int k0 = kp / (NP * NP), k1 = (kp / NP) % NP, k2 = kp % NP;
   const int2 T = up_tab[slot];
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  PartSum<float> s[4];
+#pragma unroll 4
   for (int p = T.x; p < T.x + T.y; ++p) {
-    const double* v = upart + 4 * ((size_t)(k * n_pieces + p) * P + kp);
-    s[0] += v[0], s[1] += v[1], s[2] += v[2], s[3] += v[3];
+    const float2* v = upart + 4 * (size_t)(k * n_pieces + p) * P + kp;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[c].add(v[c * P].x), s[c].lo += v[c * P].y;
   }
   const float* nd = nodes + (size_t)slot * 3 * NP;
   const size_t o = 2 * ((size_t)k * rec_stride + n + idx);
-  rec[o] = make_float4(nd[k0], nd[NP + k1], nd[2 * NP + k2], (float)s[0]);
-  rec[o + 1] = make_float4((float)s[1], (float)s[2], (float)s[3], 0.f);
+  rec[o] = make_float4(sigma * nd[k0], sigma * nd[NP + k1], sigma * nd[2 * NP + k2], s[0].hi + s[0].lo);
+  rec[o + 1] = make_float4(s[1].hi + s[1].lo, s[2].hi + s[2].lo, s[3].hi + s[3].lo, 0.f);
 }
 
-// The ordered pair of the far-field pass: A u (pair_forward: accP, accQ the
-// phi and psi rows) or A^T w (pair_transpose: the phi and psi outputs).
-template <bool TRANS, bool MASK>
-__device__ __forceinline__ void tree_pair(const float4& g, const float4& v, const float4& A, const float4& B, bool self,
-                                          const PairConst<float>& c, float& accP, float& accQ) {
-  if (TRANS)
-    pair_transpose<MASK>(g.x, g.y, g.z, v.x, v.y, v.z, A.x, A.y, A.z, A.w, B.x, B.y, B.z, self, c, accP, accQ);
-  else
-    pair_forward<MASK>(g.x, g.y, g.z, v.x, v.y, v.z, A.x, A.y, A.z, A.w, B.x, B.y, B.z, self, c, accP, accQ);
+// Two source records (packed) added to one target: S1 += s [(1 - e) a + E s^2
+// (m.d)], S3 += s^3 [(1 - t) (n.m) + (n.d) ((w - 3) s^2 (m.d) + F a)] with d =
+// target - source, which are the two outputs of both directions (pair.cuh):
+//   A u:   E = eps t - 1, F = 1 - t / eps;  phi = S1, psi = -S3;
+//   A^T w: E = 1 - t / eps, F = eps t - 1;  phi = -S3, psi = S1
+// (d changes its sign against pair_transpose, hence E and F).  The formulas
+// are placed so that no packed operand needs a negation (two logical
+// operations each).  FORM:
+//   kScaled (kappa >= 1e-6): positions and m times sigma = kappa, where kappa r
+//     = r2 s, (1 - e) s = (1 - t) s + e and (w - 3) s^2 = 3 (t - 1) s^2 + e;
+//     the sums take factors of kappa (S1) and kappa^2 (S3);
+//   kPlain (0 < kappa < 1e-6, whose scaled coordinates would overflow): sigma = 1;
+//   kLaplace (kappa = 0): e = t = 1, w = 3, only E and F remain.
+enum TreeForm { kScaled, kPlain, kLaplace };
+struct TreeConst {
+  float ef, e0, ff, f0;  // E = ef t + e0, F = ff t + f0
+  float kappa, smax;     // smax in the units of the positions
+};
+struct TreeTarget {
+  f2 x[3], n[3];
+};
+template <TreeForm FORM, bool MASK>
+__device__ __forceinline__ void tree_pair2(const TreeTarget& T, const f2* R, bool m0, bool m1, const TreeConst& c,
+                                           f2& S1, f2& S3) {
+  const f2 dx = f2_sub(T.x[0], R[0]), dy = f2_sub(T.x[1], R[1]), dz = f2_sub(T.x[2], R[2]);
+  const f2 r2 = f2_fma(dx, dx, f2_fma(dy, dy, f2_mul(dz, dz)));
+  float sa, sb;
+  f2_get(r2, sa, sb);
+  sa = fminf(rsqrt_approx(sa), c.smax), sb = fminf(rsqrt_approx(sb), c.smax);
+  if (MASK) sa = m0 ? 0.f : sa, sb = m1 ? 0.f : sb;
+  const f2 s = f2_make(sa, sb);
+  const f2 a = R[3];
+  const f2 cd = f2_fma(T.n[0], dx, f2_fma(T.n[1], dy, f2_mul(T.n[2], dz)));  // n.d
+  const f2 cm = f2_fma(R[4], dx, f2_fma(R[5], dy, f2_mul(R[6], dz)));        // m.d
+  const f2 s2 = f2_mul(s, s), s3 = f2_mul(s2, s);
+  if constexpr (FORM == kLaplace) {
+    S1 = f2_fma(f2_mul(f2_splat(c.ef + c.e0), s3), cm, S1);
+    S3 = f2_fma(f2_mul(f2_splat(c.ff + c.f0), s3), f2_mul(cd, a), S3);
+  } else {
+    const f2 cnm = f2_fma(T.n[0], R[4], f2_fma(T.n[1], R[5], f2_mul(T.n[2], R[6])));  // n.m
+    const f2 r = f2_mul(r2, s);
+    const f2 kr = FORM == kScaled ? r : f2_mul(r, f2_splat(c.kappa));
+    float ea, eb;
+    f2_get(f2_mul(kr, f2_splat(-1.4426950408889634f)), ea, eb);
+    ea = ex2_approx(ea), eb = ex2_approx(eb);
+    if (MASK) ea = m0 ? 0.f : ea, eb = m1 ? 0.f : eb;
+    const f2 e = f2_make(ea, eb);
+    const f2 t = f2_fma(e, kr, e);
+    const f2 omt = f2_sub(f2_splat(1.f), t);
+    f2 w, k1;  // (w - 3) s^2, (1 - e) s
+    if constexpr (FORM == kScaled) {
+      w = f2_fma(omt, f2_mul(f2_splat(-3.f), s2), e);
+      k1 = f2_fma(omt, s, e);
+    } else {
+      w = f2_mul(f2_fma(f2_sub(t, e), kr, f2_mul(f2_splat(-3.f), omt)), s2);
+      k1 = f2_sub(s, f2_mul(e, s));
+    }
+    const f2 E = f2_fma(f2_splat(c.ef), t, f2_splat(c.e0)), F = f2_fma(f2_splat(c.ff), t, f2_splat(c.f0));
+    S1 = f2_fma(f2_mul(E, s3), cm, f2_fma(k1, a, S1));
+    S3 = f2_fma(f2_fma(cd, f2_fma(w, cm, f2_mul(F, a)), f2_mul(omt, cnm)), s3, S3);
+  }
 }
 
 // One work item: the targets of one leaf (thread t: position lf.x + t) against
 // the records of segments [it.y, it.z).  The self pair is masked in the
 // segments that overlap the leaf's own positions.
-template <bool TRANS>
-__global__ void __launch_bounds__(kMaxLeaf) k_tree_far(const int4* __restrict__ items, const int2* __restrict__ segs,
-                                                      const int4* __restrict__ leaf_tab, const int* __restrict__ perm,
-                                                      const float4* __restrict__ tgt32,
-                                                      const float4* __restrict__ rec, int rec_stride,
-                                                      float* __restrict__ part, int n_items, int lmax,
-                                                      PairConst<float> c, const int* __restrict__ skip,
-                                                      int skip_stride) {
+//
+// Bound by the FP32 pipe: records are staged with the values of two
+// consecutive ones side by side (an odd end padded by a record without
+// strength), so each thread evaluates two pairs by 34 packed instructions, 18
+// of them multiply-adds (three register operands, which take half as long
+// again): 43 cycles a warp and source by that count, 47 measured (the scalar
+// unscaled pair took 53).  At N = 120001 the pass takes 3.13 ms (3.92 before);
+// the records of a chunk (512 against 256) and the unroll (2 against 4 and 8)
+// are worth 1 % each.  A leaf's last, partly filled warp does not lengthen the
+// pass when its idle lanes take part of the records: the other warps of its
+// processor partition set the pace.
+template <TreeForm FORM>
+__global__ void __launch_bounds__(kMaxLeaf, kFarMinB)
+    k_tree_far(const int4* __restrict__ items, const int2* __restrict__ segs, const int4* __restrict__ leaf_tab,
+               const int* __restrict__ perm, const float4* __restrict__ tgt32, const float4* __restrict__ rec,
+               int rec_stride, float* __restrict__ part, int n_items, int lmax, TreeConst c,
+               const int* __restrict__ skip, int skip_stride) {
+  // [record pair]: (x, x', y, y'), (z, z', a, a'), (mx, mx', my, my'), (mz, mz', -, -)
   __shared__ float4 sh[2 * kFarCH];
+  float* shf = reinterpret_cast<float*>(sh);
   const int k = blockIdx.y;
   if (tree_skipped(skip, skip_stride, k)) return;
   const int4 it = items[blockIdx.x];
@@ -211,63 +314,83 @@ __global__ void __launch_bounds__(kMaxLeaf) k_tree_far(const int4* __restrict__ 
   const int t = threadIdx.x;
   const bool active = t < lf.y;
   const int pos = lf.x + min(t, lf.y - 1);
-  const int e = perm[pos];
-  const float4 g = tgt32[2 * (size_t)e], v = tgt32[2 * (size_t)e + 1];
-  float accP = 0.f, accQ = 0.f;
   const float4* R = rec + 2 * (size_t)k * rec_stride;
+  const float4 g = R[2 * (size_t)pos], v = tgt32[2 * (size_t)perm[pos] + 1];
+  const TreeTarget T{{f2_splat(g.x), f2_splat(g.y), f2_splat(g.z)}, {f2_splat(v.x), f2_splat(v.y), f2_splat(v.z)}};
+  f2 S1 = f2_splat(0.f), S3 = f2_splat(0.f);
+  auto load = [&](int jj, f2* w) {
+    const float4* q = sh + 4 * jj;
+    const float4 A = q[0], B = q[1], C = q[2];
+    const float2 D = *reinterpret_cast<const float2*>(q + 3);
+    w[0] = f2_make(A.x, A.y), w[1] = f2_make(A.z, A.w), w[2] = f2_make(B.x, B.y), w[3] = f2_make(B.z, B.w);
+    w[4] = f2_make(C.x, C.y), w[5] = f2_make(C.z, C.w), w[6] = f2_make(D.x, D.y);
+  };
   for (int sg = it.y; sg < it.z; ++sg) {
     const int2 S = segs[sg];
     const bool self = S.x < lf.x + lf.y && S.x + S.y > lf.x;
     for (int j0 = 0; j0 < S.y; j0 += kFarCH) {
-      const int m = min(kFarCH, S.y - j0);
+      const int m = min(kFarCH, S.y - j0), mp = (m + 1) / 2;
       __syncthreads();
       const float4* src = R + 2 * (size_t)(S.x + j0);
-      for (int q = t; q < 2 * m; q += blockDim.x) sh[q] = src[q];
+      for (int q = t; q < 4 * mp; q += blockDim.x) {  // half q & 1 of record q / 2
+        const bool pad = q >= 2 * m;
+        float4 x = src[pad ? q - 2 : q];
+        if (pad) x = q & 1 ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(x.x, x.y, x.z, 0.f);
+        float* o = shf + 16 * (q >> 2) + 8 * (q & 1) + ((q >> 1) & 1);
+        o[0] = x.x, o[2] = x.y, o[4] = x.z, o[6] = x.w;
+      }
       __syncthreads();
       if (!active) continue;
+      f2 w[7];
       if (!self) {
-        if (m == kFarCH) {
-#pragma unroll 8
-          for (int jj = 0; jj < kFarCH; ++jj) tree_pair<TRANS, false>(g, v, sh[2 * jj], sh[2 * jj + 1], false, c, accP, accQ);
-        } else {
-          for (int jj = 0; jj < m; ++jj) tree_pair<TRANS, false>(g, v, sh[2 * jj], sh[2 * jj + 1], false, c, accP, accQ);
+#pragma unroll 2
+        for (int jj = 0; jj < mp; ++jj) {
+          load(jj, w);
+          tree_pair2<FORM, false>(T, w, false, false, c, S1, S3);
         }
       } else {
-        for (int jj = 0; jj < m; ++jj)
-          tree_pair<TRANS, true>(g, v, sh[2 * jj], sh[2 * jj + 1], S.x + j0 + jj == pos, c, accP, accQ);
+        const int own = pos - S.x - j0;
+        for (int jj = 0; jj < mp; ++jj) {
+          load(jj, w);
+          tree_pair2<FORM, true>(T, w, 2 * jj == own, 2 * jj + 1 == own, c, S1, S3);
+        }
       }
     }
   }
   if (active) {
     float* o = part + 2 * (size_t)lmax * ((size_t)k * n_items + blockIdx.x);
-    o[t] = accP;
-    o[lmax + t] = accQ;
+    o[t] = f2_sum(S1);
+    o[lmax + t] = f2_sum(S3);
   }
 }
 
-// y of element perm[t]: diag u - 1/(4 pi) (sum over the leaf's items in order),
-// the sum times the element's area for the transpose
+// y of element perm[t]: diag u - f (sum over the leaf's items in order), with f1
+// for S1 and f3 for S3 (1/(4 pi), their scale and the sign of S3); the sums
+// times the element's area, and S3 the phi output, for the transpose (area_of given)
 __global__ void k_tree_reduce(int n, const int* __restrict__ perm, const int* __restrict__ leaf_of,
                               const int4* __restrict__ leaf_tab, const float* __restrict__ part, int n_items,
                               int lmax, const int4* __restrict__ lay, const double4_32a* __restrict__ area_of,
-                              const double* __restrict__ u, double* __restrict__ y, double dphi, double dpsi,
-                              const int* __restrict__ skip, int skip_stride) {
+                              const double* __restrict__ u, double* __restrict__ y, double dphi, double dpsi, double f1,
+                              double f3, const int* __restrict__ skip, int skip_stride) {
   const int k = blockIdx.y;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n || tree_skipped(skip, skip_stride, k)) return;
   const int4 lf = leaf_tab[leaf_of[t]];
   const int local = t - lf.x;
-  double sp = 0.0, sq = 0.0;
+  PartSum<float> s1, s3;
+#pragma unroll 4
   for (int i = lf.z; i < lf.z + lf.w; ++i) {
     const float* o = part + 2 * (size_t)lmax * ((size_t)k * n_items + i);
-    sp += (double)o[local];
-    sq += (double)o[lmax + local];
+    s1.add(o[local]);
+    s3.add(o[lmax + local]);
   }
   const int4 L = lay[k];
   const int e = perm[t];
-  const double w = area_of != nullptr ? area_of[2 * (L.x + e)].w * kInv4PiT : kInv4PiT;
-  y[L.z + e] = dphi * u[L.z + e] - w * sp;
-  y[L.z + L.y + e] = dpsi * u[L.z + L.y + e] - w * sq;
+  const bool tr = area_of != nullptr;
+  const double w = tr ? area_of[2 * (L.x + e)].w : 1.0;
+  const double v1 = w * f1 * s1.value(), v3 = w * f3 * s3.value();
+  y[L.z + e] = dphi * u[L.z + e] - (tr ? v3 : v1);
+  y[L.z + L.y + e] = dpsi * u[L.z + L.y + e] - (tr ? v1 : v3);
 }
 
 // ------------------------------------------------------------------ host: tree and lists
@@ -361,20 +484,20 @@ void collect(const std::vector<Node>& nodes, int k, const double xb[3], double r
 }
 
 template <int DEG>
-void launch_up(const FarField* f, cudaStream_t st, int K, const int* skip, int skip_stride) {
-  k_tree_up<DEG><<<dim3(f->n_up, K), 256, 0, st>>>(f->up_pieces.p, f->nodes.p, f->rec_stride, f->rec.p, f->upart.p,
+void launch_up(const FarField* f, cudaStream_t st, int K, float sigma, const int* skip, int skip_stride) {
+  k_tree_up<DEG><<<dim3(f->n_up, K), 256, 0, st>>>(f->up_pieces.p, f->nodes.p, sigma, f->rec_stride, f->rec.p, f->upart.p,
                                                     f->n_up, skip, skip_stride);
 }
 template <int DEG>
-void launch_proxy(const FarField* f, cudaStream_t st, int K, const int* skip, int skip_stride) {
+void launch_proxy(const FarField* f, cudaStream_t st, int K, float sigma, const int* skip, int skip_stride) {
   constexpr int P = (DEG + 1) * (DEG + 1) * (DEG + 1);
   k_tree_proxy<DEG><<<dim3((f->n_slots * P + 255) / 256, K), 256, 0, st>>>(
-      f->n_slots, f->up_tab.p, f->nodes.p, f->upart.p, f->n_up, f->n, f->rec_stride, f->rec.p, skip, skip_stride);
+      f->n_slots, f->up_tab.p, f->nodes.p, sigma, f->upart.p, f->n_up, f->n, f->rec_stride, f->rec.p, skip, skip_stride);
 }
 
-int far_occupancy(int nt) {  // both directions have the same shape; the forward kernel sets the plan
+int far_occupancy(int nt) {  // the forms have one shape; the scaled kernel sets the plan
   int o = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_tree_far<false>, nt, 0) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_tree_far<kScaled>, nt, 0) != cudaSuccess) {
     (void)cudaGetLastError();
     o = 1;
   }
@@ -534,8 +657,8 @@ FarField* far_field(Surface* s) {
   return s->far.get();
 }
 
-void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c, bool transpose, const double* u, double* y,
-                 double dphi, double dpsi, const int* skip, int skip_stride) {
+void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c0, double kappa, bool transpose,
+                 const double* u, double* y, double dphi, double dpsi, const int* skip, int skip_stride) {
   for (int k = 0; k < L.K; ++k)
     BIPB_REQUIRE(L.geo_off[k] == 0 && L.n[k] == (int)s->n, "the far-field mat-vec covers one surface");
   FarField* f = far_field(s);
@@ -546,40 +669,42 @@ void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c, bool
   if (f->upart.ensure(std::max<size_t>(1, 4 * (size_t)P * f->n_up * K), s->stream)) ++s->alloc_gen;
   const int4* lay = s->lay_dev(L);
   const int nb = (f->n + 255) / 256;
-  k_tree_pack<<<dim3(nb, K), 256, 0, s->stream>>>(f->n, f->rec_stride, transpose, f->perm.p, s->tgt64.p, lay, u,
+  const TreeForm form = kappa == 0.0 ? kLaplace : kappa < kSymKappaMin ? kPlain : kScaled;
+  const double sigma = form == kScaled ? kappa : 1.0;
+  const float sg = (float)sigma;
+  TreeConst c;
+  c.ef = transpose ? -c0.inveps : c0.eps, c.e0 = transpose ? 1.f : -1.f;
+  c.ff = transpose ? c0.eps : -c0.inveps, c.f0 = transpose ? -1.f : 1.f;
+  c.kappa = c0.kappa, c.smax = (float)(kSMaxD / sigma);
+  k_tree_pack<<<dim3(nb, K), 256, 0, s->stream>>>(f->n, f->rec_stride, transpose, sigma, f->perm.p, s->tgt64.p, lay, u,
                                                   f->rec.p, skip, skip_stride);
   BIPB_LAUNCHED(s);
   if (f->n_up > 0) {
     switch (f->degree) {
-      case 4: launch_up<4>(f, s->stream, K, skip, skip_stride); break;
-      case 6: launch_up<6>(f, s->stream, K, skip, skip_stride); break;
-      default: launch_up<8>(f, s->stream, K, skip, skip_stride); break;
+      case 4: launch_up<4>(f, s->stream, K, sg, skip, skip_stride); break;
+      case 6: launch_up<6>(f, s->stream, K, sg, skip, skip_stride); break;
+      default: launch_up<8>(f, s->stream, K, sg, skip, skip_stride); break;
     }
     BIPB_LAUNCHED(s);
     switch (f->degree) {
-      case 4: launch_proxy<4>(f, s->stream, K, skip, skip_stride); break;
-      case 6: launch_proxy<6>(f, s->stream, K, skip, skip_stride); break;
-      default: launch_proxy<8>(f, s->stream, K, skip, skip_stride); break;
+      case 4: launch_proxy<4>(f, s->stream, K, sg, skip, skip_stride); break;
+      case 6: launch_proxy<6>(f, s->stream, K, sg, skip, skip_stride); break;
+      default: launch_proxy<8>(f, s->stream, K, sg, skip, skip_stride); break;
     }
     BIPB_LAUNCHED(s);
   }
   {
     TimedLaunch tl(s, kTMvTree);
-    if (transpose)
-      k_tree_far<true><<<dim3(f->n_items, K), f->nt, 0, s->stream>>>(f->items.p, f->segs.p, f->leaf_tab.p,
-                                                                    f->perm.p, s->tgt32.p, f->rec.p, f->rec_stride,
-                                                                    f->part.p, f->n_items, f->lmax, c, skip,
-                                                                    skip_stride);
-    else
-      k_tree_far<false><<<dim3(f->n_items, K), f->nt, 0, s->stream>>>(f->items.p, f->segs.p, f->leaf_tab.p,
-                                                                     f->perm.p, s->tgt32.p, f->rec.p, f->rec_stride,
-                                                                     f->part.p, f->n_items, f->lmax, c, skip,
-                                                                     skip_stride);
+    auto kernel = form == kScaled ? k_tree_far<kScaled> : form == kPlain ? k_tree_far<kPlain> : k_tree_far<kLaplace>;
+    kernel<<<dim3(f->n_items, K), f->nt, 0, s->stream>>>(f->items.p, f->segs.p, f->leaf_tab.p, f->perm.p, s->tgt32.p,
+                                                         f->rec.p, f->rec_stride, f->part.p, f->n_items, f->lmax, c,
+                                                         skip, skip_stride);
     BIPB_LAUNCHED(s);
   }
   k_tree_reduce<<<dim3(nb, K), 256, 0, s->stream>>>(f->n, f->perm.p, f->leaf_of.p, f->leaf_tab.p, f->part.p,
                                                     f->n_items, f->lmax, lay, transpose ? s->tgt64.p : nullptr, u, y,
-                                                    dphi, dpsi, skip, skip_stride);
+                                                    dphi, dpsi, kInv4PiT * sigma, -kInv4PiT * sigma * sigma, skip,
+                                                    skip_stride);
   BIPB_LAUNCHED(s);
 }
 

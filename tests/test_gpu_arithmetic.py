@@ -151,3 +151,24 @@ def test_multi_rhs_double_float_scaling_rule(bipb, orc, n, kappa, transpose):
         for r in (0, n_rhs - 1):
             ref = f(c, nv, a, 80.0, kappa, U[r])
             np.testing.assert_allclose(Y[r], ref, rtol=0, atol=2e-12 * np.abs(ref).max(), err_msg=f"{n_rhs} {r}")
+
+
+@pytest.mark.parametrize("n,params", [(33, (0.8, 4, 32)), (257, (0.9, 4, 32)), (1280, (0.9, 8, 33)), (1111, (0.7, 6, 64))])
+@pytest.mark.parametrize("kappa", [0.0, 9e-7, 1.1e-6, 0.4])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_treecode_forms_and_ragged_leaves(bipb, orc, n, params, kappa, transpose):
+    """The packed far-field pass in its three forms (both sides of the lines at kappa =
+    0 and 1e-6), with odd leaves and proxy counts, several elements on a group of the
+    upward pass and one leaf only: test_treecode_matvec_matches_oracle_treecode's bounds."""
+    p = synth.protein_like_problem(level=3, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, min(n, p.n), replace=False))
+    c, nv, a = p.centroids[keep], p.normals[keep], p.areas[keep]
+    u = np.random.default_rng(4).standard_normal(2 * len(keep))
+    with bipb.Surface(c, nv, a) as s:
+        s.treecode(*params)
+        y = torch.full_like(_dev(u), float("nan"))
+        s.matvec(_dev(u), y, precision=bipb.TREE32, transpose=transpose, med=bipb.medium(1.0, 80.0, kappa))
+        y = y.cpu().numpy()
+    ref = orc.treecode.matvec(c, nv, a, 80.0, kappa, u, *params, transpose=transpose)
+    assert np.linalg.norm(y - ref) < 3e-6 * np.linalg.norm(ref)
+    assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max()
