@@ -284,17 +284,21 @@ void add_part(Surface* s, const PartIn& P, std::vector<double4_32a>& tgt, std::v
   s->n += P.n;
 }
 
-// 2^(j/1024) for j < 1024 as df64 (hi, lo) pairs, two per float4: the table
-// of the df64 exp (df64.cuh)
+// 2^(j/1024) for j < 1024 as df64 (hi, lo) pairs, two per float4 (the table
+// of the df64 exp, df64.cuh), then the third floats of the FP64 values, four
+// per float4 (tf64.cuh)
 const std::vector<float4>& exp_table() {
   static const std::vector<float4> t = [] {
-    std::vector<float4> v(kExpTab / 2);
+    std::vector<float4> v(kExpTab / 2 + kExpTab / 4);
     auto hi = [](int j) { return (float)std::exp2(j / (double)kExpTab); };
     auto lo = [](int j) {
       const double x = std::exp2(j / (double)kExpTab);
       return (float)(x - (double)(float)x);
     };
+    auto third = [&](int j) { return (float)(std::exp2(j / (double)kExpTab) - (double)hi(j) - (double)lo(j)); };
     for (int i = 0; i < kExpTab / 2; ++i) v[i] = make_float4(hi(2 * i), lo(2 * i), hi(2 * i + 1), lo(2 * i + 1));
+    for (int i = 0; i < kExpTab / 4; ++i)
+      v[kExpTab / 2 + i] = make_float4(third(4 * i), third(4 * i + 1), third(4 * i + 2), third(4 * i + 3));
     return v;
   }();
   return t;

@@ -370,9 +370,9 @@ __device__ __forceinline__ void df_kernel_block(const df_pos* xi, const df* ni, 
   for (int v = 0; v < 4; ++v) k[v] = df_norm(k[v]);
 }
 
-// The symmetric pair of pair.cuh (sym_pair) in df64.  The four accumulators
+// The symmetric pair of pair.cuh in df64.  The four accumulators
 // are updated lazily (df_mac): renormalise them before use.  SCALED: the
-// records are in kappa-scaled units as in sym_pair (kappa r = r, (w - 3) s^2 =
+// records are in kappa-scaled units as there (kappa r = r, (w - 3) s^2 =
 // 3 (t - 1) s^2 + e; the caller rescales the sums); otherwise unscaled, for
 // any kappa >= 0.
 template <bool MASK, bool TRANS, bool SCALED>

@@ -295,7 +295,7 @@ struct Surface {
   // centroid (part_center), so that the FP32 copies keep the most digits.
   DevBuf<double4_32a> tgt64;  // 2n: (x, y, z, area), (nx, ny, nz, coordinate grid of the surface: df_pos)
   DevBuf<float4> tgt32;   // the same in FP32
-  DevBuf<float4> exptab;  // 2^(j/1024), j < 1024, as df64 (hi, lo) pairs: the df64 exp table
+  DevBuf<float4> exptab;  // 2^(j/1024), j < 1024, as df64 (hi, lo) pairs, then the third floats (exp_table)
 
   // per-pass scratch
   DevBuf<float4> rec32;

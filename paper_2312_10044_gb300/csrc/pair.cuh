@@ -59,15 +59,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// Precision-generic pieces of the symmetric pair: 1/sqrt (MUFU estimate in
-// FP32), min, and exp(-x) for x >= 0 (MUFU ex2 in FP32).
-__device__ __forceinline__ float rsqrt_of(float x) { return rsqrt_approx(x); }
-__device__ __forceinline__ double rsqrt_of(double x) { return rsqrt(x); }
-__device__ __forceinline__ float min_of(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double min_of(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ float exp_neg_of(float x) { return ex2_approx(x * -1.4426950408889634f); }
-__device__ __forceinline__ double exp_neg_of(double x) { return exp(-x); }
-
 // 1/r (clamped; 0 for the self pair) and exp(-kappa r) for both precisions.
 template <bool MASK>
 __device__ __forceinline__ void radial(float r2, bool self, const PairConst<float>& c, float& s,
@@ -175,58 +166,9 @@ __device__ __forceinline__ void pair_transpose(T xj, T yj, T zj, T nxj, T nyj, T
 //   kappa^2; A^T w: P by kappa^2, Q by kappa).
 // - LAPLACE (kappa = 0, unscaled): e = t = 1, w = 3, so K1 = K4 = 0 and only
 //   the double-layer terms (eps - 1) c_j s^3 and (1/eps - 1) c_i s^3 remain.
-template <bool MASK, bool TRANS, bool LAPLACE, typename T>
-__device__ __forceinline__ void sym_pair(T dx, T dy, T dz, const T* nt, T at, T alt, const T* ns, T as, T als,
-                                         bool self, const PairConst<T>& c, T& Pt, T& Qt, T& Ps, T& Qs) {
-  const T r2 = dx * dx + dy * dy + dz * dz;
-  T s = min_of(rsqrt_of(r2), c.smax);
-  if (MASK) s = self ? T(0) : s;
-  const T ci = nt[0] * dx + nt[1] * dy + nt[2] * dz;
-  const T cj = ns[0] * dx + ns[1] * dy + ns[2] * dz;
-  const T s3 = s * s * s;
-  if constexpr (LAPLACE) {
-    const T et1_s3 = c.eps * s3 - s3, te1_s3 = c.inveps * s3 - s3;  // (eps - 1) s^3, (1/eps - 1) s^3
-    if (!TRANS) {
-      Pt = (et1_s3 * cj) * als + Pt;
-      Qt = (te1_s3 * ci) * as + Qt;
-      Ps = Ps - (et1_s3 * ci) * alt;
-      Qs = Qs - (te1_s3 * cj) * at;
-    } else {
-      Pt = Pt - (et1_s3 * ci) * as;
-      Qt = Qt - (te1_s3 * cj) * als;
-      Ps = (et1_s3 * cj) * at + Ps;
-      Qs = (te1_s3 * ci) * alt + Qs;
-    }
-  } else {
-    const T kr = r2 * s;  // kappa r (0 for a masked pair)
-    const T e = exp_neg_of(kr);
-    const T t = e * kr + e;
-    const T tm1 = t - T(1);
-    const T s2 = s * s;
-    // (w - 3) s^2 = 3 (t - 1) s^2 + e (a masked pair gets e = 1, but its every coefficient carries s = 0)
-    const T wm3s2 = tm1 * (T(3) * s2) + e;
-    const T ts3 = t * s3;
-    const T cij = nt[0] * ns[0] + nt[1] * ns[1] + nt[2] * ns[2];
-    const T U = tm1 * cij - wm3s2 * (ci * cj);
-    // s and s^3 folded into the four coefficients every update uses
-    const T ome_s = s - e * s, U_s3 = U * s3;
-    const T et1_s3 = c.eps * ts3 - s3, te1_s3 = c.inveps * ts3 - s3;  // (eps t - 1) s^3, (t/eps - 1) s^3
-    if (!TRANS) {
-      Pt = (et1_s3 * cj) * als + (ome_s * as + Pt);
-      Qt = U_s3 * als + ((te1_s3 * ci) * as + Qt);
-      Ps = ome_s * at - ((et1_s3 * ci) * alt - Ps);
-      Qs = U_s3 * alt - ((te1_s3 * cj) * at - Qs);
-    } else {
-      Pt = U_s3 * als - ((et1_s3 * ci) * as - Pt);
-      Qt = ome_s * as - ((te1_s3 * cj) * als - Qt);
-      Ps = U_s3 * alt + ((et1_s3 * cj) * at + Ps);
-      Qs = ome_s * at + ((te1_s3 * ci) * alt + Qs);
-    }
-  }
-}
 
 // The symmetric pair in FP32 for two targets t (packed) and one source s (every
-// value in both halves), the formulas of sym_pair with signs placed so that no
+// value in both halves), the formulas above with signs placed so that no
 // packed operand needs a negation: 1 - t for t - 1, -U, -(eps t - 1) s^3 and
 // -(t/eps - 1) s^3, and in scaled units (1 - e) s = (1 - t) s + e (kappa r s =
 // 1).  ft: a, -alpha and alpha (A u) or -a (A^T w) of the targets; fs: a,

@@ -36,6 +36,7 @@
 #include "f32x2.cuh"
 #include "internal.cuh"
 #include "symstep.cuh"
+#include "tf64.cuh"
 
 namespace bipb {
 
@@ -54,7 +55,7 @@ constexpr double kInv4PiS = 1.0 / (4.0 * kPi);
 
 // FP64, one target per pack.  Record (x, a), (n, alpha), where (a, alpha) =
 // (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w.
-// LAPLACE: the kappa = 0 form of sym_pair (pair.cuh); otherwise the records
+// LAPLACE: the kappa = 0 form (pair.cuh); otherwise the records
 // are in kappa-scaled units (SCALED).
 template <bool TRANS, bool LAPLACE>
 struct Sym64Policy {
@@ -72,9 +73,19 @@ struct Sym64Policy {
   };
   using Red = Acc;
   struct Args {
-    PairConst<double> c;
+    TfConst c;
+    const float4* tab;  // the exp table as kept by the surface (exp_table, capi.cu)
   };
-  __device__ static void prologue(const Args&) {}
+  __device__ static float4* exp_tab() {
+    __shared__ float4 tab[kTfTab];  // 2^(j/1024) as three floats
+    return tab;
+  }
+  __device__ static void prologue(const Args& g) {
+    if (LAPLACE) return;
+    const float2* t2 = reinterpret_cast<const float2*>(g.tab);
+    const float* t3 = reinterpret_cast<const float*>(g.tab + kExpTab / 2);
+    for (int j = threadIdx.x; j < kTfTab; j += blockDim.x) exp_tab()[j] = make_float4(t2[j].x, t2[j].y, t3[j], 0.f);
+  }
   __device__ static void load(const V4* rec, const int* i, Tgt& t) { unpack(rec[2 * (size_t)i[0]], rec[2 * (size_t)i[0] + 1], t); }
   // record q of a chunk staged as planes (vector r of record q at sh[r * CH + q])
   template <int CH>
@@ -87,8 +98,10 @@ struct Sym64Policy {
   // i side of the targets t and j side of source sj for the pairs d = x_t - x_sj
   template <bool MASK>
   __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
-    sym_pair<MASK, TRANS, LAPLACE>(t.x[0] - sj.x[0], t.x[1] - sj.x[1], t.x[2] - sj.x[2], t.n, t.a, t.al, sj.n, sj.a,
-                                   sj.al, masked[0], g.c, ti.p, ti.q, tj.p, tj.q);
+    const double dx = t.x[0] - sj.x[0], dy = t.x[1] - sj.x[1], dz = t.x[2] - sj.x[2];
+    TfRadial R = tf_radial<LAPLACE>(dx * dx + dy * dy + dz * dz, g.c, LAPLACE ? nullptr : exp_tab());
+    if (MASK && masked[0]) R.k1 = R.v = R.w = R.k2 = R.k3 = 0.0;
+    sym_pair64<TRANS, LAPLACE>(dx, dy, dz, t.n, t.a, t.al, sj.n, sj.a, sj.al, R, ti.p, ti.q, tj.p, tj.q);
   }
   __device__ static void flush(Acc&, const Acc&) {}
   __device__ static Red reduced(const Acc& v) { return v; }
@@ -467,7 +480,7 @@ int blocks_of(int64_t n, int bs) { return (int)std::max<int64_t>(1, (n + bs - 1)
 // Lsrc sources; Lsrc is the candidate (the length giving 1 .. 32 waves of
 // equal pieces) whose greedy schedule (pieces sorted by size, each to the
 // first free CTA slot) finishes first.  A piece costs its
-// sources plus 32 per segment (loading a tile, storing its partials).
+// sources in blocks of 32 plus 32 per segment (loading a tile, storing its partials).
 struct HostPlan {
   std::vector<int4> items, tab;
   int n_items = 0;
@@ -534,19 +547,30 @@ HostPlan compute_sym_plan(const SysLayout& L, int T, int slots, int ch) {
     if (nT % 2) folds.push_back(Fold{k, nT / 2, -1, n - (nT / 2) * T, 0});
   }
   for (const Fold& f : folds) total += f.la + f.lb;
-  auto pieces_of = [&](const Fold& f, double Ls) {
-    return std::max(1, (int)std::lround((f.la + f.lb) / Ls));
+  // pieces of fold f: cuts at equal parts moved to whole blocks of 32 sources of their
+  // row (the kernel takes sources in blocks of 32, so a piece of 33 would cost 64: at n =
+  // 1000, T = 64 half as many blocks again); emits (first, end) along the fold
+  auto each_piece = [](const Fold& f, double Ls, auto&& emit) {
+    const int len = f.la + f.lb, P = std::max(1, (int)std::lround(len / Ls));
+    int a = 0;
+    for (int p = 1; p <= P; ++p) {
+      int b = len;
+      if (p < P) {
+        b = (int)((int64_t)p * len / P);
+        b = b < f.la ? std::min(f.la, (b + 16) / 32 * 32) : f.la + std::min(f.lb, (b - f.la + 16) / 32 * 32);
+      }
+      if (b > a) emit(a, b);
+      a = std::max(a, b);
+    }
+  };
+  // cost of a piece: its sources in blocks of 32, plus 32 per segment
+  auto cost_of = [](const Fold& f, int a, int b) {
+    const int x = std::max(0, std::min(b, f.la) - a), y = b - std::max(a, f.la);
+    return (x > 0 ? (x + 31) / 32 * 32 + 32 : 0) + (y > 0 ? (y + 31) / 32 * 32 + 32 : 0);
   };
   auto makespan = [&](double Ls) {
     std::vector<double> cost;
-    for (const Fold& f : folds) {
-      const int P = pieces_of(f, Ls), len = f.la + f.lb;
-      for (int p = 0; p < P; ++p) {
-        const int a = (int)((int64_t)p * len / P), b = (int)((int64_t)(p + 1) * len / P);
-        const int segs = (a < f.la ? 1 : 0) + (b > f.la ? 1 : 0);
-        cost.push_back((double)(b - a) + 32.0 * segs);
-      }
-    }
+    for (const Fold& f : folds) each_piece(f, Ls, [&](int a, int b) { cost.push_back(cost_of(f, a, b)); });
     std::sort(cost.begin(), cost.end(), std::greater<double>());
     std::priority_queue<double, std::vector<double>, std::greater<double>> q;
     for (int i = 0; i < slots; ++i) q.push(0.0);
@@ -578,20 +602,17 @@ HostPlan compute_sym_plan(const SysLayout& L, int T, int slots, int ch) {
   };
   std::vector<Seg> segs;
   std::vector<int> piece_cost;
-  for (const Fold& f : folds) {
-    const int P = pieces_of(f, best_L), len = f.la + f.lb;
-    for (int p = 0; p < P; ++p) {
-      const int a = (int)((int64_t)p * len / P), b = (int)((int64_t)(p + 1) * len / P);
+  for (const Fold& f : folds)
+    each_piece(f, best_L, [&](int a, int b) {
       const int id = (int)piece_cost.size();
-      piece_cost.push_back(b - a);
+      piece_cost.push_back(cost_of(f, a, b));
       const int ta = f.Ia * T;
       if (a < f.la) segs.push_back(Seg{f.k, f.Ia, ta + a, ta + std::min(b, f.la), id});
       if (b > f.la) {
         const int tb = f.Ib * T;
         segs.push_back(Seg{f.k, f.Ib, tb + std::max(a - f.la, 0), tb + (b - f.la), id});
       }
-    }
-  }
+    });
   // i-side blocks numbered row by row (system, row, first source)
   std::vector<int> order(segs.size());
   for (size_t i = 0; i < segs.size(); ++i) order[i] = (int)i;
@@ -792,26 +813,44 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
   return false;
 }
 
+// FP64 shapes: tiles of 64 targets in CTAs of 64 threads up to 32768 elements,
+// tiles and CTAs of 256 above.  Small tiles leave less of the diagonal masked
+// and more, shorter work items (N = 320 57 against 155 us, 1000 109 / 246, 7001
+// 1362 / 1463); from N = 20000 on both take the same time (10.9 ms), and
+// the j-side partials (8 n^2 / T bytes: 134 MB at 32768 with T = 64) would only grow.
+constexpr int kSym64Small = 32768;
+
 bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c0, double kappa, bool transpose,
                   const double* u, double* y, double dphi, double dpsi, const int* skip, int skip_stride) {
   PairConst<double> c = c0;
   bool lap = false;
-  if (!sym_fits(L, 256) || !sym_form(kappa, c, lap)) return false;
-#define BIPB_SYM64_RUN(TR_, LAP_)                                                                                \
-  run_sym<Sym64Policy<TR_, LAP_>, 128, 2, 64, 1>(s, TR_ ? 0x300 : 0x400, TR_ ? kTMv64T : kTMv64, L, {c}, TR_, \
-                                                      s->rec64, s->part64, u, y, dphi, dpsi, skip, skip_stride,     \
-                                                      kappa)
-  if (transpose) {
-    if (lap)
-      BIPB_SYM64_RUN(true, true);
-    else
-      BIPB_SYM64_RUN(true, false);
-  } else {
-    if (lap)
-      BIPB_SYM64_RUN(false, true);
-    else
-      BIPB_SYM64_RUN(false, false);
+  const bool small = L.max_n <= kSym64Small;
+  if (!sym_fits(L, small ? 64 : 256) || !sym_form(kappa, c, lap)) return false;
+  TfConst t;
+  t.em1 = tf_from_double(c.eps - 1.0), t.eps = tf_from_double(c.eps);
+  t.im1 = tf_from_double(c.inveps - 1.0), t.inv = tf_from_double(c.inveps);
+#define BIPB_SYM64_RUN(TR_, LAP_, V_, NT_, CH_, MINB_)                                                          \
+  run_sym<Sym64Policy<TR_, LAP_>, NT_, 1, CH_, MINB_>(s, (TR_ ? 0x300 : 0x400) + V_, TR_ ? kTMv64T : kTMv64, L, \
+                                                      {t, s->exptab.p}, TR_, s->rec64, s->part64, u, y, dphi,  \
+                                                      dpsi, skip, skip_stride, kappa)
+#define BIPB_SYM64(V_, NT_, CH_, MINB_)                    \
+  if (transpose) {                                         \
+    if (lap)                                               \
+      BIPB_SYM64_RUN(true, true, V_, NT_, CH_, MINB_);     \
+    else                                                   \
+      BIPB_SYM64_RUN(true, false, V_, NT_, CH_, MINB_);    \
+  } else {                                                 \
+    if (lap)                                               \
+      BIPB_SYM64_RUN(false, true, V_, NT_, CH_, MINB_);    \
+    else                                                   \
+      BIPB_SYM64_RUN(false, false, V_, NT_, CH_, MINB_);   \
   }
+  if (small) {
+    BIPB_SYM64(0, 64, 32, 4)
+  } else {
+    BIPB_SYM64(1, 256, 64, 1)
+  }
+#undef BIPB_SYM64
 #undef BIPB_SYM64_RUN
   return true;
 }

@@ -1,0 +1,227 @@
+// The radial factors of an FP64 pair on the FP32 pipe, in triple-float
+// arithmetic.
+//
+// GB300 executes FP64 at 2 lanes per SM per cycle against 128 for FP32: one
+// FP64 instruction takes as long as 64 FP32 instructions, and 1/sqrt and exp
+// in FP64 are some forty of them a pair.  A value here is an unevaluated sum of three
+// floats a + b + c, |b| below a few ulp of a and |c| below a few ulp of b, built from
+// the error-free transformations of df64.cuh (two of the components exact, the
+// third by FP32 multiply-adds: about 2^-65 of the value; compare Hida, Li and
+// Bailey 2001, who drop the terms below the last component alike).  The five
+// coefficients of a pair come out within half an ulp and a few 2^-60 of FP64,
+// i.e. rounded once, where the FP64 chain rounds some ten times.
+//
+//   1/sqrt(r2): the exponent of r2 is halved apart; of its mantissa one step of
+//     third order from the MUFU estimate y (error 2^-22): y (1 + h/2 + 3 h^2/8 +
+//     5 h^3/16), h = 1 - r2 y^2 to 2^-68.
+//   exp(-x): Tang's table-driven method (ACM TOMS 15, 1989), x = k L + f with L =
+//     ln2/1024 in three floats, exp(-f) = 1 - f + f^2/2 - ... to f^5, times
+//     the table's 2^(j/1024) (FP64 values, as three floats).
+//
+// About 750 FP32 and integer instructions a pair, which run beside the pair's 30
+// FP64 operations (as long as 1920) and hide behind them: those bound the
+// kernel, 18.4 of the 19.4 billion pairs a second that 2 lanes of 152 SMs
+// allow.  N = 7001 3.65 -> 1.36 ms, N = 33000 65.9 -> 29.6 ms a mat-vec, where
+// CUDA's rsqrt and exp and the chain after them were 57 of 87 FP64 operations;
+// the error against 64 bits stays the same (4.6e-16 at N = 8000: what the
+// coordinates' own rounding gives).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "df64.cuh"
+#include "pair.cuh"
+
+namespace bipb {
+
+struct tf {
+  float a, b, c;
+};
+
+__device__ __forceinline__ tf tf_mul(tf x, tf y) {
+  const df p = two_prod(x.a, y.a), q = two_prod(x.a, y.b), r = two_prod(x.b, y.a);
+  const float c = __fmaf_rn(x.a, y.c, __fmaf_rn(x.c, y.a, __fmaf_rn(x.b, y.b, __fadd_rn(q.lo, r.lo))));
+  const df s = two_sum(q.hi, r.hi), t = two_sum(p.lo, s.hi);
+  return tf{p.hi, t.hi, __fadd_rn(c, __fadd_rn(s.lo, t.lo))};
+}
+__device__ __forceinline__ tf tf_sqr(tf x) {
+  const float a2 = __fadd_rn(x.a, x.a);
+  const df p = two_prod(x.a, x.a), q = two_prod(a2, x.b);
+  const df t = two_sum(p.lo, q.hi);
+  return tf{p.hi, t.hi, __fadd_rn(__fmaf_rn(a2, x.c, __fmaf_rn(x.b, x.b, q.lo)), t.lo)};
+}
+// times a float
+__device__ __forceinline__ tf tf_mul_f(tf x, float f) {
+  const df p = two_prod(x.a, f), q = two_prod(x.b, f);
+  const df t = two_sum(p.lo, q.hi);
+  return tf{p.hi, t.hi, __fmaf_rn(x.c, f, __fadd_rn(q.lo, t.lo))};
+}
+__device__ __forceinline__ tf tf_scale(tf x, float pow2) {
+  return tf{__fmul_rn(x.a, pow2), __fmul_rn(x.b, pow2), __fmul_rn(x.c, pow2)};
+}
+// |a| >= |b| >= |c| with no overlap beyond half an ulp
+__device__ __forceinline__ tf tf_norm(tf x) {
+  const df s = fast_two_sum(x.a, x.b), t = fast_two_sum(s.lo, x.c);
+  return tf{s.hi, t.hi, t.lo};
+}
+// x - y, normalised where the leading parts cancel
+__device__ __forceinline__ tf tf_sub(tf x, tf y) {
+  const df s = two_sum(x.a, -y.a), t = two_sum(x.b, -y.b), u = two_sum(s.lo, t.hi);
+  const df v = fast_two_sum(s.hi, u.hi);
+  const df w = two_sum(v.lo, __fadd_rn(__fsub_rn(x.c, y.c), __fadd_rn(t.lo, u.lo)));
+  return tf{v.hi, w.hi, w.lo};
+}
+// f - x for a float f, |f| >= |x|
+__device__ __forceinline__ tf tf_rsub_f(float f, tf x) {
+  const df s = fast_two_sum(f, -x.a), t = two_sum(s.lo, -x.b);
+  const df v = fast_two_sum(s.hi, t.hi);
+  return tf{v.hi, v.lo, __fsub_rn(t.lo, x.c)};
+}
+
+// x 2^shift in FP64, rounded once, by integer operations (an FP64 addition
+// costs as much as 64 instructions): the leading float truncated towards zero,
+// the rest, below its ulp, rounded to the 29 bits that follow.
+__device__ __forceinline__ double tf_to_double(tf x, int shift) {
+  const tf n = tf_norm(x);
+  const int sgn = __float_as_int(n.a) & 0x80000000;
+  const float h = __int_as_float(__float_as_int(n.a) ^ sgn), m = __int_as_float(__float_as_int(n.b) ^ sgn),
+              l = __int_as_float(__float_as_int(n.c) ^ sgn);
+  const int hb = __float_as_int(h) - (m < 0.f ? 1 : 0);
+  const df t = two_sum(__fsub_rn(h, __int_as_float(hb)), m);  // in [0, ulp)
+  const float S = __int_as_float(min(306 - (hb >> 23), 254) << 23);  // 2^29 / ulp
+  const int i = __float2int_rn(__fmul_rn(t.hi, S)) + __float2int_rn(__fmul_rn(__fadd_rn(t.lo, l), S));
+  const unsigned lo0 = (unsigned)hb << 29, lo = lo0 + (unsigned)i;
+  // i >= 0 up to the rounding of its parts (a carry), or -1 (a borrow)
+  const int hi = (hb >> 3) + 0x38000000 + (int)((unsigned)shift << 20) + (i >= 0 ? (lo < lo0 ? 1 : 0) : (lo > lo0 ? -1 : 0));
+  return hb == 0 ? 0.0 : __hiloint2double(hi | sgn, (int)lo);
+}
+// the three floats of an FP64 value (host and device: constants, table)
+__host__ __device__ __forceinline__ tf tf_from_double(double v) {
+  const float a = (float)v;
+  const float b = (float)(v - (double)a);
+  return tf{a, b, (float)(v - (double)a - (double)b)};
+}
+
+constexpr int kTfTab = kExpTab;
+// ln2/1024 in three floats and 1024/ln2
+constexpr float kTfL1 = 0x1.62e43p-11f, kTfL2 = -0x1.05c61p-39f, kTfL3 = -0x1.950d88p-64f, kTfInvL = 0x1.715476p+10f;
+// constants of one launch: eps - 1, eps, 1/eps - 1, 1/eps
+struct TfConst {
+  tf em1, eps, im1, inv;
+};
+
+// exp(-x) for x >= 0 (0 above 87: below 2^-125); tab[j] = 2^(j/1024)
+__device__ __forceinline__ tf tf_exp_minus(tf x, const float4* tab) {
+  const bool big = x.a > 87.0f;
+  if (big) x = tf{87.0f, 0.f, 0.f};
+  const float mg = __fmaf_rn(x.a, kTfInvL, 12582912.0f);
+  const float k = __fsub_rn(mg, 12582912.0f);
+  const int kk = 0x4b400000 - __float_as_int(mg);  // -k
+  const float4 T = tab[kk & (kTfTab - 1)];
+  const df p = two_prod(k, kTfL1), q = two_prod(k, kTfL2);
+  const df s = two_sum(x.b, -p.lo), u = two_sum(s.hi, -q.hi), r = two_sum(__fsub_rn(x.a, p.hi), u.hi);
+  const float r2 = __fadd_rn(r.lo, __fadd_rn(__fadd_rn(s.lo, u.lo), __fmaf_rn(-k, kTfL3, __fsub_rn(x.c, q.lo))));
+  // exp(-f) - 1 = -f + f^2/2 - f^3/6 + f^4/24 - f^5/120
+  const float f = r.hi;
+  const df Q = two_prod(f, f);
+  const float ql = __fmaf_rn(__fadd_rn(f, f), r2, Q.lo);
+  const float cub = __fmaf_rn(f, __fmaf_rn(f, -1.0f / 120.0f, 1.0f / 24.0f), -1.0f / 6.0f);
+  const float tail = __fmaf_rn(__fmul_rn(f, Q.hi), cub, __fmaf_rn(0.5f, ql, -r2));
+  const df e0 = fast_two_sum(-f, __fmul_rn(0.5f, Q.hi));
+  const float p2 = __fadd_rn(e0.lo, tail);
+  const df U = two_prod(T.x, e0.hi);
+  const float v = __fmaf_rn(T.x, p2, __fmaf_rn(T.y, e0.hi, U.lo));
+  const df w = fast_two_sum(T.x, U.hi), g = two_sum(T.y, w.lo), g2 = two_sum(g.hi, v);
+  const float sc = big ? 0.f : __int_as_float((127 + (kk >> 10)) << 23);
+  return tf_scale(tf{w.hi, g2.hi, __fadd_rn(T.z, __fadd_rn(g.lo, g2.lo))}, sc);
+}
+
+// The coefficients of the kappa-scaled pair (pair.cuh) of squared distance r2 > 0:
+//   k1 = (1 - e) s, v = (t - 1) s^3, w = (w - 3) s^5, k2 = (eps t - 1) s^3, k3 = (t / eps - 1) s^3
+// LAPLACE (e = t = 1, unscaled): k2 and k3 only.
+struct TfRadial {
+  double k1, v, w, k2, k3;
+};
+template <bool LAPLACE>
+__device__ __forceinline__ TfRadial tf_radial(double r2, const TfConst& c, const float4* tab) {
+  // r2 = rho 4^q, rho in [1, 4) as three floats (its 53 bits: 24, 23 and 6)
+  const int hi = __double2hiint(r2), lo = __double2loint(r2);
+  const int ex = (hi >> 20) - 1023, q = ex >> 1, odd = ex & 1;
+  const unsigned rem = (unsigned)lo & 0x1fffffffu;
+  tf rho;
+  rho.a = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
+  const float u = __int_as_float((81 + odd) << 23);  // 2^(odd - 46)
+  rho.b = __fmul_rn(__fsub_rn(__int_as_float(0x4b000000 | (int)(rem >> 6)), 8388608.0f), u);
+  rho.c = __fmul_rn(__fsub_rn(__int_as_float(0x4b000000 | (int)(rem & 63u)), 8388608.0f), __fmul_rn(u, 0x1p-6f));
+  // sig = 1 / sqrt(rho)
+  const float y = rsqrt_approx(rho.a);
+  const df p = two_prod(y, y), A = two_prod(rho.a, p.hi), B = two_prod(rho.a, p.lo), C = two_prod(rho.b, p.hi);
+  const float hl = __fmaf_rn(rho.b, p.lo, __fmaf_rn(rho.c, p.hi, __fadd_rn(B.lo, C.lo)));
+  const df s1 = two_sum(B.hi, C.hi), s2 = two_sum(A.lo, s1.hi);
+  const df h = two_sum(__fsub_rn(1.0f, A.hi), -s2.hi);
+  const float h2 = __fsub_rn(h.lo, __fadd_rn(__fadd_rn(s1.lo, s2.lo), hl));
+  const float cor = __fmaf_rn(__fmul_rn(h.hi, h.hi), __fmaf_rn(0.3125f, h.hi, 0.375f), __fmul_rn(0.5f, h2));
+  const df g = two_prod(y, __fmul_rn(0.5f, h.hi));
+  const tf sig = tf{y, g.hi, __fmaf_rn(y, cor, g.lo)};
+  const tf sg2 = tf_sqr(sig), sg3 = tf_mul(sg2, sig);
+  TfRadial R;
+  if constexpr (LAPLACE) {
+    R.k1 = R.v = R.w = 0.0;
+    R.k2 = tf_to_double(tf_mul(c.em1, sg3), -3 * q);
+    R.k3 = tf_to_double(tf_mul(c.im1, sg3), -3 * q);
+  } else {
+    const int qc = max(-60, min(60, q));
+    const tf kr = tf_scale(tf_mul(rho, sig), __int_as_float((127 + qc) << 23));
+    const tf e = tf_exp_minus(kr, tab);
+    const tf ome = tf_rsub_f(1.0f, e);
+    const tf omt = tf_sub(ome, tf_mul(e, kr));  // 1 - t
+    const tf vs = tf_mul(omt, sg3);
+    // (w - 3) s^2 = e - 3 (1 - t) s^2
+    const tf ws = tf_sub(e, tf_mul_f(tf_scale(tf_mul(omt, sg2), __int_as_float((127 - 2 * qc) << 23)), 3.0f));
+    R.k1 = tf_to_double(tf_mul(ome, sig), -q);
+    R.v = -tf_to_double(vs, -3 * q);
+    R.w = tf_to_double(tf_mul(ws, sg3), -3 * q);
+    // eps t - 1 = (eps - 1) - eps (1 - t)
+    R.k2 = tf_to_double(tf_mul(tf_sub(c.em1, tf_mul(c.eps, omt)), sg3), -3 * q);
+    R.k3 = tf_to_double(tf_mul(tf_sub(c.im1, tf_mul(c.inv, omt)), sg3), -3 * q);
+  }
+  return R;
+}
+
+// Both directions of one unordered pair (pair.cuh) from its coefficients R (0
+// for a masked pair), 23 FP64 operations: U = (t - 1) s^3 c_ij - (w - 3) s^5 c_i c_j.
+template <bool TRANS, bool LAPLACE>
+__device__ __forceinline__ void sym_pair64(double dx, double dy, double dz, const double* nt, double at, double alt,
+                                           const double* ns, double as, double als, const TfRadial& R, double& Pt,
+                                           double& Qt, double& Ps, double& Qs) {
+  const double ci = nt[0] * dx + nt[1] * dy + nt[2] * dz;
+  const double cj = ns[0] * dx + ns[1] * dy + ns[2] * dz;
+  if constexpr (LAPLACE) {
+    if (!TRANS) {
+      Pt = (R.k2 * cj) * als + Pt;
+      Qt = (R.k3 * ci) * as + Qt;
+      Ps = Ps - (R.k2 * ci) * alt;
+      Qs = Qs - (R.k3 * cj) * at;
+    } else {
+      Pt = Pt - (R.k2 * ci) * as;
+      Qt = Qt - (R.k3 * cj) * als;
+      Ps = (R.k2 * cj) * at + Ps;
+      Qs = (R.k3 * ci) * alt + Qs;
+    }
+  } else {
+    const double cij = nt[0] * ns[0] + nt[1] * ns[1] + nt[2] * ns[2];
+    const double U = R.v * cij - R.w * (ci * cj);
+    if (!TRANS) {
+      Pt = (R.k2 * cj) * als + (R.k1 * as + Pt);
+      Qt = U * als + ((R.k3 * ci) * as + Qt);
+      Ps = R.k1 * at - ((R.k2 * ci) * alt - Ps);
+      Qs = U * alt - ((R.k3 * cj) * at - Qs);
+    } else {
+      Pt = U * als - ((R.k2 * ci) * as - Pt);
+      Qt = R.k1 * as - ((R.k3 * cj) * als - Qt);
+      Ps = U * alt + ((R.k2 * cj) * at + Ps);
+      Qs = R.k1 * at + ((R.k3 * ci) * alt + Qs);
+    }
+  }
+}
+
+}  // namespace bipb

@@ -172,3 +172,26 @@ def test_treecode_forms_and_ragged_leaves(bipb, orc, n, params, kappa, transpose
     ref = orc.treecode.matvec(c, nv, a, 80.0, kappa, u, *params, transpose=transpose)
     assert np.linalg.norm(y - ref) < 3e-6 * np.linalg.norm(ref)
     assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [2, 31, 33, 64, 65, 129, 1280])
+@pytest.mark.parametrize("scale,kappa", [(1.0, 0.0), (1.0, 0.1257), (1e-3, 1.1e-6), (1e-3, 2.5), (1e3, 2.5), (1e3, 1.1e-6)])
+def test_fp64_symmetric_pair_range(bipb, orc, n, scale, kappa):
+    """The symmetric FP64 mat-vec, its radial factors in triple-float arithmetic, from
+    kappa r = 1e-9 (t - 1 cancels) to 1e5 (e^{-kappa r} underflows), on surfaces around
+    its blocks of 32 sources and tiles of 64 targets, both directions: the FP64 bound of
+    test_matvec_fp64_and_fp32.  Without contrast and screening the kernels vanish exactly."""
+    p = synth.protein_like_problem(level=3, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, min(n, p.n), replace=False))
+    c, nv, a = scale * p.centroids[keep], p.normals[keep], scale * scale * p.areas[keep]
+    u = np.random.default_rng(9).standard_normal(2 * len(keep))
+    with bipb.Surface(c, nv, a) as s:
+        for transpose in (False, True):
+            for eps in (80.0, 1.0):
+                y = torch.full_like(_dev(u), float("nan"))
+                s.matvec(_dev(u), y, precision=bipb.FP64, transpose=transpose, med=bipb.medium(1.0, eps, kappa))
+                y = y.cpu().numpy()
+                ref = (orc.matvec_t if transpose else orc.matvec)(c, nv, a, eps, kappa, u)
+                np.testing.assert_allclose(y, ref, rtol=0, atol=1e-12 * np.abs(ref).max(), err_msg=f"{transpose} {eps}")
+                if eps == 1.0 and kappa == 0.0:
+                    np.testing.assert_array_equal(y, u)
