@@ -32,7 +32,7 @@
 // Scaling.  FP16 holds 2^-14 .. 65504 at full precision, so both operands are
 // brought to a known range by exact powers of two.  Column (j, c) of A (the
 // source unknown phi_j or psi_j) is multiplied by 2^e(j, c), chosen once per
-// surface and medium (k_tc_colexp, over all targets) so that its largest
+// surface and medium (k_tc_colmax, over all targets) so that its largest
 // value lies in [2^14, 2^15); the factors are folded into a scaled copy of
 // the source records (area times 2^e(j, 1), normal times 2^(e(j, 0) -
 // e(j, 1)): the K2 and K4 values are linear in n_j, the K1 and K3 values do
@@ -64,6 +64,7 @@
 // Every wait on an mbarrier is bounded; a wait that runs out sets an error
 // flag that the host turns into BIPB_ERR_CUDA, and the kernel still frees its
 // tensor memory.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -103,18 +104,13 @@ constexpr int kScaleTop = 14;               // scaled magnitudes lie in [2^14, 2
 constexpr int kScaleClamp = 100;            // scale exponents are clamped to [-100, 100]
 constexpr double kTcKappaMin = 1e-6;        // the kappa-scaled form from this kappa on (1/A)
 static_assert(kOffBar % 8 == 0, "mbarriers need 8-byte alignment");
+static_assert(kPerThread == 8, "two halves of four sources per thread and chunk");
 
-// floor(log2 |x|) of a normal double (-1023 for zero and subnormals, 1024
-// for infinities and NaN)
-__device__ __forceinline__ int ilog2_bits(double x) {
-  return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023;
-}
 // The exponent e that brings a magnitude of floor(log2) lg into [2^14, 2^15)
 // by a factor 2^e, clamped to [-100, 100].
 __device__ __forceinline__ int scale_exp_lg(int lg) { return max(-kScaleClamp, min(kScaleClamp, kScaleTop - lg)); }
-// 2^k for |k| <= 126, and in FP64 for |k| <= 1022
+// 2^k for |k| <= 126
 __device__ __forceinline__ float pow2f(int k) { return __uint_as_float((uint32_t)(127 + k) << 23); }
-__device__ __forceinline__ double pow2d(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
 
 // byte offset of element (row, k) of a chunk's FP16 U tile (K = 32, K-major,
 // no swizzle): core matrices of 8 rows x 8 values (16 bytes a row)
@@ -134,49 +130,103 @@ __device__ __forceinline__ void arrive_expect_tx(uint64_t* bar, uint32_t bytes) 
 }
 
 // colmax[b] = max over sources j and components c of floor(log2 |u_b(j, c)|)
-// - e(j, c), at least -1123 for a nonzero u (colmax preset to a value below
-// -2000 by a byte fill of 0x80): grid (x, nb)
-__global__ void k_colmax_u(int n, const double* __restrict__ u, const int2* __restrict__ srcexp,
-                           int* __restrict__ colmax) {
-  const int b = blockIdx.y;
-  const int64_t len = 2 * (int64_t)n;
-  const double* ub = u + (int64_t)b * len;
+// - e(j, c) (INT_MIN for a zero u): a cluster of 4 blocks per right-hand side (64 blocks with
+// atomics on a cleared word took 27 us at 64 x 40001, one block 19, this 10).
+constexpr int kMaxClu = 4;
+__global__ void __cluster_dims__(kMaxClu, 1, 1) __launch_bounds__(1024) k_colmax_u(int n, const double* __restrict__ u,
+                                                   const int2* __restrict__ srcexp, int* __restrict__ colmax) {
+  __shared__ int red[32], parts[kMaxClu];
+  chain_wait();
+  chain_release();
+  const auto cluster = cooperative_groups::this_cluster();
+  const int b = blockIdx.x / kMaxClu, rank = blockIdx.x % kMaxClu;
+  const double* ub = u + (int64_t)b * 2 * n;
   int m = INT_MIN;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += (int64_t)gridDim.x * blockDim.x) {
-    const double v = ub[e];
-    const int j = (int)(e < n ? e : e - n);
-    if (v != 0.0) m = max(m, ilog2_bits(v) - (e < n ? srcexp[j].x : srcexp[j].y));
+  // floor(log2 |v|) - e of a nonzero v by its bits (no FP64 comparison): -1023
+  // of a subnormal, 1024 of an infinity or NaN
+  auto take = [&](double v, int e) {
+    const int hi = __double2hiint(v) & 0x7fffffff;
+    if ((hi | __double2loint(v)) != 0) m = max(m, (hi >> 20) - 1023 - e);
+  };
+#pragma unroll 8
+  for (int j = rank * 1024 + threadIdx.x; j < n; j += kMaxClu * 1024) {
+    const int2 e = srcexp[j];
+    take(ub[j], e.x);
+    take(ub[n + j], e.y);
   }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xffffffffu, red[threadIdx.x]);
+    if (threadIdx.x == 0) *cluster.map_shared_rank(parts + rank, 0) = m;
+  }
+  cluster.sync();
+  if (rank == 0 && threadIdx.x == 0) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(colmax + b, m);
+    for (int r = 0; r < kMaxClu; ++r) m = max(m, parts[r]);
+    colmax[b] = m;
+  }
 }
 
 // the scale exponent f(b) of right-hand side b from colmax[b] (100 for a zero column)
 __device__ __forceinline__ int rhs_exp(int cm) { return cm < -2000 ? kScaleClamp : scale_exp_lg(cm); }
 
+// v 2^k in FP16 parts hi + lo: v's bits as a float f (24 bits, truncated) and the
+// rest, hi = round(f), lo = round(f - hi + rest).  By integer and FP32
+// operations (conversions between FP64 and FP32 run at the FP64 rate).
+__device__ __forceinline__ void split_scaled(double v, int k, unsigned short& hi, unsigned short& lo) {
+  const int vh = __double2hiint(v);
+  const unsigned vl = (unsigned)__double2loint(v);
+  const int E = (vh >> 20) & 0x7ff, fe = E + k - 896;  // exponent field of the float
+  float f = __int_as_float((vh & 0x80000000) | (fe << 23) | ((vh & 0xfffff) << 3) | (int)(vl >> 29));
+  float rest = (float)(vl & 0x1fffffffu) * __int_as_float(((vh & 0x80000000) | (max(fe - 52, 0) << 23)));
+  if (E == 0 || fe < 1) f = rest = 0.f;                 // far below the smallest FP16
+  if (fe > 254) f = __int_as_float(0x7f800000), rest = 0.f;  // beyond FP32, infinities and NaN
+  const __half h = __float2half_rn(f);
+  hi = __half_as_ushort(h);
+  lo = __half_as_ushort(__float2half_rn((f - __half2float(h)) + rest));
+}
+
 // U (FP64, system b at b * 2n: [phi; psi]) -> per chunk, u 2^(f(b) - e(j, c))
 // split into FP16 parts U_hi (rows 0..63) and U_lo (rows 64..127) in the
-// K-major core-matrix layout (row = right-hand side, K = 2 j' + c).
+// K-major core-matrix layout (row = right-hand side, K = 2 j' + c).  A thread
+// takes 4 sources (8 values, one 16-byte core-matrix row of each part); the 8
+// rows of a core matrix lie on consecutive threads, so a warp's stores are
+// contiguous and its loads whole sectors (49 -> 12 us at 64 x 40001 against one
+// value per thread in FP64).
 __global__ void k_pack_u_tc(int n, int n_rhs, int n_chunks, const double* __restrict__ u,
                             const int2* __restrict__ srcexp, const int* __restrict__ colmax,
                             __half* __restrict__ upk) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // one per (chunk, b, k)
-  if (e >= (int64_t)n_chunks * kNB * kK) return;
-  const int ch = (int)(e / (kNB * kK));
-  const int rem = (int)(e % (kNB * kK));
-  const int b = rem / kK, k = rem % kK;
-  const int j = ch * kChunk + (k >> 1), c = k & 1;
-  __half hi = __float2half_rn(0.f), lo = hi;
-  if (b < n_rhs && j < n) {
-    const int2 ej = srcexp[j];
-    const double v = u[(int64_t)b * 2 * n + (int64_t)c * n + j] * pow2d(rhs_exp(colmax[b]) - (c ? ej.y : ej.x));
-    hi = __float2half_rn((float)v);
-    lo = __float2half_rn((float)(v - (double)__half2float(hi)));
+  chain_wait();
+  chain_release();
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int kGrp = kChunk / 4;  // groups of 4 sources in a chunk
+  if (e >= (int64_t)n_chunks * kNB * kGrp) return;
+  const int r = (int)(e % (kNB * kGrp));
+  const int64_t ch = e / (kNB * kGrp);
+  const int b = (r & 7) | (r / (8 * kGrp)) << 3, g = (r >> 3) % kGrp;
+  const int j0 = (int)ch * kChunk + 4 * g;
+  unsigned hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+  if (b < n_rhs) {
+    const double* ub = u + (int64_t)b * 2 * n;
+    const int f = rhs_exp(colmax[b]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + q;
+      if (j < n) {
+        const int2 ej = srcexp[j];
+        unsigned short h0, l0, h1, l1;
+        split_scaled(ub[j], f - ej.x, h0, l0);
+        split_scaled(ub[n + j], f - ej.y, h1, l1);
+        hi[q] = h0 | (unsigned)h1 << 16;
+        lo[q] = l0 | (unsigned)l1 << 16;
+      }
+    }
   }
-  unsigned char* tile = reinterpret_cast<unsigned char*>(upk) + (int64_t)ch * kUBytes;
-  *reinterpret_cast<__half*>(tile + kmajor16_offset(b, k)) = hi;
-  *reinterpret_cast<__half*>(tile + kmajor16_offset(kNB + b, k)) = lo;
+  unsigned char* tile = reinterpret_cast<unsigned char*>(upk) + ch * kUBytes;
+  *reinterpret_cast<uint4*>(tile + kmajor16_offset(b, 8 * g)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  *reinterpret_cast<uint4*>(tile + kmajor16_offset(kNB + b, 8 * g)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
 // kernel_block for the two sources of a record pair at once, in packed FP32
@@ -244,9 +294,11 @@ __device__ __forceinline__ void kernel_block2(const f2* T, const float4& P0, con
 // i != j (the same FP32 values the tensor-core kernel generates); 0 for a
 // column of zeros (no dielectric contrast and kappa = 0), and the two kept
 // within 2^40 of each other by lowering the larger, so that the scaled
-// normal and the products formed from it stay far from the FP32 range.  Then
-// the scaled source records, pair-interleaved for kernel_block2.  One thread
-// per source.
+// normal and the products formed from it stay far from the FP32 range.  Two
+// kernels: k_tc_colmax finds the maxima (one thread per source, the targets
+// split over blockIdx.y so that the chip is full: at N = 40001 3.9 -> 2.4 ms
+// against all targets in one thread), k_tc_records the exponents and the
+// scaled source records, pair-interleaved for kernel_block2.
 //
 // A column whose values are linear in the source normal takes its scale
 // through the normal, the other through the area field: for A u the phi
@@ -261,33 +313,56 @@ __device__ __forceinline__ void kernel_block2(const f2* T, const float4& P0, con
 // divided (A u) or multiplied (A^T) by kappa, a row factor undone in the
 // epilogue, while kappa r = r2 s and (w - 3) s^2 = 3 (t - 1) s^2 + e save
 // three FP32 operations per pair.
+// The unscaled source record of element j: (x, area field), (n, 0)
 template <bool SCALED, bool TRANS>
-__global__ void __launch_bounds__(128) k_tc_colexp(int n, const float4* __restrict__ tgt32, PairConst<float> c,
-                                                   int2* __restrict__ srcexp, float4* __restrict__ src) {
+__device__ __forceinline__ void tc_source(const float4* tgt32, int j, float ks, float4& g, float4& nv) {
+  g = tgt32[2 * j], nv = tgt32[2 * j + 1];
+  g = make_float4(ks * g.x, ks * g.y, ks * g.z, TRANS ? ks * ks : ks * g.w);
+  nv = make_float4(ks * nv.x, ks * nv.y, ks * nv.z, 0.f);
+}
+// colmax[j] = largest |value| of the phi and psi column of source j over the
+// targets of split blockIdx.y, as FP32 bits (zeroed before)
+template <bool SCALED, bool TRANS>
+__global__ void __launch_bounds__(128) k_tc_colmax(int n, const float4* __restrict__ tgt32, PairConst<float> c,
+                                                   uint2* __restrict__ colmax) {
   __shared__ float4 sh[2 * 128];
   const float ks = SCALED ? c.kappa : 1.f;
   const int j = blockIdx.x * 128 + threadIdx.x;
   const int jj = min(j, n - 1);
-  float4 gj = tgt32[2 * jj], nj = tgt32[2 * jj + 1];
-  gj = make_float4(ks * gj.x, ks * gj.y, ks * gj.z, TRANS ? ks * ks : ks * gj.w);
-  nj = make_float4(ks * nj.x, ks * nj.y, ks * nj.z, 0.f);
+  float4 gj, nj;
+  tc_source<SCALED, TRANS>(tgt32, jj, ks, gj, nj);
   float m0 = 0.f, m1 = 0.f;
-  for (int i0 = 0; i0 < n; i0 += 128) {
+  const int t0 = (int)((int64_t)blockIdx.y * n / gridDim.y), t1 = (int)((int64_t)(blockIdx.y + 1) * n / gridDim.y);
+  for (int i0 = t0; i0 < t1; i0 += 128) {
     __syncthreads();
     const int il = min(i0 + (int)threadIdx.x, n - 1);
-    sh[2 * threadIdx.x] = tgt32[2 * il];
+    const float4 g = tgt32[2 * il];
+    sh[2 * threadIdx.x] = make_float4(ks * g.x, ks * g.y, ks * g.z, 0.f);
     sh[2 * threadIdx.x + 1] = tgt32[2 * il + 1];
     __syncthreads();
-    const int cnt = min(128, n - i0);
+    const int cnt = min(128, t1 - i0);
+#pragma unroll 2
     for (int ii = 0; ii < cnt; ++ii) {
       const float4 g = sh[2 * ii], nv = sh[2 * ii + 1];
       float v[4];
-      kernel_block<SCALED, TRANS>(ks * g.x, ks * g.y, ks * g.z, nv.x, nv.y, nv.z, gj, nj, i0 + ii == jj, c, v);
+      kernel_block<SCALED, TRANS>(g.x, g.y, g.z, nv.x, nv.y, nv.z, gj, nj, i0 + ii == jj, c, v);
       m0 = fmaxf(m0, fmaxf(fabsf(v[0]), fabsf(v[2])));
       m1 = fmaxf(m1, fmaxf(fabsf(v[1]), fabsf(v[3])));
     }
   }
   if (j >= n) return;
+  atomicMax(&colmax[j].x, __float_as_uint(m0));
+  atomicMax(&colmax[j].y, __float_as_uint(m1));
+}
+// the exponents from the maxima (in place: srcexp holds them) and the records
+template <bool SCALED, bool TRANS>
+__global__ void __launch_bounds__(128) k_tc_records(int n, const float4* __restrict__ tgt32, float kappa,
+                                                    int2* __restrict__ srcexp, float4* __restrict__ src) {
+  const int j = blockIdx.x * 128 + threadIdx.x;
+  if (j >= n) return;
+  float4 gj, nj;
+  tc_source<SCALED, TRANS>(tgt32, j, SCALED ? kappa : 1.f, gj, nj);
+  const float m0 = __int_as_float(srcexp[j].x), m1 = __int_as_float(srcexp[j].y);
   // floor(log2 m) of a positive normal float
   auto lg = [](float m) { return (int)((__float_as_uint(m) >> 23) & 0xffu) - 127; };
   int e0 = m0 > 0.f ? scale_exp_lg(lg(m0)) : 0, e1 = m1 > 0.f ? scale_exp_lg(lg(m1)) : 0;
@@ -318,44 +393,45 @@ __device__ __forceinline__ void split_f16x2(float a0, float a1, uint32_t& hi, ui
       : "f"(a0), "f"(a1));
 }
 
-// This thread's kPerThread sources of a chunk (pair records Sp, first index
-// jq) against target ti (splats T): the scaled pair values, two sources per
-// packed evaluation, split into FP16 parts and written into the thread's TMEM
-// lane from column acol on (tile 0 hi / lo at + 0 / + kChunk, tile 1 at
-// + 2 kChunk / + 3 kChunk).  EDGE masks pairs with no target, a source past
-// the end or the self pair.
+// Half hh of this thread's kPerThread sources of a chunk (pair records Sp,
+// first index jq) against target ti (splats T): the scaled pair values, two
+// sources per packed evaluation, split into FP16 parts.  EDGE masks pairs with
+// no target, a source past the end or the self pair.
+struct GenHalf {
+  uint32_t h0[4], l0[4], h1[4], l1[4];  // per source: the phi-row pair (K2, K1) and psi-row pair (K4, K3)
+};
 template <bool EDGE, bool SCALED, bool TRANS>
-__device__ __forceinline__ void gen_chunk(const f2* T, const float4* Sp, int jq, int ti, int n, bool tvalid,
-                                          const PairConst<float>& c, uint32_t acol) {
+__device__ __forceinline__ void gen_half(const f2* T, const float4* Sp, int hh, int jq, int ti, int n, bool tvalid,
+                                         const PairConst<float>& c, GenHalf& o) {
 #pragma unroll
-  for (int hh = 0; hh < kPerThread / 4; ++hh) {
-    uint32_t h0[4], l0[4], h1[4], l1[4];  // per source: the phi-row pair (K2, K1) and psi-row pair (K4, K3)
+  for (int pp = 0; pp < 2; ++pp) {
+    const int p = 2 * hh + pp;
+    const int ja = jq + 2 * p, jb = ja + 1;
+    const bool za = EDGE && (!tvalid || ja >= n || ja == ti), zb = EDGE && (!tvalid || jb >= n || jb == ti);
+    f2 v[4];
+    kernel_block2<EDGE, SCALED, TRANS>(T, Sp[4 * p], Sp[4 * p + 1], Sp[4 * p + 2], Sp[4 * p + 3], za, zb, c, v);
+    float a[4], b[4];
 #pragma unroll
-    for (int pp = 0; pp < 2; ++pp) {
-      const int p = 2 * hh + pp;
-      const int ja = jq + 2 * p, jb = ja + 1;
-      const bool za = EDGE && (!tvalid || ja >= n || ja == ti), zb = EDGE && (!tvalid || jb >= n || jb == ti);
-      f2 v[4];
-      kernel_block2<EDGE, SCALED, TRANS>(T, Sp[4 * p], Sp[4 * p + 1], Sp[4 * p + 2], Sp[4 * p + 3], za, zb, c, v);
-      float a[4], b[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        f2_get(v[k], a[k], b[k]);
-        if (EDGE) {
-          a[k] = za ? 0.f : a[k];
-          b[k] = zb ? 0.f : b[k];
-        }
+    for (int k = 0; k < 4; ++k) {
+      f2_get(v[k], a[k], b[k]);
+      if (EDGE) {
+        a[k] = za ? 0.f : a[k];
+        b[k] = zb ? 0.f : b[k];
       }
-      split_f16x2(a[0], a[1], h0[2 * pp], l0[2 * pp]);
-      split_f16x2(a[2], a[3], h1[2 * pp], l1[2 * pp]);
-      split_f16x2(b[0], b[1], h0[2 * pp + 1], l0[2 * pp + 1]);
-      split_f16x2(b[2], b[3], h1[2 * pp + 1], l1[2 * pp + 1]);
     }
-    tc::tmem_st4(acol + 4 * hh, h0);
-    tc::tmem_st4(acol + 4 * hh + kChunk, l0);
-    tc::tmem_st4(acol + 4 * hh + 2 * kChunk, h1);
-    tc::tmem_st4(acol + 4 * hh + 3 * kChunk, l1);
+    split_f16x2(a[0], a[1], o.h0[2 * pp], o.l0[2 * pp]);
+    split_f16x2(a[2], a[3], o.h1[2 * pp], o.l1[2 * pp]);
+    split_f16x2(b[0], b[1], o.h0[2 * pp + 1], o.l0[2 * pp + 1]);
+    split_f16x2(b[2], b[3], o.h1[2 * pp + 1], o.l1[2 * pp + 1]);
   }
+}
+// into the thread's TMEM lane from column acol on (tile 0 hi / lo at + 0 / +
+// kChunk, tile 1 at + 2 kChunk / + 3 kChunk)
+__device__ __forceinline__ void store_half(uint32_t acol, int hh, const GenHalf& o) {
+  tc::tmem_st4(acol + 4 * hh, o.h0);
+  tc::tmem_st4(acol + 4 * hh + kChunk, o.l0);
+  tc::tmem_st4(acol + 4 * hh + 2 * kChunk, o.h1);
+  tc::tmem_st4(acol + 4 * hh + 3 * kChunk, o.l1);
 }
 
 // items: {t0, c0, c1, split}; tgt32: 2 float4 per element (x, y, z, area), (n, 0).
@@ -405,8 +481,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mrhs_tc(int n, int n_rhs, int n
     tc::mbar_init(drained, kGenThreads / 32);
     tc::fence_mbar_init();
   }
-  if (tid < kNB) cinv[tid] = pow2f(-rhs_exp(colmax[tid]));
   if (warp == 0) tc::tmem_alloc(tmem_slot, kTmemCols);
+  chain_wait();  // the packed right-hand sides (no early release: this kernel is long)
+  if (tid < kNB) cinv[tid] = tid < n_rhs ? pow2f(-rhs_exp(colmax[tid])) : 0.f;
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -492,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mrhs_tc(int n, int n_rhs, int n
     const int ti = t0 + 32 * wq + lane;
     const bool tvalid = ti < n;
     const float4 gi = tgt32[2 * min(ti, n - 1)], ni = tgt32[2 * min(ti, n - 1) + 1];
-    const float ks = SCALED ? c.kappa : 1.f;  // positions in Debye lengths (k_tc_colexp)
+    const float ks = SCALED ? c.kappa : 1.f;  // positions in Debye lengths (k_tc_colmax)
     const f2 T[6] = {f2_splat(ks * gi.x), f2_splat(ks * gi.y), f2_splat(ks * gi.z),
                      f2_splat(ni.x),      f2_splat(ni.y),      f2_splat(ni.z)};
     const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
@@ -521,25 +598,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_mrhs_tc(int n, int n_rhs, int n
       __syncwarp();
       if (lane == 0) mbar_arrive(drained);
     };
+    // chunk x's tile is complete: its stores have landed, one arrival per warp
+    // (512 arrivals on one barrier word would serialise)
+    auto publish = [&](int x) {
+      tc::tmem_wait_st();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ready[x % kABuf]);
+    };
+    // Per chunk: the values of half 0; then what the tensor core's side needs
+    // (publish the previous chunk, read back the previous group once its MMAs
+    // are done, wait for the A buffer); then the stores and half 1.  The
+    // latencies of the stores and of the MMAs are so covered by half a chunk of
+    // arithmetic in each warp, where publishing a chunk at its end and waiting
+    // at the next one's start had left the schedulers idle a third of the time.
     int drained_groups = 0;
     for (int it = 0; it < n_it; ++it) {
       const int s = it % kABuf, q = it % kRing;
       ok = ok && tc::mbar_wait_timed(&sfull[q], (it / kRing) & 1, kWaitLimitNs);
-      // chunk it - kABuf's MMAs read A buffer s
-      if (it >= kABuf) ok = ok && tc::mbar_wait_timed(&afree[s], ((it - kABuf) / kABuf) & 1, kWaitLimitNs);
-      // the second chunk of group g + 1 reads back group g before its tile is
-      // generated: the first chunk of group g + 1 waits for it
-      const int d = (it % kGroup == 1 && it > kGroup) ? it / kGroup - 1 : -1;
-      if (d >= 0) ok = ok && tc::mbar_wait_timed(done, d & 1, kWaitLimitNs);
       if (!ok) break;
-      if (it >= kABuf) tc::fence_after_sync();
-      if (d >= 0) {
-        read_back();
-        drained_groups = d + 1;
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(drained);
-      }
       const int j0 = (c0 + it) * kChunk;
       // chunks at the end of the surface or over the CTA's own targets, and the
       // last target tile, mask pairs (source past the end, self pair, no target)
@@ -547,17 +624,38 @@ __global__ void __launch_bounds__(kThreads, 1) k_mrhs_tc(int n, int n_rhs, int n
       const float4* Sp = reinterpret_cast<const float4*>(smem + kOffS + q * kSBytes) + 2 * kPerThread * sq;
       const int jq = j0 + kPerThread * sq;
       const uint32_t acol = tmem + lane_base + kColA + s * kACols + kPerThread * sq;
-      // one branch per chunk: the masked form only where a chunk needs it
+      GenHalf o;
+      // one branch per half: the masked form only where a chunk needs it
       if (edge)
-        gen_chunk<true, SCALED, TRANS>(T, Sp, jq, ti, n, tvalid, c, acol);
+        gen_half<true, SCALED, TRANS>(T, Sp, 0, jq, ti, n, tvalid, c, o);
       else
-        gen_chunk<false, SCALED, TRANS>(T, Sp, jq, ti, n, tvalid, c, acol);
-      tc::tmem_wait_st();
-      tc::fence_before_sync();
-      // one arrival per warp: 512 arrivals on one barrier word would serialise
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ready[s]);
+        gen_half<false, SCALED, TRANS>(T, Sp, 0, jq, ti, n, tvalid, c, o);
+      if (it > 0) publish(it - 1);
+      // the second chunk of group g + 1 reads back group g: the first chunk of
+      // group g + 1 waits for it
+      const int d = (it % kGroup == 1 && it > kGroup) ? it / kGroup - 1 : -1;
+      if (d >= 0) ok = ok && tc::mbar_wait_timed(done, d & 1, kWaitLimitNs);
+      if (!ok) break;
+      if (d >= 0) {
+        tc::fence_after_sync();
+        read_back();
+        drained_groups = d + 1;
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(drained);
+      }
+      // chunk it - kABuf's MMAs read A buffer s
+      if (it >= kABuf) ok = ok && tc::mbar_wait_timed(&afree[s], ((it - kABuf) / kABuf) & 1, kWaitLimitNs);
+      if (!ok) break;
+      if (it >= kABuf) tc::fence_after_sync();
+      store_half(acol, 0, o);
+      if (edge)
+        gen_half<true, SCALED, TRANS>(T, Sp, 1, jq, ti, n, tvalid, c, o);
+      else
+        gen_half<false, SCALED, TRANS>(T, Sp, 1, jq, ti, n, tvalid, c, o);
+      store_half(acol, 1, o);
     }
+    if (ok && n_it > 0) publish(n_it - 1);
     for (int d = drained_groups; ok && d < n_groups; ++d) drain(d);
   }
   const bool all_ok = __syncthreads_and(ok) != 0;
@@ -673,14 +771,15 @@ void matvec_tc(Surface* s, const SysLayout& L, const PairConst<float>& c0, bool 
   if (s->alloc_gen != gen0 || s->tc_src_n[dir] != n || key3[0] != c.eps || key3[1] != c.inveps ||
       key3[2] != c.kappa) {
     const int nbk = (n + 127) / 128;
-    if (scaled && transpose)
-      k_tc_colexp<true, true><<<nbk, 128, 0, s->stream>>>(n, s->tgt32.p, c, srcexp, src);
-    else if (scaled)
-      k_tc_colexp<true, false><<<nbk, 128, 0, s->stream>>>(n, s->tgt32.p, c, srcexp, src);
-    else if (transpose)
-      k_tc_colexp<false, true><<<nbk, 128, 0, s->stream>>>(n, s->tgt32.p, c, srcexp, src);
-    else
-      k_tc_colexp<false, false><<<nbk, 128, 0, s->stream>>>(n, s->tgt32.p, c, srcexp, src);
+    const dim3 mgrid(nbk, std::min((n + 255) / 256, std::max(1, (16 * s->num_sms + nbk - 1) / nbk)));
+    auto colmax = scaled ? (transpose ? k_tc_colmax<true, true> : k_tc_colmax<true, false>)
+                         : (transpose ? k_tc_colmax<false, true> : k_tc_colmax<false, false>);
+    auto records = scaled ? (transpose ? k_tc_records<true, true> : k_tc_records<true, false>)
+                          : (transpose ? k_tc_records<false, true> : k_tc_records<false, false>);
+    BIPB_CUDA(cudaMemsetAsync(srcexp, 0, (size_t)n * sizeof(int2), s->stream));
+    colmax<<<mgrid, 128, 0, s->stream>>>(n, s->tgt32.p, c, reinterpret_cast<uint2*>(srcexp));
+    BIPB_LAUNCHED(s);
+    records<<<nbk, 128, 0, s->stream>>>(n, s->tgt32.p, c.kappa, srcexp, src);
     BIPB_LAUNCHED(s);
     s->tc_src_n[dir] = n;
     key3[0] = c.eps, key3[1] = c.inveps, key3[2] = c.kappa;
@@ -704,20 +803,17 @@ void matvec_tc(Surface* s, const SysLayout& L, const PairConst<float>& c0, bool 
     }
     const double* ub = u + (int64_t)b0 * 2 * n;
     double* yb = y + (int64_t)b0 * 2 * n;
-    const int64_t pk = (int64_t)n_chunks * kNB * kK;
+    const int64_t pk = (int64_t)n_chunks * kNB * (kChunk / 4);
     __half* upk = reinterpret_cast<__half*>(s->upk.p);
-    BIPB_CUDA(cudaMemsetAsync(s->tc_colmax.p, 0x80, kNB * sizeof(int), s->stream));
-    k_colmax_u<<<dim3((unsigned)std::min<int64_t>(64, (2 * (int64_t)n + 255) / 256), nb), 256, 0, s->stream>>>(
-        n, ub, srcexp, s->tc_colmax.p);
+    launch_chained(k_colmax_u, kMaxClu * nb, 1024, 0, s->stream, n, ub, srcexp, s->tc_colmax.p);
     BIPB_LAUNCHED(s);
-    k_pack_u_tc<<<(int)((pk + 255) / 256), 256, 0, s->stream>>>(n, nb, n_chunks, ub, srcexp,
-                                                                  s->tc_colmax.p, upk);
+    launch_chained(k_pack_u_tc, (unsigned)((pk + 255) / 256), 256, 0, s->stream, n, nb, n_chunks, ub, srcexp,
+                   s->tc_colmax.p, upk);
     BIPB_LAUNCHED(s);
     {
       TimedLaunch tl(s, kTMvTC);
-      kernel<<<plan->n_items, kThreads, kSmemBytes, s->stream>>>(n, nb, S, plan->items.p, s->tgt32.p,
-                                                               src, s->tc_colmax.p, upk, s->part32.p, c,
-                                                               s->tc_err.p);
+      launch_chained(kernel, plan->n_items, kThreads, kSmemBytes, s->stream, n, nb, S, plan->items.p, s->tgt32.p, src,
+                     s->tc_colmax.p, upk, s->part32.p, c, s->tc_err.p);
       BIPB_LAUNCHED(s);
     }
     launch_reduce_matvec32(s, Lb, tt->second->tab.p, s->part32.p, ub, yb, dphi, dpsi,

@@ -232,7 +232,7 @@ __device__ __forceinline__ void sym_pair2(const f2* xt, const f2* nt, const f2* 
 // K4_ji) in v[0], v[1], the psi row (K1_ji, K3_ji) in v[2], v[3], times the
 // record's area field (the output's area is applied to the sums), i.e.
 // ((1 - eps t) c_i s^3, K4, (1 - e) s, (1 - t/eps) c_j s^3).
-// SCALED: positions, area and normal in kappa-scaled units (k_tc_colexp,
+// SCALED: positions, area and normal in kappa-scaled units (k_tc_colmax,
 // mrhs_tc.cu: kappa r = r2 s and (w - 3) s^2 = 3 (t - 1) s^2 + e; one row
 // comes out with an extra power of kappa); c.nkl2e and c.smax are then
 // -log2(e) and the 1/r cap in those units.

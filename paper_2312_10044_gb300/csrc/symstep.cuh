@@ -26,7 +26,8 @@ struct PartSum<float> {
     hi = t.hi;
     lo = __fadd_rn(lo, t.lo);
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  // of an infinite sum the TwoSum errors are NaN and the leading part is the sum
+  __device__ __forceinline__ double value() const { return lo == lo ? (double)hi + (double)lo : (double)hi; }
 };
 
 // Sum of component c (0: phi, 1: psi) of one element of a system over a

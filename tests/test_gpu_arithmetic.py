@@ -195,3 +195,33 @@ def test_fp64_symmetric_pair_range(bipb, orc, n, scale, kappa):
                 np.testing.assert_allclose(y, ref, rtol=0, atol=1e-12 * np.abs(ref).max(), err_msg=f"{transpose} {eps}")
                 if eps == 1.0 and kappa == 0.0:
                     np.testing.assert_array_equal(y, u)
+
+
+@pytest.mark.parametrize("transpose", [False, True])
+def test_tensor_right_hand_side_packing(bipb, orc, transpose):
+    """The packing of right-hand sides by their bits: values over forty orders of
+    magnitude within one right-hand side, subnormals, an infinity and a NaN, whose
+    right-hand sides come out not finite while the others keep the FP32 bounds of
+    test_tensor_core_matvec_matches_oracle; more sources than one pass of the maximum's
+    cluster takes, an odd number."""
+    p = synth.protein_like_problem(level=4, n_charges=3)
+    n = 4099
+    keep = np.sort(np.random.default_rng(n).choice(p.n, n, replace=False))
+    c, nv, a = p.centroids[keep], p.normals[keep], p.areas[keep]
+    rng = np.random.default_rng(6)
+    U = rng.standard_normal((6, 2 * n))
+    U[1] *= 10.0 ** rng.uniform(-40, 0, 2 * n)
+    U[2, ::3] *= 1e-310
+    U[3, 5] = np.inf
+    U[4, n + 7] = np.nan
+    med = bipb.medium(p.eps_in, p.eps_out, p.kappa)
+    with bipb.Surface(c, nv, a) as s:
+        yd = torch.zeros_like(_dev(U))
+        s.matvec(_dev(U), yd, precision=bipb.TENSOR, transpose=transpose, med=med)
+        Y = yd.cpu().numpy()
+    f = orc.matvec_t if transpose else orc.matvec
+    for r in (0, 1, 2, 5):
+        ref = f(c, nv, a, p.eps_out / p.eps_in, p.kappa, U[r])
+        assert np.linalg.norm(Y[r] - ref) < 3e-6 * np.linalg.norm(ref), r
+        assert np.abs(Y[r] - ref).max() < 2e-5 * np.abs(ref).max(), r
+    assert not np.isfinite(Y[3:5]).any()
