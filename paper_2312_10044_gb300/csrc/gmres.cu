@@ -55,20 +55,24 @@ struct DevState {
 constexpr int kStateInts = (int)(sizeof(DevState) / sizeof(int));
 static_assert(offsetof(DevState, skip) == sizeof(int), "skip must be the second int");
 
+// Sum over the block in a fixed order, valid in thread 0.  One warp adds the
+// values from shared memory: a tree of shuffles in every warp would take
+// five times the FP64 additions (two lanes per SM).
 template <int NT>
 __device__ double block_sum(double v) {
-  __shared__ double red[NT / 32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ double red[NT];
   __syncthreads();
-  if (lane == 0) red[wid] = v;
+  red[threadIdx.x] = v;
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x < 32) {
-    t = threadIdx.x < NT / 32 ? red[threadIdx.x] : 0.0;
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) p[i & 3] += red[32 * i + threadIdx.x];
+    t = (p[0] + p[1]) + (p[2] + p[3]);
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
   }
-  return t;  // valid in thread 0
+  return t;
 }
 
 // Block table: blk[b] = {system, first element, end element, first block of
@@ -94,25 +98,45 @@ __device__ __forceinline__ double warp_sum_parts(const double* part, int stride,
   return __shfl_sync(0xffffffffu, s, 0);
 }
 
+// The lines of V_0 .. V_j that the block reads, into L1 (they are read in two
+// phases of the step, whose first loads would each wait for L2).
+template <int NT>
+__device__ __forceinline__ void prefetch_basis(int j, int64_t len, const double* V, int4 B, int4 Lk) {
+  const int lines = ((B.z - B.y) * 8 + 127) / 128 + 1;
+  for (int t = threadIdx.x; t < 2 * (j + 1) * lines; t += NT) {
+    const int r = t / lines, q = t % lines;
+    const double* p = V + (size_t)(r >> 1) * len + Lk.z + (r & 1) * Lk.y + min(B.y + 16 * q, B.z - 1);
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+  }
+}
+
 // part[b * m1 + i] = V_i . w over block b's unknowns, i <= j: one warp per
-// vector and half (phi, psi), the two halves added at the end.  V and w hold
-// values that other threads of the cluster or block wrote in this kernel.
+// vector (one tree of FP64 shuffles each), its phi and psi unknowns side by
+// side.  V and w hold values that other threads of the cluster or block wrote in
+// this kernel.
 template <int NT>
 __device__ __forceinline__ void block_dots(int j, int m1, int64_t len, const double* V, const double* w,
                                            double* part, int b, int4 B, int4 Lk) {
-  __shared__ double half[2 * (kMaxRestart + 1)];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = warp; t < 2 * (j + 1); t += NT / 32) {
-    const int64_t o = Lk.z + (t & 1) * Lk.y;
-    const double *v = V + (size_t)(t >> 1) * len + o, *x = w + o;
-    double acc = 0.0;
-#pragma unroll 4
-    for (int e = B.y + lane; e < B.z; e += 32) acc += v[e] * x[e];
-    acc = warp_sum(acc);
-    if (lane == 0) half[t] = acc;
+  for (int i = warp; i <= j; i += NT / 32) {
+    const double *v = V + (size_t)i * len + Lk.z, *x = w + Lk.z;
+    double acc[2] = {0.0, 0.0};
+    constexpr int U = 5;  // elements in flight, the last batch filled with zeros (sum_strided)
+    for (int e = B.y + lane; e < B.z; e += 32 * U) {
+      double p[2 * U], q[2 * U];
+#pragma unroll
+      for (int r = 0; r < 2 * U; ++r) {
+        const int o = e + 32 * (r >> 1);
+        const bool in = o < B.z;
+        p[r] = in ? v[o + (r & 1) * Lk.y] : 0.0;
+        q[r] = in ? x[o + (r & 1) * Lk.y] : 0.0;
+      }
+#pragma unroll
+      for (int r = 0; r < 2 * U; ++r) acc[r & 1] += p[r] * q[r];
+    }
+    const double t = warp_sum(acc[0] + acc[1]);
+    if (lane == 0) part[(size_t)b * m1 + i] = t;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i <= j; i += NT) part[(size_t)b * m1 + i] = half[2 * i] + half[2 * i + 1];
 }
 
 // Preconditioning by the element self blocks (Sec. 2.2.4 with one element per
@@ -145,16 +169,16 @@ struct StepArgs {
 };
 
 template <int NT, bool FUSED>
-__device__ __forceinline__ void step_dots(const StepArgs& a, int b, int4 B, int4 Lk) {
+__device__ __forceinline__ void step_dots(const StepArgs& a, int b, int4 B, int4 Lk, int4 Sm) {
   if (FUSED) {
-    const int4 S = a.mv.tab[B.x];
     const int cnt = B.z - B.y;
     for (int t = threadIdx.x; t < 2 * cnt; t += NT) {
       const int c = t < cnt ? 0 : 1, e = B.y + t - c * cnt;
-      const double acc = sym_sum(a.mv.tab, S, a.mv.part, e, c);
-      const double sc = kInv4PiG * (a.mv.transpose ? a.tgt64[2 * (Lk.x + e)].w : 1.0);
       const int64_t x = Lk.z + (int64_t)c * Lk.y + e;
-      a.w[x] = (c ? a.mv.dpsi : a.mv.dphi) * a.u[x] - sc * (c ? a.mv.f.y : a.mv.f.x) * acc;
+      const double ux = a.u[x];
+      const double sc = kInv4PiG * (a.mv.transpose ? a.tgt64[2 * (Lk.x + e)].w : 1.0);
+      const double acc = sym_sum(a.mv.tab, Sm, a.mv.part, e, c);
+      a.w[x] = (c ? a.mv.dpsi : a.mv.dphi) * ux - sc * (c ? a.mv.f.y : a.mv.f.x) * acc;
     }
     __syncthreads();  // the block's w is visible to all its threads
   }
@@ -165,9 +189,10 @@ __device__ __forceinline__ void step_dots(const StepArgs& a, int b, int4 B, int4
 // with NORM, also part1[b] = sum of the updated w^2 over block b's unknowns;
 // otherwise the block's dot products of the updated w for the second
 // Gram-Schmidt pass (block-local, so they need no reduction in between).
+// col: the system's column of H as well, in the first block.
 template <int NT, bool NORM>
 __device__ __forceinline__ void step_orth(const StepArgs& a, const double* part, int accumulate, int b, int4 B,
-                                          int4 S, int4 Lk) {
+                                          int4 S, int4 Lk, double* col) {
   const int j = a.j, m1 = a.m + 1;
   __shared__ double h[kMaxRestart + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -179,15 +204,25 @@ __device__ __forceinline__ void step_orth(const StepArgs& a, const double* part,
   __syncthreads();
   if (b == S.x) {
     double* Hs = a.H + (size_t)B.x * m1 * a.m + (size_t)j * m1;
-    for (int i = threadIdx.x; i <= j; i += NT) Hs[i] = accumulate ? Hs[i] + h[i] : h[i];
+    for (int i = threadIdx.x; i <= j; i += NT) {
+      const double v = accumulate ? Hs[i] + h[i] : h[i];
+      Hs[i] = v;
+      if (col != nullptr) col[i] = v;
+    }
   }
   double ss = 0.0;
   const int cnt = B.z - B.y;
   for (int t = threadIdx.x; t < 2 * cnt; t += NT) {
     const int64_t x = Lk.z + B.y + (t < cnt ? t : t - cnt + Lk.y);
     double p = a.w[x];
-#pragma unroll 8
-    for (int i = 0; i <= j; ++i) p -= h[i] * a.V[(size_t)i * a.len + x];
+    constexpr int U = 4;
+    for (int i0 = 0; i0 <= j; i0 += U) {
+      double v[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) v[q] = i0 + q <= j ? a.V[(size_t)(i0 + q) * a.len + x] : 0.0;
+#pragma unroll
+      for (int q = 0; q < U; ++q) p -= h[min(i0 + q, j)] * v[q];
+    }
     a.w[x] = p;
     ss += p * p;
   }
@@ -200,34 +235,54 @@ __device__ __forceinline__ void step_orth(const StepArgs& a, const double* part,
   }
 }
 
-// Per system: apply earlier rotations to column j, make rotation j, update g,
-// test.  The column (j + 2 entries, h[j + 1] = ||w||) and the earlier
-// rotations are in shared memory (ch, csh, snh), staged by the caller's
-// block in parallel, so the serial recurrence waits on no global load.
-__device__ void givens_step(int j, int m, int sys, const double* ch, const double* csh, const double* snh,
-                            double* __restrict__ H, double* __restrict__ cs, double* __restrict__ sn,
-                            double* __restrict__ g, DevState* __restrict__ st) {
-  DevState& S = st[sys];
-  const int m1 = m + 1;
-  double* h = H + (size_t)sys * m1 * m + (size_t)j * m1;
-  double* g_ = g + (size_t)sys * m1;
-  const double gj = g_[j], bnorm = S.bnorm, tol = S.tol;
-  const int iters = S.iters + 1, max_iter = S.max_iter, Sm = S.m;
-  double a = ch[0];
-  for (int i = 0; i < j; ++i) {
-    const double c = csh[i], t = snh[i], x = ch[i + 1];
-    h[i] = c * a + t * x;
-    a = c * x - t * a;
+// What the Givens step reads beside the new column: the earlier rotations and
+// the system's state.  Loaded by one warp of the system before it is needed.
+struct GivensIn {
+  double cs[kMaxRestart], sn[kMaxRestart], col[kMaxRestart + 1];
+  double gj, inv_bnorm, tol;
+  int iters, max_iter, m;
+};
+__device__ __forceinline__ void givens_load(const StepArgs& a, int sys, GivensIn& in) {
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < a.j; i += 32) in.cs[i] = a.cs[(size_t)sys * a.m + i], in.sn[i] = a.sn[(size_t)sys * a.m + i];
+  if (lane == 0) {
+    const DevState& S = a.st[sys];
+    in.gj = a.g[(size_t)sys * (a.m + 1) + a.j];
+    in.inv_bnorm = S.bnorm > 0.0 ? 1.0 / S.bnorm : 0.0;
+    in.tol = S.tol, in.iters = S.iters, in.max_iter = S.max_iter, in.m = S.m;
   }
-  const double b = ch[j + 1];
-  // den = sqrt(a^2 + b^2) = |(a, b)| of the pair scaled by a power of two near its larger part
-  const int big = max((__double2hiint(a) >> 20) & 0x7ff, (__double2hiint(b) >> 20) & 0x7ff);
+}
+
+// Per system: apply earlier rotations to column j (in.col, then b = ||w||, given
+// as b^2), make rotation j, update g, test.  One thread: the recurrence is
+// serial, one FP64 multiply-add a rotation; b and 1/|(a, b)| are both
+// taken from b^2, so the two 1/sqrt run side by side.
+__device__ void givens_step(const StepArgs& A, int sys, const GivensIn& in, double b2) {
+  const int j = A.j, m = A.m, m1 = m + 1;
+  DevState& S = A.st[sys];
+  double *cs = A.cs, *sn = A.sn;
+  double* h = A.H + (size_t)sys * m1 * m + (size_t)j * m1;
+  double* g_ = A.g + (size_t)sys * m1;
+  const double gj = in.gj, tol = in.tol;
+  const int iters = in.iters + 1, max_iter = in.max_iter, Sm = in.m;
+  double a = in.col[0];
+#pragma unroll 4
+  for (int i = 0; i < j; ++i) {
+    const double c = in.cs[i], t = in.sn[i], x = in.col[i + 1];
+    h[i] = fma(c, a, t * x);
+    a = fma(-t, a, c * x);
+  }
+  const double b = b2 > 0.0 ? b2 * rsqrt(b2) : 0.0;
+  // den = sqrt(a^2 + b^2) = |(a, b)| of the pair scaled by a power of two near its
+  // larger part; that of b is half the exponent of b^2
+  const int eb = (((__double2hiint(b2) >> 20) & 0x7ff) + 1023) >> 1;
+  const int big = max((__double2hiint(a) >> 20) & 0x7ff, b2 > 0.0 ? eb : 0);
   const int up = min(max(big, 1), 2045);
   const double down = __hiloint2double((2046 - up) << 20, 0), back = __hiloint2double(up << 20, 0);  // 2^(1023 - up), 2^(up - 1023)
-  const double as = a * down, bs = b * down, q = as * as + bs * bs;
+  const double as = a * down, q = as * as + (b2 * down) * down;
   const double inv = q > 0.0 ? rsqrt(q) : 0.0;
   const double den = q * inv * back;
-  const double c = q > 0.0 ? as * inv : 1.0, s = bs * inv;
+  const double c = q > 0.0 ? as * inv : 1.0, s = (b * down) * inv;
   h[j] = den;
   h[j + 1] = 0.0;
   cs[(size_t)sys * m + j] = c;
@@ -237,7 +292,7 @@ __device__ void givens_step(int j, int m, int sys, const double* ch, const doubl
   g_[j] = c * gj;
   S.k = j + 1;
   S.iters = iters;
-  const double est = bnorm > 0.0 ? fabs(gj1) / bnorm : 0.0;
+  const double est = fabs(gj1) * in.inv_bnorm;
   S.est = est;
   const int conv = est <= tol || b == 0.0;
   const int stop = iters >= max_iter;
@@ -246,17 +301,15 @@ __device__ void givens_step(int j, int m, int sys, const double* ch, const doubl
   if (conv || stop || j + 1 == Sm) S.skip = 1;
 }
 
-// (||w||, 1 / ||w||) of the system from the blocks' sums, in every thread (0, 0 for w = 0)
+// (||w||^2, 1 / ||w||) of the system from the blocks' sums, in each of the block's first NT threads (0, 0 for w = 0)
+template <int NT = kBS>
 __device__ __forceinline__ double2 step_norm(const double* part1, int4 S) {
   __shared__ double2 nrm;
   if (threadIdx.x < 32) {
     const double s = warp_sum_parts(part1, 1, 0, S.x, S.y);
-    if (threadIdx.x == 0) {
-      const double inv = s > 0.0 ? rsqrt(s) : 0.0;
-      nrm = make_double2(s * inv, inv);
-    }
+    if (threadIdx.x == 0) nrm = make_double2(s, s > 0.0 ? rsqrt(s) : 0.0);
   }
-  __syncthreads();
+  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
   return nrm;
 }
 
@@ -283,34 +336,24 @@ __device__ __forceinline__ void step_next(const StepArgs& a, double inv, int4 B,
   }
 }
 
-// H[j+1, j] = ||w|| and the Givens step of column j, by one warp of the system
-__device__ __forceinline__ void step_givens(const StepArgs& a, int sys, double norm) {
-  __shared__ double ch[kMaxRestart + 2], csh[kMaxRestart], snh[kMaxRestart];
-  const int j = a.j, m = a.m, lane = threadIdx.x & 31;
-  const double* Hc = a.H + (size_t)sys * (m + 1) * m + (size_t)j * (m + 1);
-  for (int i = lane; i <= j; i += 32) ch[i] = Hc[i];
-  for (int i = lane; i < j; i += 32) csh[i] = a.cs[(size_t)sys * m + i], snh[i] = a.sn[(size_t)sys * m + i];
-  if (lane == 0) ch[j + 1] = norm;
-  __syncwarp();
-  if (lane == 0) givens_step(j, m, sys, ch, csh, snh, a.H, a.cs, a.sn, a.g, a.st);
-}
-
 template <bool FUSED>
 __global__ void __launch_bounds__(kBS) k_dots(StepArgs a) {
+  // the tables are constant: read while the previous kernel ends
+  const int4 B = a.blk[blockIdx.x], Lk = a.lay[B.x], Sm = FUSED ? a.mv.tab[B.x] : make_int4(0, 0, 0, 0);
   chain_wait();
   chain_release();
-  const int4 B = a.blk[blockIdx.x];
   if (a.st[B.x].skip) return;
-  step_dots<kBS, FUSED>(a, blockIdx.x, B, a.lay[B.x]);
+  prefetch_basis<kBS>(a.j, a.len, a.V, B, Lk);
+  step_dots<kBS, FUSED>(a, blockIdx.x, B, Lk, Sm);
 }
 
 template <bool NORM>
 __global__ void __launch_bounds__(kBS) k_orth(StepArgs a, const double* part, int accumulate) {
+  const int4 B = a.blk[blockIdx.x], S = a.sysb[B.x], Lk = a.lay[B.x];
   chain_wait();
   chain_release();
-  const int4 B = a.blk[blockIdx.x];
   if (a.st[B.x].skip) return;
-  step_orth<kBS, NORM>(a, part, accumulate, blockIdx.x, B, a.sysb[B.x], a.lay[B.x]);
+  step_orth<kBS, NORM>(a, part, accumulate, blockIdx.x, B, S, Lk, nullptr);
 }
 
 // The Givens step is made by the last block of the system to finish (every
@@ -318,13 +361,12 @@ __global__ void __launch_bounds__(kBS) k_orth(StepArgs a, const double* part, in
 // arrival is counted with an atomic after a fence, no block waits).
 template <bool FUSED>
 __global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
+  const int4 B = a.blk[blockIdx.x], S = a.sysb[B.x], Lk = a.lay[B.x];
   chain_wait();
   chain_release();
-  const int4 B = a.blk[blockIdx.x];
   if (a.st[B.x].skip) return;
-  const int4 S = a.sysb[B.x];
   const double2 v = step_norm(a.part1, S);
-  step_next<kBS, FUSED>(a, v.y, B, a.lay[B.x]);
+  step_next<kBS, FUSED>(a, v.y, B, Lk);
   __shared__ int last;
   if (threadIdx.x == 0) {
     __threadfence();
@@ -334,7 +376,13 @@ __global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
   if (!last) return;
   __threadfence();
   if (threadIdx.x == 0) a.st[B.x].arrive = 0;
-  if (threadIdx.x < 32) step_givens(a, B.x, v.x);
+  if (threadIdx.x >= 32) return;
+  __shared__ GivensIn in;
+  givens_load(a, B.x, in);
+  const double* Hc = a.H + (size_t)B.x * (a.m + 1) * a.m + (size_t)a.j * (a.m + 1);
+  for (int i = threadIdx.x; i <= a.j; i += 32) in.col[i] = Hc[i];
+  __syncwarp();
+  if (threadIdx.x == 0) givens_step(a, B.x, in, v.x);
 }
 
 // The whole step in one launch: a cluster of kClu CTAs per system (its blocks).
@@ -347,27 +395,33 @@ __device__ __forceinline__ void cluster_sync() {
 }
 template <bool CGS2, bool FUSED>
 __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluNT) k_step(StepArgs a) {
+  const int4 B = a.blk[blockIdx.x], S = a.sysb[B.x], Lk = a.lay[B.x];
+  const int4 Sm = FUSED ? a.mv.tab[B.x] : make_int4(0, 0, 0, 0);
   chain_wait();
   chain_release();
-  const int4 B = a.blk[blockIdx.x];
   if (a.st[B.x].skip) return;  // the same for every CTA of the cluster
-  const int4 S = a.sysb[B.x], Lk = a.lay[B.x];
-  step_dots<kCluNT, FUSED>(a, blockIdx.x, B, Lk);
+  __shared__ GivensIn in;
+  const bool first = (int)blockIdx.x == S.x;
+  prefetch_basis<kCluNT>(a.j, a.len, a.V, B, Lk);
+  if (first && threadIdx.x >= kCluNT - 32) givens_load(a, B.x, in);
+  step_dots<kCluNT, FUSED>(a, blockIdx.x, B, Lk, Sm);
   cluster_sync();
   if (CGS2) {
-    step_orth<kCluNT, false>(a, a.part, 0, blockIdx.x, B, S, Lk);
+    step_orth<kCluNT, false>(a, a.part, 0, blockIdx.x, B, S, Lk, nullptr);
     cluster_sync();
-    step_orth<kCluNT, true>(a, a.part2, 1, blockIdx.x, B, S, Lk);
+    step_orth<kCluNT, true>(a, a.part2, 1, blockIdx.x, B, S, Lk, first ? in.col : nullptr);
   } else {
-    step_orth<kCluNT, true>(a, a.part, 0, blockIdx.x, B, S, Lk);
+    step_orth<kCluNT, true>(a, a.part, 0, blockIdx.x, B, S, Lk, first ? in.col : nullptr);
   }
   cluster_sync();  // also: every CTA has passed its skip test
   // the last warp of the system's first block makes the Givens step beside the others' vector work
-  const double2 v = step_norm(a.part1, S);
-  if (threadIdx.x < kCluNT - 32)
+  if (threadIdx.x < kCluNT - 32) {
+    const double2 v = step_norm<kCluNT - 32>(a.part1, S);
     step_next<kCluNT - 32, FUSED>(a, v.y, B, Lk);
-  else if ((int)blockIdx.x == S.x)
-    step_givens(a, B.x, v.x);
+  } else if (first) {
+    const double b2 = warp_sum_parts(a.part1, 1, 0, S.x, S.y);
+    if (threadIdx.x == kCluNT - 32) givens_step(a, B.x, in, b2);
+  }
 }
 
 // part1[b] = sum of w^2 over block b's unknowns (mode 0: systems not skipped,
@@ -404,8 +458,8 @@ __global__ void k_start(const double* __restrict__ r0, double* __restrict__ V, c
     if (tz != nullptr) tz[x] = pre.x * p, tz[y] = pre.y * q;
   }
   if (threadIdx.x == 0 && (int)blockIdx.x == S.x) {
-    st[B.x].bnorm = v.x;
-    st[B.x].beta = v.x;
+    st[B.x].bnorm = v.x * inv;
+    st[B.x].beta = v.x * inv;
   }
 }
 
@@ -474,11 +528,16 @@ __global__ void k_update(int m, int64_t len, double* __restrict__ V, double* __r
     for (int o = B.y + threadIdx.x; o < B.z; o += kBS) {
       const int64_t e = Lk.z + c * Lk.y + o;
       double dx = 0.0, v0 = 0.0;
-#pragma unroll 4
-      for (int i = 0; i <= k; ++i) {
-        double v = V[(size_t)i * len + e];
-        if (i < k) dx += y_[i] * v;
-        v0 += z_[i] * v;
+      constexpr int U = 4;
+      for (int i0 = 0; i0 <= k; i0 += U) {
+        double v[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) v[q] = i0 + q <= k ? V[(size_t)(i0 + q) * len + e] : 0.0;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          dx += (i0 + q < k ? y_[i0 + q] : 0.0) * v[q];
+          v0 += z_[min(i0 + q, k)] * v[q];
+        }
       }
       if (tz != nullptr) {
         x[e] += f * dx;

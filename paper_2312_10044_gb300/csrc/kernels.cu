@@ -12,6 +12,8 @@
 // reduction kernel adds the splits of every target in a fixed order in FP64,
 // applies 1/(4 pi) and the diagonal, and writes the output, so every pass is
 // bitwise reproducible.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 #include <algorithm>
 #include <cmath>
@@ -651,13 +653,8 @@ __global__ void k_reduce_matvec(const int4* __restrict__ lay, const int4* __rest
   // two outputs per thread
   const int i0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (i0 >= 2 * n || sys_skipped(skip, skip_stride, k)) return;
-  PartSum<PT> acc[2];
   const PT* p = part + (size_t)T.z + i0;
-#pragma unroll 8
-  for (int sp = 0; sp < T.y; ++sp) {
-    acc[0].add(p[(size_t)sp * 2 * n]);
-    acc[1].add(p[(size_t)sp * 2 * n + 1]);
-  }
+  const PartSum<PT> acc[2] = {sum_strided<8>(p, (size_t)2 * n, T.y), sum_strided<8>(p + 1, (size_t)2 * n, T.y)};
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     const int i = i0 + q;
@@ -688,35 +685,50 @@ __global__ void k_reduce_source(const int4* __restrict__ lay, const int4* __rest
   const int n = L.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * n) return;
-  double acc = 0.0;
-  for (int sp = 0; sp < T.y; ++sp) acc += part[(size_t)T.z + (size_t)sp * 2 * n + i];
-  b[L.z + i] = scale * acc;
+  b[L.z + i] = scale * sum_strided<8>(part + (size_t)T.z + i, (size_t)2 * n, T.y).value();
 }
 
-// One block per system: phi_reac_k = (1/(4 pi)) sum over splits;
-// E = KCAL/2 sum_k q_k phi_reac_k in a fixed order.
-__global__ void k_reduce_reaction(const int4* __restrict__ tab, const int4* __restrict__ lay,
-                                  const double* __restrict__ part, const double4_32a* __restrict__ chg,
-                                  double* __restrict__ phi_reac, double* __restrict__ e_out) {
-  __shared__ double red[1024];
-  const int k = blockIdx.x;
+// A cluster of blocks per system: phi_reac_k = (1/(4 pi)) sum over splits; E =
+// KCAL/2 sum_k q_k phi_reac_k in a fixed order.  A block takes tiles of 32 charges,
+// its warps one range of the splits each (few charges come with many splits:
+// one thread a charge in one block took 31 us for 1344 splits, this XX).
+constexpr int kReacClu = 8, kReacWarps = 16;
+__global__ void __cluster_dims__(kReacClu, 1, 1) __launch_bounds__(32 * kReacWarps)
+    k_reduce_reaction(const int4* __restrict__ tab, const int4* __restrict__ lay, const double* __restrict__ part,
+                      const double4_32a* __restrict__ chg, double* __restrict__ phi_reac, double* __restrict__ e_out) {
+  __shared__ double red[kReacWarps][32], sums[kReacClu];
+  const auto cluster = cooperative_groups::this_cluster();
+  const int k = blockIdx.x / kReacClu, rank = blockIdx.x % kReacClu;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int4 T = tab[k];
   const int nc = T.x, c0 = lay[k].w;
-  double local = 0.0;
-  for (int q = threadIdx.x; q < nc; q += blockDim.x) {
-    double acc = 0.0;
-    for (int sp = 0; sp < T.y; ++sp) acc += part[(size_t)T.z + (size_t)sp * nc + q];
-    acc *= kInv4Pi;
-    if (phi_reac) phi_reac[c0 + q] = acc;
-    local += chg[c0 + q].w * acc;
-  }
-  red[threadIdx.x] = local;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+  const int s0 = (int)((int64_t)warp * T.y / kReacWarps), s1 = (int)((int64_t)(warp + 1) * T.y / kReacWarps);
+  double local = 0.0;  // warp 0
+  for (int q0 = 32 * rank; q0 < nc; q0 += 32 * kReacClu) {
+    const int q = q0 + lane;
+    __syncthreads();  // the previous tile's sums have been read
+    red[warp][lane] =
+        q < nc ? sum_strided<8>(part + (size_t)T.z + (size_t)s0 * nc + q, (size_t)nc, s1 - s0).value() : 0.0;
     __syncthreads();
+    if (warp == 0 && q < nc) {
+      double acc = 0.0;
+#pragma unroll
+      for (int w = 0; w < kReacWarps; ++w) acc += red[w][lane];
+      acc *= kInv4Pi;
+      if (phi_reac) phi_reac[c0 + q] = acc;
+      local += chg[c0 + q].w * acc;
+    }
   }
-  if (threadIdx.x == 0 && e_out) e_out[k] = 0.5 * kKcal * red[0];
+  if (warp == 0) {
+    for (int o = 16; o > 0; o >>= 1) local += __shfl_down_sync(0xffffffffu, local, o);
+    if (lane == 0) *cluster.map_shared_rank(sums + rank, 0) = local;
+  }
+  cluster.sync();
+  if (rank == 0 && threadIdx.x == 0 && e_out) {
+    double t = sums[0];
+    for (int r = 1; r < kReacClu; ++r) t += sums[r];
+    e_out[k] = 0.5 * kKcal * t;
+  }
 }
 
 // Potential at points: out[k n_pts + q] (+)= scale * sum over splits of
@@ -727,8 +739,7 @@ __global__ void k_reduce_points(const int4* __restrict__ tab, const double* __re
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n_pts) return;
   const int4 T = tab[k];
-  double acc = 0.0;
-  for (int sp = 0; sp < T.y; ++sp) acc += part[(size_t)T.z + (size_t)sp * stride * n_pts + q];
+  const double acc = sum_strided<8>(part + (size_t)T.z + q, (size_t)stride * n_pts, T.y).value();
   double* o = out + (size_t)k * n_pts + q;
   *o = (accumulate ? *o : 0.0) + scale * acc;
 }
@@ -1154,7 +1165,7 @@ void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const d
   BIPB_LAUNCHED(s);
   ReactionPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, 0};
   launch_items<ReactionPolicy, float4, NT, TPT, CH>(s, kTReaction, plan, a, s->recdf.p, nullptr, 0);
-  k_reduce_reaction<<<L.K, 1024, 0, s->stream>>>(plan->tab.p, lay, s->part64.p, s->chg.p, phi_reac, e_out);
+  k_reduce_reaction<<<kReacClu * L.K, 32 * kReacWarps, 0, s->stream>>>(plan->tab.p, lay, s->part64.p, s->chg.p, phi_reac, e_out);
   BIPB_LAUNCHED(s);
 }
 

@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
   static_assert(TPT % P::PACK == 0, "whole packs of targets");
   __shared__ V4 sh[CH * P::RW];
   __shared__ typename P::Red jred[NW][CH];
-  chain_wait();  // the records of the pack kernel (no early release: this kernel is long)
+  chain_wait();  // the records of the pack kernel
+  chain_release();  // the next kernel is placed once every block of this one is, and waits there
   const int4 H = items[3 * blockIdx.x];
   const int rec_off = H.x, n = H.y, sys = H.z, jbase = H.w;
   if (skip != nullptr && skip[(size_t)sys * skip_stride] != 0) return;

@@ -30,6 +30,23 @@ struct PartSum<float> {
   __device__ __forceinline__ double value() const { return lo == lo ? (double)hi + (double)lo : (double)hi; }
 };
 
+// Sum of count values stride apart, in order, U loads in flight at a time: the last
+// batch is filled up with zeros, where a loop unrolled by U would leave up to U - 1
+// values to a rolled remainder that waits for each load in turn.  (A guard around
+// each addition lets the compiler move the load behind it, which is as slow.)
+template <int U, typename PT>
+__device__ __forceinline__ PartSum<PT> sum_strided(const PT* __restrict__ p, size_t stride, int count) {
+  PartSum<PT> acc;
+  for (int k = 0; k < count; k += U) {
+    PT v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) v[q] = k + q < count ? p[(size_t)(k + q) * stride] : PT(0);
+#pragma unroll
+    for (int q = 0; q < U; ++q) acc.add(v[q]);
+  }
+  return acc;
+}
+
 // Sum of component c (0: phi, 1: psi) of one element of a system over a
 // symmetric pass's partial sums: the i-side blocks of the element's row, then
 // the j-side values of rows 0..E, in that order.  S = {n, first row entry,
@@ -39,15 +56,19 @@ __device__ __forceinline__ double sym_sum(const int4* __restrict__ tab, const in
                                           int e, int c) {
   const int n = S.x, T = S.w, E = e / T;
   const int4 R = tab[S.y + E];
-  PartSum<PT> p;
-  const PT* b = part + (size_t)R.x + (size_t)c * T + (e - E * T);
-#pragma unroll 16
-  for (int k = 0; k < R.y; ++k) p.add(b[(size_t)k * 2 * T]);
+  PartSum<PT> p = sum_strided<sizeof(PT) == 4 ? 24 : 8>(part + (size_t)R.x + (size_t)c * T + (e - E * T), (size_t)2 * T, R.y);
   // row I starts at S.z + 2 (I n - T I (I - 1) / 2): element e of it at e - I T
-#pragma unroll 8
-  for (int I = 0; I <= E; ++I) {
-    const PT* r = part + (int64_t)S.z + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2) + (e - I * T);
-    p.add(r[c * (n - I * T)]);
+  constexpr int U = sizeof(PT) == 4 ? 8 : 4;
+  for (int I0 = 0; I0 <= E; I0 += U) {
+    PT v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int I = I0 + q;
+      const int64_t o = (int64_t)S.z + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2) + (e - I * T);
+      v[q] = I <= E ? part[o + c * (n - I * T)] : PT(0);
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) p.add(v[q]);
   }
   return p.value();
 }

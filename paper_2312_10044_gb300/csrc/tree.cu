@@ -377,13 +377,8 @@ __global__ void k_tree_reduce(int n, const int* __restrict__ perm, const int* __
   if (t >= n || tree_skipped(skip, skip_stride, k)) return;
   const int4 lf = leaf_tab[leaf_of[t]];
   const int local = t - lf.x;
-  PartSum<float> s1, s3;
-#pragma unroll 4
-  for (int i = lf.z; i < lf.z + lf.w; ++i) {
-    const float* o = part + 2 * (size_t)lmax * ((size_t)k * n_items + i);
-    s1.add(o[local]);
-    s3.add(o[lmax + local]);
-  }
+  const float* o = part + 2 * (size_t)lmax * ((size_t)k * n_items + lf.z) + local;
+  const PartSum<float> s1 = sum_strided<8>(o, (size_t)2 * lmax, lf.w), s3 = sum_strided<8>(o + lmax, (size_t)2 * lmax, lf.w);
   const int4 L = lay[k];
   const int e = perm[t];
   const bool tr = area_of != nullptr;

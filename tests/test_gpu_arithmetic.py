@@ -225,3 +225,24 @@ def test_tensor_right_hand_side_packing(bipb, orc, transpose):
         assert np.linalg.norm(Y[r] - ref) < 3e-6 * np.linalg.norm(ref), r
         assert np.abs(Y[r] - ref).max() < 2e-5 * np.abs(ref).max(), r
     assert not np.isfinite(Y[3:5]).any()
+
+
+@pytest.mark.parametrize("nc", [1, 31, 33, 257, 300])
+def test_reaction_reduction_tiles(bipb, orc, nc):
+    """The reduction of the reaction potentials over tiles of 32 charges, one block of
+    the cluster each, and ranges of the splits (many for few charges): two charge sets
+    of unequal size beside a tile's and the cluster's width, at 1e-12 as the charge passes."""
+    p = synth.protein_like_problem(level=3, n_charges=nc, seed=2)
+    u = np.random.default_rng(8).standard_normal(2 * p.n)
+    eps = p.eps_out / p.eps_in
+    q = np.asarray(p.q).reshape(-1, p.nc)[0]
+    e_ref, pr_ref = orc.energy(p.centroids, p.normals, p.areas, eps, p.kappa, p.charge_pos, q, u)
+    with bipb.Surface(p.centroids, p.normals, p.areas) as s:
+        s.set_charges(p.charge_pos, np.stack([q, -2.0 * q]))
+        pr, e = _dev(np.zeros((2, p.nc))), _dev(np.zeros(2))
+        s.reaction(_dev(np.stack([u, u])), pr, e, med=bipb.medium(p.eps_in, p.eps_out, p.kappa))
+        pr, e = pr.cpu().numpy(), e.cpu().numpy()
+    for k, f in enumerate((1.0, -2.0)):
+        np.testing.assert_allclose(pr[k], pr_ref, rtol=0, atol=1e-12 * np.abs(pr_ref).max())
+        scale = 0.5 * orc.KCAL * np.abs(f * q).sum() * np.abs(pr_ref).max()
+        assert abs(e[k] - orc.KCAL * f * e_ref) < 1e-12 * scale
