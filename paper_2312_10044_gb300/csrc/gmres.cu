@@ -153,6 +153,13 @@ __device__ __forceinline__ void block_dots(int j, int m1, int64_t len, const dou
 // records.  As three kernels (a block per about 128 elements), or, for small
 // systems, as one kernel with one cluster of CTAs per system, whose barrier
 // takes the place of the kernel boundaries.
+// What bounds the cluster's step (10.6 us at N = 1280, the tenth vector; 14.2
+// before): a chain of latencies.  So every loop keeps its loads in flight
+// together (a rolled remainder waits for each), the basis is fetched into L1 beside
+// the mat-vec's sums, tables are read before the previous kernel's end, and the Givens
+// step's state and reciprocal beside the dot products; and FP64 additions
+// (two lanes per SM), so a vector takes one tree of shuffles and a block's sum
+// one warp.
 struct StepArgs {
   int j, m;
   int64_t len;
@@ -763,8 +770,9 @@ double2 precond_factors(const bipb_medium& m) {
 // step as fast as the three kernels' launches and block reductions take only
 // for small systems, and only while every cluster has its SMs.  With the fused
 // FP32 mat-vec they also sum its partial sums.  Whole solves, cluster /
-// kernels: one system of 1280 elements 1.59 / 1.98 ms; 12 of 320 .. 5120, fused,
-// 3.00 / 2.91 ms; 16 charge sets on 5120 elements, not fused, 8.0 / 8.2 ms.
+// kernels: one system of 320 elements 1.41 / 1.74 ms, 1280 1.55 / 1.84, 2560 2.25 /
+// 2.26, 4000 3.24 / 3.31, 5120 4.20 / 3.56; 12 of 320 .. 5120, fused, 2.66 / 2.55; 16
+// charge sets on 5120 elements, not fused, 7.06 / 7.23 ms.
 bool cluster_step(const SysLayout& L, bool fused) {
   return L.max_n <= (fused ? 2560 : 5120) && L.K * kClu <= 160;
 }

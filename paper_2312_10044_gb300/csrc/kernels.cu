@@ -691,7 +691,7 @@ __global__ void k_reduce_source(const int4* __restrict__ lay, const int4* __rest
 // A cluster of blocks per system: phi_reac_k = (1/(4 pi)) sum over splits; E =
 // KCAL/2 sum_k q_k phi_reac_k in a fixed order.  A block takes tiles of 32 charges,
 // its warps one range of the splits each (few charges come with many splits:
-// one thread a charge in one block took 31 us for 1344 splits, this XX).
+// one thread a charge in one block took 31 us for 1344 splits, this 7).
 constexpr int kReacClu = 8, kReacWarps = 16;
 __global__ void __cluster_dims__(kReacClu, 1, 1) __launch_bounds__(32 * kReacWarps)
     k_reduce_reaction(const int4* __restrict__ tab, const int4* __restrict__ lay, const double* __restrict__ part,
