@@ -53,19 +53,21 @@ constexpr double kInv4PiS = 1.0 / (4.0 * kPi);
 // half per target of the pack) until a block of 32 sources is done.  Red is the
 // j side of one source over a warp.
 
-// FP64, one target per pack.  Record (x, a), (n, alpha), where (a, alpha) =
-// (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w.
-// LAPLACE: the kappa = 0 form (pair.cuh); otherwise the records
-// are in kappa-scaled units (SCALED).
+// FP64, one target per pack.  Record (a, alpha, n.x, n.y), (n.z, x.h, x.l), (x.m),
+// where (a, alpha) = (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w and the
+// position is in three floats on the surface's grid (df_pos), 9 of them from the
+// second vector's second value on.  LAPLACE: the kappa = 0 form (pair.cuh);
+// otherwise the records are in kappa-scaled units (SCALED).
 template <bool TRANS, bool LAPLACE>
 struct Sym64Policy {
   using V4 = double4_32a;
   using PT = double;  // partial sums are stored in this type
   static constexpr bool SCALED = !LAPLACE;
-  static constexpr int RW = 2, PACK = 1, UNROLL = 1;
+  static constexpr int RW = 3, PACK = 1, UNROLL = 1;
   static constexpr bool CHUNKED = false;
   struct Tgt {
-    double x[3], a, n[3], al;
+    df_pos x[3];
+    double a, n[3], al;
   };
   using Src = Tgt;
   struct Acc {
@@ -86,20 +88,27 @@ struct Sym64Policy {
     const float* t3 = reinterpret_cast<const float*>(g.tab + kExpTab / 2);
     for (int j = threadIdx.x; j < kTfTab; j += blockDim.x) exp_tab()[j] = make_float4(t2[j].x, t2[j].y, t3[j], 0.f);
   }
-  __device__ static void load(const V4* rec, const int* i, Tgt& t) { unpack(rec[2 * (size_t)i[0]], rec[2 * (size_t)i[0] + 1], t); }
+  __device__ static void load(const V4* rec, const int* i, Tgt& t) {
+    const V4* r = rec + 3 * (size_t)i[0];
+    unpack(r[0], r[1], r[2], t);
+  }
   // record q of a chunk staged as planes (vector r of record q at sh[r * CH + q])
   template <int CH>
-  __device__ static void load_src(const V4* sh, int q, Src& e) { unpack(sh[q], sh[CH + q], e); }
-  __device__ static void unpack(const V4& A, const V4& B, Tgt& e) {
-    e.x[0] = A.x, e.x[1] = A.y, e.x[2] = A.z, e.a = A.w;
-    e.n[0] = B.x, e.n[1] = B.y, e.n[2] = B.z, e.al = B.w;
+  __device__ static void load_src(const V4* sh, int q, Src& e) { unpack(sh[q], sh[CH + q], sh[2 * CH + q], e); }
+  static __device__ float2 floats(double v) { return make_float2(__int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v))); }
+  static __device__ double pair_of(float a, float b) { return __hiloint2double(__float_as_int(b), __float_as_int(a)); }
+  __device__ static void unpack(const V4& A, const V4& B, const V4& C, Tgt& e) {
+    e.a = A.x, e.al = A.y, e.n[0] = A.z, e.n[1] = A.w, e.n[2] = B.x;
+    const float2 p = floats(B.y), q = floats(B.z), r = floats(B.w), s = floats(C.x);
+    e.x[0] = df_pos{p.x, q.y, s.x}, e.x[1] = df_pos{p.y, r.x, s.y}, e.x[2] = df_pos{q.x, r.y, floats(C.y).x};
   }
   __device__ static void zero(Acc& v) { v.p = 0.0, v.q = 0.0; }
   // i side of the targets t and j side of source sj for the pairs d = x_t - x_sj
   template <bool MASK>
   __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
-    const double dx = t.x[0] - sj.x[0], dy = t.x[1] - sj.x[1], dz = t.x[2] - sj.x[2];
-    TfRadial R = tf_radial<LAPLACE>(dx * dx + dy * dy + dz * dz, g.c, LAPLACE ? nullptr : exp_tab());
+    const tf d[3] = {tf_diff(t.x[0], sj.x[0]), tf_diff(t.x[1], sj.x[1]), tf_diff(t.x[2], sj.x[2])};
+    TfRadial R = tf_radial<LAPLACE>(tf_norm2(d[0], d[1], d[2]), g.c, LAPLACE ? nullptr : exp_tab());
+    const double dx = tf_to_double(d[0], 0), dy = tf_to_double(d[1], 0), dz = tf_to_double(d[2], 0);
     if (MASK && masked[0]) R.k1 = R.v = R.w = R.k2 = R.k3 = 0.0;
     sym_pair64<TRANS, LAPLACE>(dx, dy, dz, t.n, t.a, t.al, sj.n, sj.a, sj.al, R, ti.p, ti.q, tj.p, tj.q);
   }
@@ -113,8 +122,9 @@ struct Sym64Policy {
   // a source slot q past the end of a chunk: far away, no field, no normal (adds exact zeros)
   template <int CH>
   __device__ static void pad(V4* sh, int q) {
-    sh[q] = make_double4_32a(1e4, 1e4, 1e4, 0.0);
-    sh[CH + q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    sh[q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    sh[CH + q] = make_double4_32a(0.0, pair_of(1e4f, 1e4f), pair_of(1e4f, 0.f), 0.0);
+    sh[2 * CH + q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
   }
   __device__ static PT out(double v) { return v; }
   __device__ static void store(PT* p, int T, const int* o, const bool* in, const Acc& v) {
@@ -398,7 +408,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sym(typename P::Args g, const int4
 // gscale: the power of two at or above sigma, by which the surface's coordinate grid grows with it
 __global__ void k_pack_sym64(const int4* __restrict__ lay, bool transpose, const double4_32a* __restrict__ tgt64,
                              const double* __restrict__ u, double4_32a* __restrict__ rec, const int* __restrict__ skip,
-                             int skip_stride, double sigma) {
+                             int skip_stride, double sigma, double gscale) {
   chain_wait();
   chain_release();
   const int k = blockIdx.y;
@@ -409,9 +419,14 @@ __global__ void k_pack_sym64(const int4* __restrict__ lay, bool transpose, const
   const double phi = u[L.z + j], psi = u[L.z + L.y + j];
   const double a = transpose ? phi : g.w * psi;
   const double al = sigma * (transpose ? psi : g.w * phi);
-  double4_32a* o = rec + 2 * (size_t)(L.z / 2 + j);
-  o[0] = make_double4_32a(sigma * g.x, sigma * g.y, sigma * g.z, a);
-  o[1] = make_double4_32a(v.x, v.y, v.z, al);
+  const double grid = gscale * v.w;  // of the scaled coordinates
+  const df_pos x0 = df_split_grid(sigma * g.x, grid), x1 = df_split_grid(sigma * g.y, grid),
+               x2 = df_split_grid(sigma * g.z, grid);
+  auto two = [](float p, float q) { return __hiloint2double(__float_as_int(q), __float_as_int(p)); };
+  double4_32a* o = rec + 3 * (size_t)(L.z / 2 + j);
+  o[0] = make_double4_32a(a, al, v.x, v.y);
+  o[1] = make_double4_32a(v.z, two(x0.h, x1.h), two(x2.h, x0.l), two(x1.l, x2.l));
+  o[2] = make_double4_32a(two(x0.m, x1.m), two(x2.m, 0.f), 0.0, 0.0);
 }
 
 // every value twice, with the negated fields (Sym32Policy)
@@ -730,7 +745,7 @@ void run_sym(Surface* s, int pass_id, int kind, const SysLayout& L, const typena
   if (!(stages & kSymPack)) {
   } else if constexpr (std::is_same<typename P::V4, double4_32a>::value) {
     launch_chained(k_pack_sym64, pgrid, 128, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
-                   sigma);
+                   sigma, std::exp2(std::ceil(std::log2(sigma))));
   } else if constexpr (std::is_same<typename P::PT, double>::value) {
     launch_chained(k_pack_sym_df, pgrid, 128, 0, s->stream, lay, transpose, s->tgt64.p, u, recbuf.p, skip, skip_stride,
                    sigma, std::exp2(std::ceil(std::log2(sigma))));
@@ -816,8 +831,8 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
 
 // FP64 shapes: tiles of 64 targets in CTAs of 64 threads up to 32768 elements,
 // tiles and CTAs of 256 above.  Small tiles leave less of the diagonal masked
-// and more, shorter work items (N = 320 57 against 155 us, 1000 109 / 246, 7001
-// 1362 / 1463); from N = 20000 on both take the same time (10.9 ms), and
+// and more, shorter work items (N = 320 56 against 142 us, 1000 106 / 214, 7001
+// 1155 / 1288); from N = 20000 on both take the same time (9.2 ms), and
 // the j-side partials (8 n^2 / T bytes: 134 MB at 32768 with T = 64) would only grow.
 constexpr int kSym64Small = 32768;
 
@@ -847,7 +862,7 @@ bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c0, d
       BIPB_SYM64_RUN(false, false, V_, NT_, CH_, MINB_);   \
   }
   if (small) {
-    BIPB_SYM64(0, 64, 32, 4)
+    BIPB_SYM64(0, 64, 32, 8)
   } else {
     BIPB_SYM64(1, 256, 64, 1)
   }

@@ -11,6 +11,7 @@
 // coefficients of a pair come out within half an ulp and a few 2^-60 of FP64,
 // i.e. rounded once, where the FP64 chain rounds some ten times.
 //
+//   r2 from differences of coordinates on a grid, exact to the third part.
 //   1/sqrt(r2): the exponent of r2 is halved apart; of its mantissa one step of
 //     third order from the MUFU estimate y (error 2^-22): y (1 + h/2 + 3 h^2/8 +
 //     5 h^3/16), h = 1 - r2 y^2 to 2^-68.
@@ -18,13 +19,17 @@
 //     ln2/1024 in three floats, exp(-f) = 1 - f + f^2/2 - ... to f^5, times
 //     the table's 2^(j/1024) (FP64 values, as three floats).
 //
-// About 750 FP32 and integer instructions a pair, which run beside the pair's 30
-// FP64 operations (as long as 1920) and hide behind them: those bound the
-// kernel, 18.4 of the 19.4 billion pairs a second that 2 lanes of 152 SMs
-// allow.  N = 7001 3.65 -> 1.36 ms, N = 33000 65.9 -> 29.6 ms a mat-vec, where
-// CUDA's rsqrt and exp and the chain after them were 57 of 87 FP64 operations;
-// the error against 64 bits stays the same (4.6e-16 at N = 8000: what the
-// coordinates' own rounding gives).
+// The differences of the coordinates and r2 are taken in the same arithmetic, and
+// the differences assembled for the FP64 dot products: with r2 from FP64
+// differences the error of a mat-vec was FP64's (4.7e-16 at N = 8000), now it
+// is a quarter of it.
+//
+// About 930 FP32 and integer instructions a pair, which run beside the pair's 24
+// FP64 operations (as long as 1536) and mostly hide behind them: 21.8 of the 24.3
+// billion pairs a second that 2 lanes of 152 SMs allow.  N = 7001 3.65 -> 1.16
+// ms, N = 33000 65.9 -> 25.0 ms a mat-vec, where CUDA's rsqrt and exp and the
+// chain after them were 57 of 87 FP64 operations (1.36 and 29.6 ms with the
+// differences and r2, six more operations, in FP64).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -69,6 +74,27 @@ __device__ __forceinline__ tf tf_sub(tf x, tf y) {
   const df v = fast_two_sum(s.hi, u.hi);
   const df w = two_sum(v.lo, __fadd_rn(__fsub_rn(x.c, y.c), __fadd_rn(t.lo, u.lo)));
   return tf{v.hi, w.hi, w.lo};
+}
+// x - y of grid coordinates (exact but for the third part's rounding)
+__device__ __forceinline__ tf tf_diff(df_pos x, df_pos y) {
+  const df d = fast_two_sum(__fsub_rn(x.h, y.h), __fsub_rn(x.l, y.l));
+  return tf{d.hi, d.lo, __fsub_rn(x.m, y.m)};
+}
+// |d|^2
+__device__ __forceinline__ tf tf_norm2(tf x, tf y, tf z) {
+  const float x2 = __fadd_rn(x.a, x.a), y2 = __fadd_rn(y.a, y.a), z2 = __fadd_rn(z.a, z.a);
+  const df px = two_prod(x.a, x.a), py = two_prod(y.a, y.a), pz = two_prod(z.a, z.a);
+  const df qx = two_prod(x2, x.b), qy = two_prod(y2, y.b), qz = two_prod(z2, z.b);
+  const float cx = __fmaf_rn(x2, x.c, __fmaf_rn(x.b, x.b, qx.lo)), cy = __fmaf_rn(y2, y.c, __fmaf_rn(y.b, y.b, qy.lo)),
+              cz = __fmaf_rn(z2, z.c, __fmaf_rn(z.b, z.b, qz.lo));
+  const df s = two_sum(px.hi, py.hi), t = two_sum(s.hi, pz.hi);
+  // the eight terms of the second order
+  const df a = two_sum(qx.hi, qy.hi), b = two_sum(a.hi, qz.hi), c = two_sum(px.lo, py.lo), d = two_sum(c.hi, pz.lo),
+           e = two_sum(s.lo, t.lo), f = two_sum(b.hi, d.hi), g = two_sum(f.hi, e.hi);
+  const float lo = __fadd_rn(__fadd_rn(__fadd_rn(cx, cy), __fadd_rn(cz, a.lo)),
+                             __fadd_rn(__fadd_rn(__fadd_rn(b.lo, c.lo), __fadd_rn(d.lo, e.lo)), __fadd_rn(f.lo, g.lo)));
+  const df n = fast_two_sum(t.hi, g.hi);
+  return tf{n.hi, n.lo, lo};
 }
 // f - x for a float f, |f| >= |x|
 __device__ __forceinline__ tf tf_rsub_f(float f, tf x) {
@@ -142,16 +168,10 @@ struct TfRadial {
   double k1, v, w, k2, k3;
 };
 template <bool LAPLACE>
-__device__ __forceinline__ TfRadial tf_radial(double r2, const TfConst& c, const float4* tab) {
-  // r2 = rho 4^q, rho in [1, 4) as three floats (its 53 bits: 24, 23 and 6)
-  const int hi = __double2hiint(r2), lo = __double2loint(r2);
-  const int ex = (hi >> 20) - 1023, q = ex >> 1, odd = ex & 1;
-  const unsigned rem = (unsigned)lo & 0x1fffffffu;
-  tf rho;
-  rho.a = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
-  const float u = __int_as_float((81 + odd) << 23);  // 2^(odd - 46)
-  rho.b = __fmul_rn(__fsub_rn(__int_as_float(0x4b000000 | (int)(rem >> 6)), 8388608.0f), u);
-  rho.c = __fmul_rn(__fsub_rn(__int_as_float(0x4b000000 | (int)(rem & 63u)), 8388608.0f), __fmul_rn(u, 0x1p-6f));
+__device__ __forceinline__ TfRadial tf_radial(tf r2, const TfConst& c, const float4* tab) {
+  // r2 = rho 4^q, rho in [1, 4)
+  const int q = ((__float_as_int(r2.a) >> 23) - 127) >> 1;
+  const tf rho = tf_scale(r2, __int_as_float((127 - 2 * q) << 23));
   // sig = 1 / sqrt(rho)
   const float y = rsqrt_approx(rho.a);
   const df p = two_prod(y, y), A = two_prod(rho.a, p.hi), B = two_prod(rho.a, p.lo), C = two_prod(rho.b, p.hi);
