@@ -91,8 +91,14 @@ __device__ __forceinline__ double warp_sum(double v) {
 __device__ __forceinline__ double warp_sum_parts(const double* part, int stride, int i, int b0, int b1) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
-#pragma unroll 4
-  for (int b = b0 + lane; b < b1; b += 32) s += part[(size_t)b * stride + i];
+  constexpr int U = 5;  // loads in flight, the last batch filled with zeros (sum_strided)
+  for (int b = b0 + lane; b < b1; b += 32 * U) {
+    double v[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) v[q] = b + 32 * q < b1 ? part[(size_t)(b + 32 * q) * stride + i] : 0.0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) s += v[q];
+  }
   if (b1 - b0 > 8) return warp_sum(s);
   for (int o = 4; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);  // lanes 0..7 hold all of it
   return __shfl_sync(0xffffffffu, s, 0);
@@ -372,6 +378,14 @@ __global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
   chain_wait();
   chain_release();
   if (a.st[B.x].skip) return;
+  // every block reads what the Givens step needs, beside the norm: which one makes it is known
+  // at the end only, and two rounds of loads and a division would follow
+  __shared__ GivensIn in;
+  if (threadIdx.x >= kBS - 32) {
+    givens_load(a, B.x, in);
+    const double* Hc = a.H + (size_t)B.x * (a.m + 1) * a.m + (size_t)a.j * (a.m + 1);
+    for (int i = threadIdx.x - (kBS - 32); i <= a.j; i += 32) in.col[i] = Hc[i];
+  }
   const double2 v = step_norm(a.part1, S);
   step_next<kBS, FUSED>(a, v.y, B, Lk);
   __shared__ int last;
@@ -382,14 +396,10 @@ __global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
   __syncthreads();
   if (!last) return;
   __threadfence();
-  if (threadIdx.x == 0) a.st[B.x].arrive = 0;
-  if (threadIdx.x >= 32) return;
-  __shared__ GivensIn in;
-  givens_load(a, B.x, in);
-  const double* Hc = a.H + (size_t)B.x * (a.m + 1) * a.m + (size_t)a.j * (a.m + 1);
-  for (int i = threadIdx.x; i <= a.j; i += 32) in.col[i] = Hc[i];
-  __syncwarp();
-  if (threadIdx.x == 0) givens_step(a, B.x, in, v.x);
+  if (threadIdx.x == 0) {
+    a.st[B.x].arrive = 0;
+    givens_step(a, B.x, in, v.x);
+  }
 }
 
 // The whole step in one launch: a cluster of kClu CTAs per system (its blocks).
