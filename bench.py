@@ -62,12 +62,12 @@ PAIR_PIPE_INSTR = 43
 # region (2 flop per FMA).
 FFMA_LANES_PER_SM_MEASURED = 3.65e13 / (152 * 1987e6)
 # ncu FMA-pipe busy fraction of the FP32 mat-vec pair kernel (symmetric variant
-# 9) on the Kirkwood workload, from profiles/k_sym_fp32_kirkwood.md
-NCU_FMA_PIPE_FRAC_FP32_KIRKWOOD = {9: 0.691}
+# 9) on the Kirkwood workload, from profiles/kernels_current_build.md
+NCU_FMA_PIPE_FRAC_FP32_KIRKWOOD = {9: 0.725}
 # DRAM bytes (read + write) per launch of the FP32 mat-vec kernel on the Kirkwood
 # workload, by variant, from one ncu capture of that variant's kernel (the
 # records and partial sums stay in L2); variants without a capture report null
-DRAM_BYTES_FP32_KIRKWOOD = {5: 1.369088e6, 9: 0.702976e6}
+DRAM_BYTES_FP32_KIRKWOOD = {5: 1.369088e6, 9: 1.691648e6}
 FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM per clock
 FP64_LANES_PER_SM = 2    # FP64 FMA lanes per SM per clock (1.25 TFLOP/s nominal at 2.07 GHz, 152 SMs)
 
@@ -861,7 +861,7 @@ def main():
                               "peak (can exceed 1 for the same reason)",
                 "ncu_fma_pipe_frac": ncu_pipe,
                 "ncu_note": "FMA-pipe busy fraction of this kernel from one ncu capture "
-                            "(profiles/k_sym_fp32_kirkwood.md): how busy the pipe actually is",
+                            "(profiles/kernels_current_build.md): how busy the pipe actually is",
                 "pairs_per_launch": pairs_launch, "sms": nsm, "sm_mhz": f_mhz,
                 "avg_launch_ms": avg_ms, "launches": cnt, "effective_launches": min(cnt, eff),
                 "kernel_ms": {k: v[1] for k, v in timers.items() if v[0]},

@@ -795,8 +795,11 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
   // / 26.9 / 24.7; 2500 47.2 / 37.0 / 41.1; 20480 367 / 358 / 387; 40000 1253 /
   // 1283 / 1342; 65537 3196 / 3229 / 3702.
   int shape = variant;
-  if (variant == 2) shape = L.max_n < 1536 ? 3 : L.max_n < 32768 ? 1 : 2;
   static const int kT[4] = {512, 512, 1024, 256};
+  if (variant == 2) {
+    shape = L.max_n < 1536 ? 3 : L.max_n < 32768 ? 1 : 2;
+    if (!sym_fits(L, kT[shape])) shape = 2;  // a large batch: fewer partial sums
+  }
   PairConst<float> c = c0;
   bool lap = false;
   if (!sym_fits(L, kT[shape]) || !sym_form(kappa, c, lap)) return false;
@@ -840,7 +843,7 @@ bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c0, d
                   const double* u, double* y, double dphi, double dpsi, const int* skip, int skip_stride) {
   PairConst<double> c = c0;
   bool lap = false;
-  const bool small = L.max_n <= kSym64Small;
+  const bool small = L.max_n <= kSym64Small && sym_fits(L, 64);  // else fewer partial sums
   if (!sym_fits(L, small ? 64 : 256) || !sym_form(kappa, c, lap)) return false;
   TfConst t;
   t.em1 = tf_from_double(c.eps - 1.0), t.eps = tf_from_double(c.eps);
