@@ -47,8 +47,6 @@ struct df {
   float hi, lo;
 };
 
-__device__ __forceinline__ df df_make(float hi, float lo) { return df{hi, lo}; }
-
 __device__ __forceinline__ df two_sum(float a, float b) {
   float s = __fadd_rn(a, b);
   float bb = __fsub_rn(s, a);
@@ -74,12 +72,6 @@ __device__ __forceinline__ df df_add(df x, df y) {
 }
 __device__ __forceinline__ df df_neg(df x) { return df{-x.hi, -x.lo}; }
 __device__ __forceinline__ df df_sub(df x, df y) { return df_add(x, df_neg(y)); }
-// x + f for a float f
-__device__ __forceinline__ df df_add_f(df x, float f) {
-  df s = two_sum(x.hi, f);
-  s.lo = __fadd_rn(s.lo, x.lo);
-  return fast_two_sum(s.hi, s.lo);
-}
 // Products are left unnormalised: the trailing part (the exact error of the
 // leading product plus the cross terms) is below a few ulp of the leading
 // part, so the next product or sum takes it as it is at no loss of accuracy

@@ -30,11 +30,6 @@ __device__ __forceinline__ float f2_sum(f2 a) {
   f2_get(a, lo, hi);
   return lo + hi;
 }
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-  f2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
 __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
   f2 r;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));

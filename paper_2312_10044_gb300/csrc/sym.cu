@@ -54,6 +54,7 @@ constexpr double kInv4PiS = 1.0 / (4.0 * kPi);
 // j side of one source over a warp.
 
 // FP64, one target per pack.  Record (a, alpha, n.x, n.y), (n.z, x.h, x.l), (x.m),
+// (n as integers, fix2),
 // where (a, alpha) = (ds psi, ds phi) for A u and (wphi, wpsi) for A^T w and the
 // position is in three floats on the surface's grid (df_pos), 9 of them from the
 // second vector's second value on.  LAPLACE: the kappa = 0 form (pair.cuh);
@@ -63,11 +64,12 @@ struct Sym64Policy {
   using V4 = double4_32a;
   using PT = double;  // partial sums are stored in this type
   static constexpr bool SCALED = !LAPLACE;
-  static constexpr int RW = 3, PACK = 1, UNROLL = 1;
+  static constexpr int RW = 4, PACK = 1, UNROLL = 1;
   static constexpr bool CHUNKED = false;
   struct Tgt {
     df_pos x[3];
     double a, n[3], al;
+    fix2 f[3];  // the normal as integers
   };
   using Src = Tgt;
   struct Acc {
@@ -89,15 +91,17 @@ struct Sym64Policy {
     for (int j = threadIdx.x; j < kTfTab; j += blockDim.x) exp_tab()[j] = make_float4(t2[j].x, t2[j].y, t3[j], 0.f);
   }
   __device__ static void load(const V4* rec, const int* i, Tgt& t) {
-    const V4* r = rec + 3 * (size_t)i[0];
-    unpack(r[0], r[1], r[2], t);
+    const V4* r = rec + 4 * (size_t)i[0];
+    unpack(r[0], r[1], r[2], r[3], t);
   }
   // record q of a chunk staged as planes (vector r of record q at sh[r * CH + q])
   template <int CH>
-  __device__ static void load_src(const V4* sh, int q, Src& e) { unpack(sh[q], sh[CH + q], sh[2 * CH + q], e); }
+  __device__ static void load_src(const V4* sh, int q, Src& e) { unpack(sh[q], sh[CH + q], sh[2 * CH + q], sh[3 * CH + q], e); }
   static __device__ float2 floats(double v) { return make_float2(__int_as_float(__double2loint(v)), __int_as_float(__double2hiint(v))); }
   static __device__ double pair_of(float a, float b) { return __hiloint2double(__float_as_int(b), __float_as_int(a)); }
-  __device__ static void unpack(const V4& A, const V4& B, const V4& C, Tgt& e) {
+  static __device__ fix2 ints(double v) { return fix2{__double2loint(v), __double2hiint(v)}; }
+  __device__ static void unpack(const V4& A, const V4& B, const V4& C, const V4& F, Tgt& e) {
+    e.f[0] = ints(F.x), e.f[1] = ints(F.y), e.f[2] = ints(F.z);
     e.a = A.x, e.al = A.y, e.n[0] = A.z, e.n[1] = A.w, e.n[2] = B.x;
     const float2 p = floats(B.y), q = floats(B.z), r = floats(B.w), s = floats(C.x);
     e.x[0] = df_pos{p.x, q.y, s.x}, e.x[1] = df_pos{p.y, r.x, s.y}, e.x[2] = df_pos{q.x, r.y, floats(C.y).x};
@@ -110,7 +114,8 @@ struct Sym64Policy {
     TfRadial R = tf_radial<LAPLACE>(tf_norm2(d[0], d[1], d[2]), g.c, LAPLACE ? nullptr : exp_tab());
     const double dx = tf_to_double(d[0], 0), dy = tf_to_double(d[1], 0), dz = tf_to_double(d[2], 0);
     if (MASK && masked[0]) R.k1 = R.v = R.w = R.k2 = R.k3 = 0.0;
-    sym_pair64<TRANS, LAPLACE>(dx, dy, dz, t.n, t.a, t.al, sj.n, sj.a, sj.al, R, ti.p, ti.q, tj.p, tj.q);
+    const double cij = LAPLACE ? 0.0 : fix2_dot(t.f, sj.f);
+    sym_pair64<TRANS, LAPLACE>(dx, dy, dz, cij, t.n, t.a, t.al, sj.n, sj.a, sj.al, R, ti.p, ti.q, tj.p, tj.q);
   }
   __device__ static void flush(Acc&, const Acc&) {}
   __device__ static Red reduced(const Acc& v) { return v; }
@@ -124,7 +129,7 @@ struct Sym64Policy {
   __device__ static void pad(V4* sh, int q) {
     sh[q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
     sh[CH + q] = make_double4_32a(0.0, pair_of(1e4f, 1e4f), pair_of(1e4f, 0.f), 0.0);
-    sh[2 * CH + q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    sh[2 * CH + q] = sh[3 * CH + q] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
   }
   __device__ static PT out(double v) { return v; }
   __device__ static void store(PT* p, int T, const int* o, const bool* in, const Acc& v) {
@@ -423,10 +428,15 @@ __global__ void k_pack_sym64(const int4* __restrict__ lay, bool transpose, const
   const df_pos x0 = df_split_grid(sigma * g.x, grid), x1 = df_split_grid(sigma * g.y, grid),
                x2 = df_split_grid(sigma * g.z, grid);
   auto two = [](float p, float q) { return __hiloint2double(__float_as_int(q), __float_as_int(p)); };
-  double4_32a* o = rec + 3 * (size_t)(L.z / 2 + j);
+  auto fix = [](double n) {
+    const fix2 f = fix2_from_double(n);
+    return __hiloint2double(f.l, f.h);
+  };
+  double4_32a* o = rec + 4 * (size_t)(L.z / 2 + j);
   o[0] = make_double4_32a(a, al, v.x, v.y);
   o[1] = make_double4_32a(v.z, two(x0.h, x1.h), two(x2.h, x0.l), two(x1.l, x2.l));
   o[2] = make_double4_32a(two(x0.m, x1.m), two(x2.m, 0.f), 0.0, 0.0);
+  o[3] = make_double4_32a(fix(v.x), fix(v.y), fix(v.z), 0.0);
 }
 
 // every value twice, with the negated fields (Sym32Policy)
@@ -834,8 +844,8 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
 
 // FP64 shapes: tiles of 64 targets in CTAs of 64 threads up to 32768 elements,
 // tiles and CTAs of 256 above.  Small tiles leave less of the diagonal masked
-// and more, shorter work items (N = 320 56 against 142 us, 1000 106 / 214, 7001
-// 1155 / 1288); from N = 20000 on both take the same time (9.2 ms), and
+// and more, shorter work items (N = 320 60 against 135 us, 1000 107 / 198, 7001
+// 1062 / 1167, 20000 8330 / 8490), and
 // the j-side partials (8 n^2 / T bytes: 134 MB at 32768 with T = 64) would only grow.
 constexpr int kSym64Small = 32768;
 

@@ -22,14 +22,15 @@
 // The differences of the coordinates and r2 are taken in the same arithmetic, and
 // the differences assembled for the FP64 dot products: with r2 from FP64
 // differences the error of a mat-vec was FP64's (4.7e-16 at N = 8000), now it
-// is a quarter of it.
+// is a quarter of it.  The product of the normals is an integer one.
 //
-// About 930 FP32 and integer instructions a pair, which run beside the pair's 24
-// FP64 operations (as long as 1536) and mostly hide behind them: 21.8 of the 24.3
-// billion pairs a second that 2 lanes of 152 SMs allow.  N = 7001 3.65 -> 1.16
-// ms, N = 33000 65.9 -> 25.0 ms a mat-vec, where CUDA's rsqrt and exp and the
+// About 1000 FP32 and integer instructions a pair, which run beside the pair's 21
+// FP64 operations (as long as 1344) and mostly hide behind them: 23.6 of the 27.7
+// billion pairs a second that 2 lanes of 152 SMs allow.  N = 7001 3.65 -> 1.06
+// ms, N = 33000 65.9 -> 23.1 ms a mat-vec, where CUDA's rsqrt and exp and the
 // chain after them were 57 of 87 FP64 operations (1.36 and 29.6 ms with the
-// differences and r2, six more operations, in FP64).
+// differences, r2 and the normals' product, nine more operations, in FP64; 1.16
+// and 25.0 ms with the last alone).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -127,6 +128,30 @@ __host__ __device__ __forceinline__ tf tf_from_double(double v) {
   return tf{a, b, (float)(v - (double)a - (double)b)};
 }
 
+// A unit normal's component as two integers, n = h 2^-27 + l 2^-54 (|l| <= 2^26).
+struct fix2 {
+  int h, l;
+};
+__device__ __forceinline__ fix2 fix2_from_double(double n) {
+  const int h = __double2int_rn(n * 0x1p27);
+  return fix2{h, __double2int_rn((n - h * 0x1p-27) * 0x1p54)};
+}
+// n_i . n_j in FP64 by integer multiply-adds (three FP64 operations are as long
+// as 192 instructions): exact products to 2^-54, the last rounded away (below 2^-55).
+__device__ __forceinline__ double fix2_dot(const fix2* a, const fix2* b) {
+  const long long s1 = (long long)a[0].h * b[0].h + (long long)a[1].h * b[1].h + (long long)a[2].h * b[2].h;
+  const long long s2 = (long long)a[0].h * b[0].l + (long long)a[0].l * b[0].h + (long long)a[1].h * b[1].l +
+                       (long long)a[1].l * b[1].h + (long long)a[2].h * b[2].l + (long long)a[2].l * b[2].h;
+  const long long t = s1 + ((s2 + (1ll << 26)) >> 27);  // in units of 2^-54, |t| below 2^55
+  const unsigned long long u = (unsigned long long)(t < 0 ? -t : t);
+  const int z = __clzll((long long)u);
+  const unsigned long long m = u << z;                          // bit 63 set
+  unsigned long long v = (m >> 11) + ((m >> 10) & 1ull);        // rounded to 53 bits
+  v += (unsigned long long)(1031 - z) << 52;                    // the implicit bit adds one to the exponent
+  if (u == 0) v = 0;
+  return __longlong_as_double((long long)(v | ((unsigned long long)t & 0x8000000000000000ull)));
+}
+
 constexpr int kTfTab = kExpTab;
 // ln2/1024 in three floats and 1024/ln2
 constexpr float kTfL1 = 0x1.62e43p-11f, kTfL2 = -0x1.05c61p-39f, kTfL3 = -0x1.950d88p-64f, kTfInvL = 0x1.715476p+10f;
@@ -208,11 +233,11 @@ __device__ __forceinline__ TfRadial tf_radial(tf r2, const TfConst& c, const flo
 }
 
 // Both directions of one unordered pair (pair.cuh) from its coefficients R (0
-// for a masked pair), 23 FP64 operations: U = (t - 1) s^3 c_ij - (w - 3) s^5 c_i c_j.
+// for a masked pair) and c_ij, 21 FP64 operations: U = (t - 1) s^3 c_ij - (w - 3) s^5 c_i c_j.
 template <bool TRANS, bool LAPLACE>
-__device__ __forceinline__ void sym_pair64(double dx, double dy, double dz, const double* nt, double at, double alt,
-                                           const double* ns, double as, double als, const TfRadial& R, double& Pt,
-                                           double& Qt, double& Ps, double& Qs) {
+__device__ __forceinline__ void sym_pair64(double dx, double dy, double dz, double cij, const double* nt, double at,
+                                           double alt, const double* ns, double as, double als, const TfRadial& R,
+                                           double& Pt, double& Qt, double& Ps, double& Qs) {
   const double ci = nt[0] * dx + nt[1] * dy + nt[2] * dz;
   const double cj = ns[0] * dx + ns[1] * dy + ns[2] * dz;
   if constexpr (LAPLACE) {
@@ -228,7 +253,6 @@ __device__ __forceinline__ void sym_pair64(double dx, double dy, double dz, cons
       Qs = (R.k3 * ci) * alt + Qs;
     }
   } else {
-    const double cij = nt[0] * ns[0] + nt[1] * ns[1] + nt[2] * ns[2];
     const double U = R.v * cij - R.w * (ci * cj);
     if (!TRANS) {
       Pt = (R.k2 * cj) * als + (R.k1 * as + Pt);
