@@ -493,12 +493,20 @@ __global__ void __launch_bounds__(64) k_lsq(int m, const double* __restrict__ H,
   const int k = S.k;
   if (!S.active || k == 0) return;
   const int m1 = m + 1;
-  __shared__ double c_[kMaxRestart], s_[kMaxRestart], r_[kMaxRestart + 1], z_[kMaxRestart + 1];
+  __shared__ double c_[kMaxRestart], s_[kMaxRestart], r_[kMaxRestart + 1], z_[kMaxRestart + 1], d_[kMaxRestart];
   const double* Hs = H + (size_t)sys * m1 * m;
   for (int i = threadIdx.x; i <= k; i += 64) {
-    if (i < k) c_[i] = cs[(size_t)sys * m + i], s_[i] = sn[(size_t)sys * m + i];
+    // the reciprocals of the diagonal side by side: a division in each step of the
+    // back substitution was most of this kernel
+    if (i < k) c_[i] = cs[(size_t)sys * m + i], s_[i] = sn[(size_t)sys * m + i], d_[i] = 1.0 / Hs[(size_t)i * m1 + i];
     r_[i] = g[(size_t)sys * m1 + i];
   }
+  // R as well, where it is small: each step would wait for its column from L2
+  constexpr int kR = 32;
+  __shared__ double R_[kR * kR];
+  const bool small = k <= kR;
+  if (small)
+    for (int t = threadIdx.x; t < k * k; t += 64) R_[t / k * kR + t % k] = Hs[(size_t)(t / k) * m1 + t % k];
   __syncthreads();
   const double gk = r_[k], beta = fabs(gk);
   if (threadIdx.x >= 32) {  // second warp: the restart coefficients
@@ -516,9 +524,10 @@ __global__ void __launch_bounds__(64) k_lsq(int m, const double* __restrict__ H,
     for (int i = threadIdx.x - 32; i <= k; i += 32) z[(size_t)sys * m1 + i] = z_[i];
   } else {  // first warp: back substitution by columns, the solved entries in r_
     for (int i = k - 1; i >= 0; --i) {
-      const double yi = r_[i] / Hs[(size_t)i * m1 + i];
+      const double yi = r_[i] * d_[i];
+      const double* col = small ? R_ + i * kR : Hs + (size_t)i * m1;
       __syncwarp();
-      for (int l = threadIdx.x; l < i; l += 32) r_[l] -= Hs[(size_t)i * m1 + l] * yi;
+      for (int l = threadIdx.x; l < i; l += 32) r_[l] -= col[l] * yi;
       if (threadIdx.x == 0) y[(size_t)sys * m + i] = yi;
       __syncwarp();
     }
