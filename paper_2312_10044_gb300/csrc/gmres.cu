@@ -788,12 +788,14 @@ double2 precond_factors(const bipb_medium& m) {
 // has two FP64 lanes per SM, so eight SMs make the (j + 1) 4n multiply-adds of a
 // step as fast as the three kernels' launches and block reductions take only
 // for small systems, and only while every cluster has its SMs.  With the fused
-// FP32 mat-vec they also sum its partial sums.  Whole solves, cluster /
-// kernels: one system of 320 elements 1.41 / 1.74 ms, 1280 1.55 / 1.84, 2560 2.25 /
-// 2.26, 4000 3.24 / 3.31, 5120 4.20 / 3.56; 12 of 320 .. 5120, fused, 2.66 / 2.55; 16
-// charge sets on 5120 elements, not fused, 7.06 / 7.23 ms.
+// FP32 mat-vec they also sum its partial sums, one unknown per thread up to 2048
+// elements.  Whole solves, cluster / kernels: one system of 320 elements 1.40 /
+// 1.72 ms, 1280 1.55 / 1.76, 2560 2.24 / 2.15, 5120 4.20 / 3.48; 12 of 320 .. 5120,
+// fused, 2.66 / 2.55; 16 charge sets on 5120 elements, not fused, 7.05 / 7.23 ms.
+// (Clusters of 16, one system: 2560 elements 1.97 ms, 4000 3.17 / 3.25, 5120 4.1;
+// four of up to 3000 1.23 / 1.19.)
 bool cluster_step(const SysLayout& L, bool fused) {
-  return L.max_n <= (fused ? 2560 : 5120) && L.K * kClu <= 160;
+  return L.max_n <= (fused ? 2048 : 5120) && L.K * kClu <= 160;
 }
 
 void issue_cycle(Surface* s, const SysLayout& L, GmresWork* w, const bipb_medium& med, int precision,

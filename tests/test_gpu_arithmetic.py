@@ -106,7 +106,7 @@ def test_fp32_symmetric_shapes_small_and_ragged(bipb, orc, n, transpose):
                 assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max(), (variant, kappa)
 
 
-@pytest.mark.parametrize("n,sets,precond", [(2, 1, 0), (37, 20, 1), (37, 21, 1), (2560, 1, 0), (2561, 1, 0), (2561, 2, 1)])
+@pytest.mark.parametrize("n,sets,precond", [(2, 1, 0), (37, 20, 1), (37, 21, 1), (2048, 1, 0), (2049, 1, 0), (2560, 1, 0), (2561, 2, 1)])
 def test_krylov_step_as_cluster_and_as_kernels(bipb, orc, n, sets, precond):
     """The Arnoldi step as one cluster launch per system (small systems, up to 20 of
     them) and as three kernels, on both sides of the lines between them, with the
