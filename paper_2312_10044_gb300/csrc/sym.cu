@@ -142,7 +142,7 @@ struct Sym64Policy {
 // results; measured), FADD and FMUL one, so a pair of 24 FFMA and 23 others
 // takes 59 cycles of a scheduler however it is issued, and the scalar form
 // waited for its loads, shuffles and MUFU calls on top (64.5).  Packed, they
-// hide behind it: N = 20480 0.387 -> 0.358 ms, N = 65537 3.43 -> 3.20 ms a
+// hide behind it: N = 20480 0.387 -> 0.351 ms, N = 65537 3.43 -> 3.15 ms a
 // mat-vec (59.7 cycles a pair).  Record, 5 float4, every value twice: (x, x, y, y),
 // (z, z, a, a), (nx, nx, ny, ny), (nz, nz, -alpha, -alpha), (f, f, 0, 0) with f
 // = -a (A u) or alpha (A^T w): packed FP32 has no negated operands, so every
@@ -801,13 +801,14 @@ bool matvec_sym32(Surface* s, const SysLayout& L, const PairConst<float>& c0, do
   // shape by size.  A tile of T targets evaluates n T / 2 masked pairs of its
   // own diagonal beside the n^2 / 2 real ones, and a small surface needs small
   // tiles to give every SM work, while the large tile shares each source load
-  // among more targets.  Whole mat-vec, us, tile 1024 / 512 / 256: N = 1280 34.9
-  // / 26.9 / 24.7; 2500 47.2 / 37.0 / 41.1; 20480 367 / 358 / 387; 40000 1253 /
-  // 1283 / 1342; 65537 3196 / 3229 / 3702.
+  // among more targets.  Whole mat-vec, us, tile 1024 / 512 / 256: N = 1280 28.8
+  // / 25.6 / 22; 2500 38.3 / 29.5 / 25.7; 3500 43.1 / 38.1 / 34.9; 4200 55 / 37.0 /
+  // 39.2; 20480 358 / 351 / 356; 40000 1234 / 1196 / 1300; 46000 1574 / 1578 / 1778;
+  // 65537 3138 / 3170 / 3584.
   int shape = variant;
   static const int kT[4] = {512, 512, 1024, 256};
   if (variant == 2) {
-    shape = L.max_n < 1536 ? 3 : L.max_n < 32768 ? 1 : 2;
+    shape = L.max_n < 4096 ? 3 : L.max_n < 45056 ? 1 : 2;
     if (!sym_fits(L, kT[shape])) shape = 2;  // a large batch: fewer partial sums
   }
   PairConst<float> c = c0;

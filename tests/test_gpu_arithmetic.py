@@ -84,7 +84,7 @@ def test_double_float_matvec_grid_scales_with_the_surface(bipb, orc, scale):
                 np.testing.assert_allclose(y[k], ref, rtol=0, atol=2e-12 * np.abs(ref).max(), err_msg=f"{transpose} {k}")
 
 
-@pytest.mark.parametrize("n", [2, 3, 31, 33, 255, 257, 513, 1279, 1535, 1536, 1537])
+@pytest.mark.parametrize("n", [2, 3, 31, 33, 255, 257, 513, 1279, 1536, 1537, 4095, 4096])
 @pytest.mark.parametrize("transpose", [False, True])
 def test_fp32_symmetric_shapes_small_and_ragged(bipb, orc, n, transpose):
     """Every shape of the packed symmetric FP32 mat-vec (and the default's choice by
