@@ -407,9 +407,6 @@ __global__ void __launch_bounds__(kBS) k_normalize(StepArgs a) {
 // w and H visible to the others.
 constexpr int kClu = 8;      // CTAs of a cluster (the portable size)
 constexpr int kCluNT = 512;  // threads of each
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 template <bool CGS2, bool FUSED>
 __global__ void __cluster_dims__(kClu, 1, 1) __launch_bounds__(kCluNT) k_step(StepArgs a) {
   const int4 B = a.blk[blockIdx.x], S = a.sysb[B.x], Lk = a.lay[B.x];

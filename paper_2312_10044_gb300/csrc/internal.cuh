@@ -54,6 +54,24 @@ struct Error : std::runtime_error {
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The two halves of a cluster barrier (every thread of the cluster executes both).
+// Shared memory of another CTA may be written only once that CTA is known to run: a
+// kernel that does so arrives at entry and waits just before its first remote
+// store, so that the wait hides behind its own work; the barrier after the
+// stores is another one.
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();  // the aligned forms want whole warps
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+
 template <typename... KArgs, typename... Args>
 void launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                     Args&&... args) {

@@ -697,6 +697,7 @@ __global__ void __cluster_dims__(kReacClu, 1, 1) __launch_bounds__(32 * kReacWar
     k_reduce_reaction(const int4* __restrict__ tab, const int4* __restrict__ lay, const double* __restrict__ part,
                       const double4_32a* __restrict__ chg, double* __restrict__ phi_reac, double* __restrict__ e_out) {
   __shared__ double red[kReacWarps][32], sums[kReacClu];
+  cluster_arrive();
   const auto cluster = cooperative_groups::this_cluster();
   const int k = blockIdx.x / kReacClu, rank = blockIdx.x % kReacClu;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -719,11 +720,12 @@ __global__ void __cluster_dims__(kReacClu, 1, 1) __launch_bounds__(32 * kReacWar
       local += chg[c0 + q].w * acc;
     }
   }
+  cluster_wait();  // block 0 runs: its shared memory may be written
   if (warp == 0) {
     for (int o = 16; o > 0; o >>= 1) local += __shfl_down_sync(0xffffffffu, local, o);
     if (lane == 0) *cluster.map_shared_rank(sums + rank, 0) = local;
   }
-  cluster.sync();
+  cluster_sync();
   if (rank == 0 && threadIdx.x == 0 && e_out) {
     double t = sums[0];
     for (int r = 1; r < kReacClu; ++r) t += sums[r];

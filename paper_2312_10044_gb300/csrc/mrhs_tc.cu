@@ -136,6 +136,7 @@ constexpr int kMaxClu = 4;
 __global__ void __cluster_dims__(kMaxClu, 1, 1) __launch_bounds__(1024) k_colmax_u(int n, const double* __restrict__ u,
                                                    const int2* __restrict__ srcexp, int* __restrict__ colmax) {
   __shared__ int red[32], parts[kMaxClu];
+  cluster_arrive();
   chain_wait();
   chain_release();
   const auto cluster = cooperative_groups::this_cluster();
@@ -157,11 +158,12 @@ __global__ void __cluster_dims__(kMaxClu, 1, 1) __launch_bounds__(1024) k_colmax
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
+  cluster_wait();  // block 0 runs: its shared memory may be written
   if (threadIdx.x < 32) {
     m = __reduce_max_sync(0xffffffffu, red[threadIdx.x]);
     if (threadIdx.x == 0) *cluster.map_shared_rank(parts + rank, 0) = m;
   }
-  cluster.sync();
+  cluster_sync();
   if (rank == 0 && threadIdx.x == 0) {
 #pragma unroll
     for (int r = 0; r < kMaxClu; ++r) m = max(m, parts[r]);
