@@ -251,8 +251,9 @@ ItemPlan* mrhs_df_plan(Surface* s, int n, int G, int slots, int* S_out) {
 // pair on the CUDA cores (FP32 pipe 60 % busy, tensor pipe 36 %, under the
 // generation).  At N = 20001 and 64 right-hand sides a pass takes 6.83 ms
 // (8.72 with unscaled, unfused df64 blocks and digit-by-digit rounding), and
-// a first pass in a medium 7.5 ms (18.0 when one thread per target found the
-// row scales in df64).
+// a first pass in a medium 7.96 ms (18.0 when one thread per target found the
+// row scales in df64, 7.60 with plain FP32 values of FP32 centroids, which
+// missed the largest value of rows with a close pair).
 namespace tcx {
 
 constexpr int kRHS = 64;                        // right-hand sides per CTA (all of a launch)
@@ -315,7 +316,8 @@ __device__ __forceinline__ uint32_t fields(uint32_t x, uint32_t mask, uint32_t o
   asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(off));
   return r;
 }
-// Two values (df64, normalised, below 128 in magnitude) as seven balanced
+// Two values (df64, normalised, below 128 in magnitude: from 256 on the leading
+// digit's field wraps) as seven balanced
 // base-128 digits each, in FP16 pairs (value 0 in the low half): out[k] holds
 // digit k, value = sum_k d_k 128^-k up to 2^-43.  Added to 1.5 2^23 grid units,
 // a float shows its multiple of the grid in its mantissa bits, so three
@@ -347,35 +349,80 @@ __device__ __forceinline__ void digits7_pair(df a, df b, uint32_t* out) {
   out[6] = fields(__byte_perm(__float_as_uint(va), __float_as_uint(vb), 0x5410), 0x01ff01ffu, 0xe480e480u);  // 128 + digit
 }
 
-// rowmax[i] = (largest |K2 ds|, |K1 ds| and largest |K4 ds|, |K3 ds|) over the
-// sources j != i of split blockIdx.y, as FP32 bits (zeroed before); FP32 values
-// (in the units of SCALED and TRANS) do, since a digit may exceed its range by
-// a factor near 1.  Split over blockIdx.y: one thread per target alone left the
-// chip idle (n / 128 CTAs).
+// Constants of the row maxima: eps - 1, eps, 1/eps - 1, 1/eps, kappa, -log2(e).
+struct RowConst {
+  float em1, eps, im1, inv, kappa, nl2e;
+};
+// The largest magnitudes of one pair's kernel block in its phi and its psi row
+// (df_kernel_block's values for r0 = r1 = 1), in FP32 and rounded up: never below the
+// df64 values, and above them by 2^-15 at most where no sum cancels.  A row's maximum may be
+// that of a pair of close elements, so nothing here may lose digits for them: the
+// difference comes from the grid coordinates (exact but for the last rounding; FP32
+// centroids shift n.d of a pair 0.01 A apart on a sphere of 20 A by all of its size), 1 - e and 1 - t
+// of a small kappa r from their series, and what rounding can add to n.d (below
+// 2^-21 r) and to the cancelling sums is added.  1/r has no cap, as in the df64 block.
 template <bool SCALED, bool TRANS>
-__global__ void __launch_bounds__(128) k_tcx_rowmax(int n, const float4* __restrict__ tgt32, PairConst<float> c,
+__device__ __forceinline__ void row_bound(const df_pos* xi, const float* ni, const df_pos* xj, const float* nj,
+                                          float area, const RowConst& c, float& b0, float& b1) {
+  float d[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    d[k] = __fadd_rn(__fadd_rn(__fsub_rn(xi[k].h, xj[k].h), __fsub_rn(xi[k].l, xj[k].l)), __fsub_rn(xi[k].m, xj[k].m));
+  const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+  const float s = rsqrt_approx(r2), r = r2 * s;
+  const float x = SCALED ? r : r * c.kappa;
+  const float e = ex2_approx(x * c.nl2e);
+  float ome = 1.f - e, omt = ome - e * x;  // 1 - e, 1 - t
+  if (x < 0.25f) {  // sum (-1)^(k+1) x^k / k! and sum (-1)^k (k - 1) x^k / k!, to 3e-6 of themselves
+    ome = x * (1.f + x * (-0.5f + x * (1.f / 6 + x * (-1.f / 24 + x * (1.f / 120)))));
+    omt = x * x * (0.5f + x * (-1.f / 3 + x * (1.f / 8 + x * (-1.f / 30 + x * (1.f / 144)))));
+  }
+  const float ci = ni[0] * d[0] + ni[1] * d[1] + ni[2] * d[2], cj = nj[0] * d[0] + nj[1] * d[1] + nj[2] * d[2];
+  const float cij = ni[0] * nj[0] + ni[1] * nj[1] + ni[2] * nj[2];
+  const float s2 = s * s, sa = TRANS ? s : s * area, s3 = s2 * sa, s3k = SCALED ? s3 * c.kappa : s3;
+  const float w = (SCALED ? e : e * (c.kappa * c.kappa)) - 3.f * (omt * s2);  // (w - 3) s^2
+  const float bi = fmaf(r, 0x1p-21f, fabsf(ci)), bj = fmaf(r, 0x1p-21f, fabsf(cj));
+  const float k1 = ome * sa;
+  const float k4 = fmaf(omt, 0x1p-15f, fabsf(omt * cij + w * (ci * cj))) * s3k;
+  const float et1 = fmaf(fabsf(c.em1) + c.eps * omt, 0x1p-17f, fabsf(c.em1 - c.eps * omt));
+  const float te1 = fmaf(fabsf(c.im1) + c.inv * omt, 0x1p-17f, fabsf(c.im1 - c.inv * omt));
+  if (!TRANS) {
+    b0 = fmaxf(et1 * bj * s3k, k1);
+    b1 = fmaxf(k4, te1 * bi * s3);
+  } else {
+    b0 = fmaxf(et1 * bi * s3, k4);
+    b1 = fmaxf(k1, te1 * bj * s3k);
+  }
+  b0 *= 1.f + 0x1p-16f, b1 *= 1.f + 0x1p-16f;
+}
+
+// rowmax[i] = (largest |K2 ds|, |K1 ds| and largest |K4 ds|, |K3 ds|; A^T likewise) over the
+// sources j != i of split blockIdx.y, as FP32 bits (zeroed before), bounded from
+// above (row_bound): digits7_pair wraps on a value four times its row's maximum.
+// Split over blockIdx.y: one thread per target alone left the chip idle (n / 128 CTAs).
+template <bool SCALED, bool TRANS>
+__global__ void __launch_bounds__(128) k_tcx_rowmax(int n, const float4* __restrict__ geo, RowConst c,
                                                     uint2* __restrict__ rowmax) {
-  __shared__ float4 sh[2 * 64];
-  const float ks = SCALED ? c.kappa : 1.f;
+  constexpr int kN = 64;  // sources staged at once
+  __shared__ float4 sh[kN * kGeo];
   const int i = blockIdx.x * 128 + threadIdx.x;
   const int ii = min(i, n - 1);
-  const float4 gi = tgt32[2 * ii], ni = tgt32[2 * ii + 1];
+  const GeoDF T = load_geo(geo + kGeo * (int64_t)ii);
+  const float ni[3] = {T.n[0].hi, T.n[1].hi, T.n[2].hi};
   float m0 = 0.f, m1 = 0.f;
   const int s0 = (int)((int64_t)blockIdx.y * n / gridDim.y), s1 = (int)((int64_t)(blockIdx.y + 1) * n / gridDim.y);
-  for (int j0 = s0; j0 < s1; j0 += 64) {
+  for (int j0 = s0; j0 < s1; j0 += kN) {
+    const int cnt = min(kN, s1 - j0);
     __syncthreads();
-    sh[threadIdx.x] = tgt32[2 * min(j0 + (int)threadIdx.x / 2, n - 1) + (threadIdx.x & 1)];
+    for (int q = threadIdx.x; q < kGeo * cnt; q += 128) sh[q] = geo[kGeo * (int64_t)j0 + q];
     __syncthreads();
-    const int cnt = min(64, s1 - j0);
+#pragma unroll 2
     for (int q = 0; q < cnt; ++q) {
-      const float4 g = sh[2 * q];
-      float v[4];
-      kernel_block<SCALED, TRANS>(ks * gi.x, ks * gi.y, ks * gi.z, ni.x, ni.y, ni.z,
-                                  make_float4(ks * g.x, ks * g.y, ks * g.z, TRANS ? 1.f : g.w), sh[2 * q + 1],
-                                  j0 + q == ii, c, v);
-      // the phi (A^T: psi) column takes kappa, as in df_kernel_block
-      m0 = fmaxf(m0, fmaxf(fabsf(v[0]) * (TRANS ? 1.f : ks), fabsf(v[1]) * (TRANS ? ks : 1.f)));
-      m1 = fmaxf(m1, fmaxf(fabsf(v[2]) * (TRANS ? 1.f : ks), fabsf(v[3]) * (TRANS ? ks : 1.f)));
+      const GeoDF S = load_geo(sh + kGeo * q);
+      const float nj[3] = {S.n[0].hi, S.n[1].hi, S.n[2].hi};
+      float b0, b1;
+      row_bound<SCALED, TRANS>(T.x, ni, S.x, nj, S.a.hi, c, b0, b1);
+      if (j0 + q != ii) m0 = fmaxf(m0, b0), m1 = fmaxf(m1, b1);
     }
   }
   if (i < n) {
@@ -760,21 +807,19 @@ int launch_tcx(Surface* s, int n, int nb, bool transpose, const double* ub, cons
   if (s->alloc_gen != gen0 || s->tcx_n[dir] != n || key[0] != c.eps.hi || key[1] != c.eps.lo ||
       key[2] != c.kappa.hi || key[3] != c.kappa.lo) {
     BIPB_CUDA(cudaMemsetAsync(rowexp, 0, (size_t)n * sizeof(int2), s->stream));
-    PairConst<float> pc;
-    pc.eps = c.eps.hi, pc.inveps = c.inveps.hi, pc.kappa = c.kappa.hi;
-    pc.nkl2e = sc.scaled ? -1.4426950408889634f : (float)(-(double)c.kappa.hi * 1.4426950408889634);
-    pc.smax = sc.scaled ? (float)(kSMaxD / sc.sigma) : kSMaxF;
+    const double eps = (double)c.eps.hi + (double)c.eps.lo, inv = (double)c.inveps.hi + (double)c.inveps.lo;
+    const tcx::RowConst rc{(float)(eps - 1.0), (float)eps, (float)(inv - 1.0), (float)inv, c.kappa.hi, -1.4426950408889634f};
     const int tiles = (n + 127) / 128;
     const dim3 grid(tiles, std::min((n + 255) / 256, std::max(1, (16 * s->num_sms + tiles - 1) / tiles)));
     auto* rm = reinterpret_cast<uint2*>(rowexp);
     if (sc.scaled && transpose)
-      tcx::k_tcx_rowmax<true, true><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+      tcx::k_tcx_rowmax<true, true><<<grid, 128, 0, s->stream>>>(n, s->geodf.p, rc, rm);
     else if (sc.scaled)
-      tcx::k_tcx_rowmax<true, false><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+      tcx::k_tcx_rowmax<true, false><<<grid, 128, 0, s->stream>>>(n, s->geodf.p, rc, rm);
     else if (transpose)
-      tcx::k_tcx_rowmax<false, true><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+      tcx::k_tcx_rowmax<false, true><<<grid, 128, 0, s->stream>>>(n, s->geodf.p, rc, rm);
     else
-      tcx::k_tcx_rowmax<false, false><<<grid, 128, 0, s->stream>>>(n, s->tgt32.p, pc, rm);
+      tcx::k_tcx_rowmax<false, false><<<grid, 128, 0, s->stream>>>(n, s->geodf.p, rc, rm);
     BIPB_LAUNCHED(s);
     tcx::k_tcx_rowexp<<<tiles, 128, 0, s->stream>>>(n, rowexp);
     BIPB_LAUNCHED(s);

@@ -1,0 +1,90 @@
+"""Surfaces with pairs of elements far closer than a mesh has them, against the FP64 oracle.
+
+Centroids are accepted as long as their FP32 copies differ, so no operator may lose a
+pair because its distance is near the rounding of FP32 coordinates.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def bipb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2312_10044_gb300.build import build
+
+    build()
+    import paper_2312_10044_gb300 as b
+
+    b.load_library()
+    return b
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+
+    return oracle
+
+
+def _dev(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def _paired_sphere(radius, gap, tangent, n_pairs=40, seed=3):
+    """A sphere of 320 elements, n_pairs of which get a neighbour `gap` away, along the
+    sphere or in any direction; the neighbours' elements come last."""
+    p = synth.kirkwood_problem(level=2)
+    f = radius / np.linalg.norm(p.centroids, axis=1).mean()
+    c, a = p.centroids * f, p.areas * f * f
+    nv = c / np.linalg.norm(c, axis=1, keepdims=True)
+    rng = np.random.default_rng(seed)
+    at = rng.choice(p.n, n_pairs, replace=False)
+    d = rng.standard_normal((n_pairs, 3))
+    if tangent:
+        d -= np.sum(d * nv[at], axis=1, keepdims=True) * nv[at]
+    d *= gap / np.linalg.norm(d, axis=1, keepdims=True)
+    c2 = c[at] + d
+    if tangent:  # back onto the sphere: n.d is gap^2 / (2 radius)
+        c2 *= (np.linalg.norm(c[at], axis=1) / np.linalg.norm(c2, axis=1))[:, None]
+    n2 = c2 / np.linalg.norm(c2, axis=1, keepdims=True) if tangent else nv[at]
+    return np.concatenate([c, c2]), np.concatenate([nv, n2]), np.concatenate([a, a[at]])
+
+
+@pytest.mark.parametrize("n_rhs", [4, 17])
+@pytest.mark.parametrize("kappa", [0.0, 0.1257])
+@pytest.mark.parametrize("radius,gap,tangent", [(20.0, 0.02, True), (20.0, 0.01, True), (20.0, 0.003, True),
+                                                (20.0, 1e-5, False), (100.0, 1e-5, False)])
+def test_multi_rhs_double_float_close_pairs(bipb, orc, radius, gap, tangent, kappa, n_rhs):
+    """The row scales of the exact tensor-core pass hold for the largest value of each
+    row: pairs 0.02 to 1e-5 A apart, a few FP32 spacings of their coordinates.
+
+    Bound per row, with M the row's largest coefficient bound a (s + s^2 + s^3), s = 1/r:
+    1 - e and 1 - t carry an absolute error of a few 2^-47, so each coefficient one of
+    (1 + eps) M times that, and the digits one of 2^-46 of the row's largest; 2^-40 leaves
+    a factor of about sixty for the few roundings.
+    """
+    c, nv, a = _paired_sphere(radius, gap, tangent)
+    n, eps = len(a), 80.0
+    U = np.random.default_rng(n_rhs).standard_normal((n_rhs, 2 * n))
+    r = np.linalg.norm(c[:, None] - c[None], axis=2)
+    np.fill_diagonal(r, np.inf)
+    s = 1.0 / r
+    M = s + s**2 + s**3
+    with bipb.Surface(c, nv, a) as srf:
+        for transpose in (False, True):
+            Y = torch.full_like(_dev(U), float("nan"))
+            srf.matvec(_dev(U), Y, precision=bipb.DF64, transpose=transpose, med=bipb.medium(1.0, eps, kappa))
+            Y = Y.cpu().numpy()
+            rows = a * M.max(axis=1) if transpose else (M * a).max(axis=1)
+            for k in (0, n_rhs - 1):
+                ref = (orc.matvec_t if transpose else orc.matvec)(c, nv, a, eps, kappa, U[k])
+                tol = 2.0**-40 * (1.0 + eps) * np.tile(rows, 2) * np.abs(U[k]).sum() + 2.0**-40 * np.abs(ref).max()
+                worst = np.max(np.abs(Y[k] - ref) / tol)
+                assert worst < 1.0, (transpose, k, worst)
