@@ -112,7 +112,7 @@ struct Sym64Policy {
   __device__ static void pair(const Args& g, const Tgt& t, const Src& sj, const bool* masked, Acc& ti, Acc& tj) {
     const tf d[3] = {tf_diff(t.x[0], sj.x[0]), tf_diff(t.x[1], sj.x[1]), tf_diff(t.x[2], sj.x[2])};
     TfRadial R = tf_radial<LAPLACE>(tf_norm2(d[0], d[1], d[2]), g.c, LAPLACE ? nullptr : exp_tab());
-    const double dx = tf_to_double(d[0], 0), dy = tf_to_double(d[1], 0), dz = tf_to_double(d[2], 0);
+    const double dx = tf_to_double<true>(d[0], 0), dy = tf_to_double<true>(d[1], 0), dz = tf_to_double<true>(d[2], 0);
     if (MASK && masked[0]) R.k1 = R.v = R.w = R.k2 = R.k3 = 0.0;
     const double cij = LAPLACE ? 0.0 : fix2_dot(t.f, sj.f);
     sym_pair64<TRANS, LAPLACE>(dx, dy, dz, cij, t.n, t.a, t.al, sj.n, sj.a, sj.al, R, ti.p, ti.q, tj.p, tj.q);

@@ -64,11 +64,6 @@ __device__ __forceinline__ tf tf_mul_f(tf x, float f) {
 __device__ __forceinline__ tf tf_scale(tf x, float pow2) {
   return tf{__fmul_rn(x.a, pow2), __fmul_rn(x.b, pow2), __fmul_rn(x.c, pow2)};
 }
-// |a| >= |b| >= |c| with no overlap beyond half an ulp
-__device__ __forceinline__ tf tf_norm(tf x) {
-  const df s = fast_two_sum(x.a, x.b), t = fast_two_sum(s.lo, x.c);
-  return tf{s.hi, t.hi, t.lo};
-}
 // x - y, normalised where the leading parts cancel
 __device__ __forceinline__ tf tf_sub(tf x, tf y) {
   const df s = two_sum(x.a, -y.a), t = two_sum(x.b, -y.b), u = two_sum(s.lo, t.hi);
@@ -76,10 +71,14 @@ __device__ __forceinline__ tf tf_sub(tf x, tf y) {
   const df w = two_sum(v.lo, __fadd_rn(__fsub_rn(x.c, y.c), __fadd_rn(t.lo, u.lo)));
   return tf{v.hi, w.hi, w.lo};
 }
-// x - y of grid coordinates (exact but for the third part's rounding)
+// x - y of grid coordinates (exact but for the third part's rounding).  Each part
+// is zero or at least as large as the next, but where the leading ones cancel (a
+// component below 2^(c-23)) it can have so few digits that the next is above its ulp:
+// normalised, as every product below expects.
 __device__ __forceinline__ tf tf_diff(df_pos x, df_pos y) {
   const df d = fast_two_sum(__fsub_rn(x.h, y.h), __fsub_rn(x.l, y.l));
-  return tf{d.hi, d.lo, __fsub_rn(x.m, y.m)};
+  const df e = fast_two_sum(d.lo, __fsub_rn(x.m, y.m)), u = fast_two_sum(d.hi, e.hi);
+  return tf{u.hi, u.lo, e.lo};
 }
 // |d|^2
 __device__ __forceinline__ tf tf_norm2(tf x, tf y, tf z) {
@@ -106,18 +105,20 @@ __device__ __forceinline__ tf tf_rsub_f(float f, tf x) {
 
 // x 2^shift in FP64, rounded once, by integer operations (an FP64 addition
 // costs as much as 64 instructions): the leading float truncated towards zero,
-// the rest, below its ulp, rounded to the 29 bits that follow.
+// the rest, below its ulp, rounded to the 29 bits that follow.  NORMAL: |b| is at most
+// half an ulp of a.  (c may be a few ulp of b: the integer takes it with its carry or borrow.)
+template <bool NORMAL = false>
 __device__ __forceinline__ double tf_to_double(tf x, int shift) {
-  const tf n = tf_norm(x);
-  const int sgn = __float_as_int(n.a) & 0x80000000;
-  const float h = __int_as_float(__float_as_int(n.a) ^ sgn), m = __int_as_float(__float_as_int(n.b) ^ sgn),
-              l = __int_as_float(__float_as_int(n.c) ^ sgn);
+  const df n = NORMAL ? df{x.a, x.b} : fast_two_sum(x.a, x.b);
+  const int sgn = __float_as_int(n.hi) & 0x80000000;
+  const float h = __int_as_float(__float_as_int(n.hi) ^ sgn), m = __int_as_float(__float_as_int(n.lo) ^ sgn),
+              l = __int_as_float(__float_as_int(x.c) ^ sgn);
   const int hb = __float_as_int(h) - (m < 0.f ? 1 : 0);
   const df t = two_sum(__fsub_rn(h, __int_as_float(hb)), m);  // in [0, ulp)
   const float S = __int_as_float(min(306 - (hb >> 23), 254) << 23);  // 2^29 / ulp
   const int i = __float2int_rn(__fmul_rn(t.hi, S)) + __float2int_rn(__fmul_rn(__fadd_rn(t.lo, l), S));
   const unsigned lo0 = (unsigned)hb << 29, lo = lo0 + (unsigned)i;
-  // i >= 0 up to the rounding of its parts (a carry), or -1 (a borrow)
+  // i >= 0 (a carry), or below 0 by its parts' rounding or by c (a borrow)
   const int hi = (hb >> 3) + 0x38000000 + (int)((unsigned)shift << 20) + (i >= 0 ? (lo < lo0 ? 1 : 0) : (lo > lo0 ? -1 : 0));
   return hb == 0 ? 0.0 : __hiloint2double(hi | sgn, (int)lo);
 }

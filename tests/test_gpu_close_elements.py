@@ -88,3 +88,69 @@ def test_multi_rhs_double_float_close_pairs(bipb, orc, radius, gap, tangent, kap
                 tol = 2.0**-40 * (1.0 + eps) * np.tile(rows, 2) * np.abs(U[k]).sum() + 2.0**-40 * np.abs(ref).max()
                 worst = np.max(np.abs(Y[k] - ref) / tol)
                 assert worst < 1.0, (transpose, k, worst)
+
+
+def _capped_matvec(c, nv, a, eps, kappa, u, transpose):
+    """A u or A^T u with 1/r at most 1e6 (pair.cuh) in FP64, 1 - t of small kappa r from
+    its series, and per row the bound 1e-12 sum |K u|, plus 2^-54 s^3 ds |phi| in the psi
+    row (1 - t is a difference of numbers near 1) and (1 + eps) 2^-66 s^3 ds |u| (the
+    coordinates' grid: 2^-72 of 32 A and more for a difference, twice that)."""
+    n = len(a)
+    d = c[:, None, :] - c[None, :, :]
+    r2 = np.sum(d * d, axis=2)
+    with np.errstate(divide="ignore"):
+        s = np.minimum(1.0 / np.sqrt(r2), 1e6)
+    np.fill_diagonal(s, 0.0)
+    x = kappa * r2 * s
+    e = np.exp(-x)
+    omt = np.where(x < 1e-2, x * x * (0.5 - x * (1 / 3 - x * (1 / 8 - x * (1 / 30 - x / 144)))), -np.expm1(-x) - x * e)
+    ci, cj = np.einsum("ik,ijk->ij", nv, d), np.einsum("jk,ijk->ij", nv, d)
+    w = e * kappa * kappa - 3.0 * omt * s**2  # (w - 3) s^2
+    k1 = -np.expm1(-x) * s
+    k2 = ((eps - 1.0) - eps * omt) * cj * s**3
+    k3 = ((1.0 / eps - 1.0) - omt / eps) * ci * s**3
+    k4 = (-omt * (nv @ nv.T) - w * ci * cj) * s**3
+    B = np.block([[k2, k1], [k4, k3]]) * np.tile(a, 2)[None, :] / (4.0 * np.pi)
+    g = (1.0 + eps) * 2.0**-66 * s**3
+    E = np.block([[g, g], [g + 2.0**-54 * s**3, g]]) * np.tile(a, 2)[None, :] / (4.0 * np.pi)
+    if transpose:
+        B, E = B.T, E.T
+    diag = np.repeat([0.5 * (1.0 + eps), 0.5 * (1.0 + 1.0 / eps)], n)
+    return diag * u - B @ u, 1e-12 * (np.abs(B) @ np.abs(u) + diag * np.abs(u)) + E @ np.abs(u)
+
+
+def _mirrored_surface(gap, n_pairs):
+    """Elements at x and -x in turn (their mean is the origin exactly): half an
+    icosphere of 20 A and n_pairs pairs `gap` apart near the middle, where FP32 copies
+    that close differ; without pairs, one point gap / 2 from the origin, which is a
+    pair with its mirror image."""
+    p = synth.kirkwood_problem(level=1)
+    half = p.centroids[p.centroids[:, 0] > 0.0]
+    rng = np.random.default_rng(2)
+    near = 0.2 * rng.standard_normal((n_pairs, 3))
+    d = rng.standard_normal((max(n_pairs, 1), 3))
+    d *= gap / np.linalg.norm(d, axis=1, keepdims=True)
+    pts = np.concatenate([half, near, near + d] if n_pairs else [half, 0.5 * d])
+    c = np.stack([pts, -pts], axis=1).reshape(-1, 3)
+    nv = rng.standard_normal(c.shape)
+    for _ in range(2):
+        nv /= np.linalg.norm(nv, axis=1, keepdims=True)
+    return c, nv, rng.uniform(0.5, 1.5, len(c)), rng.standard_normal(2 * len(c))
+
+
+def _check_fp64(bipb, c, nv, a, u, kappa):
+    with bipb.Surface(c, nv, a) as srf:
+        for transpose in (False, True):
+            y = torch.full_like(_dev(u), float("nan"))
+            srf.matvec(_dev(u), y, precision=bipb.FP64, transpose=transpose, med=bipb.medium(1.0, 80.0, kappa))
+            ref, tol = _capped_matvec(c, nv, a, 80.0, kappa, u, transpose)
+            worst = np.max(np.abs(y.cpu().numpy() - ref) / tol)
+            assert worst < 1.0, (transpose, worst)
+
+
+@pytest.mark.parametrize("gap", [1e-2, 1e-4, 2e-6])
+@pytest.mark.parametrize("kappa", [0.0, 0.1257])
+def test_fp64_symmetric_close_pairs(bipb, gap, kappa):
+    """Differences of the coordinates whose leading parts cancel keep FP64's digits in
+    the symmetric FP64 mat-vec: components below the leading grid (4e-6 A here)."""
+    _check_fp64(bipb, *_mirrored_surface(gap, 40), kappa)
