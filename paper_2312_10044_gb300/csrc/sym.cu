@@ -859,6 +859,7 @@ bool matvec_sym64(Surface* s, const SysLayout& L, const PairConst<double>& c0, d
   TfConst t;
   t.em1 = tf_from_double(c.eps - 1.0), t.eps = tf_from_double(c.eps);
   t.im1 = tf_from_double(c.inveps - 1.0), t.inv = tf_from_double(c.inveps);
+  tf_set_cap(t, c.smax);
 #define BIPB_SYM64_RUN(TR_, LAP_, V_, NT_, CH_, MINB_)                                                          \
   run_sym<Sym64Policy<TR_, LAP_>, NT_, 1, CH_, MINB_>(s, (TR_ ? 0x300 : 0x400) + V_, TR_ ? kTMv64T : kTMv64, L, \
                                                       {t, s->exptab.p}, TR_, s->rec64, s->part64, u, y, dphi,  \

@@ -34,6 +34,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "df64.cuh"
 #include "pair.cuh"
 
@@ -156,10 +158,21 @@ __device__ __forceinline__ double fix2_dot(const fix2* a, const fix2* b) {
 constexpr int kTfTab = kExpTab;
 // ln2/1024 in three floats and 1024/ln2
 constexpr float kTfL1 = 0x1.62e43p-11f, kTfL2 = -0x1.05c61p-39f, kTfL3 = -0x1.950d88p-64f, kTfInvL = 0x1.715476p+10f;
-// constants of one launch: eps - 1, eps, 1/eps - 1, 1/eps
+// constants of one launch: eps - 1, eps, 1/eps - 1, 1/eps; the cap of 1/r (pair.cuh) in
+// the records' units, cap 2^-qcap with cap in [0.5, 1), reached below r2 = rho_cap 4^qcap
 struct TfConst {
-  tf em1, eps, im1, inv;
+  tf em1, eps, im1, inv, cap;
+  int qcap;
+  float rho_cap;
 };
+inline void tf_set_cap(TfConst& c, double smax) {
+  int e = 0;
+  double m = std::frexp(smax, &e);
+  if (-e < -40 || -e > 40) m = 0.5, e = -e < 0 ? 40 : -40;  // kappa below 1e-6 or above 1e18: not met
+  c.cap = tf_from_double(m);
+  c.qcap = -e;
+  c.rho_cap = (float)(1.0 / (m * m));
+}
 
 // exp(-x) for x >= 0 (0 above 87: below 2^-125); tab[j] = 2^(j/1024)
 __device__ __forceinline__ tf tf_exp_minus(tf x, const float4* tab) {
@@ -187,7 +200,8 @@ __device__ __forceinline__ tf tf_exp_minus(tf x, const float4* tab) {
   return tf_scale(tf{w.hi, g2.hi, __fadd_rn(T.z, __fadd_rn(g.lo, g2.lo))}, sc);
 }
 
-// The coefficients of the kappa-scaled pair (pair.cuh) of squared distance r2 > 0:
+// The coefficients of the kappa-scaled pair (pair.cuh) of squared distance r2 >= 0
+// (s = 1/r at most its cap, kappa r = r2 s: finite at r2 = 0 and where r2 leaves the FP32 range):
 //   k1 = (1 - e) s, v = (t - 1) s^3, w = (w - 3) s^5, k2 = (eps t - 1) s^3, k3 = (t / eps - 1) s^3
 // LAPLACE (e = t = 1, unscaled): k2 and k3 only.
 struct TfRadial {
@@ -195,8 +209,8 @@ struct TfRadial {
 };
 template <bool LAPLACE>
 __device__ __forceinline__ TfRadial tf_radial(tf r2, const TfConst& c, const float4* tab) {
-  // r2 = rho 4^q, rho in [1, 4)
-  const int q = ((__float_as_int(r2.a) >> 23) - 127) >> 1;
+  // r2 = rho 4^q, rho in [1, 4), or below where q is that of the cap
+  const int q = max(((__float_as_int(r2.a) >> 23) - 127) >> 1, c.qcap);
   const tf rho = tf_scale(r2, __int_as_float((127 - 2 * q) << 23));
   // sig = 1 / sqrt(rho)
   const float y = rsqrt_approx(rho.a);
@@ -207,7 +221,8 @@ __device__ __forceinline__ TfRadial tf_radial(tf r2, const TfConst& c, const flo
   const float h2 = __fsub_rn(h.lo, __fadd_rn(__fadd_rn(s1.lo, s2.lo), hl));
   const float cor = __fmaf_rn(__fmul_rn(h.hi, h.hi), __fmaf_rn(0.3125f, h.hi, 0.375f), __fmul_rn(0.5f, h2));
   const df g = two_prod(y, __fmul_rn(0.5f, h.hi));
-  const tf sig = tf{y, g.hi, __fmaf_rn(y, cor, g.lo)};
+  const bool capped = q == c.qcap && rho.a < c.rho_cap;
+  const tf sig = capped ? c.cap : tf{y, g.hi, __fmaf_rn(y, cor, g.lo)};
   const tf sg2 = tf_sqr(sig), sg3 = tf_mul(sg2, sig);
   TfRadial R;
   if constexpr (LAPLACE) {

@@ -154,3 +154,11 @@ def test_fp64_symmetric_close_pairs(bipb, gap, kappa):
     """Differences of the coordinates whose leading parts cancel keep FP64's digits in
     the symmetric FP64 mat-vec: components below the leading grid (4e-6 A here)."""
     _check_fp64(bipb, *_mirrored_surface(gap, 40), kappa)
+
+
+@pytest.mark.parametrize("gap,n_pairs", [(3e-7, 6), (9.9e-7, 6), (1e-20, 0)])
+@pytest.mark.parametrize("kappa", [0.0, 0.1257])
+def test_fp64_symmetric_pair_keeps_the_cap_of_the_inverse_distance(bipb, gap, n_pairs, kappa):
+    """1/r is capped at 1e-6 A in the symmetric FP64 mat-vec as in the ordered one, and a
+    pair whose squared distance leaves the FP32 range stays finite."""
+    _check_fp64(bipb, *_mirrored_surface(gap, n_pairs), kappa)
