@@ -96,12 +96,14 @@ __device__ __forceinline__ uint32_t dev_bits(float v) { return __float_as_uint(v
 // Charge records (y - centre, q) of n_rhs configurations from device arrays,
 // with the checks bipb_charges_set makes on the host: every value finite, and
 // no charge on a centroid (the centroid with the same FP32 point, found in the
-// surface's hash table, compared in FP64).  A failed check sets *err.  The
+// surface's hash table, compared in FP64).  A failed check sets bit 0 of *err, a
+// coordinate above `wide` bit 1.  The
 // largest coordinate of a configuration goes into its chg_tab entry.
 __global__ void k_charges_dev(int64_t nc, int n_rhs, int n_pos_sets, const double* __restrict__ pos,
                               const double* __restrict__ q, double cx, double cy, double cz,
                               const int32_t* __restrict__ slot, uint64_t mask, const double4_32a* __restrict__ tgt64,
-                              double4_32a* __restrict__ rec, int4* __restrict__ chg_tab, int* __restrict__ err) {
+                              double4_32a* __restrict__ rec, int4* __restrict__ chg_tab, double wide,
+                              int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nc * n_rhs) return;
   const int64_t r = i / nc, k = i % nc;
@@ -124,7 +126,9 @@ __global__ void k_charges_dev(int64_t nc, int n_rhs, int n_pos_sets, const doubl
     }
   }
   if (!ok) atomicOr(err, 1);
-  const int far = __float_as_int(__double2float_ru(fmax(fabs(p0), fmax(fabs(p1), fabs(p2)))));
+  const double most = fmax(fabs(p0), fmax(fabs(p1), fabs(p2)));
+  if (ok && most > wide) atomicOr(err, 2);
+  const int far = __float_as_int(__double2float_ru(most));
   if (ok && far > chg_tab[r].z) atomicMax(&chg_tab[r].z, far);
   rec[i] = make_double4_32a(p0, p1, p2, qq);
 }
@@ -393,6 +397,9 @@ void store_charges(Surface* s, const std::vector<double4_32a>& rec, const std::v
   s->lay = std::move(lay);
   s->n_rhs = s->lay.K;
   s->have_solution = false;
+  s->chg_check_pending = false;  // of charges passed on the device before these
+  s->chg_wide = false;
+  for (size_t k = 0; k < far.size(); ++k) s->chg_wide |= far[k] > kWideSpread * s->part_far[s->batch ? k : 0];
 }
 
 // Layout of n_vec vectors for the device mat-vec entry point: replicas of a
@@ -417,7 +424,8 @@ void check_device_charges(Surface* s) {
   BIPB_CUDA(cudaMemcpyAsync(&h, s->chg_err.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
   BIPB_CUDA(cudaStreamSynchronize(s->stream));
   s->chg_check_pending = false;
-  if (h) {
+  s->chg_wide = (h & 2) != 0;
+  if (h & 1) {
     s->n_rhs = 0;
     throw Error(BIPB_ERR_INVALID_ARG, "bipb_charges_set_dev: a charge position or value is not finite, or a "
                                       "charge sits on a centroid");
@@ -534,7 +542,7 @@ bipb_status bipb_charges_set_dev(bipb_surface h, int64_t nc, const double* pos, 
     const double* c = &s->part_center[0];
     k_charges_dev<<<(unsigned)((total + 255) / 256), 256, 0, s->stream>>>(
         nc, n_rhs, n_pos_sets, pos, q, c[0], c[1], c[2], s->key_slots.p, keys.mask, s->tgt64.p, s->chg.p,
-        s->chg_tab.p, s->chg_err.p);
+        s->chg_tab.p, kWideSpread * s->part_far[0], s->chg_err.p);
     BIPB_LAUNCHED(s);
     s->nc = nc;
     s->n_pos_sets = n_pos_sets;

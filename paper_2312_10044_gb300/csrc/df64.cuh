@@ -186,15 +186,28 @@ __device__ __forceinline__ df df_norm2(const df* a) {
 struct df_pos {
   float h, l, m;
 };
-// x on the grid g (a power of two): h and l by adding and taking away 1.5 2^52 grid units
+// x on the grid g (a power of two): h and l by adding and taking away 1.5 2^52 grid units;
+// g = 0: in three floats on no grid (WIDE below)
 __device__ __forceinline__ df_pos df_split_grid(double x, double g) {
+  if (g == 0.0) {
+    const float h = __double2float_rn(x);
+    const float l = __double2float_rn(x - (double)h);
+    return df_pos{h, l, __double2float_rn(x - (double)h - (double)l)};
+  }
   const double M = 0x1.8p52 * g, M2 = 0x1.8p28 * g;
   const double h = (x + M) - M;
   const double r = x - h;
   const double l = (r + M2) - M2;
   return df_pos{__double2float_rn(h), __double2float_rn(l), __double2float_rn(r - l)};
 }
+// WIDE: of three floats on no grid, for passes whose points spread further than a
+// grid resolves; every sum recovers its error.
+template <bool WIDE = false>
 __device__ __forceinline__ df df_diff(df_pos x, df_pos y) {
+  if constexpr (WIDE) {
+    const df s = two_sum(x.h, -y.h), t = two_sum(x.l, -y.l), u = two_sum(s.hi, t.hi);
+    return fast_two_sum(u.hi, __fadd_rn(u.lo, __fadd_rn(s.lo, __fadd_rn(t.lo, __fsub_rn(x.m, y.m)))));
+  }
   df d = fast_two_sum(__fsub_rn(x.h, y.h), __fsub_rn(x.l, y.l));
   d.lo = __fadd_rn(d.lo, __fsub_rn(x.m, y.m));
   return d;
@@ -401,8 +414,9 @@ __device__ __forceinline__ void df_sym_pair(const df* d, const df* nt, df at, df
 
 // Source term of one (element, charge) pair in df64: target element (x, n),
 // charge (y, q), d = x - y:  S1 += q s,  S2 += -q (n.d) s^3  (times 4 pi eps_in).
+template <bool WIDE>
 __device__ __forceinline__ void df_source_pair(const df_pos* x, const df* nv, const df_pos* y, df q, df& s1, df& s2) {
-  const df d[3] = {df_diff(x[0], y[0]), df_diff(x[1], y[1]), df_diff(x[2], y[2])};
+  const df d[3] = {df_diff<WIDE>(x[0], y[0]), df_diff<WIDE>(x[1], y[1]), df_diff<WIDE>(x[2], y[2])};
   df s, r;
   df_rsqrt_r(df_norm2(d), s, r);
   const df qs = df_mul(q, s);
@@ -413,9 +427,10 @@ __device__ __forceinline__ void df_source_pair(const df_pos* x, const df* nv, co
 // Reaction potential at a point y from one element (record: x, a = ds psi,
 // normal n, alpha = ds phi), d = y - x (the K1, K2 terms with n_j only):
 //   4 pi phi += s (1 - e) a + s^3 (eps t - 1) alpha (n.d)
+template <bool WIDE>
 __device__ __forceinline__ void df_reaction_pair(const df_pos* y, const df_pos* x, df a, const df* nv, df al,
                                                  const DFConst& c, const df* tab, df& acc) {
-  const df d[3] = {df_diff(y[0], x[0]), df_diff(y[1], x[1]), df_diff(y[2], x[2])};
+  const df d[3] = {df_diff<WIDE>(y[0], x[0]), df_diff<WIDE>(y[1], x[1]), df_diff<WIDE>(y[2], x[2])};
   const DfRadial R = df_radial<false, false>(d, false, c, tab);
   df_mac(acc, df_neg(df_mul(R.e1, R.s)), a);
   df_mac(acc, df_norm(df_mul(df_fma_f(c.eps, R.t, -1.0f), df_cube(R.s))), df_norm(df_mul(al, df_dot(nv, d))));
@@ -425,9 +440,10 @@ __device__ __forceinline__ void df_reaction_pair(const df_pos* y, const df_pos* 
 // reaction pair), d = y - x: the exterior representation (Eq.
 // eqbim_2) with dphi2/dnu = psi / eps (flux continuity), times 4 pi:
 //   4 pi phi += s^3 t alpha (n.d) - s (1/eps) e a   (-Gk dphi2/dnu + dGk/dnu_y phi)
+template <bool WIDE>
 __device__ __forceinline__ void df_exterior_pair(const df_pos* y, const df_pos* x, df a, const df* nv, df al,
                                                  const DFConst& c, const df* tab, df& acc) {
-  const df d[3] = {df_diff(y[0], x[0]), df_diff(y[1], x[1]), df_diff(y[2], x[2])};
+  const df d[3] = {df_diff<WIDE>(y[0], x[0]), df_diff<WIDE>(y[1], x[1]), df_diff<WIDE>(y[2], x[2])};
   const DfRadial R = df_radial<false, false>(d, false, c, tab);
   // every term is proportional to e: t = e (1 + kappa r) relative to its own size
   float th = R.e.hi, tl = R.e.lo;
@@ -439,9 +455,10 @@ __device__ __forceinline__ void df_exterior_pair(const df_pos* y, const df_pos* 
 
 // Energy row of one (element, charge) pair in df64: element j (x, n), charge
 // (y, q), d = y - x (times 4 pi):  cphi += q (eps t - 1)(n.d) s^3,  cpsi += q (1 - e) s.
+template <bool WIDE>
 __device__ __forceinline__ void df_energy_row_pair(const df_pos* x, const df* nv, const df_pos* y, df q, const DFConst& c,
                                                    const df* tab, df& cphi, df& cpsi) {
-  const df d[3] = {df_diff(y[0], x[0]), df_diff(y[1], x[1]), df_diff(y[2], x[2])};
+  const df d[3] = {df_diff<WIDE>(y[0], x[0]), df_diff<WIDE>(y[1], x[1]), df_diff<WIDE>(y[2], x[2])};
   const DfRadial R = df_radial<false, false>(d, false, c, tab);
   const df qs = df_mul(q, R.s);
   df_mac(cphi, df_mul(df_fma_f(c.eps, R.t, -1.0f), df_mul(df_sqr(R.s), qs)), df_dot(nv, d));
@@ -457,9 +474,10 @@ __device__ __forceinline__ void df_energy_row_pair(const df_pos* x, const df* nv
 //   Cd = s^3 [ (t - 1) a - l - cn (3 H s^2 + eps kappa^2 e alpha) ]
 // (the y-gradients of the energy row and of the adjoint-weighted source, with
 // eps w - 3 = 3 (eps t - 1) + eps e kappa^2 r^2).
+template <bool WIDE>
 __device__ __forceinline__ void df_grad_pair(const df_pos* y, const df_pos* x, df a, const df* nv, df al, df l, df beta,
                                              const DFConst& c, const df* tab, df& v, df* g) {
-  const df d[3] = {df_diff(y[0], x[0]), df_diff(y[1], x[1]), df_diff(y[2], x[2])};
+  const df d[3] = {df_diff<WIDE>(y[0], x[0]), df_diff<WIDE>(y[1], x[1]), df_diff<WIDE>(y[2], x[2])};
   const DfRadial R = df_radial<false, false>(d, false, c, tab);
   const df s2 = df_sqr(R.s), s3 = df_mul(s2, R.s);
   const df cn = df_dot(nv, d);

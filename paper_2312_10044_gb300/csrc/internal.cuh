@@ -359,8 +359,9 @@ struct Surface {
   // table on the device for the on-centroid check, and the check's flag,
   // read by the next call that uses the charges
   DevBuf<int32_t> key_slots;
-  DevBuf<int> chg_err;
+  DevBuf<int> chg_err;  // bit 0: a check failed, bit 1: chg_wide
   bool chg_check_pending = false;
+  bool chg_wide = false;  // a charge lies more than kWideSpread times its surface's extent out
   SysLayout lay;   // the systems bipb_solve works on
 
   // surfaces of the handle (one for bipb_surface_create, several for a
@@ -504,6 +505,11 @@ void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const d
 // exterior representation (Eq. eqbim_2).  far_pts: the points' largest coordinate.
 void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
                     int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out);
+// The charge passes keep coordinates on a grid set by the farthest charge or point, which
+// resolves 2^-72 of it: at this many times the surface's largest coordinate still 2^-52 of
+// the surface (df64 values hold 2^-48).  Beyond it, coordinates on no grid and
+// differences of 17 operations in place of 7.
+constexpr double kWideSpread = 0x1p20;
 // FP32 bits of |x| rounded up (ordered like the values)
 inline int far_bits(double x) {
   float f = (float)x;

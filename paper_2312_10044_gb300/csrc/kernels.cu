@@ -97,8 +97,10 @@ struct MatvecPolicy {
 
 // Coordinate grid (df_pos) of system sys of a charge pass: 2^-23 of the power
 // of two above the largest coordinate of its surface, charges and (extra, FP32
-// bits) points.
+// bits) points; 0 (no grid) for extra = kWideCoords.
+constexpr int kWideCoords = 0x7fffffff;
 __device__ __forceinline__ double charge_grid(const int4* __restrict__ chg_tab, int sys, int extra) {
+  if (extra == kWideCoords) return 0.0;
   const int b = max(chg_tab[sys].z, extra);
   return __longlong_as_double((long long)((b >> 23) - 127 + 1 - 23 + 1023) << 52);
 }
@@ -180,6 +182,7 @@ struct MatvecDFPolicy {
 //   4 pi eps_in S1 += q s,   4 pi eps_in S2 += -q (n_i.d) s^3   (d/dnu_x = +n_x.grad_x)
 // GB300 executes FP64 at 1/64 of the FP32 rate; df64 keeps b accurate to
 // about 1e-14 relative at a fraction of the FP64 cost.
+template <bool WIDE>
 struct SourcePolicy {
   static constexpr int RW = 3;
   static constexpr int NOUT = 2;
@@ -209,7 +212,7 @@ struct SourcePolicy {
   __device__ static void pair(const Args&, const Tgt& t, const float4* r, bool, Acc& acc) {
     const float4 A = r[0], B = r[1], C = r[2];
     const df_pos y[3] = {df_pos{A.x, B.x, C.x}, df_pos{A.y, B.y, C.y}, df_pos{A.z, B.z, C.z}};
-    df_source_pair(t.x, t.n, y, df{A.w, B.w}, acc.s1, acc.s2);
+    df_source_pair<WIDE>(t.x, t.n, y, df{A.w, B.w}, acc.s1, acc.s2);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int i, const Acc& acc) {
     a.part[(size_t)out + i] = df_to_double(acc.s1);
@@ -220,6 +223,7 @@ struct SourcePolicy {
 // Reaction potential at a charge y_k from the surface in df64 (df record of
 // k_pack_df<true>: x_j, a_j = ds psi_j, n_j, alpha_j = ds phi_j), d = y_k - x_j:
 //   4 pi phi_reac += s [ (1 - e) a_j + (eps t - 1) alpha_j (n_j.d) s^2 ]  (K1 psi + K2 phi, n_j only)
+template <bool WIDE>
 struct ReactionPolicy {
   static constexpr int RW = 5;
   static constexpr int NOUT = 1;
@@ -250,7 +254,7 @@ struct ReactionPolicy {
     const float4 A = r[0], B = r[1], C = r[2], D = r[3], M = r[4];
     const df_pos xs[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
     const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_reaction_pair(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
+    df_reaction_pair<WIDE>(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
   }
   __device__ static void store(const Args& a, int out, int, int k, const Acc& acc) {
     a.part[(size_t)out + k] = df_to_double(acc.p);
@@ -260,19 +264,23 @@ struct ReactionPolicy {
 // Potential at a point y in the solvent from the surface in df64 (the same
 // df record as the reaction pass), the exterior representation:
 //   4 pi phi(y) += s [ t alpha_j (n_j.d) s^2 - (1/eps) e a_j ],  d = y - x_j
-struct ExteriorPolicy : ReactionPolicy {
+template <bool WIDE>
+struct ExteriorPolicy : ReactionPolicy<WIDE> {
+  using Base = ReactionPolicy<WIDE>;
   template <bool MASK>
-  __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
+  __device__ static void pair(const typename Base::Args& a, const typename Base::Tgt& t, const float4* r, bool,
+                              typename Base::Acc& acc) {
     const float4 A = r[0], B = r[1], C = r[2], D = r[3], M = r[4];
     const df_pos xs[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
     const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_exterior_pair(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
+    df_exterior_pair<WIDE>(t.y, xs, df{A.w, B.w}, nv, df{C.w, D.w}, a.c, df_exp_table(), acc.p);
   }
 };
 
 // Energy row c in df64: target element j, source charge k (df record
 // (y_k, q_k)), d = y_k - x_j:
 //   4 pi K2(y_k, x_j) = (eps t - 1) (n_j.d) s^3,  4 pi K1(y_k, x_j) = (1 - e) s
+template <bool WIDE>
 struct EnergyRowPolicy {
   static constexpr int RW = 3;
   static constexpr int NOUT = 2;
@@ -287,13 +295,14 @@ struct EnergyRowPolicy {
     double* part;
     DFConst c;
     const int4* chg_tab;
+    int extra;  // 0, or kWideCoords
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
   __device__ static void load(const Args& a, int i, int sys, Tgt& t) {
-    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, 0), t);
+    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) { acc.cphi = df{0.f, 0.f}, acc.cpsi = df{0.f, 0.f}; }
   __device__ static void flush(Acc& sum, const Acc& acc) {
@@ -304,7 +313,7 @@ struct EnergyRowPolicy {
   __device__ static void pair(const Args& a, const Tgt& t, const float4* r, bool, Acc& acc) {
     const float4 A = r[0], B = r[1], C = r[2];
     const df_pos y[3] = {df_pos{A.x, B.x, C.x}, df_pos{A.y, B.y, C.y}, df_pos{A.z, B.z, C.z}};
-    df_energy_row_pair(t.x, t.n, y, df{A.w, B.w}, a.c, df_exp_table(), acc.cphi, acc.cpsi);
+    df_energy_row_pair<WIDE>(t.x, t.n, y, df{A.w, B.w}, a.c, df_exp_table(), acc.cphi, acc.cpsi);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int i, const Acc& acc) {
     a.part[(size_t)out + i] = df_to_double(acc.cphi);
@@ -317,6 +326,7 @@ struct EnergyRowPolicy {
 // (n.lo, alpha.lo), (l.hi, l.lo, beta.hi, beta.lo), (x.m, 0) with a = ds psi, alpha =
 // ds phi and the adjoint lam / eps_in = [l; beta].  Outputs per charge: v
 // (dE/dq up to 1/2 and 1/(4 pi)) and the three components of the gradient g.
+template <bool WIDE>
 struct GradPolicy {
   static constexpr int RW = 6;
   static constexpr int NOUT = 4;
@@ -331,13 +341,14 @@ struct GradPolicy {
     double* part;
     DFConst c;
     const int4* chg_tab;
+    int extra;  // 0, or kWideCoords
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
   __device__ static void load(const Args& a, int k, int sys, Tgt& t) {
-    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, 0), t);
+    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) {
     acc.v = df{0.f, 0.f};
@@ -352,7 +363,7 @@ struct GradPolicy {
     const float4 A = r[0], B = r[1], C = r[2], D = r[3], E = r[4], M = r[5];
     const df_pos x[3] = {df_pos{A.x, B.x, M.x}, df_pos{A.y, B.y, M.y}, df_pos{A.z, B.z, M.z}};
     const df nv[3] = {df{C.x, D.x}, df{C.y, D.y}, df{C.z, D.z}};
-    df_grad_pair(t.y, x, df{A.w, B.w}, nv, df{C.w, D.w}, df{E.x, E.y}, df{E.z, E.w}, a.c, df_exp_table(), acc.v,
+    df_grad_pair<WIDE>(t.y, x, df{A.w, B.w}, nv, df{C.w, D.w}, df{E.x, E.y}, df{E.z, E.w}, a.c, df_exp_table(), acc.v,
                  acc.g);
   }
   __device__ static void store(const Args& a, int out, int n_tgt, int k, const Acc& acc) {
@@ -795,7 +806,8 @@ __global__ void k_energy_row_reduce(const int4* __restrict__ lay, const int4* __
 // vec_off / 2): pack_elem_df's and (l, beta) = inv_eps_in (lphi, lpsi).
 __global__ void k_pack_grad(const int4* __restrict__ lay, const int4* __restrict__ chg_tab,
                             const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
-                            const double* __restrict__ lam, double inv_eps_in, float4* __restrict__ rec) {
+                            const double* __restrict__ lam, double inv_eps_in, int extra,
+                            float4* __restrict__ rec) {
   const int k = blockIdx.y;
   const int4 L = lay[k];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -804,7 +816,7 @@ __global__ void k_pack_grad(const int4* __restrict__ lay, const int4* __restrict
   const double* lk = lam + L.z;
   const df l = df_from_double(inv_eps_in * lk[j]), beta = df_from_double(inv_eps_in * lk[L.y + j]);
   float4* o = rec + 6 * (size_t)(L.z / 2 + j);
-  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, 0), o, 5);
+  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, extra), o, 5);
   o[4] = make_float4(l.hi, l.lo, beta.hi, beta.lo);
 }
 
@@ -1133,7 +1145,9 @@ __global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const
   o[2] = make_float4(x.m, y.m, z.m, 0.f);
 }
 
-void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b) {
+template <bool WIDE>
+static void source_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, double* b) {
+  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   int n_chg = 0;
@@ -1141,40 +1155,56 @@ void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b
     sys[k] = PassSys{L.geo_off[k], L.n[k], L.chg_off[k], L.nc[k]};
     n_chg = std::max(n_chg, L.chg_off[k] + L.nc[k]);
   }
-  ItemPlan* plan = plan_pass<SourcePolicy, float4, NT, TPT, CH>(s, kPassSource, sys, CH);
+  ItemPlan* plan = plan_pass<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kPassSource, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  SourcePolicy::Args a{s->tgt64.p, s->part64.p, s->chg_tab.p, 0};
-  launch_items<SourcePolicy, float4, NT, TPT, CH>(s, kTSource, plan, a, s->chgdf.p, nullptr, 0);
+  typename SourcePolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, s->chg_tab.p, extra};
+  launch_items<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kTSource, plan, a, s->chgdf.p, nullptr, 0);
   k_reduce_source<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, kInv4Pi / m.eps_in, b);
   BIPB_LAUNCHED(s);
 }
+void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b) {
+  if (s->chg_wide)
+    source_pass_of<true>(s, L, m, b);
+  else
+    source_pass_of<false>(s, L, m, b);
+}
 
-void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, double* phi_reac,
-                   double* e_out) {
+template <bool WIDE>
+static void reaction_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u,
+                             double* phi_reac, double* e_out) {
+  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
-  ItemPlan* plan = plan_pass<ReactionPolicy, float4, NT, TPT, CH>(s, kPassReaction, sys, CH);
+  ItemPlan* plan = plan_pass<ReactionPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassReaction, sys, CH);
   s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, 0, s->tgt64.p, u,
+  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
                                                                              s->recdf.p);
   BIPB_LAUNCHED(s);
-  ReactionPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, 0};
-  launch_items<ReactionPolicy, float4, NT, TPT, CH>(s, kTReaction, plan, a, s->recdf.p, nullptr, 0);
+  typename ReactionPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  launch_items<ReactionPolicy<WIDE>, float4, NT, TPT, CH>(s, kTReaction, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_reaction<<<kReacClu * L.K, 32 * kReacWarps, 0, s->stream>>>(plan->tab.p, lay, s->part64.p, s->chg.p, phi_reac, e_out);
   BIPB_LAUNCHED(s);
 }
+void reaction_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, double* phi_reac,
+                   double* e_out) {
+  if (s->chg_wide)
+    reaction_pass_of<true>(s, L, m, u, phi_reac, e_out);
+  else
+    reaction_pass_of<false>(s, L, m, u, phi_reac, e_out);
+}
 
-void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
-                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out) {
+template <bool WIDE>
+static void potential_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
+                              int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out) {
   constexpr int NT = 128, TPT = 1, CH = 64;
-  const int extra = far_bits(far_pts);
+  const int extra = WIDE ? kWideCoords : far_bits(far_pts);
   // surface integral: targets are the points (shared by every system), sources the elements
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{0, n_pts, L.vec_off[k] / 2, L.n[k]};
@@ -1183,18 +1213,18 @@ void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const 
   k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
                                                                              s->recdf.p);
   BIPB_LAUNCHED(s);
-  ReactionPolicy::Args a{pts, nullptr, df_const_impl(s, m), s->chg_tab.p, extra};
+  typename ReactionPolicy<WIDE>::Args a{pts, nullptr, df_const_impl(s, m), s->chg_tab.p, extra};
   ItemPlan* plan;
   if (inside) {
-    plan = plan_pass<ReactionPolicy, float4, NT, TPT, CH>(s, kPassPotIn, sys, CH);
+    plan = plan_pass<ReactionPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassPotIn, sys, CH);
     s->grow(s->part64, (size_t)plan->part_len);
     a.part = s->part64.p;
-    launch_items<ReactionPolicy, float4, NT, TPT, CH>(s, kTPotential, plan, a, s->recdf.p, nullptr, 0);
+    launch_items<ReactionPolicy<WIDE>, float4, NT, TPT, CH>(s, kTPotential, plan, a, s->recdf.p, nullptr, 0);
   } else {
-    plan = plan_pass<ExteriorPolicy, float4, NT, TPT, CH>(s, kPassPotOut, sys, CH);
+    plan = plan_pass<ExteriorPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassPotOut, sys, CH);
     s->grow(s->part64, (size_t)plan->part_len);
     a.part = s->part64.p;
-    launch_items<ExteriorPolicy, float4, NT, TPT, CH>(s, kTPotential, plan, a, s->recdf.p, nullptr, 0);
+    launch_items<ExteriorPolicy<WIDE>, float4, NT, TPT, CH>(s, kTPotential, plan, a, s->recdf.p, nullptr, 0);
   }
   k_reduce_points<<<dim3(blocks_for(n_pts, 256), L.K), 256, 0, s->stream>>>(plan->tab.p, s->part64.p, n_pts, 1,
                                                                            kInv4Pi, 0, out);
@@ -1207,16 +1237,23 @@ void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const 
     n_chg = std::max(n_chg, L.chg_off[k] + L.nc[k]);
   }
   if (n_chg == 0) return;
-  ItemPlan* sp = plan_pass<SourcePolicy, float4, NT, TPT, CH>(s, kPassPotSrc, sys, CH);
+  ItemPlan* sp = plan_pass<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kPassPotSrc, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)sp->part_len);
   k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  SourcePolicy::Args b{pts2, s->part64.p, s->chg_tab.p, extra};
-  launch_items<SourcePolicy, float4, NT, TPT, CH>(s, kTPotential, sp, b, s->chgdf.p, nullptr, 0);
+  typename SourcePolicy<WIDE>::Args b{pts2, s->part64.p, s->chg_tab.p, extra};
+  launch_items<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kTPotential, sp, b, s->chgdf.p, nullptr, 0);
   k_reduce_points<<<dim3(blocks_for(n_pts, 256), L.K), 256, 0, s->stream>>>(sp->tab.p, s->part64.p, n_pts, 2,
                                                                            kInv4Pi / m.eps_in, 1, out);
   BIPB_LAUNCHED(s);
+}
+void potential_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
+                    int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out) {
+  if (far_pts > kWideSpread * s->part_far[0] || s->chg_wide)
+    potential_pass_of<true>(s, L, m, u, inside, n_pts, pts, pts2, far_pts, out);
+  else
+    potential_pass_of<false>(s, L, m, u, inside, n_pts, pts, pts2, far_pts, out);
 }
 
 void coulomb_pass(Surface* s, const SysLayout& L, const int4* tab, double* part, int* blocks) {
@@ -1227,7 +1264,9 @@ void coulomb_pass(Surface* s, const SysLayout& L, const int4* tab, double* part,
   BIPB_LAUNCHED(s);
 }
 
-void energy_row_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* c) {
+template <bool WIDE>
+static void energy_row_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, double* c) {
+  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   int n_chg = 0;
@@ -1235,35 +1274,50 @@ void energy_row_pass(Surface* s, const SysLayout& L, const bipb_medium& m, doubl
     sys[k] = PassSys{L.geo_off[k], L.n[k], L.chg_off[k], L.nc[k]};
     n_chg = std::max(n_chg, L.chg_off[k] + L.nc[k]);
   }
-  ItemPlan* plan = plan_pass<EnergyRowPolicy, float4, NT, TPT, CH>(s, kPassRow, sys, CH);
+  ItemPlan* plan = plan_pass<EnergyRowPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassRow, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  EnergyRowPolicy::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
-  launch_items<EnergyRowPolicy, float4, NT, TPT, CH>(s, kTRow, plan, a, s->chgdf.p, nullptr, 0);
+  typename EnergyRowPolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  launch_items<EnergyRowPolicy<WIDE>, float4, NT, TPT, CH>(s, kTRow, plan, a, s->chgdf.p, nullptr, 0);
   k_energy_row_reduce<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, s->tgt64.p, c);
   BIPB_LAUNCHED(s);
 }
+void energy_row_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* c) {
+  if (s->chg_wide)
+    energy_row_pass_of<true>(s, L, m, c);
+  else
+    energy_row_pass_of<false>(s, L, m, c);
+}
 
-void grad_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, const double* lam, double* dq,
-               double* dy) {
+template <bool WIDE>
+static void grad_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, const double* lam,
+                         double* dq, double* dy) {
+  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 32;
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
-  ItemPlan* plan = plan_pass<GradPolicy, float4, NT, TPT, CH>(s, kPassGrad, sys, CH);
+  ItemPlan* plan = plan_pass<GradPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassGrad, sys, CH);
   s->grow(s->recdf, (size_t)3 * L.len);  // 6 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
   k_pack_grad<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, s->tgt64.p, u, lam,
-                                                                            1.0 / m.eps_in, s->recdf.p);
+                                                                            1.0 / m.eps_in, extra, s->recdf.p);
   BIPB_LAUNCHED(s);
-  GradPolicy::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
-  launch_items<GradPolicy, float4, NT, TPT, CH>(s, kTGrad, plan, a, s->recdf.p, nullptr, 0);
+  typename GradPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  launch_items<GradPolicy<WIDE>, float4, NT, TPT, CH>(s, kTGrad, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_grad<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(plan->tab.p, lay, s->part64.p,
                                                                               s->chg.p, dq, dy);
   BIPB_LAUNCHED(s);
+}
+void grad_pass(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, const double* lam, double* dq,
+               double* dy) {
+  if (s->chg_wide)
+    grad_pass_of<true>(s, L, m, u, lam, dq, dy);
+  else
+    grad_pass_of<false>(s, L, m, u, lam, dq, dy);
 }
 
 }  // namespace bipb
