@@ -684,7 +684,8 @@ __global__ void k_reduce_matvec(const int4* __restrict__ lay, const int4* __rest
     const int e = i < n ? i : i - n;
     double sc = kInv4Pi;
     if (tgt64_for_area) sc *= tgt64_for_area[2 * (L.x + e)].w;
-    y[L.z + i] = d * u[L.z + i] - sc * acc[q].value();
+    const double total = left_range(acc[q]) ? sum_strided_fp64(p + q, (size_t)2 * n, T.y) : acc[q].value();
+    y[L.z + i] = d * u[L.z + i] - sc * total;
   }
 }
 

@@ -29,6 +29,16 @@ struct PartSum<float> {
   // of an infinite sum the TwoSum errors are NaN and the leading part is the sum
   __device__ __forceinline__ double value() const { return lo == lo ? (double)hi + (double)lo : (double)hi; }
 };
+// A sum of FP32 values may leave their range although each of them is in it: the sum is
+// then taken again in FP64 (also of infinities and NaN).
+__device__ __forceinline__ bool left_range(const PartSum<double>&) { return false; }
+__device__ __forceinline__ bool left_range(const PartSum<float>& p) { return !(fabsf(p.hi) <= 3.402823466e38f); }
+template <typename PT>
+__device__ __noinline__ double sum_strided_fp64(const PT* __restrict__ p, size_t stride, int count) {
+  double t = 0.0;
+  for (int k = 0; k < count; ++k) t += (double)p[(size_t)k * stride];
+  return t;
+}
 
 // Sum of count values stride apart, in order, U loads in flight at a time: the last
 // batch is filled up with zeros, where a loop unrolled by U would leave up to U - 1
@@ -45,6 +55,18 @@ __device__ __forceinline__ PartSum<PT> sum_strided(const PT* __restrict__ p, siz
     for (int q = 0; q < U; ++q) acc.add(v[q]);
   }
   return acc;
+}
+
+// sym_sum in FP64
+template <typename PT>
+__device__ __noinline__ double sym_sum_fp64(const int4* __restrict__ tab, const int4 S, const PT* __restrict__ part,
+                                            int e, int c) {
+  const int n = S.x, T = S.w, E = e / T;
+  const int4 R = tab[S.y + E];
+  double t = sum_strided_fp64(part + (size_t)R.x + (size_t)c * T + (e - E * T), (size_t)2 * T, R.y);
+  for (int I = 0; I <= E; ++I)
+    t += (double)part[(int64_t)S.z + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2) + (e - I * T) + c * (n - I * T)];
+  return t;
 }
 
 // Sum of component c (0: phi, 1: psi) of one element of a system over a
@@ -70,6 +92,7 @@ __device__ __forceinline__ double sym_sum(const int4* __restrict__ tab, const in
 #pragma unroll
     for (int q = 0; q < U; ++q) p.add(v[q]);
   }
+  if (left_range(p)) return sym_sum_fp64(tab, S, part, e, c);
   return p.value();
 }
 

@@ -383,7 +383,9 @@ __global__ void k_tree_reduce(int n, const int* __restrict__ perm, const int* __
   const int e = perm[t];
   const bool tr = area_of != nullptr;
   const double w = tr ? area_of[2 * (L.x + e)].w : 1.0;
-  const double v1 = w * f1 * s1.value(), v3 = w * f3 * s3.value();
+  const double t1 = left_range(s1) ? sum_strided_fp64(o, (size_t)2 * lmax, lf.w) : s1.value(),
+               t3 = left_range(s3) ? sum_strided_fp64(o + lmax, (size_t)2 * lmax, lf.w) : s3.value();
+  const double v1 = w * f1 * t1, v3 = w * f3 * t3;
   y[L.z + e] = dphi * u[L.z + e] - (tr ? v3 : v1);
   y[L.z + L.y + e] = dpsi * u[L.z + L.y + e] - (tr ? v1 : v3);
 }
