@@ -186,19 +186,21 @@ __device__ __forceinline__ df df_norm2(const df* a) {
 struct df_pos {
   float h, l, m;
 };
-// x on the grid g (a power of two): h and l by adding and taking away 1.5 2^52 grid units;
-// g = 0: in three floats on no grid (WIDE below)
+// x on the grid g (a power of two): h and l by adding and taking away 1.5 2^52 grid units
+// (of a product x the compiler's multiply-adds take the unrounded one: no branch on g here)
 __device__ __forceinline__ df_pos df_split_grid(double x, double g) {
-  if (g == 0.0) {
-    const float h = __double2float_rn(x);
-    const float l = __double2float_rn(x - (double)h);
-    return df_pos{h, l, __double2float_rn(x - (double)h - (double)l)};
-  }
   const double M = 0x1.8p52 * g, M2 = 0x1.8p28 * g;
   const double h = (x + M) - M;
   const double r = x - h;
   const double l = (r + M2) - M2;
   return df_pos{__double2float_rn(h), __double2float_rn(l), __double2float_rn(r - l)};
+}
+// x on the grid g, or for g = 0 in three floats on no grid (WIDE below)
+__device__ __forceinline__ df_pos df_split_point(double x, double g) {
+  if (g != 0.0) return df_split_grid(x, g);
+  const float h = __double2float_rn(x);
+  const float l = __double2float_rn(x - (double)h);
+  return df_pos{h, l, __double2float_rn(x - (double)h - (double)l)};
 }
 // WIDE: of three floats on no grid, for passes whose points spread further than a
 // grid resolves; every sum recovers its error.

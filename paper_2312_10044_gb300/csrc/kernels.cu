@@ -111,7 +111,7 @@ struct ElemTgtDF {
 };
 __device__ __forceinline__ void load_elem_df(const double4_32a* __restrict__ tgt, int i, double grid, ElemTgtDF& t) {
   const double4_32a g = tgt[2 * i], v = tgt[2 * i + 1];
-  t.x[0] = df_split_grid(g.x, grid), t.x[1] = df_split_grid(g.y, grid), t.x[2] = df_split_grid(g.z, grid);
+  t.x[0] = df_split_point(g.x, grid), t.x[1] = df_split_point(g.y, grid), t.x[2] = df_split_point(g.z, grid);
   t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
 }
 struct PointTgtDF {
@@ -119,7 +119,7 @@ struct PointTgtDF {
 };
 __device__ __forceinline__ void load_point_df(const double4_32a* __restrict__ pts, int k, double grid, PointTgtDF& t) {
   const double4_32a g = pts[k];
-  t.y[0] = df_split_grid(g.x, grid), t.y[1] = df_split_grid(g.y, grid), t.y[2] = df_split_grid(g.z, grid);
+  t.y[0] = df_split_point(g.x, grid), t.y[1] = df_split_point(g.y, grid), t.y[2] = df_split_point(g.z, grid);
 }
 
 // Mat-vec in double-float arithmetic (df64.cuh).  Record per source, 4 float4:
@@ -626,7 +626,7 @@ __global__ void k_pack_df(const int4* __restrict__ lay, bool transpose, const do
 // (x.m, 0) with a = ds psi, alpha = ds phi, x on the pass's grid.
 __device__ __forceinline__ void pack_elem_df(const double4_32a& g, const double4_32a& v, double phi, double psi,
                                              double grid, float4* o, int last) {
-  const df_pos x0 = df_split_grid(g.x, grid), x1 = df_split_grid(g.y, grid), x2 = df_split_grid(g.z, grid);
+  const df_pos x0 = df_split_point(g.x, grid), x1 = df_split_point(g.y, grid), x2 = df_split_point(g.z, grid);
   const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
   const df a = df_from_double(g.w * psi), al = df_from_double(g.w * phi);
   o[0] = make_float4(x0.h, x1.h, x2.h, a.hi);
@@ -1138,7 +1138,7 @@ __global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const
   if (c >= T.y) return;
   const double4_32a g = chg[T.x + c];
   const double grid = charge_grid(chg_tab, blockIdx.y, extra);
-  const df_pos x = df_split_grid(g.x, grid), y = df_split_grid(g.y, grid), z = df_split_grid(g.z, grid);
+  const df_pos x = df_split_point(g.x, grid), y = df_split_point(g.y, grid), z = df_split_point(g.z, grid);
   const df q = df_from_double(g.w);
   float4* o = rec + 3 * (size_t)(T.x + c);
   o[0] = make_float4(x.h, y.h, z.h, q.hi);
