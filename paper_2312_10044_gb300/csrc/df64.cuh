@@ -219,7 +219,7 @@ constexpr int kExpTab = 1024;  // entries of the exp table, 2^(j/1024) for j < 1
 
 struct DFConst {
   df eps, inveps, kappa;  // eps_out/eps_in, its inverse, kappa
-  float l1, l2;           // ln2/1024 = l1 + l2, l1 rounded to FP32
+  float l1, l2, l3;       // ln2/1024 = l1 + l2 + l3, l1 and l1 + l2 rounded to their digits
   float inv_l;            // 1024/ln2
   const float4* tab;      // device copy of the exp table, two df64 entries per float4
 };
@@ -244,15 +244,27 @@ __device__ __forceinline__ void df_rsqrt_r(df r2, df& s, df& r) {
   r = df{t, __fmaf_rn(t, g, tl)};
 }
 
-// exp(-x) for x >= 0 (x.hi clamped at 80), tab[j] = 2^(j/1024) as df64.
+// exp(-x) for x >= 0 (x.hi clamped at 80), tab[j] = 2^(j/1024) as df64.  The absolute error
+// is below 2^-47; relative to the value it grows as the square of the reduction's
+// trailing part (2e-13 at x = 8, 2e-12 at 32).  REL: the reduction in double-float with
+// L in three parts, 1e-14 of the value at any x (15 more operations), for sums in which
+// every term is proportional to it.
+template <bool REL = false>
 __device__ __forceinline__ df df_exp_minus(df x, const DFConst& c, const df* tab) {
   const float xh = fmaxf(-x.hi, -80.0f);
   // k = rint(x / L): adding 1.5 * 2^23 leaves the integer in the low mantissa bits
   const float km = __fmaf_rn(xh, c.inv_l, 12582912.0f);
   const int k = __float_as_int(km) - 0x4B400000;
   const float kf = __fsub_rn(km, 12582912.0f);
-  const float f = __fmaf_rn(-kf, c.l1, xh);       // exact
-  const float fl = __fmaf_rn(-kf, c.l2, -x.lo);
+  float f = __fmaf_rn(-kf, c.l1, xh);       // exact
+  float fl;
+  if constexpr (REL) {
+    const df p = two_prod(kf, c.l2), a = two_sum(-x.lo, -p.hi), g = two_sum(f, a.hi);
+    f = g.hi;
+    fl = __fadd_rn(g.lo, __fmaf_rn(-kf, c.l3, __fsub_rn(a.lo, p.lo)));
+  } else {
+    fl = __fmaf_rn(-kf, c.l2, -x.lo);
+  }
   // exp(f + fl) = 1 + f + q, q = f^2/2 + f^3/6 + fl (1 + f)
   const float q = __fmaf_rn(__fmul_rn(f, f), __fmaf_rn(f, 1.0f / 6.0f, 0.5f), __fmaf_rn(f, fl, fl));
   df ef = fast_two_sum(1.0f, f);  // |f| < 1
@@ -268,7 +280,7 @@ __device__ __forceinline__ df df_exp_minus(df x, const DFConst& c, const df* tab
 struct DfRadial {
   df s, kr, e, e1, t1, t;
 };
-template <bool MASK, bool SCALED>
+template <bool MASK, bool SCALED, bool REL = false>
 __device__ __forceinline__ DfRadial df_radial(const df* d, bool self, const DFConst& c, const df* tab) {
   DfRadial R;
   df r2 = df_norm2(d), r;
@@ -276,7 +288,7 @@ __device__ __forceinline__ DfRadial df_radial(const df* d, bool self, const DFCo
   df_rsqrt_r(r2, R.s, r);
   if (MASK && self) R.s = df{0.0f, 0.0f};
   R.kr = SCALED ? r : df_mul(r, c.kappa);
-  R.e = df_exp_minus(R.kr, c, tab);
+  R.e = df_exp_minus<REL>(R.kr, c, tab);
   const df o = fast_two_sum(-1.0f, R.e.hi);
   R.e1 = df{o.hi, __fadd_rn(o.lo, R.e.lo)};
   const df p = df_mul(R.e, R.kr);
@@ -446,12 +458,13 @@ template <bool WIDE>
 __device__ __forceinline__ void df_exterior_pair(const df_pos* y, const df_pos* x, df a, const df* nv, df al,
                                                  const DFConst& c, const df* tab, df& acc) {
   const df d[3] = {df_diff<WIDE>(y[0], x[0]), df_diff<WIDE>(y[1], x[1]), df_diff<WIDE>(y[2], x[2])};
-  const DfRadial R = df_radial<false, false>(d, false, c, tab);
-  // every term is proportional to e: t = e (1 + kappa r) relative to its own size
+  const DfRadial R = df_radial<false, false, true>(d, false, c, tab);
+  // every term is proportional to e: t = e (1 + kappa r) relative to its own size, and
+  // no product smaller than the term (they come near the end of the FP32 range)
   float th = R.e.hi, tl = R.e.lo;
   prod_sum_pos(th, tl, R.e.hi, R.kr.hi);
   const df t = df{th, __fmaf_rn(R.e.hi, R.kr.lo, __fmaf_rn(R.e.lo, R.kr.hi, tl))};
-  df_mac(acc, df_mul(t, df_cube(R.s)), df_mul(al, df_dot(nv, d)));
+  df_mac(acc, df_mul(t, R.s), df_mul(df_sqr(R.s), df_mul(al, df_dot(nv, d))));
   df_mac(acc, df_neg(df_mul(df_mul(c.inveps, R.e), R.s)), a);
 }
 

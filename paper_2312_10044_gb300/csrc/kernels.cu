@@ -870,6 +870,7 @@ DFConst df_const_impl(const Surface* s, const bipb_medium& m) {
   const double L = 0.693147180559945309417232121458 / kExpTab;
   c.l1 = (float)L;
   c.l2 = (float)(L - (double)c.l1);
+  c.l3 = (float)(L - (double)c.l1 - (double)c.l2);
   c.inv_l = (float)(kExpTab / 0.693147180559945309417232121458);
   c.tab = s->exptab.p;
   return c;

@@ -114,3 +114,29 @@ def test_gradient_beside_a_far_charge(bipb, far):
             got.append((np.ravel(s.energy())[0], np.ravel(dq)[keep], np.reshape(dy, (p.nc, 3))[keep]))
     for a, b in zip(*got):
         np.testing.assert_allclose(b, a, rtol=0, atol=1e-9 * np.abs(a).max())
+
+
+@pytest.mark.parametrize("x", [4.0, 8.0, 16.0, 32.0, 60.0])
+def test_exterior_potential_keeps_its_digits_where_it_is_screened(bipb, orc, x):
+    """Potentials at points x Debye lengths out are of the order of e^{-x}: right
+    relative to their own terms.  Bound: kappa r to a few 2^-48 of itself makes e^{-kappa r}
+    wrong by x times that; over 1280 elements its random part averages out to less than
+    x 2^-48, and 2e-14 for the other factors, both relative to the sum of the terms'
+    magnitudes."""
+    p = synth.kirkwood_problem(level=3)
+    rng = np.random.default_rng(1)
+    d = rng.standard_normal((200, 3))
+    pts = d / np.linalg.norm(d, axis=1, keepdims=True) * (x / p.kappa)
+    eps = p.eps_out / p.eps_in
+    with bipb.Surface(p.centroids, p.normals, p.areas) as s:
+        s.set_charges(p.charge_pos, p.q)
+        s.solve(eps_in=p.eps_in, eps_out=p.eps_out, kappa=p.kappa, tol=1e-12, precision=bipb.FP64)
+        phi, dphi = s.surface_potential()
+        u = np.concatenate([np.ravel(phi), np.ravel(dphi)]) / orc.KCAL
+        got = np.ravel(s.potential_at(pts, inside=False)) / orc.KCAL
+    ref = np.ravel(orc.potential(p.centroids, p.normals, p.areas, eps, p.kappa, u, pts, False))
+    r = np.linalg.norm(pts[:, None] - p.centroids[None], axis=2)
+    e = np.exp(-p.kappa * r)
+    size = ((e * (1.0 + p.kappa * r) / r**2) @ (p.areas * np.abs(u[:p.n])) + (e / r) @ (p.areas * np.abs(u[p.n:])) / eps) / (4.0 * np.pi)
+    worst = np.max(np.abs(got - ref) / size)
+    assert worst < x * 2.0**-48 + 2e-14, worst
