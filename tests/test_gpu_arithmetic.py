@@ -246,3 +246,23 @@ def test_reaction_reduction_tiles(bipb, orc, nc):
         np.testing.assert_allclose(pr[k], pr_ref, rtol=0, atol=1e-12 * np.abs(pr_ref).max())
         scale = 0.5 * orc.KCAL * np.abs(f * q).sum() * np.abs(pr_ref).max()
         assert abs(e[k] - orc.KCAL * f * e_ref) < 1e-12 * scale
+
+
+@pytest.mark.parametrize("n", [5120, 5121])
+@pytest.mark.parametrize("precision", ["FP64", "MIXED_TENSOR"])
+def test_krylov_step_without_fused_matvec_at_its_line(bipb, orc, n, precision):
+    """The Arnoldi step beside a mat-vec that is not fused into it (two Gram-Schmidt
+    passes for FP64, one for the tensor-core operator), as one cluster launch up to 5120
+    elements and as kernels above: energies against the oracle's solve, with the bounds
+    of test_krylov_step_as_cluster_and_as_kernels."""
+    p = synth.protein_like_problem(level=5, n_charges=3)
+    keep = np.sort(np.random.default_rng(n).choice(p.n, n, replace=False))
+    p.centroids, p.normals, p.areas = p.centroids[keep], p.normals[keep], p.areas[keep]
+    ref = orc.solve(p, rhs=0, method="gmres", tol=1e-12).energy_kcal
+    tol, rt = (1e-11, 1e-9) if precision == "FP64" else (1e-9, 1e-7)
+    with bipb.Surface(p.centroids, p.normals, p.areas) as s:
+        s.set_charges(p.charge_pos, p.q)
+        info = s.solve(eps_in=p.eps_in, eps_out=p.eps_out, kappa=p.kappa, tol=tol, precision=getattr(bipb, precision),
+                       precond=1)
+        assert all(i["converged"] for i in info)
+        np.testing.assert_allclose(s.energy()[0], ref, rtol=rt)
