@@ -49,12 +49,14 @@ L2_FLUSH_BYTES = 512 << 20  # > 129 MB L2
 # the pair of Eqs. 5-6 written out term by term (d, r^2, r, s^2 and s^3, the
 # exponent argument, c_i, c_j, c_ij, t and w, K1..K4, four accumulations) is
 # about 43 FP32-pipe instructions, about 20 of them FMAs, i.e. 63 flops,
-# plus 2 MUFU operations.  The kernels execute fewer (the symmetric kernel
-# about 23 FP32-pipe instructions per ordered pair, since it evaluates each
-# unordered pair once for both rows), so achieved / peak can exceed the pipe's
-# busy fraction; the ncu FMA-pipe fraction is reported beside it.
+# plus 2 MUFU operations.  The kernels execute fewer, so achieved / peak in
+# these flops can exceed the pipe's busy fraction; the ncu FMA-pipe fraction is
+# reported beside it.
 PAIR_FLOPS = 63
-PAIR_PIPE_INSTR = 43
+# FP32-pipe operations that the FP32 kernels execute per ordered pair: the
+# symmetric variants (7 on) 43 per unordered pair for both rows, 22 of them
+# multiply-adds; the folded ordered formula 39.
+PAIR_PIPE_INSTR = {"symmetric": 21.5, "ordered": 39.0}
 # Measured FP32 FFMA throughput (bench.py --mode peaks, the microbenchmark
 # microbench/alu_peaks.cu): 3.65e13 lane-ops/s on 152 SMs at a median SM clock
 # of 1987 MHz, i.e. 120.9 FMA lanes per SM per clock of the nominal 128.  The
@@ -711,9 +713,10 @@ def config4a_solves(bipb, torch):
 
 
 def run_peaks(args):
-    """Measured throughput of the FP32 FFMA, FP64 DFMA and MUFU pipes (the
-    microbenchmark microbench/alu_peaks.cu, built here with nvcc), against the
-    nominal unit counts at the SM clock sampled meanwhile."""
+    """Measured throughput of the FP32 FFMA, FP64 DFMA and MUFU pipes and of FFMA and
+    FADD with operands of their own, scalar and packed (the microbenchmark
+    microbench/alu_peaks.cu, built here with nvcc), against the nominal unit counts at
+    the SM clock sampled meanwhile."""
     here = os.path.dirname(os.path.abspath(__file__))
     src = os.path.join(here, "paper_2312_10044_gb300", "microbench", "alu_peaks.cu")
     exe = os.path.join(here, "_build", "alu_peaks")
@@ -729,7 +732,8 @@ def run_peaks(args):
     sms = int(vals["sms"])
     f = (clk["sm_mhz"] if clk else 2070.0) * 1e6
     res = {"mode": "peaks", "sms": sms, "clocks": clk}
-    for name, lanes in (("ffma", FP32_LANES_PER_SM), ("dfma", FP64_LANES_PER_SM), ("mufu", 16)):
+    f32 = [(k, FP32_LANES_PER_SM) for k in ("ffma", "ffma3", "ffma2", "fadd", "fadd2")]
+    for name, lanes in f32 + [("dfma", FP64_LANES_PER_SM), ("mufu", 16)]:
         v = float(vals[f"{name}_per_s"])
         nominal = sms * lanes * f
         res[f"{name}_per_s"] = v
@@ -840,7 +844,11 @@ def main():
     achieved = pairs_launch * PAIR_FLOPS / (avg_ms / 1e3) / 1e12
     peak = nsm * lanes_meas * 2 * f_mhz * 1e6 / 1e12
     peak_nominal = nsm * lanes * 2 * f_mhz * 1e6 / 1e12
-    instr_frac = pairs_launch * PAIR_PIPE_INSTR / (avg_ms / 1e3) / (nsm * lanes_meas * f_mhz * 1e6)
+    pair_instr = None
+    if dom == "matvec32":
+        pair_instr = PAIR_PIPE_INSTR["symmetric" if variant >= 7 else "ordered"]
+    instr_frac = None if pair_instr is None else \
+        pairs_launch * pair_instr / (avg_ms / 1e3) / (nsm * lanes_meas * f_mhz * 1e6)
     traffic = None
     if dom == "matvec32" and args.workload == "kirkwood":
         traffic = DRAM_BYTES_FP32_KIRKWOOD.get(variant)
@@ -857,8 +865,8 @@ def main():
                               "it executes fewer instructions than the algorithmic count and frac can exceed 1",
                 "peak_nominal": peak_nominal, "frac_of_nominal": achieved / peak_nominal,
                 "instr_frac": instr_frac,
-                "instr_note": f"{PAIR_PIPE_INSTR} FP32-pipe instructions per ordered pair over the measured issue "
-                              "peak (can exceed 1 for the same reason)",
+                "instr_note": f"{pair_instr} FP32-pipe instructions executed per ordered pair over the measured "
+                              "FFMA issue peak (a multiply-add with three register operands takes 1.5 issue slots)",
                 "ncu_fma_pipe_frac": ncu_pipe,
                 "ncu_note": "FMA-pipe busy fraction of this kernel from one ncu capture "
                             "(profiles/kernels_current_build.md): how busy the pipe actually is",

@@ -34,8 +34,9 @@ struct PartSum<float> {
 __device__ __forceinline__ bool left_range(const PartSum<double>&) { return false; }
 __device__ __forceinline__ bool left_range(const PartSum<float>& p) { return !(fabsf(p.hi) <= 3.402823466e38f); }
 template <typename PT>
-__device__ __noinline__ double sum_strided_fp64(const PT* __restrict__ p, size_t stride, int count) {
+__device__ __forceinline__ double sum_strided_fp64(const PT* __restrict__ p, size_t stride, int count) {
   double t = 0.0;
+#pragma unroll 1
   for (int k = 0; k < count; ++k) t += (double)p[(size_t)k * stride];
   return t;
 }
@@ -64,6 +65,7 @@ __device__ __noinline__ double sym_sum_fp64(const int4* __restrict__ tab, const 
   const int n = S.x, T = S.w, E = e / T;
   const int4 R = tab[S.y + E];
   double t = sum_strided_fp64(part + (size_t)R.x + (size_t)c * T + (e - E * T), (size_t)2 * T, R.y);
+#pragma unroll 1
   for (int I = 0; I <= E; ++I)
     t += (double)part[(int64_t)S.z + 2 * ((int64_t)I * n - (int64_t)T * I * (I - 1) / 2) + (e - I * T) + c * (n - I * T)];
   return t;
