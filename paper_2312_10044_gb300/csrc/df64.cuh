@@ -195,9 +195,10 @@ __device__ __forceinline__ df_pos df_split_grid(double x, double g) {
   const double l = (r + M2) - M2;
   return df_pos{__double2float_rn(h), __double2float_rn(l), __double2float_rn(r - l)};
 }
-// x on the grid g, or for g = 0 in three floats on no grid (WIDE below)
+// x on the grid g, or in three floats on no grid (WIDE, below)
+template <bool WIDE>
 __device__ __forceinline__ df_pos df_split_point(double x, double g) {
-  if (g != 0.0) return df_split_grid(x, g);
+  if constexpr (!WIDE) return df_split_grid(x, g);
   const float h = __double2float_rn(x);
   const float l = __double2float_rn(x - (double)h);
   return df_pos{h, l, __double2float_rn(x - (double)h - (double)l)};

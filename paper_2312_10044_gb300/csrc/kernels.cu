@@ -97,10 +97,8 @@ struct MatvecPolicy {
 
 // Coordinate grid (df_pos) of system sys of a charge pass: 2^-23 of the power
 // of two above the largest coordinate of its surface, charges and (extra, FP32
-// bits) points; 0 (no grid) for extra = kWideCoords.
-constexpr int kWideCoords = 0x7fffffff;
+// bits) points.
 __device__ __forceinline__ double charge_grid(const int4* __restrict__ chg_tab, int sys, int extra) {
-  if (extra == kWideCoords) return 0.0;
   const int b = max(chg_tab[sys].z, extra);
   return __longlong_as_double((long long)((b >> 23) - 127 + 1 - 23 + 1023) << 52);
 }
@@ -109,17 +107,19 @@ struct ElemTgtDF {
   df_pos x[3];
   df n[3];
 };
+template <bool WIDE>
 __device__ __forceinline__ void load_elem_df(const double4_32a* __restrict__ tgt, int i, double grid, ElemTgtDF& t) {
   const double4_32a g = tgt[2 * i], v = tgt[2 * i + 1];
-  t.x[0] = df_split_point(g.x, grid), t.x[1] = df_split_point(g.y, grid), t.x[2] = df_split_point(g.z, grid);
+  t.x[0] = df_split_point<WIDE>(g.x, grid), t.x[1] = df_split_point<WIDE>(g.y, grid), t.x[2] = df_split_point<WIDE>(g.z, grid);
   t.n[0] = df_from_double(v.x), t.n[1] = df_from_double(v.y), t.n[2] = df_from_double(v.z);
 }
 struct PointTgtDF {
   df_pos y[3];
 };
+template <bool WIDE>
 __device__ __forceinline__ void load_point_df(const double4_32a* __restrict__ pts, int k, double grid, PointTgtDF& t) {
   const double4_32a g = pts[k];
-  t.y[0] = df_split_point(g.x, grid), t.y[1] = df_split_point(g.y, grid), t.y[2] = df_split_point(g.z, grid);
+  t.y[0] = df_split_point<WIDE>(g.x, grid), t.y[1] = df_split_point<WIDE>(g.y, grid), t.y[2] = df_split_point<WIDE>(g.z, grid);
 }
 
 // Mat-vec in double-float arithmetic (df64.cuh).  Record per source, 4 float4:
@@ -201,7 +201,7 @@ struct SourcePolicy {
     int extra;  // FP32 bits of the largest coordinate of the targets, 0 for the surface's own elements
   };
   __device__ static void load(const Args& a, int i, int sys, Tgt& t) {
-    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, a.extra), t);
+    load_elem_df<WIDE>(a.tgt, i, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) { acc.s1 = df{0.f, 0.f}, acc.s2 = df{0.f, 0.f}; }
   __device__ static void flush(Acc& sum, const Acc& acc) {
@@ -245,7 +245,7 @@ struct ReactionPolicy {
     df_load_exp_table(df_exp_table(), a.c);
   }
   __device__ static void load(const Args& a, int k, int sys, Tgt& t) {
-    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, a.extra), t);
+    load_point_df<WIDE>(a.pts, k, charge_grid(a.chg_tab, sys, a.extra), t);
   }
   __device__ static void zero(Acc& acc) { acc.p = df{0.f, 0.f}; }
   __device__ static void flush(Acc& sum, const Acc& acc) { sum.p = df_add(sum.p, acc.p); }
@@ -295,14 +295,13 @@ struct EnergyRowPolicy {
     double* part;
     DFConst c;
     const int4* chg_tab;
-    int extra;  // 0, or kWideCoords
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
   __device__ static void load(const Args& a, int i, int sys, Tgt& t) {
-    load_elem_df(a.tgt, i, charge_grid(a.chg_tab, sys, a.extra), t);
+    load_elem_df<WIDE>(a.tgt, i, charge_grid(a.chg_tab, sys, 0), t);
   }
   __device__ static void zero(Acc& acc) { acc.cphi = df{0.f, 0.f}, acc.cpsi = df{0.f, 0.f}; }
   __device__ static void flush(Acc& sum, const Acc& acc) {
@@ -341,14 +340,13 @@ struct GradPolicy {
     double* part;
     DFConst c;
     const int4* chg_tab;
-    int extra;  // 0, or kWideCoords
   };
   template <class A>
   __device__ static void prologue(const A& a) {
     df_load_exp_table(df_exp_table(), a.c);
   }
   __device__ static void load(const Args& a, int k, int sys, Tgt& t) {
-    load_point_df(a.pts, k, charge_grid(a.chg_tab, sys, a.extra), t);
+    load_point_df<WIDE>(a.pts, k, charge_grid(a.chg_tab, sys, 0), t);
   }
   __device__ static void zero(Acc& acc) {
     acc.v = df{0.f, 0.f};
@@ -624,9 +622,10 @@ __global__ void k_pack_df(const int4* __restrict__ lay, bool transpose, const do
 // The first 4 float4 and the last one of an element's record in the charge
 // passes: (x.h, a.hi), (x.l, a.lo), (n.hi, alpha.hi), (n.lo, alpha.lo), ..,
 // (x.m, 0) with a = ds psi, alpha = ds phi, x on the pass's grid.
+template <bool WIDE>
 __device__ __forceinline__ void pack_elem_df(const double4_32a& g, const double4_32a& v, double phi, double psi,
                                              double grid, float4* o, int last) {
-  const df_pos x0 = df_split_point(g.x, grid), x1 = df_split_point(g.y, grid), x2 = df_split_point(g.z, grid);
+  const df_pos x0 = df_split_point<WIDE>(g.x, grid), x1 = df_split_point<WIDE>(g.y, grid), x2 = df_split_point<WIDE>(g.z, grid);
   const df n0 = df_from_double(v.x), n1 = df_from_double(v.y), n2 = df_from_double(v.z);
   const df a = df_from_double(g.w * psi), al = df_from_double(g.w * phi);
   o[0] = make_float4(x0.h, x1.h, x2.h, a.hi);
@@ -636,6 +635,7 @@ __device__ __forceinline__ void pack_elem_df(const double4_32a& g, const double4
   o[last] = make_float4(x0.m, x1.m, x2.m, 0.f);
 }
 // Records of the reaction pass (5 float4 per element, at vec_off / 2).
+template <bool WIDE>
 __global__ void k_pack_react(const int4* __restrict__ lay, const int4* __restrict__ chg_tab, int extra,
                              const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
                              float4* __restrict__ rec) {
@@ -644,7 +644,7 @@ __global__ void k_pack_react(const int4* __restrict__ lay, const int4* __restric
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= L.y) return;
   const double* uk = u + L.z;
-  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, extra),
+  pack_elem_df<WIDE>(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, extra),
                rec + 5 * (size_t)(L.z / 2 + j), 4);
 }
 
@@ -805,10 +805,10 @@ __global__ void k_energy_row_reduce(const int4* __restrict__ lay, const int4* __
 
 // Gradient records of every system in df64 (6 float4 per element, at
 // vec_off / 2): pack_elem_df's and (l, beta) = inv_eps_in (lphi, lpsi).
+template <bool WIDE>
 __global__ void k_pack_grad(const int4* __restrict__ lay, const int4* __restrict__ chg_tab,
                             const double4_32a* __restrict__ tgt64, const double* __restrict__ u,
-                            const double* __restrict__ lam, double inv_eps_in, int extra,
-                            float4* __restrict__ rec) {
+                            const double* __restrict__ lam, double inv_eps_in, float4* __restrict__ rec) {
   const int k = blockIdx.y;
   const int4 L = lay[k];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -817,7 +817,7 @@ __global__ void k_pack_grad(const int4* __restrict__ lay, const int4* __restrict
   const double* lk = lam + L.z;
   const df l = df_from_double(inv_eps_in * lk[j]), beta = df_from_double(inv_eps_in * lk[L.y + j]);
   float4* o = rec + 6 * (size_t)(L.z / 2 + j);
-  pack_elem_df(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, extra), o, 5);
+  pack_elem_df<WIDE>(tgt64[2 * (L.x + j)], tgt64[2 * (L.x + j) + 1], uk[j], uk[L.y + j], charge_grid(chg_tab, k, 0), o, 5);
   o[4] = make_float4(l.hi, l.lo, beta.hi, beta.lo);
 }
 
@@ -1132,6 +1132,7 @@ int autotune_matvec32(Surface* s, const SysLayout& L, const bipb_medium& m, int 
 }
 
 // df64 records of every charge: (y.h, q.hi), (y.l, q.lo), (y.m, 0), on the grid of its system's pass
+template <bool WIDE>
 __global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const double4_32a* __restrict__ chg,
                               float4* __restrict__ rec) {
   const int4 T = chg_tab[blockIdx.y];
@@ -1139,7 +1140,7 @@ __global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const
   if (c >= T.y) return;
   const double4_32a g = chg[T.x + c];
   const double grid = charge_grid(chg_tab, blockIdx.y, extra);
-  const df_pos x = df_split_point(g.x, grid), y = df_split_point(g.y, grid), z = df_split_point(g.z, grid);
+  const df_pos x = df_split_point<WIDE>(g.x, grid), y = df_split_point<WIDE>(g.y, grid), z = df_split_point<WIDE>(g.z, grid);
   const df q = df_from_double(g.w);
   float4* o = rec + 3 * (size_t)(T.x + c);
   o[0] = make_float4(x.h, y.h, z.h, q.hi);
@@ -1149,7 +1150,6 @@ __global__ void k_pack_chg_df(const int4* __restrict__ chg_tab, int extra, const
 
 template <bool WIDE>
 static void source_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, double* b) {
-  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   int n_chg = 0;
@@ -1160,9 +1160,9 @@ static void source_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m,
   ItemPlan* plan = plan_pass<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kPassSource, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<WIDE><<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  typename SourcePolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, s->chg_tab.p, extra};
+  typename SourcePolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, s->chg_tab.p, 0};
   launch_items<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kTSource, plan, a, s->chgdf.p, nullptr, 0);
   k_reduce_source<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, kInv4Pi / m.eps_in, b);
@@ -1178,7 +1178,6 @@ void source_pass(Surface* s, const SysLayout& L, const bipb_medium& m, double* b
 template <bool WIDE>
 static void reaction_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u,
                              double* phi_reac, double* e_out) {
-  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
@@ -1186,10 +1185,10 @@ static void reaction_pass_of(Surface* s, const SysLayout& L, const bipb_medium& 
   s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
+  k_pack_react<WIDE><<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, 0, s->tgt64.p, u,
                                                                              s->recdf.p);
   BIPB_LAUNCHED(s);
-  typename ReactionPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  typename ReactionPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, 0};
   launch_items<ReactionPolicy<WIDE>, float4, NT, TPT, CH>(s, kTReaction, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_reaction<<<kReacClu * L.K, 32 * kReacWarps, 0, s->stream>>>(plan->tab.p, lay, s->part64.p, s->chg.p, phi_reac, e_out);
   BIPB_LAUNCHED(s);
@@ -1206,13 +1205,13 @@ template <bool WIDE>
 static void potential_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, bool inside,
                               int n_pts, const double4_32a* pts, const double4_32a* pts2, double far_pts, double* out) {
   constexpr int NT = 128, TPT = 1, CH = 64;
-  const int extra = WIDE ? kWideCoords : far_bits(far_pts);
+  const int extra = far_bits(far_pts);
   // surface integral: targets are the points (shared by every system), sources the elements
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{0, n_pts, L.vec_off[k] / 2, L.n[k]};
   s->grow(s->recdf, (size_t)5 * L.len / 2);  // 5 float4 per element
   const int4* lay = s->lay_dev(L);
-  k_pack_react<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
+  k_pack_react<WIDE><<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, extra, s->tgt64.p, u,
                                                                              s->recdf.p);
   BIPB_LAUNCHED(s);
   typename ReactionPolicy<WIDE>::Args a{pts, nullptr, df_const_impl(s, m), s->chg_tab.p, extra};
@@ -1242,7 +1241,7 @@ static void potential_pass_of(Surface* s, const SysLayout& L, const bipb_medium&
   ItemPlan* sp = plan_pass<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kPassPotSrc, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)sp->part_len);
-  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<WIDE><<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
   typename SourcePolicy<WIDE>::Args b{pts2, s->part64.p, s->chg_tab.p, extra};
   launch_items<SourcePolicy<WIDE>, float4, NT, TPT, CH>(s, kTPotential, sp, b, s->chgdf.p, nullptr, 0);
@@ -1268,7 +1267,6 @@ void coulomb_pass(Surface* s, const SysLayout& L, const int4* tab, double* part,
 
 template <bool WIDE>
 static void energy_row_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, double* c) {
-  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 64;
   std::vector<PassSys> sys(L.K);
   int n_chg = 0;
@@ -1279,9 +1277,9 @@ static void energy_row_pass_of(Surface* s, const SysLayout& L, const bipb_medium
   ItemPlan* plan = plan_pass<EnergyRowPolicy<WIDE>, float4, NT, TPT, CH>(s, kPassRow, sys, CH);
   s->grow(s->chgdf, (size_t)3 * n_chg);
   s->grow(s->part64, (size_t)plan->part_len);
-  k_pack_chg_df<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, extra, s->chg.p, s->chgdf.p);
+  k_pack_chg_df<WIDE><<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(s->chg_tab.p, 0, s->chg.p, s->chgdf.p);
   BIPB_LAUNCHED(s);
-  typename EnergyRowPolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  typename EnergyRowPolicy<WIDE>::Args a{s->tgt64.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
   launch_items<EnergyRowPolicy<WIDE>, float4, NT, TPT, CH>(s, kTRow, plan, a, s->chgdf.p, nullptr, 0);
   k_energy_row_reduce<<<dim3(blocks_for(2 * L.max_n, 256), L.K), 256, 0, s->stream>>>(
       s->lay_dev(L), plan->tab.p, s->part64.p, s->tgt64.p, c);
@@ -1297,7 +1295,6 @@ void energy_row_pass(Surface* s, const SysLayout& L, const bipb_medium& m, doubl
 template <bool WIDE>
 static void grad_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, const double* u, const double* lam,
                          double* dq, double* dy) {
-  const int extra = WIDE ? kWideCoords : 0;
   constexpr int NT = 128, TPT = 1, CH = 32;
   std::vector<PassSys> sys(L.K);
   for (int k = 0; k < L.K; ++k) sys[k] = PassSys{L.chg_off[k], L.nc[k], L.vec_off[k] / 2, L.n[k]};
@@ -1305,10 +1302,10 @@ static void grad_pass_of(Surface* s, const SysLayout& L, const bipb_medium& m, c
   s->grow(s->recdf, (size_t)3 * L.len);  // 6 float4 per element
   s->grow(s->part64, (size_t)plan->part_len);
   const int4* lay = s->lay_dev(L);
-  k_pack_grad<<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, s->tgt64.p, u, lam,
-                                                                            1.0 / m.eps_in, extra, s->recdf.p);
+  k_pack_grad<WIDE><<<dim3(blocks_for(L.max_n, 256), L.K), 256, 0, s->stream>>>(lay, s->chg_tab.p, s->tgt64.p, u, lam,
+                                                                            1.0 / m.eps_in, s->recdf.p);
   BIPB_LAUNCHED(s);
-  typename GradPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p, extra};
+  typename GradPolicy<WIDE>::Args a{s->chg.p, s->part64.p, df_const_impl(s, m), s->chg_tab.p};
   launch_items<GradPolicy<WIDE>, float4, NT, TPT, CH>(s, kTGrad, plan, a, s->recdf.p, nullptr, 0);
   k_reduce_grad<<<dim3(blocks_for(L.max_nc, 256), L.K), 256, 0, s->stream>>>(plan->tab.p, lay, s->part64.p,
                                                                               s->chg.p, dq, dy);
