@@ -1,7 +1,9 @@
 // Packed FP32 pairs: two FP32 values in one 64-bit register and the packed
 // add / mul / fma of sm_100 and later (PTX .f32x2).  One instruction gives two
-// results at the FMA pipe's usual rate per result (measured on GB300: about
-// 120 FMAs per SM per clock either way), so a kernel bound by instruction
+// results at the scalar operation's rate per result (measured on GB300,
+// microbench/alu_peaks.cu: an fma whose three register operands are its own takes
+// 1.5 cycles of a scheduler, the packed one three for its two results, an add or
+// mul one a result), so a kernel bound by instruction
 // issue rather than by the FMA pipe runs two independent evaluations in the
 // issue slots of one.  Rounding is that of the scalar operation (.rn), and
 // an fma is a fused multiply-add exactly as fmaf.

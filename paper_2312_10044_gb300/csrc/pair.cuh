@@ -24,8 +24,9 @@
 // own targets, so the common path carries no mask).  Every other factor is
 // finite there, so both sums receive an exact zero.  Padding records carry
 // zero values and m = 0 at a far-away position, and also add exact zeros.
-// 1/r is clamped to S_MAX so that absurd inputs (distinct centroids closer
-// than 1e-6 A) stay finite; such inputs are rejected at surface creation.
+// 1/r is clamped to its value at 1e-6 A in every FP32 and FP64 pair, so that closer
+// centroids stay finite (surface creation refuses those whose FP32 copies coincide);
+// the df64 pairs (df64.cuh) have no clamp.
 #pragma once
 #include <cuda_runtime.h>
 

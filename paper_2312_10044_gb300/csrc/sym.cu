@@ -24,7 +24,8 @@
 //           numbered consecutively, in source order);
 //   j side: for row I, 2 x (n - I T) values (every element j >= I T).
 // The reduction adds, for element e of tile E, the i-side blocks of row E and
-// the j-side values of rows 0..E, in that fixed order, in FP64.
+// the j-side values of rows 0..E, in that fixed order: FP64 partials in FP64, FP32
+// ones by TwoSums (PartSum, symstep.cuh).
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -139,10 +140,10 @@ struct Sym64Policy {
 
 // FP32, two targets per pack.  What bounds it: the FP32 pipe's register ports.  An
 // FFMA with three register operands takes 1.5 issue cycles (FFMA2 three for two
-// results; measured), FADD and FMUL one, so a pair of 24 FFMA and 23 others
-// takes 59 cycles of a scheduler however it is issued, and the scalar form
+// results; microbench/alu_peaks.cu), FADD and FMUL one, so a pair of 22 FFMA and 21
+// others takes 54 cycles of a scheduler however it is issued, and the scalar form
 // waited for its loads, shuffles and MUFU calls on top (64.5).  Packed, they
-// hide behind it: N = 20480 0.387 -> 0.351 ms, N = 65537 3.43 -> 3.15 ms a
+// hide behind it: N = 20480 0.387 -> 0.350 ms, N = 65537 3.43 -> 3.15 ms a
 // mat-vec (59.7 cycles a pair).  Record, 5 float4, every value twice: (x, x, y, y),
 // (z, z, a, a), (nx, nx, ny, ny), (nz, nz, -alpha, -alpha), (f, f, 0, 0) with f
 // = -a (A u) or alpha (A^T w): packed FP32 has no negated operands, so every

@@ -85,8 +85,11 @@ __global__ void k_tree_pack(int n, int rec_stride, bool transpose, double sigma,
 // Partial proxy weights of one piece of a far cluster: for proxy q = (q0, q1, q2),
 //   upart[.][q] = sum over the piece's elements of l_q0(x) l_q1(y) l_q2(z) (a, m),
 // with l_i the barycentric Lagrange basis at the cluster's Chebyshev nodes
-// (weights (-1)^i, halved at both ends).  An element on a node takes the
-// node's basis value 1 exactly.
+// (weights (-1)^i, halved at both ends).  An element whose FP32 record is on a node
+// takes the node's basis value 1 exactly; in kappa-scaled units node and element are
+// rounded apart, and one on a node may come out an ulp beside it (its basis value then
+// differs from 1 by that ulp's share of the node spacing: the error of the
+// mat-vec is the same with nodes scaled in FP64).
 //
 // Bound by the FP32 pipe: thread (g, q0, q1) of G groups adds every G-th
 // element of a chunk to its column of DEG + 1 proxies, one multiplication and
