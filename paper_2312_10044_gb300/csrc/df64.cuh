@@ -32,7 +32,7 @@
 // unrounded product (prod_sum below: no separate TwoProduct and TwoSum), and
 // renormalising FastTwoSums are left out wherever the trailing part is taken
 // by an FP32 multiply-add anyway.  FP32 operations of one unordered pair of the
-// symmetric mat-vec: 21 differences, 20 r2, 13 1/r and r, 18 exp, 21 the
+// symmetric mat-vec: 21 differences, 20 r2, 13 1/r and r, 18 exp, 24 the
 // radial factors, 56 the dots n.d, 18 n_i.n_j, 94 coefficients, 96 the eight
 // accumulations; N = 20480, kappa = 0.1257: 3.03 -> 2.60 ms, error against
 // 64 bits 1.5e-14 -> 1.5e-15 (the second-order 1/sqrt of before was its
@@ -277,7 +277,10 @@ __device__ __forceinline__ df df_exp_minus(df x, const DFConst& c, const df* tab
 // The radial factors of a pair from d (kappa-scaled when SCALED: kappa r = r
 // then), with x = kappa r: s = 1/r, e = exp(-x), e1 = e - 1, t = e (1 + x) and
 // t1 = t - 1.  e1 + e x = t1 is ordered (1 - e >= e x), as is 1 + t1, so
-// neither needs a TwoSum.  self (MASK): s = 0, every other factor finite.
+// neither needs a TwoSum.  t1 is normalised: for small x it is x^2 / 2 beside a trailing
+// part of e's size (2^-25), and every product below would round that anew (K4, which has s^3,
+// was off by 1.4e-14 s^3 below x = 0.3 where 2e-15 s^3 is e's rounding).
+// self (MASK): s = 0, every other factor finite.
 struct DfRadial {
   df s, kr, e, e1, t1, t;
 };
@@ -294,9 +297,10 @@ __device__ __forceinline__ DfRadial df_radial(const df* d, bool self, const DFCo
   R.e1 = df{o.hi, __fadd_rn(o.lo, R.e.lo)};
   const df p = df_mul(R.e, R.kr);
   const df v = fast_two_sum(R.e1.hi, p.hi);
-  R.t1 = df{v.hi, __fadd_rn(v.lo, __fadd_rn(R.e1.lo, p.lo))};
-  const df u = fast_two_sum(1.0f, R.t1.hi);
-  R.t = df{u.hi, __fadd_rn(u.lo, R.t1.lo)};
+  const float vl = __fadd_rn(v.lo, __fadd_rn(R.e1.lo, p.lo));
+  R.t1 = fast_two_sum(v.hi, vl);  // exact enough below |vl| too: its error is 2^-24 of vl
+  const df u = fast_two_sum(1.0f, v.hi);
+  R.t = df{u.hi, __fadd_rn(u.lo, vl)};
   return R;
 }
 

@@ -162,3 +162,35 @@ def test_fp64_symmetric_pair_keeps_the_cap_of_the_inverse_distance(bipb, gap, n_
     """1/r is capped at 1e-6 A in the symmetric FP64 mat-vec as in the ordered one, and a
     pair whose squared distance leaves the FP32 range stays finite."""
     _check_fp64(bipb, *_mirrored_surface(gap, n_pairs), kappa)
+
+
+@pytest.mark.parametrize("n_rhs", [1, 5])
+@pytest.mark.parametrize("kappa", [1e-8, 1e-5])
+@pytest.mark.parametrize("gap", [0.05, 1e-3])
+def test_double_float_t_minus_one_of_close_elements(bipb, gap, kappa, n_rhs):
+    """K4 of close elements is s^3 (1 - t) with 1 - t far below e's rounding: its error
+    stays that of e, also where nothing else is as large (no dielectric contrast, hardly
+    any screening).  Bound per row: e = 1 - kappa r is held to 2^-50 (kappa r below 2^-24
+    lies in its trailing part, rounded at 2^-24 of that), 2^-49 s^3 ds |phi| in the psi row and
+    2^-48 (s + s^2) ds |u| for K1 to K3 (A^T likewise), and 2^-44 of the row's terms."""
+    c, nv, a = _paired_sphere(20.0, gap, False)
+    n = len(a)
+    U = np.random.default_rng(n_rhs).standard_normal((n_rhs, 2 * n))
+    x0 = c - c.mean(axis=0)
+    with np.errstate(divide="ignore"):
+        s = 1.0 / np.linalg.norm(x0[:, None] - x0[None], axis=2)
+    np.fill_diagonal(s, 0.0)
+    with bipb.Surface(c, nv, a) as srf:
+        for transpose in (False, True) if n_rhs == 1 else (False,):
+            Y = torch.full_like(_dev(U), float("nan"))
+            srf.matvec(_dev(U), Y, precision=bipb.DF64, transpose=transpose, med=bipb.medium(1.0, 1.0, kappa))
+            Y = Y.cpu().numpy()
+            w = (a[:, None] if transpose else a[None, :]) / (4.0 * np.pi)
+            for k in (0, n_rhs - 1):
+                phi, psi = np.abs(U[k, :n]), np.abs(U[k, n:])
+                ref, tol = _capped_matvec(x0, nv, a, 1.0, kappa, U[k], transpose)
+                e1 = 2.0**-48 * (((s + s**2) * w) @ (phi + psi))
+                e4 = 2.0**-49 * ((s**3 * w) @ (psi if transpose else phi))
+                tol = 2.0**-44 * 1e12 * tol + np.concatenate([e1 + e4, e1] if transpose else [e1, e1 + e4])
+                worst = np.max(np.abs(Y[k] - ref) / tol)
+                assert worst < 1.0, (transpose, k, worst)
