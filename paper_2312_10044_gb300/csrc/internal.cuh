@@ -460,7 +460,13 @@ struct SymStep {
   double dphi = 0.0, dpsi = 0.0;  // the diagonal
   bool transpose = false;
 };
-constexpr double kSymKappaMin = 1e-6;  // smallest kappa (1/A) of the kappa-scaled FP32 and FP64 pairs
+constexpr double kSymKappaMin = 1e-6;  // smallest kappa (1/A) of the kappa-scaled symmetric pairs
+// The same of the far-field and the multi-RHS df64 passes (a Debye length of 1000 A): their
+// sums come out divided by kappa^2 and their s^3 multiplied by 1 / kappa^3, in FP32.
+// Below it they are unscaled, as they were for every kappa (a few operations a pair
+// more): at 1e-6 values above 1e25 would leave the range, and a padding record at a
+// target's own position, where s is at its cap, would with eps above 340.
+constexpr double kScaledKappaMin = 1e-3;
 enum { kSymPack = 1, kSymPairs = 2, kSymReduce = 4, kSymAll = 7 };
 // y = A u (or A^T u) by the handle's FP32 variant if it is a symmetric one that
 // takes this layout and medium (false otherwise, nothing launched); stages is

@@ -776,15 +776,15 @@ ItemPlan* tcx_plan(Surface* s, int n, int* S_out) {
   return it->second.get();
 }
 
-// The kappa-scaled form of the multi-RHS df64 passes (kappa >= 1e-6 / A, the
-// rule of the single-system pass): sigma = kappa, else 1.
+// The kappa-scaled form of the multi-RHS df64 passes (kappa >= kScaledKappaMin):
+// sigma = kappa, else 1.
 struct MrhsScale {
   bool scaled;
   double sigma, gscale;
 };
 MrhsScale mrhs_scale(const DFConst& c) {
   const double kappa = (double)c.kappa.hi + (double)c.kappa.lo;
-  if (kappa < 1e-6) return MrhsScale{false, 1.0, 1.0};
+  if (kappa < kScaledKappaMin) return MrhsScale{false, 1.0, 1.0};
   return MrhsScale{true, kappa, std::exp2(std::ceil(std::log2(kappa)))};
 }
 

@@ -232,10 +232,10 @@ __global__ void k_tree_proxy(int n_slots, const int2* __restrict__ up_tab, const
 // (d changes its sign against pair_transpose, hence E and F).  The formulas
 // are placed so that no packed operand needs a negation (two logical
 // operations each).  FORM:
-//   kScaled (kappa >= 1e-6): positions and m times sigma = kappa, where kappa r
+//   kScaled (kappa >= kScaledKappaMin): positions and m times sigma = kappa, where kappa r
 //     = r2 s, (1 - e) s = (1 - t) s + e and (w - 3) s^2 = 3 (t - 1) s^2 + e;
 //     the sums take factors of kappa (S1) and kappa^2 (S3);
-//   kPlain (0 < kappa < 1e-6, whose scaled coordinates would overflow): sigma = 1;
+//   kPlain (0 < kappa below that): sigma = 1;
 //   kLaplace (kappa = 0): e = t = 1, w = 3, only E and F remain.
 enum TreeForm { kScaled, kPlain, kLaplace };
 struct TreeConst {
@@ -669,7 +669,7 @@ void matvec_tree(Surface* s, const SysLayout& L, const PairConst<float>& c0, dou
   if (f->upart.ensure(std::max<size_t>(1, 4 * (size_t)P * f->n_up * K), s->stream)) ++s->alloc_gen;
   const int4* lay = s->lay_dev(L);
   const int nb = (f->n + 255) / 256;
-  const TreeForm form = kappa == 0.0 ? kLaplace : kappa < kSymKappaMin ? kPlain : kScaled;
+  const TreeForm form = kappa == 0.0 ? kLaplace : kappa < kScaledKappaMin ? kPlain : kScaled;
   const double sigma = form == kScaled ? kappa : 1.0;
   const float sg = (float)sigma;
   TreeConst c;

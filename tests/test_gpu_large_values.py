@@ -47,3 +47,37 @@ def test_symmetric_sums_above_the_fp32_range(bipb, n, kappa):
         s.matvec(_dev(u * f), y, precision=bipb.FP32, med=med)
         y2 = y.cpu().numpy() / f
     np.testing.assert_allclose(y2, y1, rtol=0, atol=3e-6 * np.abs(y1).max())
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e25])
+@pytest.mark.parametrize("kappa", [1e-6, 1.1e-6, 1e-4, 9.99e-4, 1.001e-3])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_weak_screening_keeps_the_range(bipb, transpose, kappa, scale):
+    """The far-field and the multi-RHS double-float passes with Debye lengths of 1000 to
+    10^6 A, a contrast of 1000 and values up to 1e25, on both sides of the line of their
+    scaled form (1e-3): the bounds of test_treecode_matvec_matches_oracle_treecode and
+    test_multi_rhs_df64_matvec_matches_oracle."""
+    import oracle as orc
+
+    p = synth.protein_like_problem(level=3, n_charges=3)
+    keep = np.sort(np.random.default_rng(3).choice(p.n, 515, replace=False))
+    c, nv, a = p.centroids[keep], p.normals[keep], p.areas[keep]
+    n, eps = len(a), 1000.0
+    med = bipb.medium(1.0, eps, kappa)
+    U = scale * np.random.default_rng(5).standard_normal((17, 2 * n))
+    f = orc.matvec_t if transpose else orc.matvec
+    with bipb.Surface(c, nv, a) as s:
+        s.treecode(0.8, 4, 33)
+        y = torch.full_like(_dev(U[0]), float("nan"))
+        s.matvec(_dev(U[0]), y, precision=bipb.TREE32, transpose=transpose, med=med)
+        y = y.cpu().numpy()
+        ref = orc.treecode.matvec(c, nv, a, eps, kappa, U[0], 0.8, 4, 33, transpose=transpose)
+        assert np.linalg.norm((y - ref) / scale) < 3e-6 * np.linalg.norm(ref / scale)
+        assert np.abs(y - ref).max() < 2e-5 * np.abs(ref).max()
+        for k in (4, 17):
+            Y = torch.full_like(_dev(U[:k]), float("nan"))
+            s.matvec(_dev(U[:k]), Y, precision=bipb.DF64, transpose=transpose, med=med)
+            Y = Y.cpu().numpy()
+            for r in (0, k - 1):
+                ref = f(c, nv, a, eps, kappa, U[r])
+                np.testing.assert_allclose(Y[r], ref, rtol=0, atol=2e-12 * np.abs(ref).max())
