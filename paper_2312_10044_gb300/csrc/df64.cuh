@@ -33,8 +33,8 @@
 // renormalising FastTwoSums are left out wherever the trailing part is taken
 // by an FP32 multiply-add anyway.  FP32 operations of one unordered pair of the
 // symmetric mat-vec: 21 differences, 20 r2, 13 1/r and r, 18 exp, 24 the
-// radial factors, 56 the dots n.d, 18 n_i.n_j, 94 coefficients, 96 the eight
-// accumulations; N = 20480, kappa = 0.1257: 3.03 -> 2.60 ms, error against
+// radial factors, 56 the dots n.d, 18 n_i.n_j, 91 coefficients, 96 the eight
+// accumulations; N = 20480, kappa = 0.1257: 3.03 -> 2.59 ms, error against
 // 64 bits 1.5e-14 -> 1.5e-15 (the second-order 1/sqrt of before was its
 // largest part).  Reaction and source passes, 40961 elements x 4 x 2000
 // charges: 4.11 -> 3.40 ms.
@@ -409,7 +409,9 @@ __device__ __forceinline__ void df_sym_pair(const df* d, const df* nt, df at, df
   const df U = df_det(R.t1, cij, df_wm3s2<SCALED>(R, s2, c), df_mul(ci, cj));
   // s and s^3 folded into the four coefficients every update uses
   const df ome_s = df_neg(df_mul(R.e1, R.s)), U_s3 = df_mul(U, s3);
-  const df et1_s3 = df_mul(df_fma_f(c.eps, R.t, -1.0f), s3), te1_s3 = df_mul(df_fma_f(R.t, c.inveps, -1.0f), s3);
+  // t/eps - 1 left unnormalised: its trailing part is at most a few 2^-24, and the leading one is
+  // of the order of 1 unless eps is close to 1 (360 -> 357 operations)
+  const df et1_s3 = df_mul(df_fma_f(c.eps, R.t, -1.0f), s3), te1_s3 = df_mul(df_fma_lazy(R.t, c.inveps, -1.0f), s3);
   if (!TRANS) {
     df_mac(Pt, ome_s, as);
     df_mac(Pt, df_mul(et1_s3, cj), als);
